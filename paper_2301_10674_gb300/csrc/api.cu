@@ -17,7 +17,6 @@ void mlp_frag_host(const MlpBf16& h, const __nv_bfloat16* w1m, MlpFrag& G);
 }
 
 namespace fsl {
-void launch_export_owner(const Dev& s, int* out, cudaStream_t st);
 void launch_bed_height(const Dev& s, double phi_b, double* phi, double* h, cudaStream_t st);
 void launch_water_depth(const Dev& s, double* bed, double* eta, double* out, cudaStream_t st);
 int launch_bed_spectrum(const double* h, int nt, int nx, double* psd, double* work, double* peak3, cudaStream_t st);
@@ -130,6 +129,27 @@ int launch_check(fslbm* s) {
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess && !s->host_err) s->host_err = FSLBM_EDEVICE;
     return s->host_err;
+}
+
+// Whether a kernel may access [p, p + bytes) of a caller's buffer directly:
+// aligned, and its first and last byte both device memory of the current
+// device. Anything else (another device's memory, host memory passed as
+// device memory, a range that leaves its allocation) keeps the staged copy,
+// which validates it.
+bool kernel_writable(const void* p, size_t bytes, size_t align) {
+    if (reinterpret_cast<uintptr_t>(p) % align) return false;
+    int dev = -1;
+    if (cudaGetDevice(&dev) != cudaSuccess) return false;
+    const char* ends[2] = {static_cast<const char*>(p), static_cast<const char*>(p) + bytes - 1};
+    for (const char* e : ends) {
+        cudaPointerAttributes a;
+        if (cudaPointerGetAttributes(&a, e) != cudaSuccess) {
+            cudaGetLastError();
+            return false;
+        }
+        if (a.type != cudaMemoryTypeDevice || a.device != dev) return false;
+    }
+    return true;
 }
 
 cudaMemcpyKind kind_to(int on_device) { return on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost; }
@@ -724,42 +744,87 @@ int fslbm_get_fields(fslbm* s, uint32_t mask, void* const* dst, int dst_on_devic
     cudaStream_t st = s->st;
     const long long n = d.n;
     int k = 0;
+    // cell fields whose destination a kernel can write are collected here and
+    // written in one pass over the lattice; the others go one component at a
+    // time through the n-double staging buffer and a copy
+    CellOut all;
+    std::memset(&all, 0, sizeof(all));
+    bool any = false;
+    auto staged = [&](const CellOut& o, void* to, size_t bytes) {
+        launch_export(d, s->last_parity, o, st);
+        cudaMemcpyAsync(to, s->stage, bytes, kind_to(dst_on_device), st);
+    };
     for (int bit = 0; bit < 32; ++bit) {
         uint32_t b = 1u << bit;
         if (!(mask & b)) continue;
         void* out = dst[k++];
         if (!out) return FSLBM_EINVAL;
+        double* od = static_cast<double*>(out);
+        CellOut one;
+        std::memset(&one, 0, sizeof(one));
         switch (b) {
         case FSLBM_FIELD_PDF:
+            if (dst_on_device && kernel_writable(out, (size_t)27 * n * sizeof(double), sizeof(double))) {
+                all.pdf = od;
+                all.q0 = 0;
+                all.q1 = 27;
+                any = true;
+                break;
+            }
             for (int q = 0; q < 27; ++q) {
-                // one direction at a time through the n-double staging buffer
-                launch_export(d, s->last_parity, FSLBM_FIELD_PDF | (uint32_t)(q << 8), s->stage, st);
-                cudaMemcpyAsync(static_cast<double*>(out) + (size_t)q * n, s->stage, n * sizeof(double),
-                                kind_to(dst_on_device), st);
+                one.pdf = s->stage;
+                one.q0 = q;
+                one.q1 = q + 1;
+                staged(one, od + (size_t)q * n, n * sizeof(double));
             }
             break;
         case FSLBM_FIELD_TYPE:
-            launch_export_type(d, reinterpret_cast<uint8_t*>(s->stage), st);
-            cudaMemcpyAsync(out, s->stage, n, kind_to(dst_on_device), st);
+            if (dst_on_device && kernel_writable(out, n, 1)) {
+                all.type = static_cast<uint8_t*>(out);
+                any = true;
+                break;
+            }
+            one.type = reinterpret_cast<uint8_t*>(s->stage);
+            staged(one, out, n);
             break;
         case FSLBM_FIELD_OWNER:
-            launch_export_owner(d, reinterpret_cast<int*>(s->stage), st);
-            cudaMemcpyAsync(out, s->stage, n * sizeof(int), kind_to(dst_on_device), st);
+            if (dst_on_device && kernel_writable(out, n * sizeof(int), sizeof(int))) {
+                all.owner = static_cast<int*>(out);
+                any = true;
+                break;
+            }
+            one.owner = reinterpret_cast<int*>(s->stage);
+            staged(one, out, n * sizeof(int));
             break;
         case FSLBM_FIELD_MASS:
         case FSLBM_FIELD_PHI:
-        case FSLBM_FIELD_RHO:
-            launch_export(d, s->last_parity, b, s->stage, st);
-            cudaMemcpyAsync(out, s->stage, n * sizeof(double), kind_to(dst_on_device), st);
+        case FSLBM_FIELD_RHO: {
+            double* CellOut::*field = b == FSLBM_FIELD_MASS ? &CellOut::mass
+                                      : b == FSLBM_FIELD_PHI ? &CellOut::phi : &CellOut::rho;
+            if (dst_on_device && kernel_writable(out, n * sizeof(double), sizeof(double))) {
+                all.*field = od;
+                any = true;
+                break;
+            }
+            one.*field = s->stage;
+            staged(one, out, n * sizeof(double));
             break;
+        }
         case FSLBM_FIELD_U:
-        case FSLBM_FIELD_NORMAL:
+        case FSLBM_FIELD_NORMAL: {
+            const bool direct = dst_on_device && kernel_writable(out, (size_t)3 * n * sizeof(double), sizeof(double));
             for (int a = 0; a < 3; ++a) {
-                launch_export(d, s->last_parity, b | (uint32_t)(a << 8), s->stage, st);
-                cudaMemcpyAsync(static_cast<double*>(out) + (size_t)a * n, s->stage, n * sizeof(double),
-                                kind_to(dst_on_device), st);
+                if (direct) {
+                    (b == FSLBM_FIELD_U ? all.u : all.nrm)[a] = od + (size_t)a * n;
+                    any = true;
+                    continue;
+                }
+                CellOut c1 = one;
+                (b == FSLBM_FIELD_U ? c1.u : c1.nrm)[a] = s->stage;
+                staged(c1, od + (size_t)a * n, n * sizeof(double));
             }
             break;
+        }
         case FSLBM_FIELD_P_X:
             cudaMemcpyAsync(out, d.X, sizeof(double) * 3 * d.np, kind_to(dst_on_device), st);
             break;
@@ -782,6 +847,7 @@ int fslbm_get_fields(fslbm* s, uint32_t mask, void* const* dst, int dst_on_devic
             return FSLBM_EINVAL;
         }
     }
+    if (any) launch_export(d, s->last_parity, all, st);
     launch_check(s);
     return sync_check(s);
 }
@@ -799,12 +865,15 @@ int fslbm_set_fields(fslbm* s, uint32_t mask, const void* const* src, int src_on
         if (!in) return FSLBM_EINVAL;
         switch (b) {
         case FSLBM_FIELD_PDF:
+            if (src_on_device && kernel_writable(in, (size_t)27 * n * sizeof(double), sizeof(double))) {
+                launch_import_pdf(d, s->last_parity, static_cast<const double*>(in), 0, 27, true, st);
+                break;
+            }
             for (int q = 0; q < 27; ++q) {
                 cudaMemcpyAsync(s->stage, static_cast<const double*>(in) + (size_t)q * n, n * sizeof(double),
                                 kind_from(src_on_device), st);
-                launch_import_pdf(d, s->last_parity | (q << 8), s->stage, st);
+                launch_import_pdf(d, s->last_parity, s->stage, q, q + 1, q == 26, st);
             }
-            launch_import_pdf(d, s->last_parity | (27 << 8), nullptr, st);
             break;
         case FSLBM_FIELD_MASS:
             cudaMemcpyAsync(s->stage, in, n * sizeof(double), kind_from(src_on_device), st);

@@ -272,6 +272,33 @@ __device__ __forceinline__ long long nbr(const Dev& s, int x, int y, int z, int 
     return (long long)a + (long long)s.nx * ((long long)b + (long long)s.ny * c);
 }
 
+// offsets of the x, y, z neighbours (-1, 0, +1) of a cell with the wall
+// faces it touches as bits (x-, x+, y-, y+, z-, z+)
+struct NbrOffsets {
+    int ox[3], oy[3], oz[3];
+    unsigned wall;
+};
+__device__ __forceinline__ NbrOffsets nbr_offsets(const Dev& s, int x, int y, int z) {
+    const int sxy = s.nx * s.ny;
+    NbrOffsets o;
+    o.wall = 0;
+    o.ox[0] = -1; o.ox[1] = 0; o.ox[2] = 1;
+    o.oy[0] = -s.nx; o.oy[1] = 0; o.oy[2] = s.nx;
+    o.oz[0] = -sxy; o.oz[1] = 0; o.oz[2] = sxy;
+    if (x == 0) { if (s.per_x) o.ox[0] = s.nx - 1; else o.wall |= 1u; }
+    if (x == s.nx - 1) { if (s.per_x) o.ox[2] = 1 - s.nx; else o.wall |= 2u; }
+    if (y == 0) { if (s.per_y) o.oy[0] = (s.ny - 1) * s.nx; else o.wall |= 4u; }
+    if (y == s.ny - 1) { if (s.per_y) o.oy[2] = (1 - s.ny) * s.nx; else o.wall |= 8u; }
+    if (z == 0) { if (s.per_z) o.oz[0] = (s.nz - 1) * sxy; else o.wall |= 16u; }
+    if (z == s.nz - 1) { if (s.per_z) o.oz[2] = (1 - s.nz) * sxy; else o.wall |= 32u; }
+    return o;
+}
+// wall bits a direction d crosses from a cell
+__host__ __device__ constexpr unsigned wall_bits(int dx, int dy, int dz) {
+    return (dx == -1 ? 1u : 0u) | (dx == 1 ? 2u : 0u) | (dy == -1 ? 4u : 0u) | (dy == 1 ? 8u : 0u) |
+           (dz == -1 ? 16u : 0u) | (dz == 1 ? 32u : 0u);
+}
+
 // AA pattern. After an even step the post-collision PDF f*_q(x) sits in slot
 // (opp(q), x); after an odd step (and initially) it sits in slot
 // (q, x + c_q), or (opp(q), x) when x + c_q lies beyond a wall.
@@ -596,9 +623,20 @@ int launch_remap(const Dev& s, int last_parity, cudaStream_t st);
 void launch_particles_add(const Dev& s, int first, int count, cudaStream_t st);
 void launch_particle_copies(const Dev& s, cudaStream_t st);
 int launch_grid_build(const Dev& s, cudaStream_t st);
-void launch_export(const Dev& s, int last_parity, uint32_t which, double* out, cudaStream_t st);
-void launch_export_type(const Dev& s, uint8_t* out, cudaStream_t st);
-void launch_import_pdf(const Dev& s, int last_parity, const double* in, cudaStream_t st);
+// Cell fields to write in the canonical layout of the C ABI, null where not
+// wanted; PDF directions [q0, q1) go to pdf + (q - q0) n
+struct CellOut {
+    double* pdf;
+    int q0, q1;
+    double *mass, *phi, *rho;
+    double* u[3];
+    double* nrm[3];
+    uint8_t* type;
+    int* owner;
+};
+void launch_export(const Dev& s, int last_parity, const CellOut& out, cudaStream_t st);
+void launch_import_pdf(const Dev& s, int last_parity, const double* in, int q0, int q1, bool refresh,
+                       cudaStream_t st);
 void launch_import_mass(const Dev& s, const double* in, cudaStream_t st);
 void launch_reduce(const Dev& s, int last_parity, double* out, cudaStream_t st);
 int reduce_blocks(const Dev& s);

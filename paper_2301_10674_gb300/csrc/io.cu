@@ -15,100 +15,200 @@ __device__ __forceinline__ bool fluid(uint8_t fl) {
     return t == T_LIQ || t == T_IFC;
 }
 
-// which & 0xff: FSLBM_FIELD_PDF, MASS, PHI, RHO, U or NORMAL; which >> 8: the
-// direction (PDF) or component (U, NORMAL) written to out[0..n)
-__global__ void k_export(Dev s, int last_parity, uint32_t which, double* out) {
+// Sum of FP32 values carried in three FP32 words: two exact two-sums pass the
+// rounding errors on, so the value keeps more bits than an FP64 running sum
+// (72 against 53) at 12 FP32 operations per value; an FP64 add costs about
+// twice as many issue cycles here (the FP64 pipe runs at 1/64 of the FP32 rate).
+struct Sum3 {
+    float s = 0.f, e1 = 0.f, e2 = 0.f;
+    __device__ __forceinline__ static float two_sum(float a, float b, float& err) {
+        const float t = __fadd_rn(a, b), bb = __fsub_rn(t, a);
+        err = __fadd_rn(__fsub_rn(a, __fsub_rn(t, bb)), __fsub_rn(b, bb));
+        return t;
+    }
+    __device__ __forceinline__ void add(float v) {
+        float r, r2;
+        s = two_sum(s, v, r);
+        e1 = two_sum(e1, r, r2);
+        e2 += r2;
+    }
+    // (an infinite or NaN sum stands as it is: its error terms are NaN)
+    __device__ __forceinline__ double value() const {
+        return isfinite(s) ? (double)s + ((double)e1 + (double)e2) : (double)s;
+    }
+};
+
+// Slot of the post-collision PDF f*_q of a cell at height z with the neighbour
+// offsets o (the slot of fstar_slot), and the storage reference h of that
+// slot's z (0 at FP32)
+template <typename S, int LP>
+__device__ __forceinline__ long long pdf_slot(const Dev& s, int q, long long c, int z, const NbrOffsets& o, float& h) {
+    const bool own = LP == 0 || (o.wall & wall_bits(cx(q), cy(q), cz(q)));
+    h = Store<S>::HREF ? s.href[own ? z : wrap_z(s, z + cz(q))] : 0.f;
+    return own ? (long long)opp(q) * s.n + c
+               : (long long)q * s.n + c + (o.ox[1 + cx(q)] + o.oy[1 + cy(q)] + o.oz[1 + cz(q)]);
+}
+// f - w from a stored value and its slot's reference, with one rounding (the
+// same bits wherever it is inlined)
+template <typename S>
+__device__ __forceinline__ float with_ref(float v, int q, float h) {
+    return Store<S>::HREF ? __fmaf_rn(wq(q), h, v) : v;
+}
+
+// The selected cell fields in one pass, a thread per cell: the flag and the
+// 27 PDFs are read once, every output is written coalesced, with no staging
+// copy. Bound by the FP64 outputs (216 of about 270-330 bytes per cell for the
+// PDFs). A launch per component with 64-bit divisions per cell and an n-double
+// copy took 64 ms for PDF + TYPE + MASS of 3072x96x320 cells; with this kernel
+// 40 FP16 steps and that read-out went from 233 to 177 ms, 20 steps of a
+// 200x72x90 box from set PDFs to read-out from 5.2 to 2.9 ms.
+template <typename S, int LP>
+__global__ void __launch_bounds__(256) k_export(Dev s, CellOut out) {
     const long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (c >= s.n) return;
     const uint8_t fl = s.flags[c];
     const int t = fl & TYPE_MASK;
-    const uint32_t field = which & 0xffu;
-    const int sub = (int)(which >> 8);
-    if (field == FSLBM_FIELD_PDF) {
-        if (!fluid(fl)) { out[c] = 0.0; return; }
+    const bool fld = fluid(fl);
+    if (out.type) out.type[c] = (uint8_t)t;
+    if (out.owner) out.owner[c] = t == T_SOL ? s.owner[c] : -1;
+    if (out.phi) out.phi[c] = t == T_LIQ ? 1.0 : (t == T_IFC ? (double)s.phi[c] : 0.0);
+    if (out.nrm[0] || out.nrm[1] || out.nrm[2]) {
+        const float4 v = t == T_IFC ? s.nrm[c] : make_float4(0.f, 0.f, 0.f, 0.f);
+        if (out.nrm[0]) out.nrm[0][c] = v.x;
+        if (out.nrm[1]) out.nrm[1][c] = v.y;
+        if (out.nrm[2]) out.nrm[2][c] = v.z;
+    }
+    const bool want_u = out.u[0] || out.u[1] || out.u[2];
+    if (!(out.q1 > out.q0 || out.mass || out.rho || want_u)) return;
+    const bool mom = fld && want_u;
+    const bool den = mom || (fld && out.rho) || (t == T_LIQ && out.mass);
+    Sum3 d, jx, jy, jz;
+    const bool every = out.q0 == 0 && out.q1 == 27;
+    if (fld) {
+        const S* f = static_cast<const S*>(s.f);
         int x, y, z;
-        coords(s, c, x, y, z);
-        out[c] = wqd(sub) + (double)ld_any(s, s.f, fstar_slot(s, sub, x, y, z, c, last_parity));
-        return;
-    }
-    if (field == FSLBM_FIELD_NORMAL) {
-        float4 v = t == T_IFC ? s.nrm[c] : make_float4(0.f, 0.f, 0.f, 0.f);
-        out[c] = sub == 0 ? v.x : (sub == 1 ? v.y : v.z);
-        return;
-    }
-    if (field == FSLBM_FIELD_PHI) {
-        out[c] = t == T_LIQ ? 1.0 : (t == T_IFC ? (double)s.phi[c] : 0.0);
-        return;
-    }
-    double rho = 0.0, u[3] = {0, 0, 0};
-    if (fluid(fl)) {
-        float f[27];
-        load_fstar(s, c, last_parity, f);
-        double d = 0, j[3] = {0, 0, 0};
-        for (int q = 0; q < 27; ++q) {
-            d += f[q];
-            j[0] += cx(q) * (double)f[q];
-            j[1] += cy(q) * (double)f[q];
-            j[2] += cz(q) * (double)f[q];
+        coords32(s, (int)c, x, y, z);
+        const NbrOffsets o = nbr_offsets(s, x, y, z);
+        if (every || den) {
+            // all 27 loads in flight together
+            float v[27];
+#pragma unroll
+            for (int q = 0; q < 27; ++q) {
+                float h;
+                const long long a = pdf_slot<S, LP>(s, q, c, z, o, h);
+                v[q] = with_ref<S>(Store<S>::ld(f + a), q, h);
+            }
+            if (every) {
+#pragma unroll
+                for (int q = 0; q < 27; ++q) out.pdf[(long long)q * s.n + c] = wqd(q) + (double)v[q];
+            }
+            if (den) {
+#pragma unroll
+                for (int q = 0; q < 27; ++q) d.add(v[q]);
+            }
+            if (mom) {
+#pragma unroll
+                for (int q = 0; q < 27; ++q) {
+                    if (cx(q)) jx.add(cx(q) > 0 ? v[q] : -v[q]);
+                    if (cy(q)) jy.add(cy(q) > 0 ? v[q] : -v[q]);
+                    if (cz(q)) jz.add(cz(q) > 0 ? v[q] : -v[q]);
+                }
+            }
         }
-        rho = 1.0 + d;
-        u[0] = (j[0] - 0.5 * rho * s.gxd) / rho;
-        u[1] = (j[1] - 0.5 * rho * s.gyd) / rho;
-        u[2] = (j[2] - 0.5 * rho * s.gzd) / rho;
+        if (!every) {
+            // one or a few directions (the staged copy to the host)
+#pragma unroll
+            for (int q = 0; q < 27; ++q) {
+                if (q < out.q0 || q >= out.q1) continue;
+                float h;
+                const long long a = pdf_slot<S, LP>(s, q, c, z, o, h);
+                out.pdf[(long long)(q - out.q0) * s.n + c] = wqd(q) + (double)with_ref<S>(Store<S>::ld(f + a), q, h);
+            }
+        }
+    } else {
+        for (int q = out.q0; q < out.q1; ++q) out.pdf[(long long)(q - out.q0) * s.n + c] = 0.0;
     }
-    if (field == FSLBM_FIELD_MASS) out[c] = t == T_LIQ ? rho : (t == T_IFC ? (double)s.mass[c] : 0.0);
-    else if (field == FSLBM_FIELD_RHO) out[c] = rho;
-    else if (field == FSLBM_FIELD_U) out[c] = u[sub];
+    const double rho = den ? 1.0 + d.value() : 0.0;
+    if (out.mass) out.mass[c] = t == T_LIQ ? rho : (t == T_IFC ? (double)s.mass[c] : 0.0);
+    if (out.rho) out.rho[c] = rho;
+    if (want_u) {
+        if (out.u[0]) out.u[0][c] = mom ? (jx.value() - 0.5 * rho * s.gxd) / rho : 0.0;
+        if (out.u[1]) out.u[1][c] = mom ? (jy.value() - 0.5 * rho * s.gyd) / rho : 0.0;
+        if (out.u[2]) out.u[2][c] = mom ? (jz.value() - 0.5 * rho * s.gzd) / rho : 0.0;
+    }
 }
 
-__global__ void k_export_type(Dev s, uint8_t* out) {
-    const long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (c < s.n) out[c] = s.flags[c] & TYPE_MASK;
+template <typename S>
+static void export_typed(const Dev& s, int last_parity, const CellOut& out, cudaStream_t st) {
+    if (last_parity == 0) k_export<S, 0><<<blocks_for(s.n, 256), 256, 0, st>>>(s, out);
+    else k_export<S, 1><<<blocks_for(s.n, 256), 256, 0, st>>>(s, out);
 }
-__global__ void k_export_owner(Dev s, int* out) {
-    const long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (c < s.n) out[c] = (s.flags[c] & TYPE_MASK) == T_SOL ? s.owner[c] : -1;
-}
-
-void launch_export(const Dev& s, int last_parity, uint32_t which, double* out, cudaStream_t st) {
-    k_export<<<blocks_for(s.n, 128), 128, 0, st>>>(s, last_parity, which, out);
-}
-void launch_export_type(const Dev& s, uint8_t* out, cudaStream_t st) {
-    k_export_type<<<blocks_for(s.n, 256), 256, 0, st>>>(s, out);
-}
-void launch_export_owner(const Dev& s, int* out, cudaStream_t st) {
-    k_export_owner<<<blocks_for(s.n, 256), 256, 0, st>>>(s, out);
+void launch_export(const Dev& s, int last_parity, const CellOut& out, cudaStream_t st) {
+    if (s.storage == FSLBM_STORE_FP32) export_typed<float>(s, last_parity, out, st);
+    else if (s.storage == FSLBM_STORE_FP16) export_typed<__half>(s, last_parity, out, st);
+    else export_typed<__nv_bfloat16>(s, last_parity, out, st);
 }
 
-// arg & 1: layout parity, arg >> 8: direction q. For q < 27 the PDF f*_q
-// (double, canonical) becomes f - w in its AA slot (and in the side buffer of
-// interface cells); q == 27 refreshes (rho, u) and phi of interface cells.
-__global__ void k_import_pdf(Dev s, int arg, const double* in) {
+// PDFs f*_q (double, canonical, directions [q0, q1) at in + (q - q0) n) to
+// f - w in their AA slots (and in the side buffer of interface cells);
+// refresh: (rho, u) and phi of interface cells from the side buffer
+template <typename S, int LP>
+__global__ void __launch_bounds__(256) k_import_pdf(Dev s, const double* in, int q0, int q1, int refresh) {
     const long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (c >= s.n) return;
     const uint8_t fl = s.flags[c];
     if (!fluid(fl)) return;
-    const int last_parity = arg & 1;
-    const int q = arg >> 8;
     const bool ifc = (fl & TYPE_MASK) == T_IFC;
-    if (q < 27) {
-        int x, y, z;
-        coords(s, c, x, y, z);
-        const float v = (float)(in[c] - wqd(q));
-        st_any(s, s.f, fstar_slot(s, q, x, y, z, c, last_parity), v);
-        if (ifc) st_any(s, s.fs, (long long)q * s.n + c, v);
-        return;
+    S* f = static_cast<S*>(s.f);
+    S* fs = static_cast<S*>(s.fs);
+    int x, y, z;
+    coords32(s, (int)c, x, y, z);
+    const float h0 = Store<S>::HREF ? s.href[z] : 0.f;
+    const NbrOffsets o = nbr_offsets(s, x, y, z);
+    auto put = [&](int q, double f64) {
+        const float v = (float)(f64 - wqd(q));
+        float h;
+        const long long a = pdf_slot<S, LP>(s, q, c, z, o, h);
+        Store<S>::st(f + a, with_ref<S>(v, q, -h));
+        if (ifc) Store<S>::st(fs + (long long)q * s.n + c, with_ref<S>(v, q, -h0));
+    };
+    if (q0 == 0 && q1 == 27) {
+        // nine loads in flight at a time
+#pragma unroll
+        for (int k = 0; k < 27; k += 9) {
+            double g[9];
+#pragma unroll
+            for (int j = 0; j < 9; ++j) g[j] = in[(long long)(k + j) * s.n + c];
+#pragma unroll
+            for (int j = 0; j < 9; ++j) put(k + j, g[j]);
+        }
+    } else {
+#pragma unroll
+        for (int q = 0; q < 27; ++q)
+            if (q >= q0 && q < q1) put(q, in[(long long)(q - q0) * s.n + c]);
     }
-    if (!ifc) return;
-    float f[27];
-    for (int k = 0; k < 27; ++k) f[k] = ld_any(s, s.fs, (long long)k * s.n + c);
+    if (!refresh || !ifc) return;
+    float g[27];
+#pragma unroll
+    for (int k = 0; k < 27; ++k) {
+        g[k] = with_ref<S>(Store<S>::ld(fs + (long long)k * s.n + c), k, h0);
+    }
     float rho, ux, uy, uz;
-    post_moments(s, f, rho, ux, uy, uz);
+    post_moments(s, g, rho, ux, uy, uz);
     s.ru[c] = make_float4(rho, ux, uy, uz);
     s.phi[c] = s.mass[c] / rho;
 }
-void launch_import_pdf(const Dev& s, int arg, const double* in, cudaStream_t st) {
-    k_import_pdf<<<blocks_for(s.n, 128), 128, 0, st>>>(s, arg, in);
+template <typename S>
+static void import_typed(const Dev& s, int last_parity, const double* in, int q0, int q1, bool refresh,
+                         cudaStream_t st) {
+    if (last_parity == 0) k_import_pdf<S, 0><<<blocks_for(s.n, 256), 256, 0, st>>>(s, in, q0, q1, refresh);
+    else k_import_pdf<S, 1><<<blocks_for(s.n, 256), 256, 0, st>>>(s, in, q0, q1, refresh);
+}
+void launch_import_pdf(const Dev& s, int last_parity, const double* in, int q0, int q1, bool refresh,
+                       cudaStream_t st) {
+    if (s.storage == FSLBM_STORE_FP32) import_typed<float>(s, last_parity, in, q0, q1, refresh, st);
+    else if (s.storage == FSLBM_STORE_FP16) import_typed<__half>(s, last_parity, in, q0, q1, refresh, st);
+    else import_typed<__nv_bfloat16>(s, last_parity, in, q0, q1, refresh, st);
 }
 
 __global__ void k_import_mass(Dev s, const double* in) {

@@ -21,33 +21,6 @@
 
 namespace fsl {
 
-// offsets of the x, y, z neighbours (-1, 0, +1) of a cell with the wall
-// faces it touches as bits (x-, x+, y-, y+, z-, z+)
-struct NbrOffsets {
-    int ox[3], oy[3], oz[3];
-    unsigned wall;
-};
-__device__ __forceinline__ NbrOffsets nbr_offsets(const Dev& s, int x, int y, int z) {
-    const int sxy = s.nx * s.ny;
-    NbrOffsets o;
-    o.wall = 0;
-    o.ox[0] = -1; o.ox[1] = 0; o.ox[2] = 1;
-    o.oy[0] = -s.nx; o.oy[1] = 0; o.oy[2] = s.nx;
-    o.oz[0] = -sxy; o.oz[1] = 0; o.oz[2] = sxy;
-    if (x == 0) { if (s.per_x) o.ox[0] = s.nx - 1; else o.wall |= 1u; }
-    if (x == s.nx - 1) { if (s.per_x) o.ox[2] = 1 - s.nx; else o.wall |= 2u; }
-    if (y == 0) { if (s.per_y) o.oy[0] = (s.ny - 1) * s.nx; else o.wall |= 4u; }
-    if (y == s.ny - 1) { if (s.per_y) o.oy[2] = (1 - s.ny) * s.nx; else o.wall |= 8u; }
-    if (z == 0) { if (s.per_z) o.oz[0] = (s.nz - 1) * sxy; else o.wall |= 16u; }
-    if (z == s.nz - 1) { if (s.per_z) o.oz[2] = (1 - s.nz) * sxy; else o.wall |= 32u; }
-    return o;
-}
-// wall bits a direction d crosses from a cell
-__host__ __device__ constexpr unsigned wall_bits(int dx, int dy, int dz) {
-    return (dx == -1 ? 1u : 0u) | (dx == 1 ? 2u : 0u) | (dy == -1 ? 4u : 0u) | (dy == 1 ? 8u : 0u) |
-           (dz == -1 ? 16u : 0u) | (dz == 1 ? 32u : 0u);
-}
-
 // All liquid cells. Every PDF is a plain pull: PDFs from fluid cells, and
 // from solid cells the bounce-back values k_solid_links placed in the pull
 // slots. Only wall faces need handling here, and they follow from the
