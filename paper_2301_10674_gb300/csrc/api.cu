@@ -341,7 +341,7 @@ int fslbm_create(const fslbm_params* p, void* cuda_stream, fslbm** out) {
             d.bseg = dalloc<int>(s, nseg + 1, ok);
         }
         d.tl_info = dalloc<int>(s, 2 * tcap, ok);
-        counts = dalloc<int>(s, 16, ok);
+        counts = dalloc<int>(s, 32, ok);
         if (ok) {
             d.wl_count = counts;
             d.nl_count = counts + 1;
@@ -355,6 +355,7 @@ int fslbm_create(const fslbm_params* p, void* cuda_stream, fslbm** out) {
             d.bseg_count = counts + 9;
             d.cl_count = counts + 10;
             d.rtail_count = counts + 11;
+            d.g_tot = counts + 16;   // one word per CTA of the DEM cluster (8)
         }
         dd = dalloc<double>(s, 4, ok);
         if (ok) {
@@ -368,10 +369,13 @@ int fslbm_create(const fslbm_params* p, void* cuda_stream, fslbm** out) {
         d.np_cap = (int)pc;
         d.X = dalloc<double>(s, 3 * pc, ok); d.U = dalloc<double>(s, 3 * pc, ok); d.W = dalloc<double>(s, 3 * pc, ok);
         for (int k = 0; k < 2; ++k) {
-            d.dem_dx[k] = dalloc<float>(s, 3 * pc, ok);
-            d.dem_du[k] = dalloc<float>(s, 3 * pc, ok);
-            d.dem_dw[k] = dalloc<float>(s, 3 * pc, ok);
+            d.dem_x[k] = dalloc<float4>(s, pc, ok);
+            d.dem_u[k] = dalloc<float4>(s, pc, ok);
+            d.dem_w[k] = dalloc<float4>(s, pc, ok);
         }
+        d.dem_du = dalloc<float4>(s, pc, ok);
+        d.dem_dw = dalloc<float4>(s, pc, ok);
+        d.nb_xi = dalloc<float4>(s, pc * NB_ITEMS, ok);
         d.nb_d0 = dalloc<float4>(s, pc * NB_SLOTS, ok);
         d.dem_wall = dalloc<float>(s, 6 * pc, ok);
         d.dem_c = dalloc<float4>(s, pc, ok);
@@ -386,11 +390,8 @@ int fslbm_create(const fslbm_params* p, void* cuda_stream, fslbm** out) {
         d.Wf = dalloc<float4>(s, pc, ok);
         d.Fh = dalloc<double>(s, 3 * pc, ok); d.Th = dalloc<double>(s, 3 * pc, ok);
         d.Fp = dalloc<double>(s, 3 * pc, ok); d.Tp = dalloc<double>(s, 3 * pc, ok);
-        d.Fa = dalloc<double>(s, 3 * pc, ok); d.Ta = dalloc<double>(s, 3 * pc, ok);
-        d.hist_partner = dalloc<int>(s, pc * HIST_SLOTS, ok);
         d.nb = dalloc<int>(s, pc * NB_SLOTS, ok);
         d.nb_count = dalloc<int>(s, pc, ok);
-        d.hist_xi = dalloc<float>(s, pc * HIST_SLOTS * 3, ok);
         d.g_of = dalloc<int>(s, pc, ok);
         d.Xm = dalloc<double>(s, 3 * pc, ok);
         d.margin = dalloc<float>(s, pc, ok);
@@ -454,7 +455,7 @@ int fslbm_create(const fslbm_params* p, void* cuda_stream, fslbm** out) {
     cudaMemsetAsync(d.conv, 0, n, st);
     cudaMemsetAsync(d.exscale, 0, n * sizeof(float), st);
     cudaMemsetAsync(d.nrm1, 0, n * sizeof(float4), st);
-    cudaMemsetAsync(counts, 0, 16 * sizeof(int), st);
+    cudaMemsetAsync(counts, 0, 32 * sizeof(int), st);
     cudaMemsetAsync(dd, 0, 4 * sizeof(double), st);
     cudaMemsetAsync(d.viol, 0, sizeof(unsigned long long), st);
     cudaMemsetAsync(d.dirty, 0, n + 4, st);
@@ -564,6 +565,13 @@ static int enqueue_step(fslbm* s, int parity, bool capturing) {
         cudaMemsetAsync(d.Th, 0, sizeof(double) * 3 * d.np, st);
     }
     int nl = 0;
+    if (d.np > 0) {
+        // the DEM's neighbour list needs the positions alone: on the side
+        // stream from the step's start
+        cudaEventRecord(s->ev_fork, st);
+        cudaStreamWaitEvent(s->side, s->ev_fork, 0);
+        nl += launch_dem_neighbours(d, s->side);
+    }
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     if (capturing) {
         e0 = s->ev_cap[0];

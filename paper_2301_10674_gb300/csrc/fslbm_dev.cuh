@@ -50,8 +50,9 @@ constexpr int WAIT_LIMIT_DEFAULT = 1 << 22;   // polls of a bounded device wait
 
 constexpr int REDUCE_TAIL_BLOCKS = 64;   // blocks of the reduction's second level
 constexpr int REDUCE_MAX_BY = 1024;   // row blocks of the lattice reduction (several rows per thread)
-constexpr int HIST_SLOTS = 16;   // tangential-spring history slots per particle
+constexpr int HIST_SLOTS = 16;   // contacts (tangential springs) a particle may have at once
 constexpr int NB_SLOTS = 32;     // DEM neighbour-list slots per particle
+constexpr int NB_ITEMS = 40;     // spring slots per particle: its neighbours', then the six wall faces' (and two spare)
 
 struct Dev {
     // lattice
@@ -116,14 +117,18 @@ struct Dev {
     // particles (FP64 state)
     int np, np_cap;
     double* X; double* U; double* W;            // current state
-    // DEM sub-steps in FP32 (R-25): the changes of position, velocity and
-    // angular velocity since the step's start, ping-pong over the sub-steps
-    // (3 per particle each); per neighbour slot the offset of the partner's
-    // centre at the step's start, per particle the distances to the six wall
-    // faces then, (r, m, I) and the averaged hydrodynamic force plus weight
+    // DEM sub-steps in FP32 (R-25): what the particles publish to one another,
+    // the change of position since the step's start and the velocity and
+    // angular velocity (ping-pong over the sub-steps), and the changes of the
+    // last two; per neighbour slot the offset of the partner's centre at the
+    // step's start and its radius, and the tangential spring with the pair's
+    // effective mass; per particle the distances to the six wall faces at the
+    // step's start, (r, m, I) and the averaged hydrodynamic force plus weight
     // and torque, all in FP32
-    float* dem_dx[2]; float* dem_du[2]; float* dem_dw[2];
-    float4* nb_d0;                              // [np_cap][NB_SLOTS]
+    float4* dem_x[2]; float4* dem_u[2]; float4* dem_w[2];
+    float4* dem_du; float4* dem_dw;
+    float4* nb_d0;                              // [np_cap][NB_SLOTS]: offset, radius
+    float4* nb_xi;                              // [np_cap][NB_ITEMS]: spring, effective mass
     float* dem_wall;                            // [np_cap][6]: x, L_x - x, y, L_y - y, z, L_z - z
     float4* dem_c;                              // (r, m, I, 0)
     float* Faf; float* Taf;                     // [np_cap][3]
@@ -135,10 +140,7 @@ struct Dev {
     float4* Uf; float4* Wf;                     // FP32 copies of U and Omega for the links
     double* Fh; double* Th;                     // momentum exchange of this step
     double* Fp; double* Tp;                     // previous step
-    double* Fa; double* Ta;                     // two-step average
     int* nb; int* nb_count;                     // DEM neighbour list [np_cap][NB_SLOTS]
-    int* hist_partner;                          // [np_cap][HIST_SLOTS]
-    float* hist_xi;                             // [np_cap][HIST_SLOTS][3]
     double rho_p, restitution, friction, poisson, collision_time;
     double kn_coef, dn_coef, kt_ratio;          // contact law constants (host-computed)
     double gxd, gyd, gzd;
@@ -149,6 +151,7 @@ struct Dev {
     int gnx, gny, gnz;
     double ghx, ghy, ghz;
     int* g_count; int* g_start; int* g_cursor; int* g_list; int* g_of;
+    int* g_tot;                                 // the grid scan's partial totals (one per CTA of a cluster)
     double r_max;
     int* zmax_cell;
     // incremental re-mapping: position of the last map, margin to the nearest
@@ -618,6 +621,7 @@ int launch_pool_spread(const Dev& s, cudaStream_t st);
 void launch_cell_counts(const Dev& s, unsigned long long* out, cudaStream_t st);
 void launch_init_flat(const Dev& s, double H, cudaStream_t st);
 void launch_init_surface(const Dev& s, const double* H, cudaStream_t st);
+int launch_dem_neighbours(const Dev& s, cudaStream_t st);
 int launch_dem(const Dev& s, int have_prev, cudaStream_t st);
 int launch_remap(const Dev& s, int last_parity, cudaStream_t st);
 void launch_particles_add(const Dev& s, int first, int count, cudaStream_t st);

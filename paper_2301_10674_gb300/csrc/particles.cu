@@ -6,13 +6,9 @@
 // cells it covers and uncovers. Particle state and forces are FP64; the map
 // test is evaluated in FP64 without fused multiply-add so that cell types do
 // not depend on contraction choices.
-#include <limits.h>
-
 #include "fslbm_dev.cuh"
 
 namespace fsl {
-
-constexpr int HIST_EMPTY = INT_MIN;
 
 // ------------------------------------------------------------ particle grid
 __device__ __forceinline__ int gcoord(double v, double h, int g) {
@@ -20,15 +16,17 @@ __device__ __forceinline__ int gcoord(double v, double h, int g) {
     return k < 0 ? 0 : (k >= g ? g - 1 : k);
 }
 
-__global__ void k_grid_count(Dev s) {
-    int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= s.np) return;
+__device__ __forceinline__ void grid_count(const Dev& s, int p) {
     int a = gcoord(s.X[3 * p], s.ghx, s.gnx);
     int b = gcoord(s.X[3 * p + 1], s.ghy, s.gny);
     int c = gcoord(s.X[3 * p + 2], s.ghz, s.gnz);
     int g = a + s.gnx * (b + s.gny * c);
     s.g_of[p] = g;
     atomicAdd(&s.g_count[g], 1);
+}
+__global__ void k_grid_count(Dev s) {
+    const int p = blockIdx.x * blockDim.x + threadIdx.x;
+    if (p < s.np) grid_count(s, p);
 }
 
 // exclusive scan of the grid counts by one block of 32 warps: warp w owns a
@@ -75,17 +73,16 @@ __global__ void __launch_bounds__(1024) k_grid_scan(Dev s, int G) {
     }
 }
 
+__device__ __forceinline__ void grid_fill(const Dev& s, int p) {
+    s.g_list[atomicAdd(&s.g_cursor[s.g_of[p]], 1)] = p;
+}
 __global__ void k_grid_fill(Dev s) {
-    int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= s.np) return;
-    int pos = atomicAdd(&s.g_cursor[s.g_of[p]], 1);
-    s.g_list[pos] = p;
+    const int p = blockIdx.x * blockDim.x + threadIdx.x;
+    if (p < s.np) grid_fill(s, p);
 }
 
 // particles of a grid cell in index order (deterministic summation order)
-__global__ void k_grid_sort(Dev s, int G) {
-    int g = blockIdx.x * blockDim.x + threadIdx.x;
-    if (g >= G) return;
+__device__ __forceinline__ void grid_sort(const Dev& s, int g) {
     int b = s.g_start[g], e = b + s.g_count[g];
     for (int i = b + 1; i < e; ++i) {
         int v = s.g_list[i];
@@ -97,15 +94,23 @@ __global__ void k_grid_sort(Dev s, int G) {
         s.g_list[j + 1] = v;
     }
 }
+__global__ void k_grid_sort(Dev s, int G) {
+    const int g = blockIdx.x * blockDim.x + threadIdx.x;
+    if (g < G) grid_sort(s, g);
+}
 
-int launch_grid_build(const Dev& s, cudaStream_t st) {
+// the lists from the counts
+static int launch_grid_lists(const Dev& s, cudaStream_t st) {
     const int G = s.gnx * s.gny * s.gnz;
-    cudaMemsetAsync(s.g_count, 0, sizeof(int) * G, st);
-    k_grid_count<<<blocks_for(s.np, 128), 128, 0, st>>>(s);
     k_grid_scan<<<1, 1024, 0, st>>>(s, G);
     k_grid_fill<<<blocks_for(s.np, 128), 128, 0, st>>>(s);
     k_grid_sort<<<blocks_for(G, 128), 128, 0, st>>>(s, G);
-    return 4;
+    return 3;
+}
+int launch_grid_build(const Dev& s, cudaStream_t st) {
+    cudaMemsetAsync(s.g_count, 0, sizeof(int) * s.gnx * s.gny * s.gnz, st);
+    k_grid_count<<<blocks_for(s.np, 128), 128, 0, st>>>(s);
+    return 1 + launch_grid_lists(s, st);
 }
 
 // distinct grid coordinates within [k0, k1] along one axis
@@ -132,50 +137,6 @@ __device__ __forceinline__ GRange grange(int k0, int k1, int g, int periodic) {
 }
 
 // ------------------------------------------------------------ DEM
-__global__ void k_force_avg(Dev s, int have_prev) {
-    int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= 3 * s.np) return;
-    double fh = s.Fh[k], th = s.Th[k];
-    const double fa = have_prev ? 0.5 * (fh + s.Fp[k]) : fh;
-    const double ta = have_prev ? 0.5 * (th + s.Tp[k]) : th;
-    s.Fa[k] = fa;
-    s.Ta[k] = ta;
-    s.Fp[k] = fh;
-    s.Tp[k] = th;
-    // the sub-steps' FP32 copies: averaged hydrodynamic force plus the weight
-    const int a = k % 3;
-    const double g = a == 0 ? s.gxd : (a == 1 ? s.gyd : s.gzd);
-    s.Faf[k] = (float)(fa + s.M[k / 3] * g);
-    s.Taf[k] = (float)ta;
-}
-
-// The history slot of a partner among the particle's slots held in
-// registers: its own, else the first empty one, whose spring starts at zero;
-// -1 (and the sticky history bit) when none is left.
-__device__ __forceinline__ int hist_slot(const Dev& s, int p, int partner, int (&hpart)[HIST_SLOTS],
-                                         unsigned& seen) {
-    int found = -1, freeslot = -1;
-#pragma unroll
-    for (int k = 0; k < HIST_SLOTS; ++k) {
-        if (hpart[k] == partner && found < 0) found = k;
-        if (hpart[k] == HIST_EMPTY && freeslot < 0) freeslot = k;
-    }
-    if (found < 0) {
-        if (freeslot < 0) {
-            set_error(s, ERR_HISTORY);
-            return -1;
-        }
-        found = freeslot;
-#pragma unroll
-        for (int k = 0; k < HIST_SLOTS; ++k)
-            if (k == found) hpart[k] = partner;
-        float* xi = s.hist_xi + ((long long)p * HIST_SLOTS + found) * 3;
-        xi[0] = xi[1] = xi[2] = 0.f;
-    }
-    seen |= 1u << found;
-    return found;
-}
-
 // minimal image of an integer displacement along a periodic axis
 __device__ __forceinline__ int wrap_int(int d, int L, int periodic) {
     if (periodic) {
@@ -239,19 +200,32 @@ __device__ __forceinline__ bool dem_partner(const Dev& s, int p, int j, const fl
 // step: particles whose surfaces are within 3/4 cell (beyond the
 // lubrication range; the motion within a step is far below the margin).
 // With it the FP32 start of the sub-steps (R-25): per neighbour slot the
-// partner's centre offset, per mobile particle the distances to the wall
-// faces, and zero changes of position, velocity and angular velocity.
+// partner's centre offset and radius, the pair's effective mass and the
+// tangential spring carried over from the last step's list; per mobile
+// particle the distances to the wall faces; and the values the particles
+// publish to one another: zero change of position, velocity and angular
+// velocity at the step's start.
 // A warp per particle: lane t scans grid cell t of the (up to) 3x3x3 cells
 // around the particle's, in the order (z, y, x) of the cells and of the
 // particles within a cell; the accepted partners are compacted into the
 // slots in that order (a warp prefix sum over the lanes' counts).
 __global__ void k_dem_neighbours(Dev s) {
+    __shared__ int found_s[4][NB_SLOTS];
     const unsigned full = 0xffffffffu;
     const int p = (int)(((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
     const int lane = threadIdx.x & 31;
     if (p >= s.np) return;   // whole warps leave together
-    if (lane < 3) s.dem_dx[0][3 * p + lane] = s.dem_du[0][3 * p + lane] = s.dem_dw[0][3 * p + lane] = 0.f;
-    if (s.fixed[p]) {
+    int* found = found_s[threadIdx.x >> 5];
+    const bool fixed = s.fixed[p] != 0;
+    if (lane < 2) {
+        // both buffers: a fixed particle's values stay as they are
+        s.dem_x[lane][p] = make_float4(0.f, 0.f, 0.f, 0.f);
+        s.dem_u[lane][p] = s.Uf[p];
+        s.dem_w[lane][p] = s.Wf[p];
+    } else if (lane == 2) {
+        s.dem_du[p] = s.dem_dw[p] = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    if (fixed) {
         if (lane == 0) s.nb_count[p] = 0;
         return;
     }
@@ -290,32 +264,45 @@ __global__ void k_dem_neighbours(Dev s) {
         const int t = __shfl_up_sync(full, incl, o);
         if (lane >= o) incl += t;
     }
-    const int total = __shfl_sync(full, incl, 31);
+    const int total = min(__shfl_sync(full, incl, 31), NB_SLOTS);
+    if (lane == 31 && incl > NB_SLOTS) set_error(s, ERR_HISTORY);
     int slot = incl - mine;
     for (int k = b; k < e; ++k) {
         const int j = s.g_list[k];
         if (!dem_partner(s, p, j, xri)) continue;
-        if (slot < NB_SLOTS) {
-            s.nb[(long long)p * NB_SLOTS + slot] = j;
-            const int4 ij = s.Xi[j];
-            const float4 fj = s.Xfr[j];
-            s.nb_d0[(long long)p * NB_SLOTS + slot] =
-                make_float4((float)wrap_int(ij.x - ip.x, s.nx, s.per_x) + (fj.x - fp.x),
-                            (float)wrap_int(ij.y - ip.y, s.ny, s.per_y) + (fj.y - fp.y),
-                            (float)wrap_int(ij.z - ip.z, s.nz, s.per_z) + (fj.z - fp.z), 0.f);
-        }
+        if (slot < NB_SLOTS) found[slot] = j;
         ++slot;
     }
-    if (lane == 0) {
-        if (total > NB_SLOTS) set_error(s, ERR_HISTORY);
-        s.nb_count[p] = total > NB_SLOTS ? NB_SLOTS : total;
+    __syncwarp();
+    // lane t: the old list's slot t, then the new list's
+    const int oldn = s.nb_count[p];
+    const long long row = (long long)p * NB_ITEMS;
+    const int oj = lane < oldn ? s.nb[(long long)p * NB_SLOTS + lane] : -1;
+    const float4 oxi = lane < oldn ? s.nb_xi[row + lane] : make_float4(0.f, 0.f, 0.f, 0.f);
+    const int nj = lane < total ? found[lane] : -1;
+    float4 xi = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int t = 0; t < oldn; ++t) {
+        const int j = __shfl_sync(full, oj, t);
+        const float a0 = __shfl_sync(full, oxi.x, t), a1 = __shfl_sync(full, oxi.y, t), a2 = __shfl_sync(full, oxi.z, t);
+        if (nj == j) xi = make_float4(a0, a1, a2, 0.f);
     }
+    if (nj >= 0) {
+        const float4 cp = s.dem_c[p], cj = s.dem_c[nj];
+        const int4 ij = s.Xi[nj];
+        const float4 fj = s.Xfr[nj];
+        s.nb[(long long)p * NB_SLOTS + lane] = nj;
+        s.nb_d0[(long long)p * NB_SLOTS + lane] =
+            make_float4((float)wrap_int(ij.x - ip.x, s.nx, s.per_x) + (fj.x - fp.x),
+                        (float)wrap_int(ij.y - ip.y, s.ny, s.per_y) + (fj.y - fp.y),
+                        (float)wrap_int(ij.z - ip.z, s.nz, s.per_z) + (fj.z - fp.z), cj.x);
+        xi.w = cp.y * cj.y / (cp.y + cj.y);
+        s.nb_xi[row + lane] = xi;
+    }
+    if (lane == 0) s.nb_count[p] = total;
 }
 
 // FP32 copies of the particle state used by the lattice kernels
-__global__ void k_particle_copies(Dev s) {
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= s.np) return;
+__device__ __forceinline__ void particle_copies(const Dev& s, int p) {
     const double X = s.X[3 * p], Y = s.X[3 * p + 1], Z = s.X[3 * p + 2];
     const double r = s.R[p];
     s.Xr[p] = make_float4((float)X, (float)Y, (float)Z, s.fixed[p] ? -(float)r : (float)r);
@@ -326,14 +313,18 @@ __global__ void k_particle_copies(Dev s) {
     s.Wf[p] = make_float4((float)s.W[3 * p], (float)s.W[3 * p + 1], (float)s.W[3 * p + 2], 0.f);
     s.dem_c[p] = make_float4((float)r, (float)s.M[p], (float)s.I[p], 0.f);
 }
+__global__ void k_particle_copies(Dev s) {
+    const int p = blockIdx.x * blockDim.x + threadIdx.x;
+    if (p < s.np) particle_copies(s, p);
+}
 
 void launch_particle_copies(const Dev& s, cudaStream_t st) {
     if (s.np > 0) k_particle_copies<<<blocks_for(s.np, 128), 128, 0, st>>>(s);
 }
 
 // FP32 linear spring-dashpot with tangential history (same law as above)
-__device__ void contact_f(const Dev& s, float meff, const float n[3], float delta, const float vrel[3], float* xi,
-                          float dts, float F[3], float Ft[3]) {
+__device__ __forceinline__ void contact_f(const Dev& s, float meff, const float n[3], float delta,
+                                          const float vrel[3], float xi[3], float dts, float F[3], float Ft[3]) {
     const float kn = meff * (float)s.kn_coef;
     const float dn = meff * (float)s.dn_coef;
     const float kt = kn * (float)s.kt_ratio;
@@ -360,181 +351,281 @@ __device__ void contact_f(const Dev& s, float meff, const float n[3], float delt
     }
 }
 
-// One DEM sub-step, a thread per particle over its neighbour list and the
-// walls, in FP32 (R-25): a particle's position, velocity and angular velocity
-// are its FP64 state at the step's start plus the changes dx, du, dw the
-// sub-steps have made (small numbers, exact to FP32 rounding of themselves);
-// the offset to a partner is the start offset (formed in FP64 with the
-// neighbour list) plus the difference of their dx, a wall distance the start
-// distance plus or minus dx. Contact law and sums in FP32, semi-implicit
-// Euler on the changes; the last sub-step adds them to the FP64 state.
-__global__ void __launch_bounds__(64) k_dem_substep(Dev s, const float* __restrict__ dxa,
-                                                   const float* __restrict__ dua, const float* __restrict__ dwa,
-                                                   float* dxb, float* dub, float* dwb, float dts, int last) {
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= s.np) return;
-    const float dx[3] = {dxa[3 * p], dxa[3 * p + 1], dxa[3 * p + 2]};
-    const float du[3] = {dua[3 * p], dua[3 * p + 1], dua[3 * p + 2]};
-    const float dw[3] = {dwa[3 * p], dwa[3 * p + 1], dwa[3 * p + 2]};
+// One DEM sub-step of particle p by the DEM_LANES lanes of a group (l: the
+// lane in the group, gm: the group's lanes), in FP32 (R-25): a particle's
+// position, velocity and angular velocity are its FP64 state at the step's
+// start plus the changes dx, du, dw the sub-steps have made (small numbers,
+// exact to FP32 rounding of themselves); the offset to a partner is the start
+// offset plus the difference of their dx, a wall distance the start distance
+// plus or minus dx. The particles publish dx, u and w (buffers a read, b
+// written). Lane l takes neighbour slots l, l + DEM_LANES, ... and then wall
+// face l; the lanes' forces join in a fixed tree; lanes 0 to 2 advance one
+// axis each (semi-implicit Euler on the changes). The first sub-step averages
+// the hydrodynamic force over two steps, the last adds the changes to the
+// FP64 state, forms the FP32 copies and counts the particle in its grid cell.
+// Bound by latency: a thread per particle ran its dozen partners one after
+// the other (about 3000 dependent instructions, 18 to 21 us a sub-step whatever
+// the particle count), and searched its 16 spring slots for every contact. Eight
+// lanes per particle with the spring stored beside the partner's slot: 9.7 us
+// for 4 712 particles (19.2 before), 16.5 us for 30 696 (21.4).
+constexpr int DEM_LANES = 8;
+static_assert(NB_SLOTS % DEM_LANES == 0 && NB_ITEMS == NB_SLOTS + DEM_LANES, "one wall face per lane");
+
+__device__ __forceinline__ void dem_substep(const Dev& s, int p, int l, unsigned gm, int a, bool have_prev,
+                                            float dts, bool first, bool last) {
+    const int b = 1 - a;
     if (s.fixed[p]) {
-        for (int a = 0; a < 3; ++a) { dxb[3 * p + a] = dx[a]; dub[3 * p + a] = du[a]; dwb[3 * p + a] = dw[a]; }
-        // the top of the particle cells counts the fixed particles too
-        if (last) atomicMax(s.zmax_cell, (int)ceil(s.X[3 * p + 2] + s.R[p]) + 2);
+        // the top of the particle cells and the grid count the fixed particles too
+        if (last && l == 0) {
+            atomicMax(s.zmax_cell, (int)ceil(s.X[3 * p + 2] + s.R[p]) + 2);
+            atomicAdd(&s.g_count[s.g_of[p]], 1);
+        }
         return;
     }
     const float4 cp = s.dem_c[p];
-    const float rif = cp.x, mif = cp.y, Iif = cp.z;
-    const float4 u0 = s.Uf[p], w0 = s.Wf[p];
-    const float Uf[3] = {u0.x + du[0], u0.y + du[1], u0.z + du[2]};
-    const float Wf[3] = {w0.x + dw[0], w0.y + dw[1], w0.z + dw[2]};
-    float F[3] = {s.Faf[3 * p], s.Faf[3 * p + 1], s.Faf[3 * p + 2]};
-    float T[3] = {s.Taf[3 * p], s.Taf[3 * p + 1], s.Taf[3 * p + 2]};
-    unsigned seen = 0;
-    // the particle's tangential-history partners, held in registers for the
-    // sub-step (slot k: partner index, a wall code, or HIST_EMPTY)
-    int hpart[HIST_SLOTS];
-    {
-        const int4* hp4 = reinterpret_cast<const int4*>(s.hist_partner + (long long)p * HIST_SLOTS);
-#pragma unroll
-        for (int k = 0; k < HIST_SLOTS / 4; ++k) {
-            const int4 v = hp4[k];
-            hpart[4 * k] = v.x; hpart[4 * k + 1] = v.y; hpart[4 * k + 2] = v.z; hpart[4 * k + 3] = v.w;
+    const float4 xa4 = s.dem_x[a][p], ua4 = s.dem_u[a][p], wa4 = s.dem_w[a][p];
+    const int nbc = s.nb_count[p];
+    const float rif = cp.x;
+    // lane k < 3: the outer force and torque along axis k
+    float Fo = 0.f, To = 0.f;
+    if (l < 3) {
+        const int k = 3 * p + l;
+        if (first) {
+            const double fh = s.Fh[k], th = s.Th[k];
+            const double fa = have_prev ? 0.5 * (fh + s.Fp[k]) : fh;
+            const double ta = have_prev ? 0.5 * (th + s.Tp[k]) : th;
+            s.Fp[k] = fh;
+            s.Tp[k] = th;
+            // averaged hydrodynamic force plus the weight
+            const double g = l == 0 ? s.gxd : (l == 1 ? s.gyd : s.gzd);
+            Fo = (float)(fa + s.M[p] * g);
+            To = (float)ta;
+            s.Faf[k] = Fo;
+            s.Taf[k] = To;
+        } else {
+            Fo = s.Faf[k];
+            To = s.Taf[k];
         }
     }
-    const int nbc = s.nb_count[p];
-    const int* nbl = s.nb + (long long)p * NB_SLOTS;
-    const float4* nd0 = s.nb_d0 + (long long)p * NB_SLOTS;
-    // neighbours four at a time: their indices, offsets and changes load together
-    for (int k0 = 0; k0 < nbc; k0 += 4) {
-        int jj[4];
-        float4 d0[4], cj[4];
-        float dxj[4][3];
+    float F[3] = {0.f, 0.f, 0.f}, T[3] = {0.f, 0.f, 0.f};
+    int touching = 0;
+    const int nround = (nbc + DEM_LANES - 1) / DEM_LANES;   // rounds of neighbours, then one of wall faces
+#pragma unroll 1
+    for (int r = 0; r <= nround; ++r) {
+        const bool wall = r == nround;
+        const int slot = wall ? NB_SLOTS + l : r * DEM_LANES + l;
+        bool near = false, touch = false;
+        float n[3] = {0.f, 0.f, 0.f}, delta = 0.f, rj = 0.f;
+        float4 uj = make_float4(0.f, 0.f, 0.f, 0.f), wj = uj, xi4 = uj;
+        if (!wall) {
+            if (slot < nbc) {
+                const int j = s.nb[(long long)p * NB_SLOTS + slot];
+                const float4 d0 = s.nb_d0[(long long)p * NB_SLOTS + slot];
+                xi4 = s.nb_xi[(long long)p * NB_ITEMS + slot];
+                const float4 xj = s.dem_x[a][j];
+                uj = s.dem_u[a][j];
+                wj = s.dem_w[a][j];
+                rj = d0.w;
+                const float d[3] = {d0.x + (xj.x - xa4.x), d0.y + (xj.y - xa4.y), d0.z + (xj.z - xa4.z)};
+                const float dist2 = d[0] * d[0] + d[1] * d[1] + d[2] * d[2];
+                const float rs = rif + rj;
+                touch = dist2 < rs * rs;
+                near = touch || (s.lub && dist2 < (rs + LUB_HC) * (rs + LUB_HC));
+                const float dist = sqrtf(dist2);
+                const float inv = 1.f / dist;
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            jj[u] = k0 + u < nbc ? nbl[k0 + u] : -1;
-            d0[u] = k0 + u < nbc ? nd0[k0 + u] : make_float4(0.f, 0.f, 0.f, 0.f);
+                for (int k = 0; k < 3; ++k) n[k] = d[k] * inv;
+                delta = rs - dist;
+            }
+        } else if (l < 6) {
+            const int ax = l >> 1;
+            if (!(ax == 0 ? s.per_x : (ax == 1 ? s.per_y : s.per_z))) {
+                const float dxa = ax == 0 ? xa4.x : (ax == 1 ? xa4.y : xa4.z);
+                const float dist = (l & 1) ? s.dem_wall[6 * p + l] - dxa : s.dem_wall[6 * p + l] + dxa;
+                delta = rif - dist;
+                touch = delta > 0.f;
+                near = touch || (s.lub && -delta < LUB_HC);
+                const float sg = (l & 1) ? 1.f : -1.f;
+#pragma unroll
+                for (int k = 0; k < 3; ++k) n[k] = k == ax ? sg : 0.f;
+                xi4 = s.nb_xi[(long long)p * NB_ITEMS + slot];
+                xi4.w = cp.y;   // the wall's mass is infinite
+            }
         }
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            cj[u] = jj[u] >= 0 ? s.dem_c[jj[u]] : make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-            for (int a = 0; a < 3; ++a) dxj[u][a] = jj[u] >= 0 ? dxa[3 * jj[u] + a] : 0.f;
-        }
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const int j = jj[u];
-            if (j < 0) continue;
-            const float d[3] = {d0[u].x + (dxj[u][0] - dx[0]), d0[u].y + (dxj[u][1] - dx[1]),
-                                d0[u].z + (dxj[u][2] - dx[2])};
-            const float rjf = cj[u].x;
-            const float dist2 = d[0] * d[0] + d[1] * d[1] + d[2] * d[2];
-            const float rs = rif + rjf;
-            const bool touch = dist2 < rs * rs;
-            const bool lub = s.lub && dist2 < (rs + LUB_HC) * (rs + LUB_HC);
-            if (!touch && !lub) continue;
-            const float dist = sqrtf(dist2);
-            const float inv = 1.f / dist;
-            const float n[3] = {d[0] * inv, d[1] * inv, d[2] * inv};
-            const float delta = rs - dist;
-            const float4 uj0 = s.Uf[j], wj0 = s.Wf[j];
-            const float Uj[3] = {uj0.x + dua[3 * j], uj0.y + dua[3 * j + 1], uj0.z + dua[3 * j + 2]};
-            const float Wj[3] = {wj0.x + dwa[3 * j], wj0.y + dwa[3 * j + 1], wj0.z + dwa[3 * j + 2]};
-            float wsum[3];
-            for (int a = 0; a < 3; ++a) wsum[a] = rif * Wf[a] + rjf * Wj[a];
+        if (near) {
+            const float wsum[3] = {rif * wa4.x + rj * wj.x, rif * wa4.y + rj * wj.y, rif * wa4.z + rj * wj.z};
             const float wn[3] = {wsum[1] * n[2] - wsum[2] * n[1], wsum[2] * n[0] - wsum[0] * n[2],
                                  wsum[0] * n[1] - wsum[1] * n[0]};
-            float vrel[3];
-            for (int a = 0; a < 3; ++a) vrel[a] = Uf[a] - Uj[a] + wn[a];
-            if (lub) {
+            const float vrel[3] = {ua4.x - uj.x + wn[0], ua4.y - uj.y + wn[1], ua4.z - uj.z + wn[2]};
+            float Ft[3] = {0.f, 0.f, 0.f};   // tangential, for the torque
+            if (s.lub && delta > -LUB_HC) {
                 float Fl[3], Ftl[3];
-                lub_f(s, rif * rjf / rs, n, -delta, vrel, Fl, Ftl);
-                const float tq[3] = {rif * (n[1] * Ftl[2] - n[2] * Ftl[1]), rif * (n[2] * Ftl[0] - n[0] * Ftl[2]),
-                                     rif * (n[0] * Ftl[1] - n[1] * Ftl[0])};
-                for (int a = 0; a < 3; ++a) { F[a] += Fl[a]; T[a] += tq[a]; }
-            }
-            if (!touch) continue;
-            const float mj = cj[u].y;
-            const float meff = mif * mj / (mif + mj);
-            const int slot = hist_slot(s, p, j, hpart, seen);
-            if (slot < 0) continue;
-            float* xi = s.hist_xi + ((long long)p * HIST_SLOTS + slot) * 3;
-            float Fc[3], Ft[3];
-            contact_f(s, meff, n, delta, vrel, xi, dts, Fc, Ft);
-            const float tq[3] = {rif * (n[1] * Ft[2] - n[2] * Ft[1]), rif * (n[2] * Ft[0] - n[0] * Ft[2]),
-                                 rif * (n[0] * Ft[1] - n[1] * Ft[0])};
-            for (int a = 0; a < 3; ++a) { F[a] += Fc[a]; T[a] += tq[a]; }
-        }
-    }
-    // walls on non-periodic axes
-    const int per[3] = {s.per_x, s.per_y, s.per_z};
-    for (int a = 0; a < 3; ++a) {
-        if (per[a]) continue;
-        for (int side = 0; side < 2; ++side) {
-            const float dist = side == 0 ? s.dem_wall[6 * p + 2 * a] + dx[a] : s.dem_wall[6 * p + 2 * a + 1] - dx[a];
-            const float delta = rif - dist;
-            const bool lub = s.lub && -delta < LUB_HC;
-            if (delta <= 0.f && !lub) continue;
-            float n[3] = {0.f, 0.f, 0.f};
-            n[a] = side == 0 ? -1.f : 1.f;
-            const float rw[3] = {rif * Wf[0], rif * Wf[1], rif * Wf[2]};
-            const float wn[3] = {rw[1] * n[2] - rw[2] * n[1], rw[2] * n[0] - rw[0] * n[2],
-                                 rw[0] * n[1] - rw[1] * n[0]};
-            const float vrel[3] = {Uf[0] + wn[0], Uf[1] + wn[1], Uf[2] + wn[2]};
-            if (lub) {
-                float Fl[3], Ftl[3];
-                lub_f(s, rif, n, -delta, vrel, Fl, Ftl);
-                const float tq[3] = {rif * (n[1] * Ftl[2] - n[2] * Ftl[1]), rif * (n[2] * Ftl[0] - n[0] * Ftl[2]),
-                                     rif * (n[0] * Ftl[1] - n[1] * Ftl[0])};
-                for (int b = 0; b < 3; ++b) { F[b] += Fl[b]; T[b] += tq[b]; }
-            }
-            if (delta <= 0.f) continue;
-            const int slot = hist_slot(s, p, -1 - (2 * a + side), hpart, seen);
-            if (slot < 0) continue;
-            float* xi = s.hist_xi + ((long long)p * HIST_SLOTS + slot) * 3;
-            float Fc[3], Ft[3];
-            contact_f(s, mif, n, delta, vrel, xi, dts, Fc, Ft);
-            const float tq[3] = {rif * (n[1] * Ft[2] - n[2] * Ft[1]), rif * (n[2] * Ft[0] - n[0] * Ft[2]),
-                                 rif * (n[0] * Ft[1] - n[1] * Ft[0])};
-            for (int b = 0; b < 3; ++b) { F[b] += Fc[b]; T[b] += tq[b]; }
-        }
-    }
-    // partners not met in this sub-step lose their springs
-    {
-        int4* hp4 = reinterpret_cast<int4*>(s.hist_partner + (long long)p * HIST_SLOTS);
+                lub_f(s, wall ? rif : rif * rj / (rif + rj), n, -delta, vrel, Fl, Ftl);
 #pragma unroll
-        for (int k = 0; k < HIST_SLOTS / 4; ++k) {
-            int4 v;
-            v.x = (seen >> (4 * k)) & 1u ? hpart[4 * k] : HIST_EMPTY;
-            v.y = (seen >> (4 * k + 1)) & 1u ? hpart[4 * k + 1] : HIST_EMPTY;
-            v.z = (seen >> (4 * k + 2)) & 1u ? hpart[4 * k + 2] : HIST_EMPTY;
-            v.w = (seen >> (4 * k + 3)) & 1u ? hpart[4 * k + 3] : HIST_EMPTY;
-            hp4[k] = v;
+                for (int k = 0; k < 3; ++k) { F[k] += Fl[k]; Ft[k] = Ftl[k]; }
+            }
+            if (touch) {
+                float xi[3] = {xi4.x, xi4.y, xi4.z}, Fc[3], Ftc[3];
+                contact_f(s, xi4.w, n, delta, vrel, xi, dts, Fc, Ftc);
+                s.nb_xi[(long long)p * NB_ITEMS + slot] = make_float4(xi[0], xi[1], xi[2], xi4.w);
+#pragma unroll
+                for (int k = 0; k < 3; ++k) { F[k] += Fc[k]; Ft[k] += Ftc[k]; }
+            }
+            T[0] += rif * (n[1] * Ft[2] - n[2] * Ft[1]);
+            T[1] += rif * (n[2] * Ft[0] - n[0] * Ft[2]);
+            T[2] += rif * (n[0] * Ft[1] - n[1] * Ft[0]);
         }
+        // a partner not touched in this sub-step loses its spring
+        if (!touch && (xi4.x != 0.f || xi4.y != 0.f || xi4.z != 0.f))
+            s.nb_xi[(long long)p * NB_ITEMS + slot] = make_float4(0.f, 0.f, 0.f, xi4.w);
+        touching += touch ? 1 : 0;
     }
-    // semi-implicit Euler on the changes
-    const float im = 1.f / mif, iI = 1.f / Iif;
-    float dxn[3], dun[3], dwn[3];
-    for (int a = 0; a < 3; ++a) {
-        dun[a] = du[a] + dts * F[a] * im;
-        dwn[a] = dw[a] + dts * T[a] * iI;
-        const float u0a = a == 0 ? u0.x : (a == 1 ? u0.y : u0.z);
-        dxn[a] = dx[a] + dts * (u0a + dun[a]);
-        dxb[3 * p + a] = dxn[a];
-        dub[3 * p + a] = dun[a];
-        dwb[3 * p + a] = dwn[a];
+#pragma unroll
+    for (int o = 1; o < DEM_LANES; o <<= 1) {
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            F[k] += __shfl_xor_sync(gm, F[k], o);
+            T[k] += __shfl_xor_sync(gm, T[k], o);
+        }
+        touching += __shfl_xor_sync(gm, touching, o);
+    }
+    if (touching > HIST_SLOTS && l == 0) set_error(s, ERR_HISTORY);
+    // lane l < 3 (the others repeat lane 2's) advances axis l
+    const int ax = l < 3 ? l : 2;
+    auto sel = [ax](float v0, float v1, float v2) { return ax == 0 ? v0 : (ax == 1 ? v1 : v2); };
+    const float dxo = sel(xa4.x, xa4.y, xa4.z);
+    float* duo = reinterpret_cast<float*>(s.dem_du + p) + ax;
+    float* dwo = reinterpret_cast<float*>(s.dem_dw + p) + ax;
+    const float4 u0 = s.Uf[p], w0 = s.Wf[p];
+    const float u0a = sel(u0.x, u0.y, u0.z), w0a = sel(w0.x, w0.y, w0.z);
+    const float dun = *duo + dts * (Fo + sel(F[0], F[1], F[2])) * (1.f / cp.y);
+    const float dwn = *dwo + dts * (To + sel(T[0], T[1], T[2])) * (1.f / cp.z);
+    const float dxn = dxo + dts * (u0a + dun);
+    __syncwarp(gm);   // every lane has read du and dw, and the copies Uf and Wf
+    if (l < 3 && !last) {
+        *duo = dun;
+        *dwo = dwn;
+        reinterpret_cast<float*>(s.dem_x[b] + p)[l] = dxn;
+        reinterpret_cast<float*>(s.dem_u[b] + p)[l] = u0a + dun;
+        reinterpret_cast<float*>(s.dem_w[b] + p)[l] = w0a + dwn;
     }
     if (last) {
-        // the FP64 state of the step's end (positions wrapped on periodic axes)
-        const int L[3] = {s.nx, s.ny, s.nz};
-        for (int a = 0; a < 3; ++a) {
-            double x = s.X[3 * p + a] + (double)dxn[a];
-            if (per[a]) x = x < 0.0 ? x + L[a] : (x >= L[a] ? x - L[a] : x);
-            s.X[3 * p + a] = x;
-            s.U[3 * p + a] += (double)dun[a];
-            s.W[3 * p + a] += (double)dwn[a];
+        // the FP64 state of the step's end (positions wrapped on periodic
+        // axes), its FP32 copies and the grid cell
+        int g = 0;
+        if (l < 3) {
+            const int L = l == 0 ? s.nx : (l == 1 ? s.ny : s.nz);
+            double x = s.X[3 * p + l] + (double)dxn;
+            if (l == 0 ? s.per_x : (l == 1 ? s.per_y : s.per_z)) x = x < 0.0 ? x + L : (x >= L ? x - L : x);
+            const double u = s.U[3 * p + l] + (double)dun, w = s.W[3 * p + l] + (double)dwn;
+            s.X[3 * p + l] = x;
+            s.U[3 * p + l] = u;
+            s.W[3 * p + l] = w;
+            const double fl = floor(x);
+            reinterpret_cast<float*>(s.Xr + p)[l] = (float)x;
+            reinterpret_cast<int*>(s.Xi + p)[l] = (int)fl;
+            reinterpret_cast<float*>(s.Xfr + p)[l] = (float)(x - fl);
+            reinterpret_cast<float*>(s.Uf + p)[l] = (float)u;
+            reinterpret_cast<float*>(s.Wf + p)[l] = (float)w;
+            if (l == 2) atomicMax(s.zmax_cell, (int)ceil(x + s.R[p]) + 2);
+            g = l == 0 ? gcoord(x, s.ghx, s.gnx)
+                       : (l == 1 ? s.gnx * gcoord(x, s.ghy, s.gny) : s.gnx * s.gny * gcoord(x, s.ghz, s.gnz));
         }
-        atomicMax(s.zmax_cell, (int)ceil(s.X[3 * p + 2] + s.R[p]) + 2);
+        g += __shfl_xor_sync(gm, g, 1);
+        g += __shfl_xor_sync(gm, g, 2);
+        if (l == 0) {
+            s.g_of[p] = g;
+            atomicAdd(&s.g_count[g], 1);
+        }
     }
+}
+
+// one sub-step; the first of several also clears what the last one counts
+__global__ void __launch_bounds__(128) k_dem_substep(Dev s, int a, int have_prev, int G, float dts, int first,
+                                                     int last) {
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (first && !last) {
+        for (int g = t; g < G; g += gridDim.x * blockDim.x) s.g_count[g] = 0;
+        if (t == 0) *s.zmax_cell = 0;
+    }
+    const int p = t / DEM_LANES, l = t % DEM_LANES;
+    const unsigned gm = ((1u << DEM_LANES) - 1u) << ((threadIdx.x & 31) / DEM_LANES * DEM_LANES);
+    if (p < s.np) dem_substep(s, p, l, gm, a, have_prev != 0, dts, first != 0, last != 0);
+}
+
+// The sub-steps of a step and the particle grid in one thread-block cluster,
+// for up to DEM_CLUSTER_MAX particles: the cluster's hardware barrier
+// (release at arrival, acquire at the wait) stands between the phases that
+// read other particles' values, so nothing is launched between the sub-steps.
+// Measured for the whole DEM half (ten sub-steps and the grid): 52 us for 34
+// particles, 113 us for 1 008 (two per lane group), against ten launches of
+// 9.7 us plus three of the grid; beyond 1 024 particles a lane group would take
+// three and more in turn, and the launches win.
+constexpr int DEM_CLUSTER_MAX = 1024;
+constexpr int DEM_CLUSTER_CTAS = 8;
+constexpr int DEM_CLUSTER_THREADS = 512;
+
+__device__ __forceinline__ void cluster_barrier() {
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+__global__ void __launch_bounds__(DEM_CLUSTER_THREADS) k_dem_cluster(Dev s, int have_prev, int G, float dts) {
+    __shared__ int wtot[DEM_CLUSTER_THREADS / 32];
+    const int nt = gridDim.x * blockDim.x, tid = blockIdx.x * blockDim.x + threadIdx.x;   // one cluster: the grid
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    const unsigned full = 0xffffffffu;
+    const int l = tid % DEM_LANES;
+    const unsigned gm = ((1u << DEM_LANES) - 1u) << (lane / DEM_LANES * DEM_LANES);
+    for (int g = tid; g < G; g += nt) s.g_count[g] = 0;
+    if (tid == 0) *s.zmax_cell = 0;
+    cluster_barrier();
+    for (int k = 0; k < s.dem_substeps; ++k) {
+        for (int p = tid / DEM_LANES; p < s.np; p += nt / DEM_LANES)
+            dem_substep(s, p, l, gm, k & 1, have_prev != 0, dts, k == 0, k == s.dem_substeps - 1);
+        cluster_barrier();
+    }
+    // exclusive scan of the grid counts: each CTA scans a contiguous run of
+    // rows of 32 counts, a warp a part of it; the CTAs' totals pass through g_tot
+    const int rows = (G + 31) / 32;
+    const int cper = (rows + gridDim.x - 1) / gridDim.x;
+    const int c0 = blockIdx.x * cper, c1 = min(rows, c0 + cper);
+    const int per = (cper + nw - 1) / nw;
+    const int r0 = min(c1, c0 + warp * per), r1 = min(c1, r0 + per);
+    int sum = 0;
+    for (int r = r0; r < r1; ++r) {
+        const int i = 32 * r + lane;
+        sum += i < G ? s.g_count[i] : 0;
+    }
+    for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(full, sum, o);
+    if (lane == 0) wtot[warp] = sum;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        int t = 0;
+        for (int w = 0; w < nw; ++w) t += wtot[w];
+        s.g_tot[blockIdx.x] = t;
+    }
+    cluster_barrier();
+    int run = 0;
+    for (int c = 0; c < (int)blockIdx.x; ++c) run += s.g_tot[c];
+    for (int w = 0; w < warp; ++w) run += wtot[w];
+    for (int r = r0; r < r1; ++r) {
+        const int i = 32 * r + lane;
+        const int c = i < G ? s.g_count[i] : 0;
+        int v = c;
+        for (int o = 1; o < 32; o <<= 1) {
+            const int u = __shfl_up_sync(full, v, o);
+            if (lane >= o) v += u;
+        }
+        if (i < G) {
+            s.g_start[i] = run + v - c;
+            s.g_cursor[i] = run + v - c;
+        }
+        run += __shfl_sync(full, v, 31);
+    }
+    cluster_barrier();
+    for (int p = tid; p < s.np; p += nt) grid_fill(s, p);
+    cluster_barrier();
+    for (int g = tid; g < G; g += nt) grid_sort(s, g);
 }
 
 // ------------------------------------------------------------ particle map
@@ -983,28 +1074,49 @@ __global__ void k_repair(Dev s) {
     }
 }
 
-// The particle part of a step in two halves. The DEM half (force average,
-// neighbour list, sub-steps, FP32 copies, particle grid) reads and writes
-// particle state only, so it can run beside the free-surface conversion,
-// which reads and writes cell state only; the re-map half needs both.
+// The particle part of a step in two halves. The DEM half (neighbour list,
+// force average, sub-steps, FP32 copies, particle grid) reads and writes
+// particle state only, so it can run beside the fluid kernels and the
+// free-surface conversion, which read and write cell state only; the re-map
+// half needs both. The neighbour list needs the positions alone, so it is
+// launched at the step's start, the rest once the particle forces are complete.
+int launch_dem_neighbours(const Dev& s, cudaStream_t st) {
+    if (s.np == 0) return 0;
+    k_dem_neighbours<<<blocks_for(32LL * s.np, 128), 128, 0, st>>>(s);
+    return 1;
+}
+
 int launch_dem(const Dev& s, int have_prev, cudaStream_t st) {
     if (s.np == 0) return 0;
-    int launches = 0;
-    const int n3 = 3 * s.np;
-    const int ns = s.dem_substeps;
-    k_force_avg<<<blocks_for(n3, 128), 128, 0, st>>>(s, have_prev);
-    k_dem_neighbours<<<blocks_for(32LL * s.np, 128), 128, 0, st>>>(s);
-    cudaMemsetAsync(s.zmax_cell, 0, sizeof(int), st);
-    launches += 2 + ns;
+    const int ns = s.dem_substeps, G = s.gnx * s.gny * s.gnz;
     const float dts = 1.f / (float)ns;
-    for (int k = 0; k < ns; ++k) {
-        const int a = k % 2, b = 1 - a;
-        k_dem_substep<<<blocks_for(s.np, 64), 64, 0, st>>>(s, s.dem_dx[a], s.dem_du[a], s.dem_dw[a], s.dem_dx[b],
-                                                          s.dem_du[b], s.dem_dw[b], dts, k == ns - 1);
+    if (s.np <= DEM_CLUSTER_MAX) {
+        // as many CTAs (a power of two) as give one warp per scheduler
+        int ctas = 1;
+        while (ctas < DEM_CLUSTER_CTAS && ctas * 128 < s.np * DEM_LANES) ctas *= 2;
+        int threads = ((s.np * DEM_LANES + ctas - 1) / ctas + 31) / 32 * 32;
+        threads = threads < 128 ? 128 : (threads > DEM_CLUSTER_THREADS ? DEM_CLUSTER_THREADS : threads);
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3((unsigned)ctas);
+        cfg.blockDim = dim3((unsigned)threads);
+        cfg.stream = st;
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = (unsigned)ctas;
+        at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+        cfg.attrs = at;
+        cfg.numAttrs = 1;
+        cudaLaunchKernelEx(&cfg, k_dem_cluster, s, have_prev, G, dts);
+        return 1;
     }
-    k_particle_copies<<<blocks_for(s.np, 128), 128, 0, st>>>(s);
-    launches += 1 + launch_grid_build(s, st);
-    return launches;
+    if (ns == 1) {
+        cudaMemsetAsync(s.g_count, 0, sizeof(int) * G, st);
+        cudaMemsetAsync(s.zmax_cell, 0, sizeof(int), st);
+    }
+    for (int k = 0; k < ns; ++k)
+        k_dem_substep<<<blocks_for((long long)DEM_LANES * s.np, 128), 128, 0, st>>>(s, k & 1, have_prev, G, dts, k == 0,
+                                                                                   k == ns - 1);
+    return ns + launch_grid_lists(s, st);
 }
 
 int launch_remap(const Dev& s, int last_parity, cudaStream_t st) {
@@ -1032,9 +1144,9 @@ __global__ void k_init_particles(Dev s, int first, int count, double rho_p) {
     for (int a = 0; a < 3; ++a) {
         s.U[3 * p + a] = s.W[3 * p + a] = 0.0;
         s.Fh[3 * p + a] = s.Th[3 * p + a] = s.Fp[3 * p + a] = s.Tp[3 * p + a] = 0.0;
-        s.Fa[3 * p + a] = s.Ta[3 * p + a] = 0.0;
     }
-    for (int j = 0; j < HIST_SLOTS; ++j) s.hist_partner[(long long)p * HIST_SLOTS + j] = HIST_EMPTY;
+    s.nb_count[p] = 0;
+    for (int j = 0; j < NB_ITEMS; ++j) s.nb_xi[(long long)p * NB_ITEMS + j] = make_float4(0.f, 0.f, 0.f, 0.f);
     s.margin[p] = 0.f;
     // the set-up map (k_remap_all) flags every particle that shares a cell;
     // the others re-map their thin shell from the first step on
