@@ -348,7 +348,7 @@ int fslbm_create(const fslbm_params* p, void* cuda_stream, fslbm** out) {
             d.tl_count = counts + 2;
             d.zmax_cell = counts + 3;
             d.err = counts + 4;
-            d.act_count = counts + 5;
+            d.cls_done = counts + 5;
             d.dl_count = counts + 6;
             d.sl_count = counts + 7;
             d.tile_count = counts + 8;
@@ -388,15 +388,14 @@ int fslbm_create(const fslbm_params* p, void* cuda_stream, fslbm** out) {
         d.Xfr = dalloc<float4>(s, pc, ok);
         d.Uf = dalloc<float4>(s, pc, ok);
         d.Wf = dalloc<float4>(s, pc, ok);
-        d.Fh = dalloc<double>(s, 3 * pc, ok); d.Th = dalloc<double>(s, 3 * pc, ok);
+        d.Fh = dalloc<double>(s, 6 * pc, ok);   // force, then torque: one clear
+        d.Th = d.Fh + 3 * pc;
         d.Fp = dalloc<double>(s, 3 * pc, ok); d.Tp = dalloc<double>(s, 3 * pc, ok);
         d.nb = dalloc<int>(s, pc * NB_SLOTS, ok);
         d.nb_count = dalloc<int>(s, pc, ok);
         d.g_of = dalloc<int>(s, pc, ok);
         d.Xm = dalloc<double>(s, 3 * pc, ok);
-        d.margin = dalloc<float>(s, pc, ok);
         d.shared = dalloc<int>(s, pc, ok);
-        d.act = dalloc<int>(s, pc, ok);
         d.dirty = dalloc<uint8_t>(s, n + 4, ok);
         d.scratch_a = dalloc<uint8_t>(s, n, ok);
         d.scratch_b = dalloc<uint8_t>(s, n, ok);
@@ -462,7 +461,7 @@ int fslbm_create(const fslbm_params* p, void* cuda_stream, fslbm** out) {
     cudaMemsetAsync(d.fixowner, 0xff, n * sizeof(int), st);
     cudaMemsetAsync(d.segflag, 0, (size_t)d.nsegx * p->ny * p->nz + 4, st);
     launch_init_flat(d, p->liquid_height, st);
-    launch_classify(d, st);
+    launch_classify(d, false, st);
     launch_normals(d, d.nrm, st);
     if (launch_check(s) || sync_check(s)) {
         int e = s->host_err;
@@ -531,7 +530,7 @@ int fslbm_add_spheres(fslbm* s, int64_t n, const double* xyz, const double* radi
         cudaMemcpyAsync(d.R, R.data(), sizeof(double) * n, cudaMemcpyHostToDevice, st);
         cudaMemcpyAsync(d.fixed, F.data(), n, cudaMemcpyHostToDevice, st);
         launch_particles_add(d, 0, (int)n, st);
-        launch_classify(d, st);
+        launch_classify(d, false, st);
         launch_normals(d, d.nrm, st);
     }
     s->spheres_added = true;
@@ -547,7 +546,7 @@ int fslbm_init_surface(fslbm* s, const double* height_xy, int on_device) {
     const size_t cnt = (size_t)d.nx * d.ny;
     cudaMemcpyAsync(s->stage, height_xy, cnt * sizeof(double), kind_from(on_device), s->st);
     launch_init_surface(d, s->stage, s->st);
-    launch_classify(d, s->st);
+    launch_classify(d, false, s->st);
     launch_normals(d, d.nrm, s->st);
     launch_check(s);
     return sync_check(s);
@@ -561,8 +560,7 @@ static int enqueue_step(fslbm* s, int parity, bool capturing) {
     Dev& d = s->d;
     cudaStream_t st = s->st;
     if (d.np > 0) {
-        cudaMemsetAsync(d.Fh, 0, sizeof(double) * 3 * d.np, st);
-        cudaMemsetAsync(d.Th, 0, sizeof(double) * 3 * d.np, st);
+        cudaMemset2DAsync(d.Fh, sizeof(double) * 3 * d.np_cap, 0, sizeof(double) * 3 * d.np, 2, st);
     }
     int nl = 0;
     if (d.np > 0) {
@@ -607,7 +605,7 @@ static int enqueue_step(fslbm* s, int parity, bool capturing) {
         cudaStreamWaitEvent(st, s->ev_join, 0);
         nl += launch_remap(d, parity, st);
     }
-    nl += launch_classify(d, st);
+    nl += launch_classify(d, true, st);
     nl += launch_pool_spread(d, st);
     nl += launch_normals(d, d.nrm, st);
     return nl;

@@ -93,6 +93,7 @@ struct Dev {
     // z that of the cell whose index the slot carries
     const float* href;
     // work lists (device counts)
+    int* cls_done;                              // blocks of the classification done
     int* wl; int* wl_count; int wl_cap;        // interface cells
     int* nl; int* nl_count; int nl_cap;        // cells becoming interface this step
     int* cl; int* cl_count;                    // interface cells converting this step (capacity wl_cap)
@@ -154,10 +155,8 @@ struct Dev {
     int* g_tot;                                 // the grid scan's partial totals (one per CTA of a cluster)
     double r_max;
     int* zmax_cell;
-    // incremental re-mapping: position of the last map, margin to the nearest
-    // cell centre, shared-cell flag, active particles and their cells
+    // incremental re-mapping: position of the last map, shared-cell flag
     double* Xm;
-    float* margin;
     // learned normal: operand copies of the network (null: Parker-Youngs)
     // and counters of stencils evaluated / normals taken from the network
     const struct MlpBf16* mlp;
@@ -168,7 +167,6 @@ struct Dev {
     const struct MlpFrag* mlp_frag;
     int mlp_mirror;
     int* shared;
-    int* act; int* act_count;
     uint8_t* dirty;
     uint8_t* scratch_a; uint8_t* scratch_b;     // byte fields for the neighbourhood OR
     int* dl; int* dl_count; int dl_cap;
@@ -585,6 +583,55 @@ __device__ __forceinline__ void store_fstar(const Dev& s, long long cell, int la
 #pragma unroll
     for (int q = 0; q < 27; ++q) st_any(s, s.f, fstar_slot(s, q, x, y, z, cell, last_parity), f[q]);
 }
+// Slot of the post-collision PDF f*_q of a cell at height z with the neighbour
+// offsets o (the slot of fstar_slot), and the storage reference h of that
+// slot's z (0 at FP32)
+template <typename S, int LP>
+__device__ __forceinline__ long long pdf_slot(const Dev& s, int q, long long c, int z, const NbrOffsets& o, float& h) {
+    const bool own = LP == 0 || (o.wall & wall_bits(cx(q), cy(q), cz(q)));
+    h = Store<S>::HREF ? s.href[own ? z : wrap_z(s, z + cz(q))] : 0.f;
+    return own ? (long long)opp(q) * s.n + c
+               : (long long)q * s.n + c + (o.ox[1 + cx(q)] + o.oy[1 + cy(q)] + o.oz[1 + cz(q)]);
+}
+// f - w from a stored value and its slot's reference, with one rounding (the
+// same bits wherever it is inlined)
+template <typename S>
+__device__ __forceinline__ float with_ref(float v, int q, float h) {
+    return Store<S>::HREF ? __fmaf_rn(wq(q), h, v) : v;
+}
+// f - w of all 27 post-collision PDFs of a cell, the loads in flight together
+template <typename S, int LP>
+__device__ __forceinline__ void load_cell(const Dev& s, int c, int x, int y, int z, float (&f)[27]) {
+    const S* base = static_cast<const S*>(s.f);
+    const NbrOffsets o = nbr_offsets(s, x, y, z);
+#pragma unroll
+    for (int q = 0; q < 27; ++q) {
+        float h;
+        const long long a = pdf_slot<S, LP>(s, q, c, z, o, h);
+        f[q] = with_ref<S>(Store<S>::ld(base + a), q, h);
+    }
+}
+// Neighbour c + c_q of a cell for a direction known at run time only (a lane
+// per direction), -1 beyond a wall face
+__device__ __forceinline__ int nbr_q(const Dev& s, int x, int y, int z, int q) {
+    const int a = shift(x, q % 3 - 1, s.nx, s.per_x);
+    const int b = shift(y, (q / 3) % 3 - 1, s.ny, s.per_y);
+    const int d = shift(z, q / 9 - 1, s.nz, s.per_z);
+    return (a | b | d) < 0 ? -1 : a + s.nx * (b + s.ny * d);
+}
+// the same cell's slot of f*_q, from that neighbour, and its reference
+template <typename S, int LP>
+__device__ __forceinline__ long long lane_slot(const Dev& s, int q, int c, int nb, int z, float& h) {
+    const bool own = LP == 0 || nb < 0;
+    h = Store<S>::HREF ? s.href[own ? z : wrap_z(s, z + q / 9 - 1)] : 0.f;
+    return own ? (long long)(26 - q) * s.n + c : (long long)q * s.n + nb;
+}
+__device__ __forceinline__ float warp_sum_f(float v) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+}
+
 // density and collision velocity from post-collision PDFs (f - w):
 // rho = 1 + sum, u = (sum c f* - rho g / 2) / rho
 __device__ __forceinline__ void post_moments(const Dev& s, const float (&f)[27], float& rho, float& ux, float& uy,
@@ -611,7 +658,7 @@ __device__ __forceinline__ void post_moments(const Dev& s, const float (&f)[27],
 // step are complete: after the link pass, or after the sweep with fluid-side
 // links
 int launch_stream_collide(const Dev& s, int parity, cudaStream_t st, cudaEvent_t links_done);
-int launch_classify(const Dev& s, cudaStream_t st);
+int launch_classify(const Dev& s, bool spread, cudaStream_t st);
 void launch_check_invariant(const Dev& s, cudaStream_t st);
 int launch_normals(const Dev& s, float4* out, cudaStream_t st);
 void launch_log_stencils(const Dev& s, long long cap, float* fill, float* target, float* fd, int* cells,

@@ -38,23 +38,6 @@ struct Sum3 {
     }
 };
 
-// Slot of the post-collision PDF f*_q of a cell at height z with the neighbour
-// offsets o (the slot of fstar_slot), and the storage reference h of that
-// slot's z (0 at FP32)
-template <typename S, int LP>
-__device__ __forceinline__ long long pdf_slot(const Dev& s, int q, long long c, int z, const NbrOffsets& o, float& h) {
-    const bool own = LP == 0 || (o.wall & wall_bits(cx(q), cy(q), cz(q)));
-    h = Store<S>::HREF ? s.href[own ? z : wrap_z(s, z + cz(q))] : 0.f;
-    return own ? (long long)opp(q) * s.n + c
-               : (long long)q * s.n + c + (o.ox[1 + cx(q)] + o.oy[1 + cy(q)] + o.oz[1 + cz(q)]);
-}
-// f - w from a stored value and its slot's reference, with one rounding (the
-// same bits wherever it is inlined)
-template <typename S>
-__device__ __forceinline__ float with_ref(float v, int q, float h) {
-    return Store<S>::HREF ? __fmaf_rn(wq(q), h, v) : v;
-}
-
 // The selected cell fields in one pass, a thread per cell: the flag and the
 // 27 PDFs are read once, every output is written coalesced, with no staging
 // copy. Bound by the FP64 outputs (216 of about 270-330 bytes per cell for the

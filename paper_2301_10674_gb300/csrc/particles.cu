@@ -648,16 +648,26 @@ __device__ __forceinline__ double image_centre(int k, double X, int L, int perio
     return c;
 }
 
+// grid coordinates along one axis that particles covering cell k can have:
+// those of [k + 1/2 - r_max, k + 1/2 + r_max], in FP32 with a margin above its
+// rounding (the division in FP64 cost more than all the rest of a cell's
+// map; a grid cell too many only adds candidates). Grid cells are at least
+// 2 r_max + 1 wide, so the range holds two of them (three for very large radii).
+__device__ __forceinline__ GRange cover_range(int k, double r_max, double h, int g, int periodic) {
+    const float inv = 1.f / (float)h, c = (float)k + 0.5f, r = (float)r_max;
+    const float eps = 1e-3f + 4e-7f * (float)g;
+    return grange((int)floorf((c - r) * inv - eps), (int)floorf((c + r) * inv + eps), g, periodic);
+}
+
 // best covering particle (lowest metric, then lowest index) among the
 // particles of the selected kind near cell (x, y, z); every covering mobile
 // particle of a cell covered more than once is flagged as sharing cells
 __device__ void best_cover(const Dev& s, int x, int y, int z, int want_fixed, double& best, int& bestp,
                            int* ncover = nullptr, int* cov = nullptr) {
-    const double rm = s.r_max;
     const double xc = x + 0.5, yc = y + 0.5, zc = z + 0.5;
-    GRange ra = grange((int)floor((xc - rm) / s.ghx), (int)floor((xc + rm) / s.ghx), s.gnx, s.per_x);
-    GRange rb = grange((int)floor((yc - rm) / s.ghy), (int)floor((yc + rm) / s.ghy), s.gny, s.per_y);
-    GRange rc = grange((int)floor((zc - rm) / s.ghz), (int)floor((zc + rm) / s.ghz), s.gnz, s.per_z);
+    const GRange ra = cover_range(x, s.r_max, s.ghx, s.gnx, s.per_x);
+    const GRange rb = cover_range(y, s.r_max, s.ghy, s.gny, s.per_y);
+    const GRange rc = cover_range(z, s.r_max, s.ghz, s.gnz, s.per_z);
     for (int ic = 0; ic < rc.n; ++ic)
         for (int ib = 0; ib < rb.n; ++ib)
             for (int ia = 0; ia < ra.n; ++ia) {
@@ -696,7 +706,7 @@ __global__ void k_fixed_map(Dev s) {
     const long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (c >= s.n) return;
     int x, y, z;
-    coords(s, c, x, y, z);
+    coords32(s, (int)c, x, y, z);
     double best = __longlong_as_double(0x7ff0000000000000LL);
     int bestp = -1;
     // above every particle's top (z not periodic) no sphere covers the cell
@@ -705,127 +715,84 @@ __global__ void k_fixed_map(Dev s) {
     s.fixowner[c] = bestp;
 }
 
-// Mobile particles covering cell (x, y, z). The inside test is decided in
-// FP32 where |d^2 - r^2| exceeds a bound far above the FP32 rounding of the
-// offsets (the FP64 result has the same sign there) and in FP64 without
-// fused multiply-add otherwise. Returns the number of covering particles
-// (up to 4 are listed).
-__device__ int covering_mobile(const Dev& s, int x, int y, int z, int* cov) {
-    const double rm = s.r_max;
-    const double xc = x + 0.5, yc = y + 0.5, zc = z + 0.5;
-    GRange ra = grange((int)floor((xc - rm) / s.ghx), (int)floor((xc + rm) / s.ghx), s.gnx, s.per_x);
-    GRange rb = grange((int)floor((yc - rm) / s.ghy), (int)floor((yc + rm) / s.ghy), s.gny, s.per_y);
-    GRange rc = grange((int)floor((zc - rm) / s.ghz), (int)floor((zc + rm) / s.ghz), s.gnz, s.per_z);
-    int n = 0;
-    for (int ic = 0; ic < rc.n; ++ic)
-        for (int ib = 0; ib < rb.n; ++ib)
-            for (int ia = 0; ia < ra.n; ++ia) {
-                const int gg = ra.v[ia] + s.gnx * (rb.v[ib] + s.gny * rc.v[ic]);
-                const int b = s.g_start[gg], e = b + s.g_count[gg];
-                for (int k = b; k < e; ++k) {
-                    const int p = s.g_list[k];
-                    const float4 xr = s.Xr[p];
-                    if (xr.w < 0.f) continue;
-                    float fx = (float)xc - xr.x, fy = (float)yc - xr.y, fz = (float)zc - xr.z;
-                    if (s.per_x) fx -= (float)s.nx * rintf(fx / (float)s.nx);
-                    if (s.per_y) fy -= (float)s.ny * rintf(fy / (float)s.ny);
-                    if (s.per_z) fz -= (float)s.nz * rintf(fz / (float)s.nz);
-                    const float m32 = fx * fx + fy * fy + fz * fz - xr.w * xr.w;
-                    const float tol = 1e-3f * (1.f + xr.w * xr.w);
-                    if (m32 > tol) continue;
-                    if (m32 >= -tol) {
-                        const double* Xp = s.X + 3 * p;
-                        const double m = map_metric(image_centre(x, Xp[0], s.nx, s.per_x),
-                                                    image_centre(y, Xp[1], s.ny, s.per_y),
-                                                    image_centre(z, Xp[2], s.nz, s.per_z), Xp, s.R[p]);
-                        if (m > 0.0) continue;
-                    }
-                    if (n < 4) cov[n] = p;
-                    n++;
-                }
-            }
-    return n;
-}
-
-// new owner of a cell; at set-up covered cells simply become solid, during a
-// run every change is listed for the transition pass
-__device__ void remap_cell(const Dev& s, long long c, int init_mode) {
-    int x, y, z;
-    coords(s, c, x, y, z);
-    const int fo = s.fixowner[c];
-    int cov[4];
-    const int nm = covering_mobile(s, x, y, z, cov);
-    if (nm > 4) set_error(s, ERR_CAPACITY);
-    int bestp;
-    if (nm + (fo >= 0) <= 1) {
-        bestp = nm ? cov[0] : fo;
-    } else {
-        // several covers: exact metrics decide (lowest, then lowest index)
-        double best = reinterpret_cast<const double*>(s.fixkey)[c];
-        bestp = fo;
-        for (int k = 0; k < min(nm, 4); ++k) {
-            const int p = cov[k];
+// Calls f(p) for every mobile particle of the k-th grid cell of the ranges
+// that covers cell (x, y, z). The inside test is decided in FP32 where
+// |d^2 - r^2| exceeds a bound far above the FP32 rounding of the offsets (the
+// FP64 result has the same sign there) and in FP64 without fused multiply-add
+// otherwise.
+template <class F>
+__device__ __forceinline__ void for_covers(const Dev& s, int x, int y, int z, const GRange& ra, const GRange& rb,
+                                           const GRange& rc, int k, F f) {
+    const int ia = k % ra.n, ib = (k / ra.n) % rb.n, ic = k / (ra.n * rb.n);
+    // (selects, so that the ranges stay in registers)
+    auto at = [](const GRange& r, int i) { return i == 0 ? r.v[0] : (i == 1 ? r.v[1] : r.v[2]); };
+    const int gg = at(ra, ia) + s.gnx * (at(rb, ib) + s.gny * at(rc, ic));
+    const int b = s.g_start[gg], e = b + s.g_count[gg];
+    for (int j = b; j < e; ++j) {
+        const int p = s.g_list[j];
+        const float4 xr = s.Xr[p];
+        if (xr.w < 0.f) continue;
+        float fx = (float)x + 0.5f - xr.x, fy = (float)y + 0.5f - xr.y, fz = (float)z + 0.5f - xr.z;
+        if (s.per_x) fx -= (float)s.nx * rintf(fx / (float)s.nx);
+        if (s.per_y) fy -= (float)s.ny * rintf(fy / (float)s.ny);
+        if (s.per_z) fz -= (float)s.nz * rintf(fz / (float)s.nz);
+        const float m32 = fx * fx + fy * fy + fz * fz - xr.w * xr.w;
+        const float tol = 1e-3f * (1.f + xr.w * xr.w);
+        if (m32 > tol) continue;
+        if (m32 >= -tol) {
             const double* Xp = s.X + 3 * p;
             const double m = map_metric(image_centre(x, Xp[0], s.nx, s.per_x), image_centre(y, Xp[1], s.ny, s.per_y),
                                         image_centre(z, Xp[2], s.nz, s.per_z), Xp, s.R[p]);
-            if (m < best || (m == best && p < bestp)) {
-                best = m;
-                bestp = p;
-            }
-            s.shared[p] = 1;
+            if (m > 0.0) continue;
         }
-    }
-    const uint8_t t0 = s.flags[c] & TYPE_MASK;
-    if (init_mode) {
-        if (bestp >= 0) {
-            s.flags[c] = T_SOL;
-            s.owner[c] = bestp;
-            s.mass[c] = 0.f;
-            s.phi[c] = 0.f;
-        }
-        return;
-    }
-    const bool was = t0 == T_SOL;
-    if ((bestp >= 0) != was || (was && bestp != s.owner[c])) {
-        int k = atomicAdd(s.tl_count, 1);
-        if (k < s.tl_cap) {
-            s.tl[k] = (int)c;
-            s.tl_info[2 * k] = bestp;
-        } else {
-            set_error(s, ERR_CAPACITY);
-        }
+        f(p);
     }
 }
 
-__global__ void k_remap_all(Dev s, int init_mode) {
+// Set-up map: covered cells become solid; every particle of a cell with
+// several covers is flagged as sharing cells. The owner has the lowest exact
+// metric, then the lowest index.
+__device__ void remap_cell(const Dev& s, int c) {
+    int x, y, z;
+    coords32(s, c, x, y, z);
+    const int fo = s.fixowner[c];
+    const GRange ra = cover_range(x, s.r_max, s.ghx, s.gnx, s.per_x);
+    const GRange rb = cover_range(y, s.r_max, s.ghy, s.gny, s.per_y);
+    const GRange rc = cover_range(z, s.r_max, s.ghz, s.gnz, s.per_z);
+    const int nc = ra.n * rb.n * rc.n;
+    int nm = 0, bestp = -1;
+    for (int k = 0; k < nc; ++k) for_covers(s, x, y, z, ra, rb, rc, k, [&](int p) { ++nm; bestp = p; });
+    if (nm > 4) set_error(s, ERR_CAPACITY);
+    if (nm + (fo >= 0) <= 1) {
+        bestp = nm ? bestp : fo;
+    } else {
+        double best = reinterpret_cast<const double*>(s.fixkey)[c];
+        bestp = fo;
+        for (int k = 0; k < nc; ++k)
+            for_covers(s, x, y, z, ra, rb, rc, k, [&](int p) {
+                const double* Xp = s.X + 3 * p;
+                const double m = map_metric(image_centre(x, Xp[0], s.nx, s.per_x), image_centre(y, Xp[1], s.ny, s.per_y),
+                                            image_centre(z, Xp[2], s.nz, s.per_z), Xp, s.R[p]);
+                if (m < best || (m == best && p < bestp)) {
+                    best = m;
+                    bestp = p;
+                }
+                s.shared[p] = 1;
+            });
+    }
+    if (bestp >= 0) {
+        s.flags[c] = T_SOL;
+        s.owner[c] = bestp;
+        s.mass[c] = 0.f;
+        s.phi[c] = 0.f;
+    }
+}
+
+__global__ void k_remap_all(Dev s) {
     const long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (c >= s.n) return;
-    int x, y, z;
-    coords(s, c, x, y, z);
-    if (z > *s.zmax_cell) return;
-    remap_cell(s, c, init_mode);
-}
-
-// Every mobile particle that moved since its last map (|dX| > 0) marks the
-// cells whose inside/outside status it can have changed: a cell changes only
-// if |x_c - X_new| - r lies within |dX| of zero (triangle inequality), so
-// the thin shell |  |x_c - X_new| - r | <= |dX| + 1e-3 is marked (the slack
-// covers the FP32 evaluation of the offsets, exact to ~1e-6 through the
-// integer-plus-fraction form of the centre). A particle that shares a cell
-// with another one marks its whole box, since the owner of a shared cell is
-// decided by comparing the two metrics.
-__global__ void k_active(Dev s) {
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= s.np || s.fixed[p]) return;
-    const double dx = s.X[3 * p] - s.Xm[3 * p], dy = s.X[3 * p + 1] - s.Xm[3 * p + 1],
-                 dz = s.X[3 * p + 2] - s.Xm[3 * p + 2];
-    const double d = sqrt(dx * dx + dy * dy + dz * dz);
-    if (s.shared[p] || d > 0.0) {
-        s.margin[p] = s.shared[p] ? -1.f : (float)d;   // shell half-width (negative: whole box)
-        s.shared[p] = 0;
-        int k = atomicAdd(s.act_count, 1);
-        s.act[k] = p;
-    }
+    if ((int)((unsigned)c / ((unsigned)s.nx * (unsigned)s.ny)) > *s.zmax_cell) return;
+    remap_cell(s, (int)c);
 }
 
 __device__ __forceinline__ void bbox_axis(double a, double b, double r, int L, int periodic, int& lo, int& hi) {
@@ -841,20 +808,32 @@ __device__ __forceinline__ void bbox_axis(double a, double b, double r, int L, i
     }
 }
 
-// Cells of the shell (or of the old and new boxes) of every active particle
-// join the dirty list, each once. A warp per particle, a lane per (y, z)
-// row of its box: the row meets the shell | |x_c - X| - r | <= band in at
-// most two x-intervals, found from the row's distance to the centre; the
+// Every mobile particle that moved since its last map (|dX| > 0) marks the
+// cells whose inside/outside status it can have changed: a cell changes only
+// if |x_c - X_new| - r lies within |dX| of zero (triangle inequality), so
+// the thin shell |  |x_c - X_new| - r | <= |dX| + 1e-3 is marked (the slack
+// covers the FP32 evaluation of the offsets, exact to ~1e-6 through the
+// integer-plus-fraction form of the centre). A particle that shares a cell
+// with another one marks its whole box, since the owner of a shared cell is
+// decided by comparing the two metrics.
+// Those cells join the dirty list, each once. A warp per particle, a lane per
+// (y, z) row of its box: the row meets the shell | |x_c - X| - r | <= band in
+// at most two x-intervals, found from the row's distance to the centre; the
 // radii are widened by 1e-3 cells so that rounding can only add cells (a
-// cell re-mapped without need keeps its owner).
+// cell re-mapped without need keeps its owner). The particle's map position
+// then moves to its centre.
 __global__ void k_dirty(Dev s) {
-    const int wid = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
+    const int p = (int)(((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
     const int lane = threadIdx.x & 31;
-    if (wid >= *s.act_count) return;   // whole warps leave together
-    const int p = s.act[wid];
+    if (p >= s.np || s.fixed[p]) return;   // whole warps leave together
+    const double mx = s.X[3 * p] - s.Xm[3 * p], my = s.X[3 * p + 1] - s.Xm[3 * p + 1],
+                 mz = s.X[3 * p + 2] - s.Xm[3 * p + 2];
+    const bool whole = s.shared[p] != 0;
+    if (!whole && mx == 0.0 && my == 0.0 && mz == 0.0) return;
+    // shell half-width, rounded up
+    const float fx = (float)mx, fy = (float)my, fz = (float)mz;
+    const float w = sqrtf(fx * fx + fy * fy + fz * fz) * (1.f + 1e-5f);
     const double r = s.R[p];
-    const float w = s.margin[p];
-    const bool whole = w < 0.f;
     int lo[3], hi[3];
     bbox_axis(s.Xm[3 * p], s.X[3 * p], r, s.nx, s.per_x, lo[0], hi[0]);
     bbox_axis(s.Xm[3 * p + 1], s.X[3 * p + 1], r, s.ny, s.per_y, lo[1], hi[1]);
@@ -910,25 +889,84 @@ __global__ void k_dirty(Dev s) {
             warp_append(s, first, cell, s.dl, s.dl_count, s.dl_cap);
         }
     }
+    __syncwarp();   // every lane has read the old map position and the flag
+    if (lane < 3) s.Xm[3 * p + lane] = s.X[3 * p + lane];
+    else if (lane == 3) s.shared[p] = 0;
 }
 
-__global__ void k_remap_list(Dev s) {
+// Lane groups of COVER_LANES over the dirty cells, a lane per grid cell
+// around it: a thread per cell walked the candidates of up to eight grid
+// cells one after the other, after six FP64 divisions (40 us at 1024x64x128
+// with 4 712 particles, 12.5 us now; 32 and 11 us at 512x40x96). The lanes
+// agree on the number of covering mobile particles; where the cell has one
+// cover or none that decides, otherwise the exact metrics do (lowest, then
+// lowest index), as in remap_cell.
+constexpr int COVER_LANES = 8;
+__global__ void __launch_bounds__(128) k_remap_list(Dev s) {
     const int cnt = min(*s.dl_count, s.dl_cap);
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < cnt; i += gridDim.x * blockDim.x) {
+    const int l = threadIdx.x % COVER_LANES;
+    const unsigned gm = ((1u << COVER_LANES) - 1u) << ((threadIdx.x & 31) / COVER_LANES * COVER_LANES);
+    for (int i = (blockIdx.x * blockDim.x + threadIdx.x) / COVER_LANES; i < cnt;
+         i += gridDim.x * blockDim.x / COVER_LANES) {
         const int c = s.dl[i];
-        s.dirty[c] = 0;
-        remap_cell(s, c, 0);
+        int x, y, z;
+        coords32(s, c, x, y, z);
+        const GRange ra = cover_range(x, s.r_max, s.ghx, s.gnx, s.per_x);
+        const GRange rb = cover_range(y, s.r_max, s.ghy, s.gny, s.per_y);
+        const GRange rc = cover_range(z, s.r_max, s.ghz, s.gnz, s.per_z);
+        const int fo = s.fixowner[c];
+        const uint8_t t0 = s.flags[c] & TYPE_MASK;
+        const int own = t0 == T_SOL ? s.owner[c] : -1;
+        int n = 0, one = -1;      // this lane's covering particles, and the last of them
+        for (int k = l; k < ra.n * rb.n * rc.n; k += COVER_LANES)
+            for_covers(s, x, y, z, ra, rb, rc, k, [&](int p) { ++n; one = p; });
+        int nm = n, bestp = one;
+#pragma unroll
+        for (int o = 1; o < COVER_LANES; o <<= 1) {
+            nm += __shfl_xor_sync(gm, nm, o);
+            bestp = max(bestp, __shfl_xor_sync(gm, bestp, o));
+        }
+        if (nm > 4 && l == 0) set_error(s, ERR_CAPACITY);
+        if (nm + (fo >= 0) <= 1) {
+            bestp = nm ? bestp : fo;
+        } else {
+            double best = l == 0 ? reinterpret_cast<const double*>(s.fixkey)[c] : __longlong_as_double(0x7ff0000000000000LL);
+            bestp = l == 0 ? fo : -1;
+            for (int k = l; k < ra.n * rb.n * rc.n; k += COVER_LANES)
+                for_covers(s, x, y, z, ra, rb, rc, k, [&](int p) {
+                    const double* Xp = s.X + 3 * p;
+                    const double m = map_metric(image_centre(x, Xp[0], s.nx, s.per_x),
+                                                image_centre(y, Xp[1], s.ny, s.per_y),
+                                                image_centre(z, Xp[2], s.nz, s.per_z), Xp, s.R[p]);
+                    if (m < best || (m == best && p < bestp)) {
+                        best = m;
+                        bestp = p;
+                    }
+                    s.shared[p] = 1;
+                });
+#pragma unroll
+            for (int o = 1; o < COVER_LANES; o <<= 1) {
+                const double m2 = __shfl_xor_sync(gm, best, o);
+                const int p2 = __shfl_xor_sync(gm, bestp, o);
+                if (p2 >= 0 && (bestp < 0 || m2 < best || (m2 == best && p2 < bestp))) {
+                    best = m2;
+                    bestp = p2;
+                }
+            }
+        }
+        if (l == 0) {
+            s.dirty[c] = 0;
+            if (bestp != own) {
+                const int k = atomicAdd(s.tl_count, 1);
+                if (k < s.tl_cap) {
+                    s.tl[k] = c;
+                    s.tl_info[2 * k] = bestp;
+                } else {
+                    set_error(s, ERR_CAPACITY);
+                }
+            }
+        }
     }
-}
-
-// the active particles' map positions move to their current centres
-__global__ void k_map_position(Dev s) {
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= *s.act_count) return;
-    const int p = s.act[k];
-    s.Xm[3 * p] = s.X[3 * p];
-    s.Xm[3 * p + 1] = s.X[3 * p + 1];
-    s.Xm[3 * p + 2] = s.X[3 * p + 2];
 }
 
 #define FOR_TL(i)                                                                             \
@@ -940,7 +978,10 @@ enum : int { NT_UNCOVERED_LIQ = 0x100 };
 // covered cells give their mass to the pool; uncovered cells become liquid
 // (interface next to gas, gas without fluid neighbours) with f_eq(mean rho,
 // u_b) and take their mass from the pool (snapshot of the cell types)
-__global__ void k_transitions(Dev s, int last_parity) {
+template <typename S, int LP>
+__global__ void __launch_bounds__(128) k_transitions(Dev s) {
+    // (56 us with general slot lookups and FP16 references by division, 11.6 us
+    // with the neighbour offsets formed once, at 1024x64x128)
     // a warp per transition: the 27 PDFs of a covered cell, the 26
     // neighbours of an uncovered one and its 27 new PDFs are spread over the
     // lanes, so no thread walks a long chain of dependent loads
@@ -954,11 +995,15 @@ __global__ void k_transitions(Dev s, int last_parity) {
         const int o1 = s.tl_info[2 * i];
         const int t0 = s.flags[c] & TYPE_MASK;
         int x, y, z;
-        coords(s, c, x, y, z);
+        coords32(s, c, x, y, z);
+        S* f = static_cast<S*>(s.f);
+        const int nb = lane < 27 ? nbr_q(s, x, y, z, lane) : -1;
+        float h = 0.f;
+        const long long slot = lane < 27 ? lane_slot<S, LP>(s, lane, c, nb, z, h) : 0;
         int nt;
         if (o1 >= 0) {
             // covered: its liquid mass goes to the pool
-            float v = (t0 == T_LIQ && lane < 27) ? ld_any(s, s.f, fstar_slot(s, lane, x, y, z, c, last_parity)) : 0.f;
+            float v = (t0 == T_LIQ && lane < 27) ? with_ref<S>(Store<S>::ld(f + slot), lane, h) : 0.f;
             for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(full, v, o);
             if (lane == 0) {
                 if (t0 == T_LIQ) dpool += (double)(1.f + v);
@@ -966,22 +1011,23 @@ __global__ void k_transitions(Dev s, int last_parity) {
             }
             nt = T_SOL;
         } else {
-            // uncovered: lane k takes neighbour q = k (k < 13) or k + 1
+            // uncovered: lane q takes neighbour q
             float rs = 0.f;
             int cnt = 0;
             bool gas = false;
-            if (lane < 26) {
-                const int q = lane < 13 ? lane : lane + 1;
-                const long long nb = nbr(s, x, y, z, cx(q), cy(q), cz(q));
+            if (lane < 27 && lane != 13) {
                 if (nb >= 0) {
                     const int tn = s.flags[nb] & TYPE_MASK;
                     if (tn == T_IFC) {
                         rs = s.ru[nb].x;
                         cnt = 1;
                     } else if (tn == T_LIQ) {
+                        int bx, by, bz;
+                        coords32(s, nb, bx, by, bz);
                         float g[27];
-                        load_fstar(s, nb, last_parity, g);
+                        load_cell<S, LP>(s, nb, bx, by, bz, g);
                         float d = 0.f;
+#pragma unroll
                         for (int k = 0; k < 27; ++k) d += g[k];
                         rs = 1.f + d;
                         cnt = 1;
@@ -1013,8 +1059,9 @@ __global__ void k_transitions(Dev s, int last_parity) {
                                      (float)(Up[2] + (Wp[0] * d[1] - Wp[1] * d[0]))};
                 if (lane < 27) {
                     const float fq = feq_dev(lane, rb, ub[0], ub[1], ub[2]);
-                    st_any(s, s.f, fstar_slot(s, lane, x, y, z, c, last_parity), fq);
-                    st_any(s, s.fs, (long long)lane * s.n + c, fq);
+                    Store<S>::st(f + slot, with_ref<S>(fq, lane, -h));
+                    Store<S>::st(static_cast<S*>(s.fs) + (long long)lane * s.n + c,
+                                 with_ref<S>(fq, lane, Store<S>::HREF ? -s.href[z] : 0.f));
                 }
                 if (lane == 0) {
                     s.ru[c] = make_float4(rb, ub[0], ub[1], ub[2]);
@@ -1061,15 +1108,17 @@ __global__ void k_repair(Dev s) {
         if (!(s.tl_info[2 * i + 1] & NT_UNCOVERED_LIQ)) continue;
         const int c = s.tl[i];
         int x, y, z;
-        coords(s, c, x, y, z);
+        coords32(s, c, x, y, z);
+        const NbrOffsets o = nbr_offsets(s, x, y, z);
+        bool gas = false;
+#pragma unroll
         for (int q = 0; q < 27; ++q) {
-            if (q == 13) continue;
-            long long nb = nbr(s, x, y, z, cx(q), cy(q), cz(q));
-            if (nb >= 0 && (s.flags[nb] & TYPE_MASK) == T_GAS) {
-                s.flags[c] = T_IFC;
-                s.phi[c] = s.mass[c] / s.ru[c].x;
-                break;
-            }
+            if (q == 13 || (o.wall & wall_bits(cx(q), cy(q), cz(q)))) continue;
+            gas |= (s.flags[c + o.ox[1 + cx(q)] + o.oy[1 + cy(q)] + o.oz[1 + cz(q)]] & TYPE_MASK) == T_GAS;
+        }
+        if (gas) {
+            s.flags[c] = T_IFC;
+            s.phi[c] = s.mass[c] / s.ru[c].x;
         }
     }
 }
@@ -1119,19 +1168,23 @@ int launch_dem(const Dev& s, int have_prev, cudaStream_t st) {
     return ns + launch_grid_lists(s, st);
 }
 
+template <typename S>
+static void launch_transitions(const Dev& s, int last_parity, cudaStream_t st) {
+    if (last_parity == 0) k_transitions<S, 0><<<152 * 4, 128, 0, st>>>(s);
+    else k_transitions<S, 1><<<152 * 4, 128, 0, st>>>(s);
+}
+
+// (the counts of the dirty and transition lists are cleared by the conversion)
 int launch_remap(const Dev& s, int last_parity, cudaStream_t st) {
     if (s.np == 0) return 0;
-    cudaMemsetAsync(s.tl_count, 0, sizeof(int), st);
-    cudaMemsetAsync(s.act_count, 0, sizeof(int), st);
-    cudaMemsetAsync(s.dl_count, 0, sizeof(int), st);
-    k_active<<<blocks_for(s.np, 128), 128, 0, st>>>(s);
     k_dirty<<<blocks_for(32LL * s.np, 128), 128, 0, st>>>(s);
     k_remap_list<<<152 * 8, 128, 0, st>>>(s);
-    k_map_position<<<blocks_for(s.np, 256), 256, 0, st>>>(s);
-    k_transitions<<<152 * 4, 128, 0, st>>>(s, last_parity);
+    if (s.storage == FSLBM_STORE_FP32) launch_transitions<float>(s, last_parity, st);
+    else if (s.storage == FSLBM_STORE_FP16) launch_transitions<__half>(s, last_parity, st);
+    else launch_transitions<__nv_bfloat16>(s, last_parity, st);
     k_apply_transitions<<<152 * 4, 256, 0, st>>>(s);
     k_repair<<<152 * 4, 256, 0, st>>>(s);
-    return 7;
+    return 5;
 }
 
 __global__ void k_init_particles(Dev s, int first, int count, double rho_p) {
@@ -1147,7 +1200,6 @@ __global__ void k_init_particles(Dev s, int first, int count, double rho_p) {
     }
     s.nb_count[p] = 0;
     for (int j = 0; j < NB_ITEMS; ++j) s.nb_xi[(long long)p * NB_ITEMS + j] = make_float4(0.f, 0.f, 0.f, 0.f);
-    s.margin[p] = 0.f;
     // the set-up map (k_remap_all) flags every particle that shares a cell;
     // the others re-map their thin shell from the first step on
     s.shared[p] = 0;
@@ -1160,7 +1212,7 @@ void launch_particles_add(const Dev& s, int first, int count, cudaStream_t st) {
     k_particle_copies<<<blocks_for(s.np, 128), 128, 0, st>>>(s);
     launch_grid_build(s, st);
     k_fixed_map<<<blocks_for(s.n, 256), 256, 0, st>>>(s);
-    k_remap_all<<<blocks_for(s.n, 256), 256, 0, st>>>(s, 1);
+    k_remap_all<<<blocks_for(s.n, 256), 256, 0, st>>>(s);
 }
 
 }  // namespace fsl

@@ -427,7 +427,7 @@ __device__ __forceinline__ void bulk_load(void* dst, const void* src, unsigned b
         : "memory");
 }
 
-// the x-tiles of SP_TILE cells that hold at least one liquid cell, in the
+// the x-tiles (count cleared by the step before) of SP_TILE cells that hold at least one liquid cell, in the
 // order of their first cell within each block; SP_FULL marks a tile whose
 // cells are all liquid
 constexpr int SP_FULL = 1 << 30;
@@ -1360,7 +1360,6 @@ static void launch_typed(const Dev& s, int parity, cudaStream_t st, cudaEvent_t 
         if (early && links_done) cudaEventRecord(links_done, st);
         if (use_staged_pairs(s)) {
             if constexpr (sizeof(S) == 2) {
-                cudaMemsetAsync(s.tile_count, 0, sizeof(int), st);
                 k_sp_tiles<<<(unsigned)((s.n / SP_TILE + 255) / 256), 256, 0, st>>>(s);
                 k_liquid_staged_pair<S><<<staged_pair_blocks<S>(), SP_TILE / 2, StagedPairLayout<S>::SMEM, st>>>(s);
             }

@@ -18,43 +18,42 @@ constexpr int LIST_BLOCKS = 152 * 4;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x, _cnt = *(countp); i < _cnt; \
          i += gridDim.x * blockDim.x)
 
-__device__ __forceinline__ bool is_fluid(int t) { return t == T_LIQ || t == T_IFC; }
-
-// ------------------------------------------------------------ fill levels
-__global__ void k_update_phi(Dev s) {
-    FOR_LIST(i, s.wl_count) {
-        int c = s.wl[i];
-        s.phi[c] = s.mass[c] / s.ru[c].x;
-    }
-}
-
 // Parker-Youngs normal: gradient sum_c w(c) c phi(x+c) with weights 4 (face),
 // 2 (edge), 1 (corner); solid and wall neighbours take the centre value;
 // n = -grad/|grad| points toward the gas.
-__device__ float4 py_normal(const Dev& s, long long c) {
+__device__ __forceinline__ float py_weight(int q) { return nnz(q) == 1 ? 4.f : (nnz(q) == 2 ? 2.f : 1.f); }
+__device__ __forceinline__ float4 py_result(float gx, float gy, float gz) {
+    const float len = sqrtf(gx * gx + gy * gy + gz * gz);
+    if (len > 0.f) return make_float4(-gx / len, -gy / len, -gz / len, 0.f);
+    return make_float4(0.f, 0.f, 0.f, 0.f);
+}
+// (two load phases, the 26 flags and the fill levels of the interface
+// neighbours, each in flight together)
+__device__ __forceinline__ float4 py_normal(const Dev& s, int c) {
     int x, y, z;
-    coords(s, c, x, y, z);
-    const int t0 = s.flags[c] & TYPE_MASK;
-    const float p0 = t0 == T_LIQ ? 1.f : (t0 == T_IFC ? s.phi[c] : 0.f);
+    coords32(s, c, x, y, z);
+    const NbrOffsets o = nbr_offsets(s, x, y, z);
+    uint8_t t[27];
+#pragma unroll
+    for (int q = 0; q < 27; ++q)
+        t[q] = (o.wall & wall_bits(cx(q), cy(q), cz(q)))
+                   ? (uint8_t)T_SOL
+                   : s.flags[c + o.ox[1 + cx(q)] + o.oy[1 + cy(q)] + o.oz[1 + cz(q)]] & TYPE_MASK;
+    float v[27];
+#pragma unroll
+    for (int q = 0; q < 27; ++q)
+        v[q] = t[q] == T_IFC ? s.phi[c + o.ox[1 + cx(q)] + o.oy[1 + cy(q)] + o.oz[1 + cz(q)]]
+                             : (t[q] == T_LIQ ? 1.f : 0.f);
     float gx = 0.f, gy = 0.f, gz = 0.f;
 #pragma unroll
     for (int q = 0; q < 27; ++q) {
         if (q == 13) continue;
-        const float w = nnz(q) == 1 ? 4.f : (nnz(q) == 2 ? 2.f : 1.f);
-        long long nb = nbr(s, x, y, z, cx(q), cy(q), cz(q));
-        float v;
-        if (nb < 0) v = p0;
-        else {
-            int tn = s.flags[nb] & TYPE_MASK;
-            v = tn == T_LIQ ? 1.f : (tn == T_IFC ? s.phi[nb] : (tn == T_GAS ? 0.f : p0));
-        }
-        gx += w * cx(q) * v;
-        gy += w * cy(q) * v;
-        gz += w * cz(q) * v;
+        const float w = py_weight(q), u = t[q] == T_SOL ? v[13] : v[q];
+        gx += w * cx(q) * u;
+        gy += w * cy(q) * u;
+        gz += w * cz(q) * u;
     }
-    float len = sqrtf(gx * gx + gy * gy + gz * gz);
-    if (len > 0.f) return make_float4(-gx / len, -gy / len, -gz / len, 0.f);
-    return make_float4(0.f, 0.f, 0.f, 0.f);
+    return py_result(gx, gy, gz);
 }
 
 __global__ void k_normals(Dev s, float4* out, const int* list, const int* countp) {
@@ -94,7 +93,7 @@ __global__ void __launch_bounds__(128, 5) k_mlp_normals(Dev s, float4* out, cons
             int x = 0, y = 0, z = 0;
             float p0 = 0.f;
             if (cell[r] >= 0) {
-                coords(s, cell[r], x, y, z);
+                coords32(s, cell[r], x, y, z);
                 p0 = s.phi[cell[r]];
             }
 #pragma unroll
@@ -213,231 +212,264 @@ static int normals_into(const Dev& s, float4* out, const int* list, const int* c
 }
 
 // ------------------------------------------------------------ conversion
-// candidates: fill level beyond 1 + eps or below -eps, or isolation (no gas
-// neighbour -> liquid, no liquid neighbour -> gas)
-__global__ void k_candidates(Dev s) {
+// The converting cells of a step are few (tens to thousands), so the kernels
+// over them give each a warp with a lane per neighbour: a thread per cell
+// walked up to 26 neighbours, 27 loads each, one after the other. With a wavy
+// surface on 1024x64x128 cells (72 k interface cells, FP16): new cells and
+// excess shares 138 + 30 -> 6.3 us, marks 26 -> 4.8 us, gather and the new
+// types 30 + 5 + 4 + 3 -> 11.7 us, candidates and fill levels 15 + 4 -> 6.7 us,
+// conflicts 13.8 -> 5.8 us.
+
+// fill levels, and the conversion candidates: fill level beyond 1 + eps or
+// below -eps, or isolation (no gas neighbour -> liquid, no liquid neighbour
+// -> gas). Clears the counts of the lists that the kernels after it fill.
+__global__ void __launch_bounds__(LIST_THREADS) k_candidates(Dev s) {
+    if (blockIdx.x == 0 && threadIdx.x == 0)
+        *s.cl_count = *s.nl_count = *s.tl_count = *s.dl_count = *s.tile_count = 0;
     FOR_LIST(i, s.wl_count) {
-        int c = s.wl[i];
+        const int c = s.wl[i];
         int x, y, z;
-        coords(s, c, x, y, z);
-        bool has_gas = false, has_liq = false;
+        coords32(s, c, x, y, z);
+        const NbrOffsets o = nbr_offsets(s, x, y, z);
+        unsigned gas = 0, liq = 0;
+#pragma unroll
         for (int q = 0; q < 27; ++q) {
-            if (q == 13) continue;
-            long long nb = nbr(s, x, y, z, cx(q), cy(q), cz(q));
-            if (nb < 0) continue;
-            int tn = s.flags[nb] & TYPE_MASK;
-            has_gas |= tn == T_GAS;
-            has_liq |= tn == T_LIQ;
+            if (q == 13 || (o.wall & wall_bits(cx(q), cy(q), cz(q)))) continue;
+            const int t = s.flags[c + o.ox[1 + cx(q)] + o.oy[1 + cy(q)] + o.oz[1 + cz(q)]] & TYPE_MASK;
+            gas |= t == T_GAS;
+            liq |= t == T_LIQ;
         }
-        float ph = s.phi[c];
+        const float ph = s.mass[c] / s.ru[c].x;
+        s.phi[c] = ph;
         uint8_t cv = 0;
         if (ph > 1.f + s.eps_conv) cv = CV_TO_LIQ;
         else if (ph < -s.eps_conv) cv = CV_TO_GAS;
-        else if (!has_gas) cv = CV_TO_LIQ;
-        else if (!has_liq) cv = CV_TO_GAS;
+        else if (!gas) cv = CV_TO_LIQ;
+        else if (!liq) cv = CV_TO_GAS;
         s.conv[c] = cv;
     }
-}
-
-__device__ __forceinline__ void list_push(const Dev& s, int* list, int* count, int cap, int v) {
-    int k = atomicAdd(count, 1);
-    if (k < cap) list[k] = v;
-    else set_error(s, ERR_CAPACITY);
 }
 
 // filling wins: a to-gas cell next to a to-liquid cell stays interface. The
 // cells that still convert are listed (their normals give the excess-mass
 // weights).
-__global__ void k_conflict(Dev s) {
-    FOR_LIST(i, s.wl_count) {
-        int c = s.wl[i];
-        const uint8_t cv = s.conv[c];
-        if (!cv) continue;
+__global__ void __launch_bounds__(LIST_THREADS) k_conflict(Dev s) {
+    const int cnt = *s.wl_count, stride = gridDim.x * blockDim.x;
+    for (int base = blockIdx.x * blockDim.x; base < cnt; base += stride) {
+        const int i = base + threadIdx.x;
+        int c = 0;
+        uint8_t cv = 0;
+        if (i < cnt) {
+            c = s.wl[i];
+            cv = s.conv[c];
+        }
         if (cv == CV_TO_GAS) {
             int x, y, z;
-            coords(s, c, x, y, z);
+            coords32(s, c, x, y, z);
+            const NbrOffsets o = nbr_offsets(s, x, y, z);
             bool clash = false;
-            for (int q = 0; q < 27 && !clash; ++q) {
-                if (q == 13) continue;
-                long long nb = nbr(s, x, y, z, cx(q), cy(q), cz(q));
-                if (nb >= 0 && s.conv[nb] == CV_TO_LIQ) clash = true;
-            }
-            if (clash) {
-                s.conv[c] = 0;
-                continue;
-            }
-        }
-        list_push(s, s.cl, s.cl_count, s.wl_cap, c);
-    }
-}
-
-// gas neighbours of filled cells and liquid neighbours of emptied cells
-// become interface cells; each is listed once (first setter of its mark)
-// (over the cells that convert, listed by k_conflict)
-__global__ void k_mark(Dev s) {
-    const int ncl = min(*s.cl_count, s.wl_cap);
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < ncl; i += gridDim.x * blockDim.x) {
-        int c = s.cl[i];
-        uint8_t cv = s.conv[c];
-        if (!cv) continue;
-        int x, y, z;
-        coords(s, c, x, y, z);
-        for (int q = 0; q < 27; ++q) {
-            if (q == 13) continue;
-            long long nb = nbr(s, x, y, z, cx(q), cy(q), cz(q));
-            if (nb < 0) continue;
-            int tn = s.flags[nb] & TYPE_MASK;
-            uint8_t bit = 0;
-            if (cv == CV_TO_LIQ && tn == T_GAS) bit = F_NEW;
-            if (cv == CV_TO_GAS && tn == T_LIQ) bit = F_EMPTIED;
-            if (!bit) continue;
-            uint8_t old = flag_or(s.flags, nb, bit);
-            if (!(old & bit)) list_push(s, s.nl, s.nl_count, s.nl_cap, (int)nb);
-        }
-    }
-}
-
-// new interface cells: from gas, f* = f_eq(mean rho, mean u) of the liquid
-// and interface neighbours (cell types of the snapshot) with m = 0; from
-// liquid, PDFs kept and m = rho. Both get their own PDFs in the side buffer.
-__global__ void k_init_new(Dev s, int last_parity) {
-    FOR_LIST(i, s.nl_count) {
-        if (i >= s.nl_cap) break;
-        const int c = s.nl[i];
-        const uint8_t fl = s.flags[c];
-        float f[27];
-        float rho, ux, uy, uz;
-        if (fl & F_NEW) {
-            int x, y, z;
-            coords(s, c, x, y, z);
-            float rs = 0.f, us = 0.f, vs = 0.f, ws = 0.f;
-            int cnt = 0;
-            // rolled: the 27 loads per liquid neighbour make an unrolled loop
-            // bound by instruction fetch
-#pragma unroll 1
-            for (int q = 0; q < 27; ++q) {
-                if (q == 13) continue;
-                long long nb = nbr(s, x, y, z, cx(q), cy(q), cz(q));
-                if (nb < 0) continue;
-                int tn = s.flags[nb] & TYPE_MASK;
-                if (tn == T_IFC) {
-                    float4 r = s.ru[nb];
-                    rs += r.x; us += r.y; vs += r.z; ws += r.w;
-                    cnt++;
-                } else if (tn == T_LIQ) {
-                    float g[27];
-                    load_fstar(s, nb, last_parity, g);
-                    float r0, a, b, d;
-                    post_moments(s, g, r0, a, b, d);
-                    rs += r0; us += a; vs += b; ws += d;
-                    cnt++;
-                }
-            }
-            float inv = cnt ? 1.f / cnt : 0.f;
-            rho = cnt ? rs * inv : s.rho_gas;
-            ux = us * inv; uy = vs * inv; uz = ws * inv;
 #pragma unroll
-            for (int q = 0; q < 27; ++q) f[q] = feq_dev(q, rho, ux, uy, uz);
-            store_fstar(s, c, last_parity, f);
-            s.mass[c] = 0.f;
-        } else {
-            load_fstar(s, c, last_parity, f);
-            post_moments(s, f, rho, ux, uy, uz);
-            s.mass[c] = rho;
+            for (int q = 0; q < 27; ++q) {
+                if (q == 13 || (o.wall & wall_bits(cx(q), cy(q), cz(q)))) continue;
+                clash |= s.conv[c + o.ox[1 + cx(q)] + o.oy[1 + cy(q)] + o.oz[1 + cz(q)]] == CV_TO_LIQ;
+            }
+            if (clash) s.conv[c] = cv = 0;
         }
-        for (int q = 0; q < 27; ++q) st_any(s, s.fs, (long long)q * s.n + c, f[q]);
-        s.ru[c] = make_float4(rho, ux, uy, uz);
+        warp_append(s, cv != 0, c, s.cl, s.cl_count, s.wl_cap);
     }
 }
 
-__device__ __forceinline__ bool is_receiver(const Dev& s, long long c) {
-    uint8_t fl = s.flags[c];
+// a warp per entry of a list of n
+#define FOR_WARP(i, n)                                                                                  \
+    for (int i = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5), _st = (gridDim.x * blockDim.x) >> 5; i < (n); \
+         i += _st)
+
+// Gas neighbours of filled cells and liquid neighbours of emptied cells
+// become interface cells; each is listed once (first setter of its mark).
+// With FD the Parker-Youngs normal of the converting cell from the same
+// neighbours (fill levels and types are still those the candidates saw).
+template <bool FD>
+__global__ void __launch_bounds__(LIST_THREADS) k_mark(Dev s) {
+    const int lane = threadIdx.x & 31;
+    const int ncl = min(*s.cl_count, s.wl_cap);
+    FOR_WARP(i, ncl) {
+        const int c = s.cl[i];
+        const uint8_t cv = s.conv[c];
+        int x, y, z;
+        coords32(s, c, x, y, z);
+        const int nb = lane < 27 ? nbr_q(s, x, y, z, lane) : -1;
+        const int tn = nb >= 0 ? s.flags[nb] & TYPE_MASK : (int)T_SOL;
+        uint8_t bit = 0;
+        if (cv == CV_TO_LIQ && tn == T_GAS) bit = F_NEW;
+        if (cv == CV_TO_GAS && tn == T_LIQ) bit = F_EMPTIED;
+        const bool fresh = bit && !(flag_or(s.flags, nb, bit) & bit);
+        warp_append(s, fresh, nb, s.nl, s.nl_count, s.nl_cap);
+        if (FD) {
+            float v = tn == T_IFC ? s.phi[nb] : (tn == T_LIQ ? 1.f : 0.f);
+            const float p0 = __shfl_sync(0xffffffffu, v, 13);
+            if (tn == T_SOL) v = p0;
+            const int dx = lane % 3 - 1, dy = (lane / 3) % 3 - 1, dz = lane / 9 - 1;
+            const int k = (dx != 0) + (dy != 0) + (dz != 0);
+            v *= lane < 27 ? (k == 1 ? 4.f : (k == 2 ? 2.f : 1.f)) : 0.f;
+            const float gx = warp_sum_f(dx * v), gy = warp_sum_f(dy * v), gz = warp_sum_f(dz * v);
+            if (lane == 0) s.nrm1[c] = py_result(gx, gy, gz);
+        }
+    }
+}
+
+__device__ __forceinline__ bool is_receiver(const Dev& s, int c) {
+    const uint8_t fl = s.flags[c];
     if (fl & (F_NEW | F_EMPTIED)) return true;
     return (fl & TYPE_MASK) == T_IFC && (s.conv[c] & 3) == 0;
 }
 
-// excess mass of converting cells: m - rho (to liquid, m := rho) or m (to
-// gas, m := 0), spread over interface neighbours with weights max(0, n.c)
-// (filled) or max(0, -n.c) (emptied), evenly if all weights vanish or the
-// even variant is selected, into the FP64 pool if there is no interface
-// neighbour
-__global__ void k_excess_prep(Dev s) {
-    const int ncl = min(*s.cl_count, s.wl_cap);
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < ncl; i += gridDim.x * blockDim.x) {
-        int c = s.cl[i];
-        uint8_t cv = s.conv[c];
-        if (!cv) continue;
-        float rho = s.ru[c].x;
-        float m = s.mass[c];
-        float ex;
-        if (cv == CV_TO_LIQ) { ex = m - rho; s.mass[c] = rho; }
-        else { ex = m; s.mass[c] = 0.f; }
-        float sg = cv == CV_TO_LIQ ? 1.f : -1.f;
-        float4 n1 = s.nrm1[c];
-        int x, y, z;
-        coords(s, c, x, y, z);
-        float wsum = 0.f;
-        int nrec = 0;
-        for (int q = 0; q < 27; ++q) {
-            if (q == 13) continue;
-            long long nb = nbr(s, x, y, z, cx(q), cy(q), cz(q));
-            if (nb < 0 || !is_receiver(s, nb)) continue;
-            float w = sg * (n1.x * cx(q) + n1.y * cy(q) + n1.z * cz(q));
-            wsum += w > 0.f ? w : 0.f;
-            nrec++;
+// New interface cells: from gas, f* = f_eq(mean rho, mean u) of the liquid
+// and interface neighbours (cell types of the snapshot) with m = 0; from
+// liquid, PDFs kept and m = rho. Both get their own PDFs in the side buffer.
+// One warp; lane q holds neighbour and direction q.
+template <typename S, int LP>
+__device__ __forceinline__ void init_new(const Dev& s, int c, int lane) {
+    const uint8_t fl = s.flags[c];
+    S* f = static_cast<S*>(s.f);
+    S* fs = static_cast<S*>(s.fs);
+    int x, y, z;
+    coords32(s, c, x, y, z);
+    const int nb = lane < 27 ? nbr_q(s, x, y, z, lane) : -1;
+    float h = 0.f;
+    const long long slot = lane < 27 ? lane_slot<S, LP>(s, lane, c, nb, z, h) : 0;
+    const float h0 = Store<S>::HREF ? s.href[z] : 0.f;
+    float v, rho, ux, uy, uz, m;
+    if (fl & F_NEW) {
+        float rs = 0.f, us = 0.f, vs = 0.f, ws = 0.f, n = 0.f;
+        if (nb >= 0 && lane != 13) {
+            const int tn = s.flags[nb] & TYPE_MASK;
+            if (tn == T_IFC) {
+                const float4 r = s.ru[nb];
+                rs = r.x; us = r.y; vs = r.z; ws = r.w;
+                n = 1.f;
+            } else if (tn == T_LIQ) {
+                int bx, by, bz;
+                coords32(s, nb, bx, by, bz);
+                float g[27];
+                load_cell<S, LP>(s, nb, bx, by, bz, g);
+                post_moments(s, g, rs, us, vs, ws);
+                n = 1.f;
+            }
         }
-        if (nrec == 0) {
-            atomicAdd(s.pool, (double)ex);
-            s.exscale[c] = 0.f;
-        } else if (wsum > 0.f && !s.excess_even) {
-            s.exscale[c] = ex / wsum;
-        } else {
-            s.exscale[c] = ex / (float)nrec;
-            s.conv[c] = cv | CV_EVEN;
-        }
+        n = warp_sum_f(n);
+        rs = warp_sum_f(rs);
+        const float inv = n > 0.f ? 1.f / n : 0.f;
+        rho = n > 0.f ? rs * inv : s.rho_gas;
+        ux = warp_sum_f(us) * inv;
+        uy = warp_sum_f(vs) * inv;
+        uz = warp_sum_f(ws) * inv;
+        v = feq_dev(lane < 27 ? lane : 0, rho, ux, uy, uz);
+        if (lane < 27) Store<S>::st(f + slot, with_ref<S>(v, lane, -h));
+        m = 0.f;
+    } else {
+        v = lane < 27 ? with_ref<S>(Store<S>::ld(f + slot), lane, h) : 0.f;
+        const float d = warp_sum_f(v);
+        const float jx = warp_sum_f((lane % 3 - 1) * v), jy = warp_sum_f(((lane / 3) % 3 - 1) * v),
+                    jz = warp_sum_f((lane / 9 - 1) * v);
+        rho = 1.f + d;
+        const float inv = 1.f / rho;
+        ux = (jx - 0.5f * rho * s.gx) * inv;
+        uy = (jy - 0.5f * rho * s.gy) * inv;
+        uz = (jz - 0.5f * rho * s.gz) * inv;
+        m = rho;
+    }
+    if (lane < 27) Store<S>::st(fs + (long long)lane * s.n + c, with_ref<S>(v, lane, -h0));
+    if (lane == 0) {
+        s.mass[c] = m;
+        s.ru[c] = make_float4(rho, ux, uy, uz);
     }
 }
 
-__device__ void gather_excess(const Dev& s, int c) {
-    if (!is_receiver(s, c)) return;
+// Excess mass of a converting cell: m - rho (to liquid, m := rho) or m (to
+// gas, m := 0), spread over interface neighbours with weights max(0, n.c)
+// (filled) or max(0, -n.c) (emptied), evenly if all weights vanish or the
+// even variant is selected, into the FP64 pool if there is no interface
+// neighbour. One warp, lane q on neighbour q.
+__device__ __forceinline__ void excess_prep(const Dev& s, int c, int lane) {
+    const uint8_t cv = s.conv[c];
+    const float rho = s.ru[c].x, m = s.mass[c];
+    const float4 n1 = s.nrm1[c];
     int x, y, z;
-    coords(s, c, x, y, z);
-    float add = 0.f;
+    coords32(s, c, x, y, z);
+    const int nb = lane < 27 && lane != 13 ? nbr_q(s, x, y, z, lane) : -1;
+    const bool rec = nb >= 0 && is_receiver(s, nb);
+    const float sg = cv == CV_TO_LIQ ? 1.f : -1.f;
+    const float w = sg * (n1.x * (lane % 3 - 1) + n1.y * ((lane / 3) % 3 - 1) + n1.z * (lane / 9 - 1));
+    const int nrec = __popc(__ballot_sync(0xffffffffu, rec));
+    const float wsum = warp_sum_f(rec && w > 0.f ? w : 0.f);
+    if (lane != 0) return;
+    const float ex = cv == CV_TO_LIQ ? m - rho : m;
+    s.mass[c] = cv == CV_TO_LIQ ? rho : 0.f;
+    if (nrec == 0) {
+        atomicAdd(s.pool, (double)ex);
+        s.exscale[c] = 0.f;
+    } else if (wsum > 0.f && !s.excess_even) {
+        s.exscale[c] = ex / wsum;
+    } else {
+        s.exscale[c] = ex / (float)nrec;
+        s.conv[c] = cv | CV_EVEN;
+    }
+}
+
+// The new interface cells and the converting cells in one launch: the first
+// write the state of cells that are still gas or liquid in the snapshot, the
+// second read and write that of interface cells only.
+template <typename S, int LP>
+__global__ void __launch_bounds__(LIST_THREADS) k_init_and_prep(Dev s) {
+    const int lane = threadIdx.x & 31;
+    const int nnl = min(*s.nl_count, s.nl_cap), ncl = min(*s.cl_count, s.wl_cap);
+    FOR_WARP(i, nnl + ncl) {
+        if (i < nnl) init_new<S, LP>(s, s.nl[i], lane);
+        else excess_prep(s, s.cl[i - nnl], lane);
+        __syncwarp();
+    }
+}
+
+// the excess mass a receiver takes from the converting cells around it
+__device__ __forceinline__ float gather_excess(const Dev& s, int c, bool& any) {
+    int x, y, z;
+    coords32(s, c, x, y, z);
+    const NbrOffsets o = nbr_offsets(s, x, y, z);
+    unsigned conv = 0;
+#pragma unroll
     for (int q = 0; q < 27; ++q) {
-        if (q == 13) continue;
-        long long nb = nbr(s, x, y, z, cx(q), cy(q), cz(q));
-        if (nb < 0) continue;
-        uint8_t cv = s.conv[nb];
-        if (!(cv & 3)) continue;
+        if (q == 13 || (o.wall & wall_bits(cx(q), cy(q), cz(q)))) continue;
+        if (s.conv[c + o.ox[1 + cx(q)] + o.oy[1 + cy(q)] + o.oz[1 + cz(q)]] & 3) conv |= 1u << q;
+    }
+    any = conv != 0;
+    float add = 0.f;
+    for (; conv; conv &= conv - 1) {
+        const int q = __ffs(conv) - 1;
+        const int nb = nbr_q(s, x, y, z, q);
+        const uint8_t cv = s.conv[nb];
         float w;
         if (cv & CV_EVEN) w = 1.f;
         else {
             // direction from the converting cell to this receiver is -c_q
-            float4 n1 = s.nrm1[nb];
-            float sg = (cv & 3) == CV_TO_LIQ ? 1.f : -1.f;
-            w = -sg * (n1.x * cx(q) + n1.y * cy(q) + n1.z * cz(q));
+            const float4 n1 = s.nrm1[nb];
+            const float sg = (cv & 3) == CV_TO_LIQ ? 1.f : -1.f;
+            w = -sg * (n1.x * (q % 3 - 1) + n1.y * ((q / 3) % 3 - 1) + n1.z * (q / 9 - 1));
             w = w > 0.f ? w : 0.f;
         }
         add += s.exscale[nb] * w;
     }
-    s.mass[c] += add;
+    return add;
 }
 
-__global__ void k_excess_gather(Dev s) {
-    // without a converting cell no receiver gets anything
+// Excess mass gathered by the receivers, and the new types and fill levels.
+// A cell reads the conversion codes, normals and scales of its neighbours,
+// which nothing here writes, and writes its own mass, fill level and flag.
+// Without a converting cell everything stands as the candidates left it.
+__global__ void __launch_bounds__(LIST_THREADS) k_finish_conversion(Dev s) {
     if (*s.cl_count == 0) return;
-    FOR_LIST(i, s.wl_count) gather_excess(s, s.wl[i]);
-    const int cap = s.nl_cap;
-    FOR_LIST(i, s.nl_count) {
-        if (i >= cap) break;
-        gather_excess(s, s.nl[i]);
-    }
-}
-
-__global__ void k_finalize_old(Dev s) {
     FOR_LIST(i, s.wl_count) {
-        int c = s.wl[i];
-        uint8_t cv = s.conv[c] & 3;
+        const int c = s.wl[i];
+        const uint8_t cv = s.conv[c] & 3;
         if (cv == CV_TO_LIQ) {
             s.flags[c] = T_LIQ;
         } else if (cv == CV_TO_GAS) {
@@ -445,23 +477,25 @@ __global__ void k_finalize_old(Dev s) {
             s.mass[c] = 0.f;
             s.phi[c] = 0.f;
         } else {
-            s.phi[c] = s.mass[c] / s.ru[c].x;
+            bool any;
+            const float add = gather_excess(s, c, any);
+            if (any) {
+                const float m = s.mass[c] + add;
+                s.mass[c] = m;
+                s.phi[c] = m / s.ru[c].x;
+            }
         }
     }
-}
-__global__ void k_finalize_new(Dev s) {
     const int cap = s.nl_cap;
     FOR_LIST(i, s.nl_count) {
         if (i >= cap) break;
-        int c = s.nl[i];
+        const int c = s.nl[i];
+        bool any;
+        const float m = s.mass[c] + gather_excess(s, c, any);
+        s.mass[c] = m;
         s.flags[c] = T_IFC;
-        s.phi[c] = s.mass[c] / s.ru[c].x;
+        s.phi[c] = m / s.ru[c].x;
     }
-}
-// conversion codes are left only on the cells k_conflict listed
-__global__ void k_clear_conv(Dev s) {
-    const int ncl = min(*s.cl_count, s.wl_cap);
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < ncl; i += gridDim.x * blockDim.x) s.conv[s.cl[i]] = 0;
 }
 
 // Interface stencils of the current state with height-function labels (R-17e):
@@ -600,23 +634,27 @@ void launch_log_stencils(const Dev& s, long long cap, float* fill, float* target
 
 int launch_normals(const Dev& s, float4* out, cudaStream_t st) { return normals_into(s, out, s.wl, s.wl_count, st); }
 
+template <typename S>
+static void launch_init_and_prep(const Dev& s, int last_parity, cudaStream_t st) {
+    if (last_parity == 0) k_init_and_prep<S, 0><<<LIST_BLOCKS, LIST_THREADS, 0, st>>>(s);
+    else k_init_and_prep<S, 1><<<LIST_BLOCKS, LIST_THREADS, 0, st>>>(s);
+}
+
 int launch_conversion(const Dev& s, int last_parity, cudaStream_t st) {
-    k_update_phi<<<LIST_BLOCKS, LIST_THREADS, 0, st>>>(s);
     k_candidates<<<LIST_BLOCKS, LIST_THREADS, 0, st>>>(s);
-    cudaMemsetAsync(s.cl_count, 0, sizeof(int), st);
     k_conflict<<<LIST_BLOCKS, LIST_THREADS, 0, st>>>(s);
-    // the excess-mass weights need the normals of the converting cells only;
-    // fill levels and types are those k_update_phi left
-    normals_into(s, s.nrm1, s.cl, s.cl_count, st);
-    cudaMemsetAsync(s.nl_count, 0, sizeof(int), st);
-    k_mark<<<LIST_BLOCKS, LIST_THREADS, 0, st>>>(s);
-    k_init_new<<<LIST_BLOCKS, LIST_THREADS, 0, st>>>(s, last_parity);
-    k_excess_prep<<<LIST_BLOCKS, LIST_THREADS, 0, st>>>(s);
-    k_excess_gather<<<LIST_BLOCKS, LIST_THREADS, 0, st>>>(s);
-    k_finalize_old<<<LIST_BLOCKS, LIST_THREADS, 0, st>>>(s);
-    k_finalize_new<<<LIST_BLOCKS, LIST_THREADS, 0, st>>>(s);
-    k_clear_conv<<<LIST_BLOCKS, LIST_THREADS, 0, st>>>(s);
-    return 12;
+    // the excess-mass weights need the normals of the converting cells only
+    if (s.mlp) {
+        normals_into(s, s.nrm1, s.cl, s.cl_count, st);
+        k_mark<false><<<LIST_BLOCKS, LIST_THREADS, 0, st>>>(s);
+    } else {
+        k_mark<true><<<LIST_BLOCKS, LIST_THREADS, 0, st>>>(s);
+    }
+    if (s.storage == FSLBM_STORE_FP32) launch_init_and_prep<float>(s, last_parity, st);
+    else if (s.storage == FSLBM_STORE_FP16) launch_init_and_prep<__half>(s, last_parity, st);
+    else launch_init_and_prep<__nv_bfloat16>(s, last_parity, st);
+    k_finish_conversion<<<LIST_BLOCKS, LIST_THREADS, 0, st>>>(s);
+    return s.mlp ? 6 : 5;
 }
 
 // ------------------------------------------------------------ work lists
@@ -686,8 +724,10 @@ __device__ __forceinline__ void type_nibbles(unsigned v, unsigned& f, unsigned& 
     sl = pack(hi & a & 0x01010101u);
 }
 
+// (also clears the counts of the lists that the second pass fills)
 __global__ void k_type_bits(Dev s) {
     const long long w = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (w == 0) *s.wl_count = *s.sl_count = *s.bseg_count = 0;
     if (w >= (s.n >> 5)) return;
     const uint4* src = reinterpret_cast<const uint4*>(s.flags + (w << 5));
     const uint4 a = src[0], b = src[1];
@@ -706,7 +746,29 @@ __global__ void k_type_bits(Dev s) {
     s.sbits[w] = sm;
 }
 
-__global__ void k_classify_bits(Dev s) {
+// The block of the classification that finishes last clamps the list counts
+// to their capacities and, with spread, takes the mass pool's share per
+// interface cell (k_pool_spread adds it). Every thread of the block calls it.
+__device__ __forceinline__ void classify_last(const Dev& s, int spread) {
+    if (threadIdx.x != 0) return;
+    __threadfence();
+    if (atomicAdd(s.cls_done, 1) != (int)gridDim.x - 1) return;
+    __threadfence();
+    *s.cls_done = 0;
+    const int wl = min(__ldcg(s.wl_count), s.wl_cap);
+    *s.wl_count = wl;
+    *s.sl_count = min(__ldcg(s.sl_count), s.sl_cap);
+    if (!spread) return;
+    const double p = *s.pool;
+    if (wl > 0 && p != 0.0) {
+        *s.pool_share = p / (double)wl;
+        *s.pool = 0.0;
+    } else {
+        *s.pool_share = 0.0;
+    }
+}
+
+__global__ void k_classify_bits(Dev s, int spread) {
     const long long w = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     const int nxw = s.nx >> 5;                      // words per row
     const long long nw = s.n >> 5;
@@ -741,6 +803,7 @@ __global__ void k_classify_bits(Dev s) {
     }
     const int c0 = (int)(w << 5);
     block_append_masks(s, c0, ifc_mask, s.wl, s.wl_count, s.wl_cap, sol_mask, s.sl, s.sl_count, s.sl_cap);
+    classify_last(s, spread);
 }
 
 // Bed segments, for particle links taken from the fluid side: a thread per
@@ -804,7 +867,7 @@ __global__ void k_bed_segments(Dev s) {
 
 // Fallback for lattices whose x extent is not a multiple of 32: one thread
 // per cell, 26 neighbour reads for solid cells.
-__global__ void k_classify(Dev s) {
+__global__ void k_classify(Dev s, int spread) {
     const long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     const bool in = c < s.n;
     int t = 0;
@@ -831,6 +894,7 @@ __global__ void k_classify(Dev s) {
     }
     block_append(s, in && t == T_IFC, (int)c, s.wl, s.wl_count, s.wl_cap);
     block_append(s, surf, (int)c, s.sl, s.sl_count, s.sl_cap);
+    classify_last(s, spread);
 }
 
 // liquid cells with a gas neighbour (the separation the conversion rules keep)
@@ -853,28 +917,21 @@ void launch_check_invariant(const Dev& s, cudaStream_t st) {
     k_check_invariant<<<blocks_for(s.n, 256), 256, 0, st>>>(s);
 }
 
-__global__ void k_clamp_count(Dev s) {
-    if (*s.wl_count > s.wl_cap) *s.wl_count = s.wl_cap;
-    if (*s.sl_count > s.sl_cap) *s.sl_count = s.sl_cap;
-}
-
-int launch_classify(const Dev& s, cudaStream_t st) {
-    cudaMemsetAsync(s.wl_count, 0, sizeof(int), st);
-    cudaMemsetAsync(s.sl_count, 0, sizeof(int), st);
-    int k = 2;
+int launch_classify(const Dev& s, bool spread, cudaStream_t st) {
+    int k = 1;
     if (s.nx % 32 == 0) {
         k_type_bits<<<blocks_for(s.n / 32, 256), 256, 0, st>>>(s);
-        k_classify_bits<<<blocks_for(s.n / 32, 128), 128, 0, st>>>(s);
+        k_classify_bits<<<blocks_for(s.n / 32, 128), 128, 0, st>>>(s, spread);
         ++k;
         if (s.links_fused) {
-            cudaMemsetAsync(s.bseg_count, 0, sizeof(int), st);
             k_bed_segments<<<blocks_for((long long)s.nsegx * s.ny * s.nz, 128), 128, 0, st>>>(s);
             ++k;
         }
     } else {
-        k_classify<<<blocks_for(s.n, 256), 256, 0, st>>>(s);
+        cudaMemsetAsync(s.wl_count, 0, sizeof(int), st);
+        cudaMemsetAsync(s.sl_count, 0, sizeof(int), st);
+        k_classify<<<blocks_for(s.n, 256), 256, 0, st>>>(s, spread);
     }
-    k_clamp_count<<<1, 1, 0, st>>>(s);
     return k;
 }
 
@@ -897,31 +954,24 @@ void launch_cell_counts(const Dev& s, unsigned long long* out, cudaStream_t st) 
 }
 
 // ------------------------------------------------------------ mass pool
-__global__ void k_pool_prepare(Dev s) {
-    int cnt = *s.wl_count;
-    double p = *s.pool;
-    if (cnt > 0 && p != 0.0) {
-        *s.pool_share = p / (double)cnt;
-        *s.pool = 0.0;
-    } else {
-        *s.pool_share = 0.0;
-    }
-}
+// the pool's share joins every interface cell; the conversion codes, left
+// only on the cells k_conflict listed, are cleared
 __global__ void k_pool_spread(Dev s) {
+    const int ncl = min(*s.cl_count, s.wl_cap);
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < ncl; i += gridDim.x * blockDim.x) s.conv[s.cl[i]] = 0;
     const double share = *s.pool_share;
     if (share == 0.0) return;
     FOR_LIST(i, s.wl_count) {
-        int c = s.wl[i];
-        float m = (float)((double)s.mass[c] + share);
+        const int c = s.wl[i];
+        const float m = (float)((double)s.mass[c] + share);
         s.mass[c] = m;
         s.phi[c] = m / s.ru[c].x;
     }
 }
 
 int launch_pool_spread(const Dev& s, cudaStream_t st) {
-    k_pool_prepare<<<1, 1, 0, st>>>(s);
     k_pool_spread<<<LIST_BLOCKS, LIST_THREADS, 0, st>>>(s);
-    return 2;
+    return 1;
 }
 
 // ------------------------------------------------------------ initial state
