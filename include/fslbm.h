@@ -300,7 +300,7 @@ int fslbm_transport_numbers(fslbm* s, double d50, double out[6]);
  * toward +x, and amplitude 2 sqrt(psd / (nt nx)) (exact for a single
  * travelling sine on the grid's frequencies). 2 <= nt <= 65535,
  * 2 <= nx <= 2^20, dx, dt > 0, else FSLBM_EINVAL. Needs no handle;
- * allocates 16 (nx + nt + nt nx) + 32 bytes of device scratch for the call
+ * allocates at most 16 (nx + nt + nt nx) + 16384 bytes of device scratch for the call
  * (FSLBM_ENOMEM if that fails) and synchronises cuda_stream (NULL: the
  * legacy default stream). FSLBM_EDEVICE on a CUDA error. */
 int fslbm_bed_spectrum(const double* h, int64_t nt, int64_t nx, double dx, double dt, double* psd, double peak[4],

@@ -19,6 +19,7 @@ void mlp_frag_host(const MlpBf16& h, const __nv_bfloat16* w1m, MlpFrag& G);
 namespace fsl {
 void launch_bed_height(const Dev& s, double phi_b, double* phi, double* h, cudaStream_t st);
 void launch_water_depth(const Dev& s, double* bed, double* eta, double* out, cudaStream_t st);
+size_t bed_spectrum_work(long long nt, long long nx);
 int launch_bed_spectrum(const double* h, int nt, int nx, double* psd, double* work, double* peak3, cudaStream_t st);
 }
 
@@ -1066,9 +1067,7 @@ int fslbm_bed_spectrum(const double* h, int64_t nt, int64_t nx, double dx, doubl
     if (!h || !psd || !peak || nt < 2 || nx < 2 || nt > 65535 || nx > (1 << 20)) return FSLBM_EINVAL;
     if (!(dx > 0.0) || !(dt > 0.0) || !std::isfinite(dx) || !std::isfinite(dt)) return FSLBM_EINVAL;
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
-    // scratch: twiddles (nx + nt complex), the x-transformed series (nt nx
-    // complex), the mean, and the peak (value, l, j)
-    const size_t work_doubles = 2 * ((size_t)nx + nt + (size_t)nt * nx) + 4;
+    const size_t work_doubles = bed_spectrum_work(nt, nx);   // the peak (value, l, j) at its end
     double* work = nullptr;
     if (cudaMalloc(&work, work_doubles * sizeof(double)) != cudaSuccess) {
         cudaGetLastError();

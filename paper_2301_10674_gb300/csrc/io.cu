@@ -1046,7 +1046,288 @@ __global__ void k_psd_peak(const double* psd, int nt, int nx, double* out) {
     }
 }
 
+// ------------------------------------------------------------ bed spectrum, factored
+// Series whose rows and columns fit shared memory (both extents up to
+// FFT_MAX) take mixed-radix transforms instead of the direct sums: FP64 runs
+// at 1/64 of the FP32 rate here, so the operation count is the bound
+// (500 x 3072 samples: 2.4e10 FP64 operations directly, 1.6e8 factored; the call
+// went from 24.7 ms to 0.42 ms, of which 0.11 ms are each of the two transforms;
+// the mean and the peak, each by one block before, took 0.45 ms apiece).
+// Stockham passes between two shared buffers: with L the product of the
+// radices done, Y_L[j][k] = sum_b x[k + (N/L) b] W_L^(b j) (index j N/L + k), a
+// pass of radix r forms Y_rL[j + L c][k] = sum_a W_r^(a c) (W_rL^(a j)
+// Y_L[j][k + M a]), M = N/(r L). Radices 4, 2, 3 and 5 are butterflies, any
+// other prime factor a direct sum over its r inputs.
+constexpr int FFT_MAX = 7168;            // two buffers of complex FP64: 224 KB
+constexpr int FFT_THREADS = 512;
+constexpr int FFT_SUMS = 64;             // partial sums of the mean
+constexpr int FFT_BLOCKS = 512;          // column blocks, one partial peak each
+
+struct Radices {
+    int n;
+    int r[16];                           // 7168 < 2^13
+};
+
+static Radices factor(int N) {
+    Radices f = {};
+    for (int p : {4, 2, 3, 5})
+        while (N % p == 0) { f.r[f.n++] = p; N /= p; }
+    for (int p = 7; N > 1; p += 2)
+        while (N % p == 0) { f.r[f.n++] = p; N /= p; }
+    return f;
+}
+
+__device__ __forceinline__ double2 c_add(double2 a, double2 b) { return make_double2(a.x + b.x, a.y + b.y); }
+__device__ __forceinline__ double2 c_sub(double2 a, double2 b) { return make_double2(a.x - b.x, a.y - b.y); }
+__device__ __forceinline__ double2 c_mul(double2 a, double2 b) {
+    return make_double2(fma(a.x, b.x, -a.y * b.y), fma(a.x, b.y, a.y * b.x));
+}
+__device__ __forceinline__ double2 c_mji(double2 a) { return make_double2(a.y, -a.x); }   // -i a
+
+template <int R>
+__device__ __forceinline__ void butterfly(double2 (&v)[R]) {
+    if constexpr (R == 2) {
+        const double2 t = v[1];
+        v[1] = c_sub(v[0], t);
+        v[0] = c_add(v[0], t);
+    } else if constexpr (R == 3) {
+        constexpr double s3 = 0.86602540378443864676;
+        const double2 t = c_add(v[1], v[2]), d = c_mji(c_sub(v[1], v[2]));
+        const double2 m = make_double2(fma(-0.5, t.x, v[0].x), fma(-0.5, t.y, v[0].y));
+        v[0] = c_add(v[0], t);
+        v[1] = make_double2(fma(s3, d.x, m.x), fma(s3, d.y, m.y));
+        v[2] = make_double2(fma(-s3, d.x, m.x), fma(-s3, d.y, m.y));
+    } else if constexpr (R == 4) {
+        const double2 a = c_add(v[0], v[2]), b = c_sub(v[0], v[2]), c = c_add(v[1], v[3]), d = c_mji(c_sub(v[1], v[3]));
+        v[0] = c_add(a, c);
+        v[1] = c_add(b, d);
+        v[2] = c_sub(a, c);
+        v[3] = c_sub(b, d);
+    } else {
+        // cos and sin of 2 pi / 5 and 4 pi / 5
+        constexpr double c1 = 0.30901699437494742410, c2 = -0.80901699437494742410;
+        constexpr double s1 = 0.95105651629515357212, s2 = 0.58778525229247312917;
+        const double2 p = c_add(v[1], v[4]), q = c_add(v[2], v[3]);
+        const double2 d = c_mji(c_sub(v[1], v[4])), e = c_mji(c_sub(v[2], v[3]));
+        const double2 m1 = make_double2(fma(c1, p.x, fma(c2, q.x, v[0].x)), fma(c1, p.y, fma(c2, q.y, v[0].y)));
+        const double2 m2 = make_double2(fma(c2, p.x, fma(c1, q.x, v[0].x)), fma(c2, p.y, fma(c1, q.y, v[0].y)));
+        const double2 n1 = make_double2(fma(s1, d.x, s2 * e.x), fma(s1, d.y, s2 * e.y));
+        const double2 n2 = make_double2(fma(s2, d.x, -s1 * e.x), fma(s2, d.y, -s1 * e.y));
+        v[0] = c_add(v[0], c_add(p, q));
+        v[1] = c_add(m1, n1);
+        v[2] = c_add(m2, n2);
+        v[3] = c_sub(m2, n2);
+        v[4] = c_sub(m1, n1);
+    }
+}
+
+template <int R>
+__device__ __forceinline__ void fft_pass(const double2* in, double2* out, const double2* tw, int N, int batch, int L) {
+    const unsigned M = (unsigned)(N / (L * R)), nb = (unsigned)(N / R);
+    for (unsigned t = threadIdx.x; t < nb * (unsigned)batch; t += blockDim.x) {
+        const unsigned col = t / nb, u = t - col * nb;
+        const unsigned j = u / M, k = u - j * M;
+        const double2* src = in + col * (unsigned)N + j * (R * M) + k;
+        double2 v[R];
+#pragma unroll
+        for (int a = 0; a < R; ++a) v[a] = src[a * M];
+#pragma unroll
+        for (int a = 1; a < R; ++a) v[a] = c_mul(v[a], tw[a * j * M]);
+        butterfly<R>(v);
+        double2* dst = out + col * (unsigned)N + j * M + k;
+#pragma unroll
+        for (int c = 0; c < R; ++c) dst[(unsigned)c * (unsigned)L * M] = v[c];
+    }
+}
+// any radix r: one output per thread
+__device__ __forceinline__ void fft_pass_any(const double2* in, double2* out, const double2* tw, int N, int batch, int L,
+                                             int r) {
+    const unsigned M = (unsigned)(N / (L * r)), rl = (unsigned)(L * r);
+    for (unsigned t = threadIdx.x; t < (unsigned)N * (unsigned)batch; t += blockDim.x) {
+        const unsigned col = t / (unsigned)N, u = t - col * (unsigned)N;
+        const unsigned jj = u / M, k = u - jj * M;       // output Y_rL[jj][k]
+        const double2* src = in + col * (unsigned)N + (jj % (unsigned)L) * ((unsigned)r * M) + k;
+        double2 acc = make_double2(0.0, 0.0);
+        unsigned w = 0;                                   // a jj mod rL
+        for (int a = 0; a < r; ++a) {
+            const double2 x = src[(unsigned)a * M], e = tw[w * M];
+            acc.x = fma(x.x, e.x, fma(-x.y, e.y, acc.x));
+            acc.y = fma(x.x, e.y, fma(x.y, e.x, acc.y));
+            w += jj;
+            if (w >= rl) w -= rl;
+        }
+        out[col * (unsigned)N + u] = acc;
+    }
+}
+// transforms `batch` sequences of N values in a (column by column), between
+// a and b; returns the buffer that holds the result. Every thread of the
+// block calls it, after a barrier behind the loads of a.
+__device__ __forceinline__ double2* block_fft(double2* a, double2* b, const double2* tw, int N, int batch,
+                                              const Radices& f) {
+    int L = 1;
+    for (int i = 0; i < f.n; ++i) {
+        const int r = f.r[i];
+        if (r == 4) fft_pass<4>(a, b, tw, N, batch, L);
+        else if (r == 2) fft_pass<2>(a, b, tw, N, batch, L);
+        else if (r == 3) fft_pass<3>(a, b, tw, N, batch, L);
+        else if (r == 5) fft_pass<5>(a, b, tw, N, batch, L);
+        else fft_pass_any(a, b, tw, N, batch, L, r);
+        L *= r;
+        double2* t = a;
+        a = b;
+        b = t;
+        __syncthreads();
+    }
+    return a;
+}
+
+// twiddles exp(-2 pi i k / N) of both extents, and the series' partial sums
+// (block b adds values b, b + FFT_SUMS, ... of 256 each, in a fixed order)
+__global__ void __launch_bounds__(256) k_fft_setup(const double* h, long long n, double2* twx, int nx, double2* twt,
+                                                   int nt, double* sums) {
+    __shared__ double sh[256];
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    for (int k = t; k < nx + nt; k += gridDim.x * blockDim.x) {
+        const bool x = k < nx;
+        double sn, cs;
+        sincospi(2.0 * (double)(x ? k : k - nx) / (double)(x ? nx : nt), &sn, &cs);
+        (x ? twx : twt)[x ? k : k - nx] = make_double2(cs, -sn);
+    }
+    double v = 0.0;
+#pragma unroll 4
+    for (long long i = t; i < n; i += (long long)gridDim.x * blockDim.x) v += h[i];
+    sh[threadIdx.x] = v;
+    __syncthreads();
+    for (int off = 128; off > 0; off >>= 1) {
+        if ((int)threadIdx.x < off) sh[threadIdx.x] += sh[threadIdx.x + off];
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) sums[blockIdx.x] = sh[0];
+}
+
+// X1[t][j], j = 0 .. nx/2: the transforms along x of two rows at once, as the
+// real and the imaginary part of one sequence (X_t[j] = (Z[j] + conj Z[-j])/2,
+// X_t+1[j] = (Z[j] - conj Z[-j])/2i); the upper half follows by symmetry
+__global__ void __launch_bounds__(FFT_THREADS) k_fft_x(const double* h, const double* sums, const double2* tw, int nt,
+                                                       int nx, Radices f, double2* X1) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    double2* a = reinterpret_cast<double2*>(smem_raw);
+    const int t = 2 * blockIdx.x, hx = nx / 2 + 1;
+    double m = 0.0;
+    for (int k = 0; k < FFT_SUMS; ++k) m += sums[k];
+    m /= (double)nt * (double)nx;
+    const double* h0 = h + (long long)t * nx;
+    const bool two = t + 1 < nt;
+    for (int x = threadIdx.x; x < nx; x += blockDim.x) a[x] = make_double2(h0[x] - m, two ? h0[nx + x] - m : 0.0);
+    __syncthreads();
+    const double2* Z = block_fft(a, a + nx, tw, nx, 1, f);
+    for (int j = threadIdx.x; j < hx; j += blockDim.x) {
+        const double2 p = Z[j], q = Z[j == 0 ? 0 : nx - j];
+        X1[(long long)t * hx + j] = make_double2(0.5 * (p.x + q.x), 0.5 * (p.y - q.y));
+        if (two) X1[(long long)(t + 1) * hx + j] = make_double2(0.5 * (p.y + q.y), 0.5 * (q.x - p.x));
+    }
+}
+
+// psd[l][j] = |transform of X1 along t|^2 / (nt nx) and its mirror image
+// psd[-l][-j], `cols` adjacent wavenumbers per pass of a block; the block's
+// largest value at wavenumbers j >= 1 (ties: the lowest l, then j)
+__global__ void __launch_bounds__(FFT_THREADS) k_fft_t(const double2* X1, const double2* tw, int nt, int nx, int cols,
+                                                       Radices f, double* psd, double* peaks) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ double sv[FFT_THREADS / 32];
+    __shared__ long long si[FFT_THREADS / 32];
+    double2* a = reinterpret_cast<double2*>(smem_raw);
+    const int hx = nx / 2 + 1, jm = nx / 2;
+    const double norm = (double)nt * (double)nx;
+    double best = -1.0;
+    long long bi = 0x7fffffffffffffffLL;
+    for (int j0 = blockIdx.x * cols; j0 < hx; j0 += gridDim.x * cols) {
+        const int nc = min(cols, hx - j0);
+        for (int i = threadIdx.x; i < nt * nc; i += blockDim.x) {
+            const int t = i / nc, c = i - t * nc;
+            a[c * nt + t] = X1[(long long)t * hx + j0 + c];
+        }
+        __syncthreads();
+        const double2* Y = block_fft(a, a + nt * cols, tw, nt, nc, f);
+        for (int i = threadIdx.x; i < nt * nc; i += blockDim.x) {
+            const int l = i / nc, c = i - l * nc, j = j0 + c;
+            const double2 v = Y[c * nt + l];
+            const double p = (v.x * v.x + v.y * v.y) / norm;
+            psd[(long long)l * nx + j] = p;
+            if (j > 0 && 2 * j != nx) psd[(long long)(l == 0 ? 0 : nt - l) * nx + (nx - j)] = p;
+            if (j > 0) {
+                const long long id = (long long)l * jm + (j - 1);
+                if (p > best || (p == best && id < bi)) { best = p; bi = id; }
+            }
+        }
+        __syncthreads();
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+        const double v = __shfl_xor_sync(0xffffffffu, best, o);
+        const long long i = __shfl_xor_sync(0xffffffffu, bi, o);
+        if (v > best || (v == best && i < bi)) { best = v; bi = i; }
+    }
+    if ((threadIdx.x & 31) == 0) { sv[threadIdx.x >> 5] = best; si[threadIdx.x >> 5] = bi; }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int w = 1; w < FFT_THREADS / 32; ++w)
+            if (sv[w] > best || (sv[w] == best && si[w] < bi)) { best = sv[w]; bi = si[w]; }
+        peaks[2 * blockIdx.x] = best;
+        peaks[2 * blockIdx.x + 1] = (double)bi;
+    }
+}
+// out[0] value, out[1] l, out[2] j of the blocks' largest
+__global__ void k_fft_peak(const double* peaks, int n, int nx, double* out) {
+    double best = -1.0, bi = 1e300;
+    for (int k = threadIdx.x; k < n; k += 32) {
+        const double v = peaks[2 * k], i = peaks[2 * k + 1];
+        if (v > best || (v == best && i < bi)) { best = v; bi = i; }
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+        const double v = __shfl_xor_sync(0xffffffffu, best, o), i = __shfl_xor_sync(0xffffffffu, bi, o);
+        if (v > best || (v == best && i < bi)) { best = v; bi = i; }
+    }
+    if (threadIdx.x == 0) {
+        // no value at all (a series with NaN): index -1, as k_psd_peak
+        const long long i = best < 0.0 ? -1 : (long long)bi, jm = nx / 2;
+        out[0] = best;
+        out[1] = (double)(i / jm);
+        out[2] = (double)(1 + i % jm);
+    }
+}
+
+static bool fft_fits(long long nt, long long nx) { return nt <= FFT_MAX && nx <= FFT_MAX; }
+
+// doubles of device scratch of launch_bed_spectrum
+size_t bed_spectrum_work(long long nt, long long nx) {
+    const size_t tw = 2 * ((size_t)nx + nt);
+    if (fft_fits(nt, nx)) return tw + 2 * (size_t)nt * (nx / 2 + 1) + FFT_SUMS + 2 * FFT_BLOCKS + 3;
+    return tw + 2 * (size_t)nt * nx + 4;
+}
+
 int launch_bed_spectrum(const double* h, int nt, int nx, double* psd, double* work, double* peak3, cudaStream_t st) {
+    if (fft_fits(nt, nx)) {
+        // twiddles, the half-spectrum rows, partial sums and peaks
+        double2* twx = reinterpret_cast<double2*>(work);
+        double2* twt = twx + nx;
+        double2* X1 = twt + nt;
+        double* sums = reinterpret_cast<double*>(X1 + (size_t)nt * (nx / 2 + 1));
+        double* peaks = sums + FFT_SUMS;
+        // columns per block pass: whole 64-byte segments while two buffers of
+        // them fit twice on an SM, or as many as fit at all
+        int cols = 4;
+        while (cols > 1 && cols * nt > FFT_MAX) cols /= 2;
+        const int hx = nx / 2 + 1;
+        const int blocks = std::min(FFT_BLOCKS, (hx + cols - 1) / cols);
+        const int smx = 2 * nx * (int)sizeof(double2), smt = 2 * cols * nt * (int)sizeof(double2);
+        cudaFuncSetAttribute(k_fft_x, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * FFT_MAX * (int)sizeof(double2));
+        cudaFuncSetAttribute(k_fft_t, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * FFT_MAX * (int)sizeof(double2));
+        k_fft_setup<<<FFT_SUMS, 256, 0, st>>>(h, (long long)nt * nx, twx, nx, twt, nt, sums);
+        k_fft_x<<<(unsigned)((nt + 1) / 2), FFT_THREADS, smx, st>>>(h, sums, twx, nt, nx, factor(nx), X1);
+        k_fft_t<<<blocks, FFT_THREADS, smt, st>>>(X1, twt, nt, nx, cols, factor(nt), psd, peaks);
+        k_fft_peak<<<1, 32, 0, st>>>(peaks, blocks, nx, peak3);
+        return 4;
+    }
     // work: nx + nt twiddles, nt * nx transformed values (complex), the mean
     double2* twx = reinterpret_cast<double2*>(work);
     double2* twt = twx + nx;
