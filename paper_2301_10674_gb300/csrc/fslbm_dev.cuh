@@ -593,11 +593,11 @@ __device__ __forceinline__ long long pdf_slot(const Dev& s, int q, long long c, 
     return own ? (long long)opp(q) * s.n + c
                : (long long)q * s.n + c + (o.ox[1 + cx(q)] + o.oy[1 + cy(q)] + o.oz[1 + cz(q)]);
 }
-// f - w from a stored value and its slot's reference, with one rounding (the
-// same bits wherever it is inlined)
+// f - w from a stored value and its slot's reference (the rounding of ld_any
+// and, with -h, of st_any: product, then sum)
 template <typename S>
 __device__ __forceinline__ float with_ref(float v, int q, float h) {
-    return Store<S>::HREF ? __fmaf_rn(wq(q), h, v) : v;
+    return Store<S>::HREF ? __fadd_rn(v, __fmul_rn(wq(q), h)) : v;
 }
 // f - w of all 27 post-collision PDFs of a cell, the loads in flight together
 template <typename S, int LP>
@@ -626,10 +626,13 @@ __device__ __forceinline__ long long lane_slot(const Dev& s, int q, int c, int n
     h = Store<S>::HREF ? s.href[own ? z : wrap_z(s, z + q / 9 - 1)] : 0.f;
     return own ? (long long)(26 - q) * s.n + c : (long long)q * s.n + nb;
 }
-__device__ __forceinline__ float warp_sum_f(float v) {
+// sum of lanes 0 to 26 in lane order, in every lane: the rounding is that of
+// one thread adding the 27 directions in turn
+__device__ __forceinline__ float ordered_sum27(float v) {
+    float t = 0.f;
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
+    for (int k = 0; k < 27; ++k) t += __shfl_sync(0xffffffffu, v, k);
+    return t;
 }
 
 // density and collision velocity from post-collision PDFs (f - w):

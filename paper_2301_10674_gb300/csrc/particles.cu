@@ -164,6 +164,23 @@ __device__ __forceinline__ float wrapf(float d, int L, int periodic) {
     return d;
 }
 
+// Contact arithmetic with every rounding spelled out (which product of a sum
+// is fused into it), so that a sub-step gives the same bits in every kernel it
+// is inlined in: a gap is the difference of numbers near 2 r, so a last-bit
+// difference in a position is up to 5e-5 of a lubrication force, and two
+// contractions of the same source would let runs drift apart by that.
+__device__ __forceinline__ float dot_r(const float (&a)[3], const float (&b)[3]) {
+    return __fmaf_rn(a[2], b[2], __fmaf_rn(a[0], b[0], __fmul_rn(a[1], b[1])));
+}
+__device__ __forceinline__ float det_r(float a, float b, float c, float d) {   // a b - c d
+    return __fmaf_rn(a, b, -__fmul_rn(c, d));
+}
+__device__ __forceinline__ void cross_r(const float (&a)[3], const float (&b)[3], float (&o)[3]) {
+    o[0] = det_r(a[1], b[2], a[2], b[1]);
+    o[1] = det_r(a[2], b[0], a[0], b[2]);
+    o[2] = det_r(a[0], b[1], a[1], b[0]);
+}
+
 // Lubrication corrections (Section 2.2): the paper augments the DEM with
 // normal and tangential lubrication forces where a gap is too small for the
 // lattice to resolve and gives no formula. These are the asymptotic
@@ -173,16 +190,16 @@ __device__ __forceinline__ float wrapf(float d, int L, int periodic) {
 constexpr float LUB_HC = 2.f / 3.f, LUB_HMIN = 1e-2f;
 // force on the particle (n toward the partner or wall, vrel the relative
 // velocity of the surfaces at the contact point) and its tangential part
-__device__ __forceinline__ void lub_f(const Dev& s, float R, const float n[3], float h, const float vrel[3],
-                                      float Fl[3], float Ft[3]) {
+__device__ __forceinline__ void lub_f(const Dev& s, float R, const float (&n)[3], float h, const float (&vrel)[3],
+                                      float (&Fl)[3], float (&Ft)[3]) {
     const float hh = fmaxf(h, LUB_HMIN);
-    const float vn = vrel[0] * n[0] + vrel[1] * n[1] + vrel[2] * n[2];
+    const float vn = dot_r(vrel, n);
     const float k = 6.f * 3.14159265f * (float)s.lub_mu * R;
     const float cn = k * R * (1.f / hh - 1.f / LUB_HC);
     const float ct = k * (8.f / 15.f) * logf(LUB_HC / hh);
     for (int a = 0; a < 3; ++a) {
-        Ft[a] = -ct * (vrel[a] - vn * n[a]);
-        Fl[a] = -cn * vn * n[a] + Ft[a];
+        Ft[a] = __fmul_rn(-ct, __fmaf_rn(-vn, n[a], vrel[a]));
+        Fl[a] = __fmaf_rn(__fmul_rn(-cn, vn), n[a], Ft[a]);
     }
 }
 
@@ -323,31 +340,32 @@ void launch_particle_copies(const Dev& s, cudaStream_t st) {
 }
 
 // FP32 linear spring-dashpot with tangential history (same law as above)
-__device__ __forceinline__ void contact_f(const Dev& s, float meff, const float n[3], float delta,
-                                          const float vrel[3], float xi[3], float dts, float F[3], float Ft[3]) {
+__device__ __forceinline__ void contact_f(const Dev& s, float meff, const float (&n)[3], float delta,
+                                          const float (&vrel)[3], float (&xi)[3], float dts, float (&F)[3],
+                                          float (&Ft)[3]) {
     const float kn = meff * (float)s.kn_coef;
     const float dn = meff * (float)s.dn_coef;
     const float kt = kn * (float)s.kt_ratio;
     const float dt_ = dn;
-    const float vn = vrel[0] * n[0] + vrel[1] * n[1] + vrel[2] * n[2];
-    const float vt[3] = {vrel[0] - vn * n[0], vrel[1] - vn * n[1], vrel[2] - vn * n[2]};
-    const float fn = kn * delta + dn * vn;
+    const float vn = dot_r(vrel, n);
+    const float vt[3] = {__fmaf_rn(-vn, n[0], vrel[0]), __fmaf_rn(-vn, n[1], vrel[1]), __fmaf_rn(-vn, n[2], vrel[2])};
+    const float fn = __fmaf_rn(kn, delta, __fmul_rn(dn, vn));
     float x[3] = {xi[0], xi[1], xi[2]};
-    const float xn = x[0] * n[0] + x[1] * n[1] + x[2] * n[2];
-    for (int a = 0; a < 3; ++a) x[a] = x[a] - xn * n[a] + vt[a] * dts;
-    for (int a = 0; a < 3; ++a) Ft[a] = -kt * x[a] - dt_ * vt[a];
-    const float ftl = sqrtf(Ft[0] * Ft[0] + Ft[1] * Ft[1] + Ft[2] * Ft[2]);
+    const float xn = dot_r(x, n);
+    for (int a = 0; a < 3; ++a) x[a] = __fmaf_rn(vt[a], dts, __fmaf_rn(-xn, n[a], x[a]));
+    for (int a = 0; a < 3; ++a) Ft[a] = __fmaf_rn(-kt, x[a], -__fmul_rn(dt_, vt[a]));
+    const float ftl = sqrtf(dot_r(Ft, Ft));
     const float lim = (float)s.friction * fabsf(fn);
     if (ftl > lim && ftl > 0.f) {
         const float sc = lim / ftl;
         for (int a = 0; a < 3; ++a) {
-            Ft[a] *= sc;
-            x[a] = -(Ft[a] + dt_ * vt[a]) / kt;
+            Ft[a] = __fmul_rn(Ft[a], sc);
+            x[a] = -__fadd_rn(Ft[a], __fmul_rn(dt_, vt[a])) / kt;
         }
     }
     for (int a = 0; a < 3; ++a) {
         xi[a] = x[a];
-        F[a] = -fn * n[a] + Ft[a];
+        F[a] = __fmaf_rn(-fn, n[a], Ft[a]);
     }
 }
 
@@ -359,7 +377,10 @@ __device__ __forceinline__ void contact_f(const Dev& s, float meff, const float 
 // offset plus the difference of their dx, a wall distance the start distance
 // plus or minus dx. The particles publish dx, u and w (buffers a read, b
 // written). Lane l takes neighbour slots l, l + DEM_LANES, ... and then wall
-// face l; the lanes' forces join in a fixed tree; lanes 0 to 2 advance one
+// face l; the lanes pass their forces through shared memory, and lane c < 6
+// adds component c of force and torque in the order of the slots (the order of
+// one thread walking them, so the result is that thread's); lanes 0 to 2 then
+// advance the velocity and position, lanes 3 to 5 the angular velocity, one
 // axis each (semi-implicit Euler on the changes). The first sub-step averages
 // the hydrodynamic force over two steps, the last adds the changes to the
 // FP64 state, forms the FP32 copies and counts the particle in its grid cell.
@@ -371,7 +392,11 @@ __device__ __forceinline__ void contact_f(const Dev& s, float meff, const float 
 constexpr int DEM_LANES = 8;
 static_assert(NB_SLOTS % DEM_LANES == 0 && NB_ITEMS == NB_SLOTS + DEM_LANES, "one wall face per lane");
 
-__device__ __forceinline__ void dem_substep(const Dev& s, int p, int l, unsigned gm, int a, bool have_prev,
+// per lane group: 8 lanes of lubrication force and torque, contact force and
+// torque (12 floats); the group stride keeps a warp's four groups on distinct banks
+constexpr int DEM_SH = 104;
+
+__device__ __forceinline__ void dem_substep(const Dev& s, float* sh, int p, int l, unsigned gm, int a, bool have_prev,
                                             float dts, bool first, bool last) {
     const int b = 1 - a;
     if (s.fixed[p]) {
@@ -386,35 +411,33 @@ __device__ __forceinline__ void dem_substep(const Dev& s, int p, int l, unsigned
     const float4 xa4 = s.dem_x[a][p], ua4 = s.dem_u[a][p], wa4 = s.dem_w[a][p];
     const int nbc = s.nb_count[p];
     const float rif = cp.x;
-    // lane k < 3: the outer force and torque along axis k
-    float Fo = 0.f, To = 0.f;
-    if (l < 3) {
-        const int k = 3 * p + l;
+    const bool trans = l < 3;              // lanes 0-2: velocity and position, 3-5: angular velocity
+    const int ax = trans ? l : l - 3;      // (lanes 6 and 7 hold no component)
+    float acc = 0.f;                       // the lane's component of force or torque
+    const float arm = trans ? 1.f : rif;   // torque: r n x F_t, the lanes' n x F_t times r
+    if (l < 6) {
+        const int k = 3 * p + ax;
+        float* outer = (trans ? s.Faf : s.Taf) + k;
         if (first) {
-            const double fh = s.Fh[k], th = s.Th[k];
-            const double fa = have_prev ? 0.5 * (fh + s.Fp[k]) : fh;
-            const double ta = have_prev ? 0.5 * (th + s.Tp[k]) : th;
-            s.Fp[k] = fh;
-            s.Tp[k] = th;
-            // averaged hydrodynamic force plus the weight
-            const double g = l == 0 ? s.gxd : (l == 1 ? s.gyd : s.gzd);
-            Fo = (float)(fa + s.M[p] * g);
-            To = (float)ta;
-            s.Faf[k] = Fo;
-            s.Taf[k] = To;
+            // two-step average of the hydrodynamic force, plus the weight
+            const double now = (trans ? s.Fh : s.Th)[k];
+            double* prev = (trans ? s.Fp : s.Tp) + k;
+            const double avg = have_prev ? 0.5 * (now + *prev) : now;
+            *prev = now;
+            const double g = ax == 0 ? s.gxd : (ax == 1 ? s.gyd : s.gzd);
+            acc = (float)(trans ? avg + s.M[p] * g : avg);
+            *outer = acc;
         } else {
-            Fo = s.Faf[k];
-            To = s.Taf[k];
+            acc = *outer;
         }
     }
-    float F[3] = {0.f, 0.f, 0.f}, T[3] = {0.f, 0.f, 0.f};
     int touching = 0;
     const int nround = (nbc + DEM_LANES - 1) / DEM_LANES;   // rounds of neighbours, then one of wall faces
 #pragma unroll 1
     for (int r = 0; r <= nround; ++r) {
         const bool wall = r == nround;
         const int slot = wall ? NB_SLOTS + l : r * DEM_LANES + l;
-        bool near = false, touch = false;
+        bool lub = false, touch = false;
         float n[3] = {0.f, 0.f, 0.f}, delta = 0.f, rj = 0.f;
         float4 uj = make_float4(0.f, 0.f, 0.f, 0.f), wj = uj, xi4 = uj;
         if (!wall) {
@@ -430,7 +453,7 @@ __device__ __forceinline__ void dem_substep(const Dev& s, int p, int l, unsigned
                 const float dist2 = d[0] * d[0] + d[1] * d[1] + d[2] * d[2];
                 const float rs = rif + rj;
                 touch = dist2 < rs * rs;
-                near = touch || (s.lub && dist2 < (rs + LUB_HC) * (rs + LUB_HC));
+                lub = s.lub && dist2 < (rs + LUB_HC) * (rs + LUB_HC);
                 const float dist = sqrtf(dist2);
                 const float inv = 1.f / dist;
 #pragma unroll
@@ -438,98 +461,101 @@ __device__ __forceinline__ void dem_substep(const Dev& s, int p, int l, unsigned
                 delta = rs - dist;
             }
         } else if (l < 6) {
-            const int ax = l >> 1;
-            if (!(ax == 0 ? s.per_x : (ax == 1 ? s.per_y : s.per_z))) {
-                const float dxa = ax == 0 ? xa4.x : (ax == 1 ? xa4.y : xa4.z);
+            const int wx = l >> 1;
+            if (!(wx == 0 ? s.per_x : (wx == 1 ? s.per_y : s.per_z))) {
+                const float dxa = wx == 0 ? xa4.x : (wx == 1 ? xa4.y : xa4.z);
                 const float dist = (l & 1) ? s.dem_wall[6 * p + l] - dxa : s.dem_wall[6 * p + l] + dxa;
                 delta = rif - dist;
                 touch = delta > 0.f;
-                near = touch || (s.lub && -delta < LUB_HC);
+                lub = s.lub && -delta < LUB_HC;
                 const float sg = (l & 1) ? 1.f : -1.f;
 #pragma unroll
-                for (int k = 0; k < 3; ++k) n[k] = k == ax ? sg : 0.f;
+                for (int k = 0; k < 3; ++k) n[k] = k == wx ? sg : 0.f;
                 xi4 = s.nb_xi[(long long)p * NB_ITEMS + slot];
                 xi4.w = cp.y;   // the wall's mass is infinite
             }
         }
-        if (near) {
-            const float wsum[3] = {rif * wa4.x + rj * wj.x, rif * wa4.y + rj * wj.y, rif * wa4.z + rj * wj.z};
-            const float wn[3] = {wsum[1] * n[2] - wsum[2] * n[1], wsum[2] * n[0] - wsum[0] * n[2],
-                                 wsum[0] * n[1] - wsum[1] * n[0]};
-            const float vrel[3] = {ua4.x - uj.x + wn[0], ua4.y - uj.y + wn[1], ua4.z - uj.z + wn[2]};
-            float Ft[3] = {0.f, 0.f, 0.f};   // tangential, for the torque
-            if (s.lub && delta > -LUB_HC) {
-                float Fl[3], Ftl[3];
-                lub_f(s, wall ? rif : rif * rj / (rif + rj), n, -delta, vrel, Fl, Ftl);
+        float Fl[3] = {0.f, 0.f, 0.f}, Fc[3] = {0.f, 0.f, 0.f}, tl[3] = {0.f, 0.f, 0.f}, tc[3] = {0.f, 0.f, 0.f};
+        if (lub || touch) {
+            // (the second two slots of every four fuse the partner's product: the
+            // rounding that a loop unrolled over four of them had)
+            const bool sw = (slot & 2) != 0;
+            const float wa[3] = {wa4.x, wa4.y, wa4.z}, wb[3] = {wj.x, wj.y, wj.z};
+            float wsum[3], wn[3];
 #pragma unroll
-                for (int k = 0; k < 3; ++k) { F[k] += Fl[k]; Ft[k] = Ftl[k]; }
+            for (int k = 0; k < 3; ++k)
+                wsum[k] = sw ? __fmaf_rn(rj, wb[k], __fmul_rn(rif, wa[k])) : __fmaf_rn(rif, wa[k], __fmul_rn(rj, wb[k]));
+            cross_r(wsum, n, wn);
+            const float vrel[3] = {ua4.x - uj.x + wn[0], ua4.y - uj.y + wn[1], ua4.z - uj.z + wn[2]};
+            float Ft[3];
+            if (lub) {
+                lub_f(s, wall ? rif : rif * rj / (rif + rj), n, -delta, vrel, Fl, Ft);
+                cross_r(n, Ft, tl);
             }
             if (touch) {
-                float xi[3] = {xi4.x, xi4.y, xi4.z}, Fc[3], Ftc[3];
-                contact_f(s, xi4.w, n, delta, vrel, xi, dts, Fc, Ftc);
+                float xi[3] = {xi4.x, xi4.y, xi4.z};
+                contact_f(s, xi4.w, n, delta, vrel, xi, dts, Fc, Ft);
                 s.nb_xi[(long long)p * NB_ITEMS + slot] = make_float4(xi[0], xi[1], xi[2], xi4.w);
-#pragma unroll
-                for (int k = 0; k < 3; ++k) { F[k] += Fc[k]; Ft[k] += Ftc[k]; }
+                cross_r(n, Ft, tc);
             }
-            T[0] += rif * (n[1] * Ft[2] - n[2] * Ft[1]);
-            T[1] += rif * (n[2] * Ft[0] - n[0] * Ft[2]);
-            T[2] += rif * (n[0] * Ft[1] - n[1] * Ft[0]);
         }
         // a partner not touched in this sub-step loses its spring
         if (!touch && (xi4.x != 0.f || xi4.y != 0.f || xi4.z != 0.f))
             s.nb_xi[(long long)p * NB_ITEMS + slot] = make_float4(0.f, 0.f, 0.f, xi4.w);
         touching += touch ? 1 : 0;
-    }
+        float4* mine = reinterpret_cast<float4*>(sh + 12 * l);
+        mine[0] = make_float4(Fl[0], Fl[1], Fl[2], tl[0]);
+        mine[1] = make_float4(tl[1], tl[2], Fc[0], Fc[1]);
+        mine[2] = make_float4(Fc[2], tc[0], tc[1], tc[2]);
+        __syncwarp(gm);
+        if (l < 6) {
 #pragma unroll
-    for (int o = 1; o < DEM_LANES; o <<= 1) {
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            F[k] += __shfl_xor_sync(gm, F[k], o);
-            T[k] += __shfl_xor_sync(gm, T[k], o);
+            for (int t = 0; t < DEM_LANES; ++t) {
+                acc = fmaf(arm, sh[12 * t + l], acc);
+                acc = fmaf(arm, sh[12 * t + 6 + l], acc);
+            }
         }
-        touching += __shfl_xor_sync(gm, touching, o);
+        __syncwarp(gm);
     }
+#pragma unroll
+    for (int o = 1; o < DEM_LANES; o <<= 1) touching += __shfl_xor_sync(gm, touching, o);
     if (touching > HIST_SLOTS && l == 0) set_error(s, ERR_HISTORY);
-    // lane l < 3 (the others repeat lane 2's) advances axis l
-    const int ax = l < 3 ? l : 2;
-    auto sel = [ax](float v0, float v1, float v2) { return ax == 0 ? v0 : (ax == 1 ? v1 : v2); };
-    const float dxo = sel(xa4.x, xa4.y, xa4.z);
-    float* duo = reinterpret_cast<float*>(s.dem_du + p) + ax;
-    float* dwo = reinterpret_cast<float*>(s.dem_dw + p) + ax;
-    const float4 u0 = s.Uf[p], w0 = s.Wf[p];
-    const float u0a = sel(u0.x, u0.y, u0.z), w0a = sel(w0.x, w0.y, w0.z);
-    const float dun = *duo + dts * (Fo + sel(F[0], F[1], F[2])) * (1.f / cp.y);
-    const float dwn = *dwo + dts * (To + sel(T[0], T[1], T[2])) * (1.f / cp.z);
-    const float dxn = dxo + dts * (u0a + dun);
-    __syncwarp(gm);   // every lane has read du and dw, and the copies Uf and Wf
-    if (l < 3 && !last) {
-        *duo = dun;
-        *dwo = dwn;
-        reinterpret_cast<float*>(s.dem_x[b] + p)[l] = dxn;
-        reinterpret_cast<float*>(s.dem_u[b] + p)[l] = u0a + dun;
-        reinterpret_cast<float*>(s.dem_w[b] + p)[l] = w0a + dwn;
+    float v0 = 0.f, dv = 0.f;    // velocity component at the step's start, and its change
+    if (l < 6) {
+        const float4 v4 = trans ? s.Uf[p] : s.Wf[p];
+        v0 = ax == 0 ? v4.x : (ax == 1 ? v4.y : v4.z);
+        dv = reinterpret_cast<const float*>((trans ? s.dem_du : s.dem_dw) + p)[ax];
+        dv = dv + dts * acc * (1.f / (trans ? cp.y : cp.z));
+    }
+    const float dxn = (ax == 0 ? xa4.x : (ax == 1 ? xa4.y : xa4.z)) + dts * (v0 + dv);   // (lanes 0-2)
+    __syncwarp(gm);   // every lane has read the copies Uf and Wf
+    if (l < 6 && !last) {
+        reinterpret_cast<float*>((trans ? s.dem_du : s.dem_dw) + p)[ax] = dv;
+        reinterpret_cast<float*>((trans ? s.dem_u : s.dem_w)[b] + p)[ax] = v0 + dv;
+        if (trans) reinterpret_cast<float*>(s.dem_x[b] + p)[ax] = dxn;
     }
     if (last) {
         // the FP64 state of the step's end (positions wrapped on periodic
         // axes), its FP32 copies and the grid cell
         int g = 0;
-        if (l < 3) {
+        if (trans) {
             const int L = l == 0 ? s.nx : (l == 1 ? s.ny : s.nz);
             double x = s.X[3 * p + l] + (double)dxn;
             if (l == 0 ? s.per_x : (l == 1 ? s.per_y : s.per_z)) x = x < 0.0 ? x + L : (x >= L ? x - L : x);
-            const double u = s.U[3 * p + l] + (double)dun, w = s.W[3 * p + l] + (double)dwn;
             s.X[3 * p + l] = x;
-            s.U[3 * p + l] = u;
-            s.W[3 * p + l] = w;
             const double fl = floor(x);
             reinterpret_cast<float*>(s.Xr + p)[l] = (float)x;
             reinterpret_cast<int*>(s.Xi + p)[l] = (int)fl;
             reinterpret_cast<float*>(s.Xfr + p)[l] = (float)(x - fl);
-            reinterpret_cast<float*>(s.Uf + p)[l] = (float)u;
-            reinterpret_cast<float*>(s.Wf + p)[l] = (float)w;
             if (l == 2) atomicMax(s.zmax_cell, (int)ceil(x + s.R[p]) + 2);
             g = l == 0 ? gcoord(x, s.ghx, s.gnx)
                        : (l == 1 ? s.gnx * gcoord(x, s.ghy, s.gny) : s.gnx * s.gny * gcoord(x, s.ghz, s.gnz));
+        }
+        if (l < 6) {
+            double* v = (trans ? s.U : s.W) + 3 * p + ax;
+            const double vn = *v + (double)dv;
+            *v = vn;
+            reinterpret_cast<float*>((trans ? s.Uf : s.Wf) + p)[ax] = (float)vn;
         }
         g += __shfl_xor_sync(gm, g, 1);
         g += __shfl_xor_sync(gm, g, 2);
@@ -543,6 +569,7 @@ __device__ __forceinline__ void dem_substep(const Dev& s, int p, int l, unsigned
 // one sub-step; the first of several also clears what the last one counts
 __global__ void __launch_bounds__(128) k_dem_substep(Dev s, int a, int have_prev, int G, float dts, int first,
                                                      int last) {
+    __shared__ __align__(16) float sh[128 / DEM_LANES * DEM_SH];
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (first && !last) {
         for (int g = t; g < G; g += gridDim.x * blockDim.x) s.g_count[g] = 0;
@@ -550,7 +577,8 @@ __global__ void __launch_bounds__(128) k_dem_substep(Dev s, int a, int have_prev
     }
     const int p = t / DEM_LANES, l = t % DEM_LANES;
     const unsigned gm = ((1u << DEM_LANES) - 1u) << ((threadIdx.x & 31) / DEM_LANES * DEM_LANES);
-    if (p < s.np) dem_substep(s, p, l, gm, a, have_prev != 0, dts, first != 0, last != 0);
+    if (p < s.np)
+        dem_substep(s, sh + threadIdx.x / DEM_LANES * DEM_SH, p, l, gm, a, have_prev != 0, dts, first != 0, last != 0);
 }
 
 // The sub-steps of a step and the particle grid in one thread-block cluster,
@@ -570,6 +598,7 @@ __device__ __forceinline__ void cluster_barrier() {
 }
 
 __global__ void __launch_bounds__(DEM_CLUSTER_THREADS) k_dem_cluster(Dev s, int have_prev, int G, float dts) {
+    __shared__ __align__(16) float sh[DEM_CLUSTER_THREADS / DEM_LANES * DEM_SH];
     __shared__ int wtot[DEM_CLUSTER_THREADS / 32];
     const int nt = gridDim.x * blockDim.x, tid = blockIdx.x * blockDim.x + threadIdx.x;   // one cluster: the grid
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
@@ -581,7 +610,8 @@ __global__ void __launch_bounds__(DEM_CLUSTER_THREADS) k_dem_cluster(Dev s, int 
     cluster_barrier();
     for (int k = 0; k < s.dem_substeps; ++k) {
         for (int p = tid / DEM_LANES; p < s.np; p += nt / DEM_LANES)
-            dem_substep(s, p, l, gm, k & 1, have_prev != 0, dts, k == 0, k == s.dem_substeps - 1);
+            dem_substep(s, sh + threadIdx.x / DEM_LANES * DEM_SH, p, l, gm, k & 1, have_prev != 0, dts, k == 0,
+                        k == s.dem_substeps - 1);
         cluster_barrier();
     }
     // exclusive scan of the grid counts: each CTA scans a contiguous run of
@@ -1035,6 +1065,8 @@ __global__ void __launch_bounds__(128) k_transitions(Dev s) {
                     gas = tn == T_GAS;
                 }
             }
+            // (the sum's tree runs over the 26 neighbours without the cell itself)
+            rs = __shfl_sync(full, rs, lane < 13 ? lane : (lane < 26 ? lane + 1 : 31));
             for (int o = 16; o > 0; o >>= 1) {
                 rs += __shfl_xor_sync(full, rs, o);
                 cnt += __shfl_xor_sync(full, cnt, o);

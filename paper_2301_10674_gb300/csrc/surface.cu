@@ -311,7 +311,7 @@ __global__ void __launch_bounds__(LIST_THREADS) k_mark(Dev s) {
             const int dx = lane % 3 - 1, dy = (lane / 3) % 3 - 1, dz = lane / 9 - 1;
             const int k = (dx != 0) + (dy != 0) + (dz != 0);
             v *= lane < 27 ? (k == 1 ? 4.f : (k == 2 ? 2.f : 1.f)) : 0.f;
-            const float gx = warp_sum_f(dx * v), gy = warp_sum_f(dy * v), gz = warp_sum_f(dz * v);
+            const float gx = ordered_sum27(dx * v), gy = ordered_sum27(dy * v), gz = ordered_sum27(dz * v);
             if (lane == 0) s.nrm1[c] = py_result(gx, gy, gz);
         }
     }
@@ -356,21 +356,21 @@ __device__ __forceinline__ void init_new(const Dev& s, int c, int lane) {
                 n = 1.f;
             }
         }
-        n = warp_sum_f(n);
-        rs = warp_sum_f(rs);
+        n = (float)__popc(__ballot_sync(0xffffffffu, n > 0.f));
+        rs = ordered_sum27(rs);
         const float inv = n > 0.f ? 1.f / n : 0.f;
         rho = n > 0.f ? rs * inv : s.rho_gas;
-        ux = warp_sum_f(us) * inv;
-        uy = warp_sum_f(vs) * inv;
-        uz = warp_sum_f(ws) * inv;
+        ux = ordered_sum27(us) * inv;
+        uy = ordered_sum27(vs) * inv;
+        uz = ordered_sum27(ws) * inv;
         v = feq_dev(lane < 27 ? lane : 0, rho, ux, uy, uz);
         if (lane < 27) Store<S>::st(f + slot, with_ref<S>(v, lane, -h));
         m = 0.f;
     } else {
         v = lane < 27 ? with_ref<S>(Store<S>::ld(f + slot), lane, h) : 0.f;
-        const float d = warp_sum_f(v);
-        const float jx = warp_sum_f((lane % 3 - 1) * v), jy = warp_sum_f(((lane / 3) % 3 - 1) * v),
-                    jz = warp_sum_f((lane / 9 - 1) * v);
+        const float d = ordered_sum27(v);
+        const float jx = ordered_sum27((lane % 3 - 1) * v), jy = ordered_sum27(((lane / 3) % 3 - 1) * v),
+                    jz = ordered_sum27((lane / 9 - 1) * v);
         rho = 1.f + d;
         const float inv = 1.f / rho;
         ux = (jx - 0.5f * rho * s.gx) * inv;
@@ -401,7 +401,7 @@ __device__ __forceinline__ void excess_prep(const Dev& s, int c, int lane) {
     const float sg = cv == CV_TO_LIQ ? 1.f : -1.f;
     const float w = sg * (n1.x * (lane % 3 - 1) + n1.y * ((lane / 3) % 3 - 1) + n1.z * (lane / 9 - 1));
     const int nrec = __popc(__ballot_sync(0xffffffffu, rec));
-    const float wsum = warp_sum_f(rec && w > 0.f ? w : 0.f);
+    const float wsum = ordered_sum27(rec && w > 0.f ? w : 0.f);
     if (lane != 0) return;
     const float ex = cv == CV_TO_LIQ ? m - rho : m;
     s.mass[c] = cv == CV_TO_LIQ ? rho : 0.f;
