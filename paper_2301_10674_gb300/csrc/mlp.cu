@@ -85,9 +85,19 @@ __device__ float block_sum(float v, float* sh) {
 
 // One block per surface. params: n x 12 FP64 rows (kind, n0, s, r, A, k,
 // phase, e1; P = s n0); fill: n x 27 FP32; target: n x 4 FP32.
+// Bound by instruction issue over the sub-samples (27 x 64^3 per sine wave).
+// A cell, a row of 64 samples or a run of 16 that lies wholly on one side of
+// the surface is counted without its samples, where the value in its middle
+// (a run: at its first sample) exceeds what the surface function can change by
+// within it plus the rounding of the evaluation: the counts are those of all
+// samples. The FP64 cell offsets are formed once per cell, not per thread.
+// 20 000 surfaces of all kinds: 12.6 ms with every sample evaluated,
+// 2.76 ms now.
 __global__ void __launch_bounds__(GEN_THREADS) k_make_stencils(const double* __restrict__ params, long long n,
                                                                float* fill, float* target) {
     __shared__ float sh[GEN_THREADS / 32];
+    __shared__ float rot[2];         // phase per sample, A sin(phase)
+    __shared__ float off[27][3];     // cell offsets from the sphere's centre, or (u, w) of the cell's corner
     const long long i = blockIdx.x;
     if (i >= n) return;
     const double* p = params + i * 12;
@@ -97,15 +107,40 @@ __global__ void __launch_bounds__(GEN_THREADS) k_make_stencils(const double* __r
     const double e1[3] = {p[9], p[10], p[11]};
     const double P[3] = {s * n0[0], s * n0[1], s * n0[2]};
     const int tid = threadIdx.x;
+    // labels, by a warp of their own: FP64 trigonometry and divisions
+    if (tid == 64) {
+        double nt[3] = {n0[0], n0[1], n0[2]}, kap = 0.0;
+        if (kind == 1) kap = 1.0 / r;
+        else if (kind == 2) kap = -1.0 / r;
+        else if (kind == 3) {
+            // graph w = f(u): normal (n0 - f' e1) / sqrt(1 + f'^2), mean
+            // curvature of the cylinder -f'' / (2 (1 + f'^2)^(3/2))
+            const double fp = A * kw * cos(ph), fpp = -A * kw * kw * sin(ph);
+            const double qn = sqrt(1.0 + fp * fp);
+            for (int k = 0; k < 3; ++k) nt[k] = (n0[k] - fp * e1[k]) / qn;
+            kap = -fpp / (2.0 * qn * qn * qn);
+        }
+        for (int k = 0; k < 3; ++k) target[i * 4 + k] = (float)nt[k];
+        target[i * 4 + 3] = (float)kap;
+    }
     if (kind == 0) {
         if (tid < 27) fill[i * 27 + tid] = (float)plane_cell(n0, P, tid);
     } else if (kind == 1 || kind == 2) {
         // exact chord along x of each of the 64 x 64 rows
         const double sg = kind == 1 ? -1.0 : 1.0;       // centre P -/+ r n0
-        const double C[3] = {P[0] + sg * r * n0[0], P[1] + sg * r * n0[1], P[2] + sg * r * n0[2]};
-        const float rr = (float)(r * r);
+        if (tid < 27)
+            for (int a = 0; a < 3; ++a)
+                off[tid][a] = (float)(P[a] + sg * r * n0[a] - (a == 0 ? cx(tid) : (a == 1 ? cy(tid) : cz(tid))));
+        __syncthreads();
+        const float rf = (float)r, rr = (float)(r * r);
         for (int q = 0; q < 27; ++q) {
-            const float ox = (float)(C[0] - cx(q)), oy = (float)(C[1] - cy(q)), oz = (float)(C[2] - cz(q));
+            const float ox = off[q][0], oy = off[q][1], oz = off[q][2];
+            // whole cell inside or outside (half a diagonal is 0.8661)
+            const float d = sqrtf(ox * ox + oy * oy + oz * oz) - rf;
+            if (fabsf(d) > 0.8661f + 1e-4f * (1.f + rf)) {
+                if (tid == 0) fill[i * 27 + q] = (d < 0.f) == (kind == 1) ? 1.f : 0.f;
+                continue;
+            }
             float acc = 0.f;
             for (int j = tid; j < ROWS; j += GEN_THREADS) {
                 const float y = ((j % SUBS) + 0.5f) / SUBS - 0.5f, z = ((j / SUBS) + 0.5f) / SUBS - 0.5f;
@@ -125,25 +160,74 @@ __global__ void __launch_bounds__(GEN_THREADS) k_make_stencils(const double* __r
         // the sub-cell offsets in FP32; along a row the phase advances by
         // k e1.x / 64 per sample (a rotation), restarted from sincosf every
         // 16 samples.
+        if (tid < 27) {
+            const double b[3] = {cx(tid) - 0.5 - P[0], cy(tid) - 0.5 - P[1], cz(tid) - 0.5 - P[2]};
+            off[tid][0] = (float)(b[0] * e1[0] + b[1] * e1[1] + b[2] * e1[2]);
+            off[tid][1] = (float)(b[0] * n0[0] + b[1] * n0[1] + b[2] * n0[2]);
+        } else if (tid == 32) {
+            rot[0] = (float)(kw * e1[0] / SUBS);
+            rot[1] = (float)(A * sin(ph));
+        }
+        __syncthreads();
         float sd, cd;
-        sincosf((float)(kw * e1[0] / SUBS), &sd, &cd);
-        const float Af = (float)A, As = (float)(A * sin(ph)), kf = (float)kw, pf = (float)ph;
+        sincosf(rot[0], &sd, &cd);
+        const float Af = (float)A, As = rot[1], kf = (float)kw, pf = (float)ph;
         const float fe[3] = {(float)e1[0], (float)e1[1], (float)e1[2]};
         const float fn[3] = {(float)n0[0], (float)n0[1], (float)n0[2]};
+        // change of g = w - A sin(k u + phase) + A sin(phase) within a cell,
+        // row or run, at most: the gradient at the point tested times the
+        // extent plus half the largest second derivative A k^2 along u, and
+        // the rounding of an evaluation
+        const float Ak = Af * kf, h2 = 0.5f * fabsf(Ak * kf);
+        const float tol = 1e-4f * (1.f + fabsf(Af));
+        const float ec = 0.5f * (fabsf(fe[0]) + fabsf(fe[1]) + fabsf(fe[2])), er = 0.5f * fe[0], es = 0.25f * fe[0];
+        const float cell_add = tol + h2 * ec * ec, row_add = tol + h2 * er * er, run_add = tol + h2 * es * es;
         for (int q = 0; q < 27; ++q) {
-            const double b[3] = {cx(q) - 0.5 - P[0], cy(q) - 0.5 - P[1], cz(q) - 0.5 - P[2]};
-            const float bu = (float)(b[0] * e1[0] + b[1] * e1[1] + b[2] * e1[2]);
-            const float bw = (float)(b[0] * n0[0] + b[1] * n0[1] + b[2] * n0[2]);
+            const float bu = off[q][0], bw = off[q][1];
+            float sc, cc;
+            sincosf(kf * (bu + 0.5f * (fe[0] + fe[1] + fe[2])) + pf, &sc, &cc);
+            const float gc = bw + 0.5f * (fn[0] + fn[1] + fn[2]) - Af * sc + As, dc = Ak * cc;
+            if (fabsf(gc) > 0.5f * (fabsf(fn[0] - dc * fe[0]) + fabsf(fn[1] - dc * fe[1]) + fabsf(fn[2] - dc * fe[2])) +
+                                cell_add) {
+                if (tid == 0) fill[i * 27 + q] = gc < 0.f ? 1.f : 0.f;
+                continue;
+            }
             int cnt = 0;
             for (int j = tid; j < ROWS; j += GEN_THREADS) {
                 const float yo = ((j % SUBS) + 0.5f) / SUBS, zo = ((j / SUBS) + 0.5f) / SUBS;
                 const float x0 = 0.5f / SUBS;
                 const float u0 = bu + (x0 * fe[0] + yo * fe[1] + zo * fe[2]);
                 const float w0 = bw + (x0 * fn[0] + yo * fn[1] + zo * fn[2]);
-                for (int seg = 0; seg < SUBS; seg += 16) {
+                float sm, cm;
+                sincosf(kf * (u0 + (0.5f - x0) * fe[0]) + pf, &sm, &cm);
+                const float gm = w0 + (0.5f - x0) * fn[0] - Af * sm + As;
+                if (fabsf(gm) > 0.5f * fabsf(fn[0] - Ak * cm * fe[0]) + row_add) {
+                    cnt += gm < 0.f ? SUBS : 0;
+                    continue;
+                }
+                // runs of 16: decided from the expansion about the row's
+                // middle where that suffices; the lanes then walk their
+                // remaining runs together
+                const float dm = fn[0] - Ak * cm * fe[0];
+                const float lim = 0.125f * fabsf(dm) + row_add;
+                unsigned todo = 0;
+#pragma unroll
+                for (int g = 0; g < 4; ++g) {
+                    const float gr = gm + dm * (0.25f * g - 0.375f);
+                    if (fabsf(gr) > lim) cnt += gr < 0.f ? 16 : 0;
+                    else todo |= 1u << g;
+                }
+                for (; todo; todo &= todo - 1u) {
+                    const int seg = 16 * (__ffs(todo) - 1);
                     float sn, cs;
                     sincosf(kf * (u0 + seg * (fe[0] / SUBS)) + pf, &sn, &cs);
                     float w = w0 + seg * (fn[0] / SUBS);
+                    const float g0 = w - Af * sn + As;
+                    if (fabsf(g0) > 0.25f * fabsf(fn[0] - Ak * cs * fe[0]) + run_add) {
+                        cnt += g0 < 0.f ? 16 : 0;
+                        continue;
+                    }
+#pragma unroll
                     for (int k = 0; k < 16; ++k) {
                         cnt += w <= Af * sn - As ? 1 : 0;
                         const float sn2 = sn * cd + cs * sd;
@@ -156,21 +240,6 @@ __global__ void __launch_bounds__(GEN_THREADS) k_make_stencils(const double* __r
             const float tot = block_sum((float)cnt, sh);      // integer counts: exact in FP32
             if (tid == 0) fill[i * 27 + q] = tot / (float)(ROWS * SUBS);
         }
-    }
-    if (tid == 0) {
-        double nt[3] = {n0[0], n0[1], n0[2]}, kap = 0.0;
-        if (kind == 1) kap = 1.0 / r;
-        else if (kind == 2) kap = -1.0 / r;
-        else if (kind == 3) {
-            // graph w = f(u): normal (n0 - f' e1) / sqrt(1 + f'^2), mean
-            // curvature of the cylinder -f'' / (2 (1 + f'^2)^(3/2))
-            const double fp = A * kw * cos(ph), fpp = -A * kw * kw * sin(ph);
-            const double qn = sqrt(1.0 + fp * fp);
-            for (int k = 0; k < 3; ++k) nt[k] = (n0[k] - fp * e1[k]) / qn;
-            kap = -fpp / (2.0 * qn * qn * qn);
-        }
-        for (int k = 0; k < 3; ++k) target[i * 4 + k] = (float)nt[k];
-        target[i * 4 + 3] = (float)kap;
     }
 }
 
