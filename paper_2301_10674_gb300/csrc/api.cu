@@ -339,6 +339,7 @@ int fslbm_create(const fslbm_params* p, void* cuda_stream, fslbm** out) {
         d.fbits = dalloc<unsigned>(s, n / 32 + 1, ok);
         d.ibits = dalloc<unsigned>(s, n / 32 + 1, ok);
         d.sbits = dalloc<unsigned>(s, n / 32 + 1, ok);
+        d.tw = p->storage != FSLBM_STORE_FP32 && d.idx32 && p->nx % 32 == 0 ? dalloc<unsigned>(s, n / 8 + 1, ok) : nullptr;
         d.tiles = dalloc<int>(s, n / fsl::SP_TILE + 1, ok);
         {
             const long long nseg = (long long)d.nsegx * p->ny * p->nz;

@@ -108,6 +108,10 @@ struct Dev {
     uint8_t* segflag;                           // [nz][ny][nsegx]
     int* bseg; int* bseg_count;
     unsigned* fbits; unsigned* ibits; unsigned* sbits;   // per 32 cells of a row: fluid / interface / solid bits
+    // 2-bit types of the 16 cells 8k - 4 .. 8k + 11 of a row, per word k of the
+    // row, up to the cells above the particles' (null where the link pass
+    // reads the flag bytes: FP32, nx no multiple of 32, 64-bit indices)
+    unsigned* tw;
     int* tl_info;                               // per transition: new owner / new type
     double* pool;
     double* pool_share;

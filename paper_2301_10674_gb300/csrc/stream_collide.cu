@@ -666,6 +666,26 @@ __device__ __forceinline__ PData particle_data(const Dev& s, int p) {
     return d;
 }
 
+// R-12a: the net injection leaves the pool (one FP64 atomic per block; every
+// thread of the block calls it)
+__device__ __forceinline__ void link_injection(const Dev& s, float injected) {
+    if (!s.link_corr) return;
+    __shared__ float red[8];
+    for (int off = 16; off > 0; off >>= 1) injected += __shfl_xor_sync(0xffffffffu, injected, off);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = injected;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        float t = 0.f;
+        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += red[w];
+        if (t != 0.f) atomicAdd(s.pool, -(double)t);
+    }
+}
+
+// block size and resident blocks per SM of the link pass over type words (96
+// registers); large flume, FP16, sweep: 128 x 5 3.06 ms, 128 x 4 3.17, 128 x 6 3.13
+// (spills), 256 x 2 3.17, 64 x 10 3.06
+constexpr int LINK_THREADS = 128, LINK_BLOCKS = 5;
+
 // Moving bounce-back and momentum exchange (Section 2.2), from the solid
 // side: for every surface solid cell s (owner p) and every fluid neighbour
 // x = s + c_q, the PDF x will pull from s in direction q is
@@ -792,18 +812,158 @@ __global__ void __launch_bounds__(256, 3) k_solid_links(Dev s) {
         }
         flush_mem(s, key, F, T);
     }
-    // R-12a: the net injection leaves the pool (one FP64 atomic per block)
-    if (s.link_corr) {
-        __shared__ float red[8];
-        for (int off = 16; off > 0; off >>= 1) injected += __shfl_xor_sync(0xffffffffu, injected, off);
-        if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = injected;
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            float t = 0.f;
-            for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += red[w];
-            if (t != 0.f) atomicAdd(s.pool, -(double)t);
+    link_injection(s, injected);
+}
+
+// The same links with the neighbours' types from the overlapping type words
+// (s.tw): nine 4-byte loads instead of 26 bytes, one word per row of the 3x3x3
+// block, and loaded one list entry ahead together with the owner, so that an
+// entry waits for one memory latency (its PDFs and its particle's data) where
+// the kernel above waits for three in turn. For 16-bit storage (rows of 32
+// cells, 32-bit indices), where the pass is bound by latency: the sweep of the
+// 3072x96x320 flume at FP16 went from 3.39 to 3.06 ms, of 1024x64x128 from 0.349
+// to 0.315 ms. At FP32 the pass moves its 9 GB at the HBM rate either way
+// (sweep 4.00 ms with the kernel above, 4.02 to 4.08 ms with this one), so it
+// stays with the flag bytes and saves the words.
+// bit of direction q in the per-plane masks: 2 (c_x + 1) + 6 (c_y + 1) of plane c_z + 1
+__device__ __forceinline__ bool fluid_bit(const unsigned (&m)[3], int q) {
+    return (m[cz(q) + 1] >> (2 * (cx(q) + 1) + 6 * (cy(q) + 1))) & 1u;
+}
+
+template <typename S, int PAR>
+__global__ void __launch_bounds__(LINK_THREADS, LINK_BLOCKS) k_solid_links_words(Dev s) {
+    const int count = min(*s.sl_count, s.sl_cap);
+    const int stride = gridDim.x * blockDim.x;
+    const unsigned un = (unsigned)s.n;
+    const int nxw = s.nx >> 3;
+    S* f = static_cast<S*>(s.f);
+    float injected = 0.f;   // mass the moving bounce-back adds to liquid cells
+    // types of the block around a cell, as 18 bits per plane
+    auto types = [&](int x, int y, int z, unsigned (&w)[9]) {
+        const int k = x >> 3;
+#pragma unroll
+        for (int r = 0; r < 9; ++r) {
+            const int yy = shift(y, r % 3 - 1, s.ny, s.per_y), zz = shift(z, r / 3 - 1, s.nz, s.per_z);
+            w[r] = (yy | zz) >= 0 ? s.tw[(unsigned)(zz * s.ny + yy) * (unsigned)nxw + (unsigned)k] : 0u;
         }
+    };
+    int i = blockIdx.x * blockDim.x + threadIdx.x;
+    int cell = i < count ? s.sl[i] : 0;
+    int ahead = i + stride < count ? s.sl[i + stride] : 0;
+    int x, y, z;
+    coords32(s, cell, x, y, z);
+    unsigned w[9];
+    types(x, y, z, w);
+    int p = s.owner[cell];
+    for (int base = blockIdx.x * blockDim.x; base < count; base += stride) {
+        i = base + threadIdx.x;
+        unsigned fm[3], lm[3];
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+            const int sh = 2 * ((x & 7) + 3);
+            const unsigned t = ((w[3 * d] >> sh) & 0x3fu) | (((w[3 * d + 1] >> sh) & 0x3fu) << 6) |
+                               (((w[3 * d + 2] >> sh) & 0x3fu) << 12);
+            fm[d] = i < count ? (t ^ (t >> 1)) & 0x15555u : 0u;   // liquid or interface
+            lm[d] = t & ~(t >> 1) & 0x15555u;
+        }
+        int key = -1;
+        if (i < count) {
+            if (p < 0 || p >= s.np) {
+                if (fm[0] | fm[1] | fm[2]) set_error(s, ERR_INVARIANT);
+                fm[0] = fm[1] = fm[2] = 0u;
+            } else {
+                key = p;
+            }
+        }
+        const NbrOffsets o = nbr_offsets(s, x, y, z);
+        // the post-collision PDFs the fluid neighbours send here
+        float fo[27];
+#pragma unroll
+        for (int q = 0; q < 27; ++q) {
+            if (q == 13) continue;
+            const unsigned xn = (unsigned)(cell + o.ox[1 + cx(q)] + o.oy[1 + cy(q)] + o.oz[1 + cz(q)]);
+            const unsigned a = PAR == 0 ? (unsigned)opp(q) * un + (unsigned)cell : (unsigned)q * un + xn;
+            fo[q] = fluid_bit(fm, q) ? Store<S>::ld(f + a) : 0.f;
+        }
+        const PData P = particle_data(s, key < 0 ? 0 : key);
+        // the next entry's types and owner
+        const int ncell = ahead;
+        ahead = i + 2 * stride < count ? s.sl[i + 2 * stride] : 0;
+        int nx_, ny_, nz_;
+        coords32(s, ncell, nx_, ny_, nz_);
+        unsigned nw[9];
+        types(nx_, ny_, nz_, nw);
+        const int np_ = s.owner[ncell];
+        float F[3] = {0.f, 0.f, 0.f}, T[3] = {0.f, 0.f, 0.f};
+        // bounce-back values and momentum exchange, as above
+        if (fm[0] | fm[1] | fm[2]) {
+            const float ddx = (float)wrap_int(x - P.xi.x, s.nx, s.per_x) + 0.5f - P.xf.x;
+            const float ddy = (float)wrap_int(y - P.xi.y, s.ny, s.per_y) + 0.5f - P.xf.y;
+            const float ddz = (float)wrap_int(z - P.xi.z, s.nz, s.per_z) + 0.5f - P.xf.z;
+            const float usx = P.u.x + (P.w.y * ddz - P.w.z * ddy);
+            const float usy = P.u.y + (P.w.z * ddx - P.w.x * ddz);
+            const float usz = P.u.z + (P.w.x * ddy - P.w.y * ddx);
+            // 16-bit storage: references of the solid cell's z and of the
+            // neighbour's (an even step reads at the solid cell and writes
+            // at the neighbour, an odd step the other way round)
+            const float hz = Store<S>::HREF ? s.href[z] : 0.f;
+            const int zm = wrap_z(s, z - 1), zp = wrap_z(s, z + 1);
+            const float hm = Store<S>::HREF ? s.href[zm] : 0.f, hp = Store<S>::HREF ? s.href[zp] : 0.f;
+            float Ax = 0.f, Ay = 0.f, Az = 0.f, B = 0.f, Cx = 0.f, Cy = 0.f, Cz = 0.f, D = 0.f;
+            float Mxx = 0.f, Myy = 0.f, Mzz = 0.f, Mxy = 0.f, Mxz = 0.f, Myz = 0.f;
+#pragma unroll
+            for (int q = 0; q < 27; ++q) {
+                if (!fluid_bit(fm, q)) continue;
+                const float hn = cz(q) == 0 ? hz : (cz(q) < 0 ? hm : hp);
+                if (Store<S>::HREF) fo[q] += wq(q) * (PAR == 0 ? hz : hn);
+                const unsigned xn = (unsigned)(cell + o.ox[1 + cx(q)] + o.oy[1 + cy(q)] + o.oz[1 + cz(q)]);
+                // c_q.u_s with the signs of c_q
+                float cu = 0.f;
+                if (cx(q)) cu = cx(q) > 0 ? cu + usx : cu - usx;
+                if (cy(q)) cu = cy(q) > 0 ? cu + usy : cu - usy;
+                if (cz(q)) cu = cz(q) > 0 ? cu + usz : cu - usz;
+                const float corr = (6.f * wq(q)) * cu;
+                const float val = fo[q] + corr;
+                if (fluid_bit(lm, q)) injected += corr;
+                const unsigned dst = PAR == 0 ? (unsigned)q * un + xn : (unsigned)opp(q) * un + (unsigned)cell;
+                Store<S>::st(f + dst, Store<S>::HREF ? val - wq(q) * (PAR == 0 ? hn : hz) : val);
+                const float t = fmaf(2.f, fo[q], corr);
+                if (cx(q)) { Ax = cx(q) > 0 ? Ax + t : Ax - t; Cx = cx(q) > 0 ? Cx + corr : Cx - corr; Mxx += corr; }
+                if (cy(q)) { Ay = cy(q) > 0 ? Ay + t : Ay - t; Cy = cy(q) > 0 ? Cy + corr : Cy - corr; Myy += corr; }
+                if (cz(q)) { Az = cz(q) > 0 ? Az + t : Az - t; Cz = cz(q) > 0 ? Cz + corr : Cz - corr; Mzz += corr; }
+                if (cx(q) && cy(q)) Mxy = cx(q) * cy(q) > 0 ? Mxy + corr : Mxy - corr;
+                if (cx(q) && cz(q)) Mxz = cx(q) * cz(q) > 0 ? Mxz + corr : Mxz - corr;
+                if (cy(q) && cz(q)) Myz = cy(q) * cz(q) > 0 ? Myz + corr : Myz - corr;
+                B += corr;
+                D += (float)nnz(q) * corr;
+            }
+            const float hx = 0.5f * (P.w.y * Cz - P.w.z * Cy);
+            const float hy = 0.5f * (P.w.z * Cx - P.w.x * Cz);
+            const float hzz = 0.5f * (P.w.x * Cy - P.w.y * Cx);
+            F[0] = fmaf(usx, B, hx) - Ax;
+            F[1] = fmaf(usy, B, hy) - Ay;
+            F[2] = fmaf(usz, B, hzz) - Az;
+            // M W
+            const float mwx = Mxx * P.w.x + Mxy * P.w.y + Mxz * P.w.z;
+            const float mwy = Mxy * P.w.x + Myy * P.w.y + Myz * P.w.z;
+            const float mwz = Mxz * P.w.x + Myz * P.w.y + Mzz * P.w.z;
+            const float gx = (Cy * usz - Cz * usy) + 0.5f * (P.w.x * D - mwx);
+            const float gy = (Cz * usx - Cx * usz) + 0.5f * (P.w.y * D - mwy);
+            const float gz = (Cx * usy - Cy * usx) + 0.5f * (P.w.z * D - mwz);
+            T[0] = (ddy * F[2] - ddz * F[1]) + 0.5f * gx;
+            T[1] = (ddz * F[0] - ddx * F[2]) + 0.5f * gy;
+            T[2] = (ddx * F[1] - ddy * F[0]) + 0.5f * gz;
+        }
+        flush_mem(s, key, F, T);
+        cell = ncell;
+        x = nx_;
+        y = ny_;
+        z = nz_;
+        p = np_;
+#pragma unroll
+        for (int r = 0; r < 9; ++r) w[r] = nw[r];
     }
+    link_injection(s, injected);
 }
 
 // ---------------------------------------------------------------- bed segments
@@ -1317,6 +1477,18 @@ static int staged_pair_blocks() {
     return blocks;
 }
 
+template <typename S, int PAR>
+static int link_word_blocks() {
+    static int blocks = 0;
+    if (blocks == 0) {
+        int per_sm = 0, dev = 0, sms = 0;
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_solid_links_words<S, PAR>, LINK_THREADS, 0);
+        cudaGetDevice(&dev);
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        blocks = (per_sm > 0 ? per_sm : 1) * (sms > 0 ? sms : 1);
+    }
+    return blocks;
+}
 // blocks of the link pass: one resident wave (the kernel strides over the
 // list), found once per storage format and parity
 template <typename S, int PAR>
@@ -1330,6 +1502,17 @@ static int link_blocks() {
         blocks = (per_sm > 0 ? per_sm : 1) * (sms > 0 ? sms : 1);
     }
     return blocks;
+}
+
+template <typename S, int PAR>
+static void launch_links(const Dev& s, cudaStream_t st) {
+    if constexpr (sizeof(S) == 2) {
+        if (s.tw) {
+            k_solid_links_words<S, PAR><<<link_word_blocks<S, PAR>(), LINK_THREADS, 0, st>>>(s);
+            return;
+        }
+    }
+    k_solid_links<S, PAR><<<link_blocks<S, PAR>(), 256, 0, st>>>(s);
 }
 
 // blocks of the bed kernel: one resident wave (the kernel strides over the
@@ -1356,7 +1539,9 @@ static void launch_typed(const Dev& s, int parity, cudaStream_t st, cudaEvent_t 
     // liquid kernels: threads along x, blocks over the rows (y, z)
     const dim3 lgrid((unsigned)((s.nx + 255) / 256), (unsigned)(s.ny * s.nz < 65535 ? s.ny * s.nz : 65535));
     if (parity == 0) {
-        if (s.np > 0 && !s.links_fused) k_solid_links<S, 0><<<link_blocks<S, 0>(), 256, 0, st>>>(s);
+        if (s.np > 0 && !s.links_fused) {
+            launch_links<S, 0>(s, st);
+        }
         if (early && links_done) cudaEventRecord(links_done, st);
         if (use_staged_pairs(s)) {
             if constexpr (sizeof(S) == 2) {
@@ -1371,7 +1556,9 @@ static void launch_typed(const Dev& s, int parity, cudaStream_t st, cudaEvent_t 
         if (s.np > 0 && s.links_fused) k_liquid_pair_bed<S, 0><<<bed_blocks<S, 0>(), 128, 0, st>>>(s);
         k_interface<S, 0><<<lb, 128, 0, st>>>(s);
     } else {
-        if (s.np > 0 && !s.links_fused) k_solid_links<S, 1><<<link_blocks<S, 1>(), 256, 0, st>>>(s);
+        if (s.np > 0 && !s.links_fused) {
+            launch_links<S, 1>(s, st);
+        }
         if (early && links_done) cudaEventRecord(links_done, st);
         if (use_split(s)) {
             k_liquid_pair<S, 1, 1><<<lgrid, 128, 0, st>>>(s);

@@ -744,6 +744,27 @@ __global__ void k_type_bits(Dev s) {
     s.fbits[w] = fm;
     s.ibits[w] = im;
     s.sbits[w] = sm;
+    if (!s.tw || s.np == 0) return;
+    // overlapping words of 2-bit types for the link pass, up to the cells
+    // above the particles'
+    const unsigned nxw = (unsigned)s.nx >> 5, row = (unsigned)w / nxw, xw = (unsigned)w - row * nxw;
+    if (!s.per_z && (int)(row / (unsigned)s.ny) > *s.zmax_cell + 1) return;
+    // four type bytes to one byte: bits 0, 8, 16, 24 to 24, 26, 28, 30
+    auto pack = [](unsigned v) { return ((v & 0x03030303u) * 0x01041040u) >> 24; };
+    unsigned lo = 0, hi = 0;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        lo |= pack(words[k]) << (8 * k);
+        hi |= pack(words[4 + k]) << (8 * k);
+    }
+    // the four cells before and behind (across the seam, or gas beyond a wall)
+    const uint8_t* rf = s.flags + (long long)row * s.nx;
+    const int xl = xw > 0 ? (int)(32 * xw) - 4 : (s.per_x ? s.nx - 4 : -1);
+    const int xr = xw + 1 < nxw ? (int)(32 * xw) + 32 : (s.per_x ? 0 : -1);
+    const unsigned L = xl >= 0 ? pack(*reinterpret_cast<const unsigned*>(rf + xl)) : 0u;
+    const unsigned R = xr >= 0 ? pack(*reinterpret_cast<const unsigned*>(rf + xr)) : 0u;
+    const uint4 out = make_uint4(L | (lo << 8), (lo >> 8) | (hi << 24), (lo >> 24) | (hi << 8), (hi >> 8) | (R << 24));
+    *reinterpret_cast<uint4*>(s.tw + 4 * w) = out;
 }
 
 // The block of the classification that finishes last clamps the list counts
