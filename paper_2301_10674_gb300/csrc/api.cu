@@ -334,8 +334,10 @@ int fslbm_create(const fslbm_params* p, void* cuda_stream, fslbm** out) {
         if (tcap > n) tcap = n;
         d.tl_cap = (int)tcap;
         d.tl = dalloc<int>(s, tcap, ok);
-        d.sl_cap = (int)n;
-        d.sl = dalloc<int>(s, n, ok);
+        // (with the fill-up to groups of 32 per 4096 cells)
+        const long long scap = std::min(n + 32 * (n / 4096 + 1), (1LL << 31) - 1);
+        d.sl_cap = (int)scap;
+        d.sl = dalloc<int>(s, scap, ok);
         d.fbits = dalloc<unsigned>(s, n / 32 + 1, ok);
         d.ibits = dalloc<unsigned>(s, n / 32 + 1, ok);
         d.sbits = dalloc<unsigned>(s, n / 32 + 1, ok);

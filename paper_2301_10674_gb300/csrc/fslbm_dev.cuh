@@ -98,7 +98,7 @@ struct Dev {
     int* nl; int* nl_count; int nl_cap;        // cells becoming interface this step
     int* cl; int* cl_count;                    // interface cells converting this step (capacity wl_cap)
     int* tl; int* tl_count; int tl_cap;        // particle map transitions
-    int* sl; int* sl_count; int sl_cap;        // solid cells with a fluid neighbour
+    int* sl; int* sl_count; int sl_cap;        // solid cells with a fluid neighbour (-1: none)
     int* tiles; int* tile_count;               // SP_TILE-cell x-tiles holding a liquid cell
     // particle links taken from the fluid side: the bed segments (BED_SEG-cell
     // x-ranges of a row holding a liquid cell with a solid neighbour) are

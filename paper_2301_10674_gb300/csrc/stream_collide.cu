@@ -295,11 +295,7 @@ __device__ __forceinline__ void pair_update(const Dev& s, S* f, int x, int row, 
     pair_finish<S, PAR>(s, f, x, row, liq, interior, v, ref, wt);
 }
 
-// PART 1 keeps to the interior pairs of an odd step (all 26 neighbours of
-// both cells inside the lattice, no wrap), so that the kernel of the bulk
-// carries no boundary code; k_liquid_pair_edges takes the others. PART 0:
-// every pair (even steps).
-template <typename S, int PAR, int PART>
+template <typename S, int PAR>
 __global__ void __launch_bounds__(128, liquid_pair_min_blocks<S, PAR>()) k_liquid_pair(Dev s) {
     __shared__ int ps[128];      // (x << 2 | liquid bits) of the compacted pairs
     __shared__ int wn[4];
@@ -315,11 +311,8 @@ __global__ void __launch_bounds__(128, liquid_pair_min_blocks<S, PAR>()) k_liqui
         const int x0 = blockIdx.x * 256 + 2 * (int)threadIdx.x;
         unsigned lm = 0;
         if (x0 < s.nx) {
-            const bool inner_pair = !face_row && x0 > 0 && x0 + 1 < s.nx - 1;
-            if (PART == 0 || inner_pair) {
-                const uchar2 fl = *reinterpret_cast<const uchar2*>(s.flags + x0 + (long long)s.nx * row);
-                lm = ((fl.x & TYPE_MASK) == T_LIQ ? 1u : 0u) | ((fl.y & TYPE_MASK) == T_LIQ ? 2u : 0u);
-            }
+            const uchar2 fl = *reinterpret_cast<const uchar2*>(s.flags + x0 + (long long)s.nx * row);
+            lm = ((fl.x & TYPE_MASK) == T_LIQ ? 1u : 0u) | ((fl.y & TYPE_MASK) == T_LIQ ? 2u : 0u);
         }
         const unsigned m = __ballot_sync(0xffffffffu, lm != 0);
         if (lane == 0) wn[warp] = __popc(m);
@@ -337,12 +330,61 @@ __global__ void __launch_bounds__(128, liquid_pair_min_blocks<S, PAR>()) k_liqui
         if (e < 0) continue;
         const int x = e >> 2;
         const bool interior =
-            PAR == 0 || PART == 1 || (x > 0 && x + 1 < s.nx - 1 && !face_row);
+            PAR == 0 || (x > 0 && x + 1 < s.nx - 1 && !face_row);
         pair_update<S, PAR>(s, f, x, row, (unsigned)e & 3u, interior);
     }
 }
 
-// The pairs of an odd step that k_liquid_pair<S, 1, 1> leaves out, one per
+// The same for 16-bit storage with a warp per 256-cell segment and no
+// block-wide barrier: the warp compacts the segment's liquid pairs into its
+// own list and takes them 32 at a time, so a warp waits for its own loads
+// only. Bound by issue and latency (the collision alone is about 430 packed
+// operations per pair). Sweep of the 3072x96x320 flume at FP16, even steps over
+// the staged kernel and odd steps over the block's compaction: 3.06 ms before,
+// 2.84 ms; 128 cells per warp 3.07 ms, 512 cells 2.85 ms; 4, 6, 7 resident blocks per
+// SM 2.90, 2.86, 2.84 ms. PART 1 keeps to the interior pairs of an odd step (all 26
+// neighbours of both cells inside the lattice, no wrap), so that the kernel of
+// the bulk carries no boundary code; k_liquid_pair_edges takes the others. PART
+// 0: every pair (even steps). At FP32, bound by HBM, the block's compaction (four
+// warps on adjacent cells) is 2% faster and stays.
+constexpr int SEG_CELLS = 256;
+template <typename S, int PAR, int PART>
+__global__ void __launch_bounds__(128, 7) k_liquid_pair_warps(Dev s) {
+    __shared__ int ps[4][SEG_CELLS / 2];      // (x << 2 | liquid bits) of each warp's compacted pairs
+    const int lane = threadIdx.x & 31;
+    int* mine = ps[threadIdx.x >> 5];
+    S* f = static_cast<S*>(s.f);
+    const int nsegrow = (s.nx + SEG_CELLS - 1) / SEG_CELLS;
+    const int seg = blockIdx.x * 4 + (threadIdx.x >> 5);
+    const int row = seg / nsegrow, xb = (seg - row * nsegrow) * SEG_CELLS;
+    if (row >= s.ny * s.nz) return;           // whole warps leave together
+    // the bed kernel takes the segments with particle links
+    if (s.links_fused && s.segflag[row * s.nsegx + xb / BED_SEG]) return;
+    const int yr = row % s.ny, zr = row / s.ny;
+    if (PART == 1 && (yr == 0 || yr == s.ny - 1 || zr == 0 || zr == s.nz - 1)) return;
+    const uint8_t* fl = s.flags + (long long)s.nx * row;
+    int tot = 0;
+#pragma unroll
+    for (int k = 0; k < SEG_CELLS / 64; ++k) {
+        const int x0 = xb + 64 * k + 2 * lane;
+        unsigned lm = 0;
+        if (x0 < s.nx && (PART == 0 || (x0 > 0 && x0 + 1 < s.nx - 1))) {
+            const uchar2 t = *reinterpret_cast<const uchar2*>(fl + x0);
+            lm = ((t.x & TYPE_MASK) == T_LIQ ? 1u : 0u) | ((t.y & TYPE_MASK) == T_LIQ ? 2u : 0u);
+        }
+        const unsigned m = __ballot_sync(0xffffffffu, lm != 0);
+        if (lm) mine[tot + __popc(m & ((1u << lane) - 1u))] = (x0 << 2) | (int)lm;
+        tot += __popc(m);
+    }
+    __syncwarp();
+#pragma unroll 1
+    for (int i = lane; i < tot; i += 32) {
+        const int e = mine[i];
+        pair_update<S, PAR>(s, f, e >> 2, row, (unsigned)e & 3u, true);   // no boundary in an even step or PART 1
+    }
+}
+
+// The pairs of an odd step that k_liquid_pair_warps<S, 1, 1> leaves out, one per
 // thread: every pair of the rows on the y and z faces, then the pairs at
 // x = 0 and x = nx - 2 of the other rows (ny, nz >= 3 and nx >= 4, so that
 // no pair is listed twice).
@@ -666,20 +708,31 @@ __device__ __forceinline__ PData particle_data(const Dev& s, int p) {
     return d;
 }
 
-// R-12a: the net injection leaves the pool (one FP64 atomic per block; every
-// thread of the block calls it)
-__device__ __forceinline__ void link_injection(const Dev& s, float injected) {
-    if (!s.link_corr) return;
-    __shared__ float red[8];
-    for (int off = 16; off > 0; off >>= 1) injected += __shfl_xor_sync(0xffffffffu, injected, off);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = injected;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        float t = 0.f;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += red[w];
-        if (t != 0.f) atomicAdd(s.pool, -(double)t);
+// R-12a: the net injection leaves the pool. A thread adds its entries'
+// injections with their rounding errors carried on, so that the sum does not
+// depend on which entries a thread takes beyond FP64 rounding; one FP64 atomic
+// per block (every thread of the block calls flush).
+struct Injection {
+    float hi = 0.f, lo = 0.f;
+    __device__ __forceinline__ void add(float v) {
+        const float t = __fadd_rn(hi, v), bb = __fsub_rn(t, hi);
+        lo += __fadd_rn(__fsub_rn(hi, __fsub_rn(t, bb)), __fsub_rn(v, bb));
+        hi = t;
     }
-}
+    __device__ __forceinline__ void flush(const Dev& s) {
+        if (!s.link_corr) return;
+        __shared__ double red[8];
+        double v = (double)hi + (double)lo;
+        for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+        if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            double t = 0.0;
+            for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += red[w];
+            if (t != 0.0) atomicAdd(s.pool, -t);
+        }
+    }
+};
 
 // block size and resident blocks per SM of the link pass over type words (96
 // registers); large flume, FP16, sweep: 128 x 5 3.06 ms, 128 x 4 3.17, 128 x 6 3.13
@@ -701,7 +754,7 @@ template <typename S, int PAR>
 __global__ void __launch_bounds__(256, 3) k_solid_links(Dev s) {
     const int count = min(*s.sl_count, s.sl_cap);
     const int stride = gridDim.x * blockDim.x;
-    float injected = 0.f;   // mass the moving bounce-back adds to liquid cells
+    Injection injection;    // mass the moving bounce-back adds to liquid cells
     // the list entry of the next pass is loaded one pass ahead
     int next = blockIdx.x * blockDim.x + threadIdx.x < count ? s.sl[blockIdx.x * blockDim.x + threadIdx.x] : 0;
     for (int base = blockIdx.x * blockDim.x; base < count; base += stride) {
@@ -709,8 +762,9 @@ __global__ void __launch_bounds__(256, 3) k_solid_links(Dev s) {
         const int cell = next;
         next = i + stride < count ? s.sl[i + stride] : 0;
         int key = -1;
+        float injected = 0.f;
         float F[3] = {0.f, 0.f, 0.f}, T[3] = {0.f, 0.f, 0.f};
-        if (i < count) {
+        if (i < count && cell >= 0) {
             int x, y, z;
             coords32(s, cell, x, y, z);
             const int p = s.owner[cell];
@@ -811,8 +865,9 @@ __global__ void __launch_bounds__(256, 3) k_solid_links(Dev s) {
             }
         }
         flush_mem(s, key, F, T);
+        injection.add(injected);
     }
-    link_injection(s, injected);
+    injection.flush(s);
 }
 
 // The same links with the neighbours' types from the overlapping type words
@@ -837,7 +892,7 @@ __global__ void __launch_bounds__(LINK_THREADS, LINK_BLOCKS) k_solid_links_words
     const unsigned un = (unsigned)s.n;
     const int nxw = s.nx >> 3;
     S* f = static_cast<S*>(s.f);
-    float injected = 0.f;   // mass the moving bounce-back adds to liquid cells
+    Injection injection;    // mass the moving bounce-back adds to liquid cells
     // types of the block around a cell, as 18 bits per plane
     auto types = [&](int x, int y, int z, unsigned (&w)[9]) {
         const int k = x >> 3;
@@ -848,8 +903,10 @@ __global__ void __launch_bounds__(LINK_THREADS, LINK_BLOCKS) k_solid_links_words
         }
     };
     int i = blockIdx.x * blockDim.x + threadIdx.x;
-    int cell = i < count ? s.sl[i] : 0;
-    int ahead = i + stride < count ? s.sl[i + stride] : 0;
+    // (-1: no entry; the cell loads then go to cell 0)
+    int listed = i < count ? s.sl[i] : -1;
+    int ahead = i + stride < count ? s.sl[i + stride] : -1;
+    int cell = max(listed, 0);
     int x, y, z;
     coords32(s, cell, x, y, z);
     unsigned w[9];
@@ -863,11 +920,12 @@ __global__ void __launch_bounds__(LINK_THREADS, LINK_BLOCKS) k_solid_links_words
             const int sh = 2 * ((x & 7) + 3);
             const unsigned t = ((w[3 * d] >> sh) & 0x3fu) | (((w[3 * d + 1] >> sh) & 0x3fu) << 6) |
                                (((w[3 * d + 2] >> sh) & 0x3fu) << 12);
-            fm[d] = i < count ? (t ^ (t >> 1)) & 0x15555u : 0u;   // liquid or interface
+            fm[d] = listed >= 0 ? (t ^ (t >> 1)) & 0x15555u : 0u;   // liquid or interface
             lm[d] = t & ~(t >> 1) & 0x15555u;
         }
         int key = -1;
-        if (i < count) {
+        float injected = 0.f;
+        if (listed >= 0) {
             if (p < 0 || p >= s.np) {
                 if (fm[0] | fm[1] | fm[2]) set_error(s, ERR_INVARIANT);
                 fm[0] = fm[1] = fm[2] = 0u;
@@ -887,8 +945,9 @@ __global__ void __launch_bounds__(LINK_THREADS, LINK_BLOCKS) k_solid_links_words
         }
         const PData P = particle_data(s, key < 0 ? 0 : key);
         // the next entry's types and owner
-        const int ncell = ahead;
-        ahead = i + 2 * stride < count ? s.sl[i + 2 * stride] : 0;
+        listed = ahead;
+        const int ncell = max(ahead, 0);
+        ahead = i + 2 * stride < count ? s.sl[i + 2 * stride] : -1;
         int nx_, ny_, nz_;
         coords32(s, ncell, nx_, ny_, nz_);
         unsigned nw[9];
@@ -955,6 +1014,7 @@ __global__ void __launch_bounds__(LINK_THREADS, LINK_BLOCKS) k_solid_links_words
             T[2] = (ddx * F[1] - ddy * F[0]) + 0.5f * gz;
         }
         flush_mem(s, key, F, T);
+        injection.add(injected);
         cell = ncell;
         x = nx_;
         y = ny_;
@@ -963,7 +1023,7 @@ __global__ void __launch_bounds__(LINK_THREADS, LINK_BLOCKS) k_solid_links_words
 #pragma unroll
         for (int r = 0; r < 9; ++r) w[r] = nw[r];
     }
-    link_injection(s, injected);
+    injection.flush(s);
 }
 
 // ---------------------------------------------------------------- bed segments
@@ -1455,9 +1515,17 @@ static bool use_pairs(const Dev& s) { return s.idx32 && (s.nx % 2) == 0 && !s.ga
 static bool use_split(const Dev& s) {
     return use_pairs(s) && s.storage != FSLBM_STORE_FP32 && s.nx >= 4 && s.ny >= 3 && s.nz >= 3;
 }
-// the staged even step: 16-bit storage, nx a multiple of the tile
+// the staged even step: 16-bit storage, nx a multiple of the tile, and few
+// enough tiles: with six and fewer per resident CTA its prefetch is the
+// faster one (256x40x96, 4.2 tiles per CTA: step 0.188 ms against 0.194 ms with
+// k_liquid_pair_warps), beyond that its block barriers cost more (512x40x96,
+// 8.4 tiles: 0.198 against 0.188 ms; the large flume 3.49 against 3.36 ms)
+template <typename S>
+static int staged_pair_blocks();
 static bool use_staged_pairs(const Dev& s) {
-    return s.idx32 && s.storage != FSLBM_STORE_FP32 && (s.nx % SP_TILE) == 0 && !s.galilean;
+    if (!s.idx32 || s.storage == FSLBM_STORE_FP32 || s.nx % SP_TILE != 0 || s.galilean) return false;
+    const int ctas = s.storage == FSLBM_STORE_FP16 ? staged_pair_blocks<__half>() : staged_pair_blocks<__nv_bfloat16>();
+    return s.n / SP_TILE <= 6LL * ctas;
 }
 
 // CTAs of the staged even step: as many as fit on the SMs at once, found
@@ -1538,6 +1606,8 @@ static void launch_typed(const Dev& s, int parity, cudaStream_t st, cudaEvent_t 
     const bool early = s.np > 0 && !s.links_fused;
     // liquid kernels: threads along x, blocks over the rows (y, z)
     const dim3 lgrid((unsigned)((s.nx + 255) / 256), (unsigned)(s.ny * s.nz < 65535 ? s.ny * s.nz : 65535));
+    // a warp per 256-cell segment of a row
+    const unsigned wblocks = (unsigned)(((long long)((s.nx + SEG_CELLS - 1) / SEG_CELLS) * s.ny * s.nz + 3) / 4);
     if (parity == 0) {
         if (s.np > 0 && !s.links_fused) {
             launch_links<S, 0>(s, st);
@@ -1549,7 +1619,8 @@ static void launch_typed(const Dev& s, int parity, cudaStream_t st, cudaEvent_t 
                 k_liquid_staged_pair<S><<<staged_pair_blocks<S>(), SP_TILE / 2, StagedPairLayout<S>::SMEM, st>>>(s);
             }
         } else if (use_pairs(s)) {
-            k_liquid_pair<S, 0, 0><<<lgrid, 128, 0, st>>>(s);
+            if constexpr (sizeof(S) == 2) k_liquid_pair_warps<S, 0, 0><<<wblocks, 128, 0, st>>>(s);
+            else k_liquid_pair<S, 0><<<lgrid, 128, 0, st>>>(s);
         } else {
             k_liquid<S, 0><<<lgrid, 256, 0, st>>>(s);
         }
@@ -1561,12 +1632,12 @@ static void launch_typed(const Dev& s, int parity, cudaStream_t st, cudaEvent_t 
         }
         if (early && links_done) cudaEventRecord(links_done, st);
         if (use_split(s)) {
-            k_liquid_pair<S, 1, 1><<<lgrid, 128, 0, st>>>(s);
+            if constexpr (sizeof(S) == 2) k_liquid_pair_warps<S, 1, 1><<<wblocks, 128, 0, st>>>(s);
             const long long ne = (2LL * s.nz + 2LL * (s.ny > 2 ? s.ny - 2 : 0)) * (s.nx / 2) +
                                  2LL * (s.ny > 2 ? s.ny - 2 : 0) * (s.nz > 2 ? s.nz - 2 : 0);
             k_liquid_pair_edges<S><<<blocks_for(ne, 128), 128, 0, st>>>(s);
         } else if (use_pairs(s)) {
-            k_liquid_pair<S, 1, 0><<<lgrid, 128, 0, st>>>(s);
+            k_liquid_pair<S, 1><<<lgrid, 128, 0, st>>>(s);
         } else {
             k_liquid<S, 1><<<lgrid, 256, 0, st>>>(s);
         }

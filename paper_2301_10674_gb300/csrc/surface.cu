@@ -662,12 +662,15 @@ int launch_conversion(const Dev& s, int last_parity, cudaStream_t st) {
 // thread's two 32-bit masks, ma to list la and mb to list lb: one scan of
 // both counts (list a in the low 16 bits, list b in the high ones; a block
 // holds at most 32 x 32 bits per warp), one atomic per list and block. The
-// cells of a block keep their order in each list. Every thread of the block
-// must call it.
+// cells of a block keep their order in each list. List b takes whole groups
+// of 32 entries per block, the last one filled up with -1: the link pass forms
+// FP32 sums over 32 consecutive entries, and with whole groups they hold the
+// same cells in the same order whichever block appends first (runs then repeat
+// to the order of FP64 atomics). Every thread of the block must call it.
 __device__ __forceinline__ void block_append_masks(const Dev& s, int c0, unsigned ma, int* la, int* ca, int capa,
                                                    unsigned mb, int* lb, int* cb, int capb) {
     __shared__ int warp_tot[32];
-    __shared__ int base_a, base_b;
+    __shared__ int base_a, base_b, total_b;
     const unsigned full = 0xffffffffu;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const int na = __popc(ma), nb = __popc(mb);
@@ -688,7 +691,8 @@ __device__ __forceinline__ void block_append_masks(const Dev& s, int c0, unsigne
             tb += c >> 16;
         }
         base_a = ta ? atomicAdd(ca, ta) : 0;
-        base_b = tb ? atomicAdd(cb, tb) : 0;
+        base_b = tb ? atomicAdd(cb, (tb + 31) & ~31) : 0;
+        total_b = tb;
     }
     __syncthreads();
     const int pre = warp_tot[wid];
@@ -702,6 +706,8 @@ __device__ __forceinline__ void block_append_masks(const Dev& s, int c0, unsigne
         if (kb < capb) lb[kb] = c0 + __ffs(m) - 1;
         else set_error(s, ERR_CAPACITY);
     }
+    const int pad = total_b + (int)threadIdx.x;   // (blocks have at least 32 threads)
+    if (pad < ((total_b + 31) & ~31) && base_b + pad < capb) lb[base_b + pad] = -1;
     __syncthreads();
 }
 
