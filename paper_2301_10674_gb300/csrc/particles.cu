@@ -746,10 +746,13 @@ __global__ void k_fixed_map(Dev s) {
 }
 
 // Calls f(p) for every mobile particle of the k-th grid cell of the ranges
-// that covers cell (x, y, z). The inside test is decided in FP32 where
-// |d^2 - r^2| exceeds a bound far above the FP32 rounding of the offsets (the
-// FP64 result has the same sign there) and in FP64 without fused multiply-add
-// otherwise.
+// that covers cell (x, y, z). |d^2 - r^2| is taken from the FP32 centre first
+// (rounded by up to 1e-4 cells at x = 3072), within its margin from the integer
+// and fraction of the centre (offsets exact to 1e-7, so the sum to 1e-6 of
+// 1 + r^2), and only within the margin of that (1e-5) in FP64 without fused
+// multiply-add, which decides: with the FP64 test for the whole first margin
+// every listed cell took it, and the kernel was bound by the FP64 pipe (70 us on
+// the large flume, 38 us now).
 template <class F>
 __device__ __forceinline__ void for_covers(const Dev& s, int x, int y, int z, const GRange& ra, const GRange& rb,
                                            const GRange& rc, int k, F f) {
@@ -770,10 +773,20 @@ __device__ __forceinline__ void for_covers(const Dev& s, int x, int y, int z, co
         const float tol = 1e-3f * (1.f + xr.w * xr.w);
         if (m32 > tol) continue;
         if (m32 >= -tol) {
-            const double* Xp = s.X + 3 * p;
-            const double m = map_metric(image_centre(x, Xp[0], s.nx, s.per_x), image_centre(y, Xp[1], s.ny, s.per_y),
-                                        image_centre(z, Xp[2], s.nz, s.per_z), Xp, s.R[p]);
-            if (m > 0.0) continue;
+            const int4 xi = s.Xi[p];
+            const float4 xf = s.Xfr[p];
+            const float ex = (float)wrap_int(x - xi.x, s.nx, s.per_x) + (0.5f - xf.x),
+                        ey = (float)wrap_int(y - xi.y, s.ny, s.per_y) + (0.5f - xf.y),
+                        ez = (float)wrap_int(z - xi.z, s.nz, s.per_z) + (0.5f - xf.z);
+            const float m2 = ex * ex + ey * ey + ez * ez - xr.w * xr.w;
+            if (m2 > 1e-2f * tol) continue;
+            if (m2 >= -1e-2f * tol) {
+                const double* Xp = s.X + 3 * p;
+                const double m = map_metric(image_centre(x, Xp[0], s.nx, s.per_x),
+                                            image_centre(y, Xp[1], s.ny, s.per_y),
+                                            image_centre(z, Xp[2], s.nz, s.per_z), Xp, s.R[p]);
+                if (m > 0.0) continue;
+            }
         }
         f(p);
     }
@@ -825,10 +838,13 @@ __global__ void k_remap_all(Dev s) {
     remap_cell(s, (int)c);
 }
 
-__device__ __forceinline__ void bbox_axis(double a, double b, double r, int L, int periodic, int& lo, int& hi) {
-    double mn = a < b ? a : b, mx = a < b ? b : a;
-    lo = (int)floor(mn - r - 0.5) - 1;
-    hi = (int)ceil(mx + r - 0.5) + 1;
+// cells along one axis that a sphere of radius r at a or b can cover, with a
+// cell to spare on each side (the FP32 rounding of the coordinates, below 0.07
+// at 2^20 cells, stays within it)
+__device__ __forceinline__ void bbox_axis(float a, float b, float r, int L, int periodic, int& lo, int& hi) {
+    const float mn = fminf(a, b), mx = fmaxf(a, b);
+    lo = (int)floorf(mn - r - 0.5f) - 1;
+    hi = (int)ceilf(mx + r - 0.5f) + 1;
     if (!periodic) {
         lo = lo < 0 ? 0 : lo;
         hi = hi > L - 1 ? L - 1 : hi;
@@ -856,21 +872,37 @@ __global__ void k_dirty(Dev s) {
     const int p = (int)(((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
     const int lane = threadIdx.x & 31;
     if (p >= s.np || s.fixed[p]) return;   // whole warps leave together
-    const double mx = s.X[3 * p] - s.Xm[3 * p], my = s.X[3 * p + 1] - s.Xm[3 * p + 1],
-                 mz = s.X[3 * p + 2] - s.Xm[3 * p + 2];
     const bool whole = s.shared[p] != 0;
-    if (!whole && mx == 0.0 && my == 0.0 && mz == 0.0) return;
+    // lane a < 3: axis a, its FP64 work once (the FP64 pipe issues a warp
+    // instruction in about 59 cycles, and there is a warp per particle;
+    // 17.6 -> 11.5 us for 4 712 particles)
+    double xa = 0.0, dm = 0.0;
+    if (lane < 3) {
+        xa = s.X[3 * p + lane];
+        dm = xa - s.Xm[3 * p + lane];
+    }
+    if (!whole && !__any_sync(0xffffffffu, dm != 0.0)) return;
+    const float df = (float)dm, xf32 = (float)xa;
+    const float fx = __shfl_sync(0xffffffffu, df, 0), fy = __shfl_sync(0xffffffffu, df, 1),
+                fz = __shfl_sync(0xffffffffu, df, 2);
     // shell half-width, rounded up
-    const float fx = (float)mx, fy = (float)my, fz = (float)mz;
     const float w = sqrtf(fx * fx + fy * fy + fz * fz) * (1.f + 1e-5f);
-    const double r = s.R[p];
+    const float r = fabsf(s.Xr[p].w);
     int lo[3], hi[3];
-    bbox_axis(s.Xm[3 * p], s.X[3 * p], r, s.nx, s.per_x, lo[0], hi[0]);
-    bbox_axis(s.Xm[3 * p + 1], s.X[3 * p + 1], r, s.ny, s.per_y, lo[1], hi[1]);
-    bbox_axis(s.Xm[3 * p + 2], s.X[3 * p + 2], r, s.nz, s.per_z, lo[2], hi[2]);
+    {
+        const int L = lane == 0 ? s.nx : (lane == 1 ? s.ny : s.nz);
+        const int per = lane == 0 ? s.per_x : (lane == 1 ? s.per_y : s.per_z);
+        int l = 0, h = 0;
+        bbox_axis(xf32 - df, xf32, r, L, per, l, h);
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            lo[k] = __shfl_sync(0xffffffffu, l, k);
+            hi[k] = __shfl_sync(0xffffffffu, h, k);
+        }
+    }
     const int4 xi = s.Xi[p];
     const float4 xf = s.Xfr[p];
-    const float rf = (float)r, band = w + 1e-3f;
+    const float rf = r, band = w + 1e-3f;
     const float ro = rf + band + 1e-3f, ri = fmaxf(rf - band - 1e-3f, 0.f);
     const int ex = hi[0] - lo[0] + 1, ey = hi[1] - lo[1] + 1, ez = hi[2] - lo[2] + 1;
     const int rows = ey * ez;
@@ -920,14 +952,14 @@ __global__ void k_dirty(Dev s) {
         }
     }
     __syncwarp();   // every lane has read the old map position and the flag
-    if (lane < 3) s.Xm[3 * p + lane] = s.X[3 * p + lane];
+    if (lane < 3) s.Xm[3 * p + lane] = xa;
     else if (lane == 3) s.shared[p] = 0;
 }
 
 // Lane groups of COVER_LANES over the dirty cells, a lane per grid cell
 // around it: a thread per cell walked the candidates of up to eight grid
 // cells one after the other, after six FP64 divisions (40 us at 1024x64x128
-// with 4 712 particles, 12.5 us now; 32 and 11 us at 512x40x96). The lanes
+// with 4 712 particles, 11.6 us now; 32 and 10.7 us at 512x40x96). The lanes
 // agree on the number of covering mobile particles; where the cell has one
 // cover or none that decides, otherwise the exact metrics do (lowest, then
 // lowest index), as in remap_cell.

@@ -799,34 +799,47 @@ __global__ void k_classify_bits(Dev s, int spread) {
     const long long w = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     const int nxw = s.nx >> 5;                      // words per row
     const long long nw = s.n >> 5;
-    unsigned ifc_mask = 0, sol_mask = 0;
+    unsigned ifc_mask = 0, sol_mask = 0, sol = 0;
     if (w < nw) {
-        const int xw = (int)(w % nxw);
-        const long long row = w / nxw;
-        const int y = (int)(row % s.ny), z = (int)(row / s.ny);
+        sol = s.sbits[w];
+        ifc_mask = s.ibits[w];
+    }
+    // the solid words' neighbourhood, only in warps that hold one; a lane's
+    // x-neighbour words are its neighbour lanes' own, but for the warp's and
+    // the rows' ends (27 words per lane, for every lane: 87 us on the large
+    // flume, 71 us now; 17.6 -> 14.5 us at 1024x64x128)
+    if (__any_sync(0xffffffffu, sol != 0)) {
+        const unsigned full = 0xffffffffu;
+        const int lane = threadIdx.x & 31;
+        const unsigned wc = (unsigned)(w < nw ? w : nw - 1);
+        const int xw = (int)(wc % (unsigned)nxw);
+        const unsigned row = wc / (unsigned)nxw;
+        const int y = (int)(row % (unsigned)s.ny), z = (int)(row / (unsigned)s.ny);
         // x-neighbour words (periodic wrap, or none beyond a wall face)
         const int xl = xw > 0 ? xw - 1 : (s.per_x ? nxw - 1 : -1);
         const int xr = xw < nxw - 1 ? xw + 1 : (s.per_x ? 0 : -1);
+        const bool own_l = lane == 0 || xw == 0, own_r = lane == 31 || xw == nxw - 1 || w + 1 >= nw;
+        unsigned cw[9], lw[9], rw[9];
+#pragma unroll
+        for (int k = 0; k < 9; ++k) {
+            const int yy = shift(y, k % 3 - 1, s.ny, s.per_y), zz = shift(z, k / 3 - 1, s.nz, s.per_z);
+            const bool in = (yy | zz) >= 0;
+            const unsigned* rb = s.fbits + (unsigned)(in ? zz * s.ny + yy : 0) * (unsigned)nxw;
+            cw[k] = in ? rb[xw] : 0u;
+            lw[k] = in && own_l && xl >= 0 ? rb[xl] : 0u;
+            rw[k] = in && own_r && xr >= 0 ? rb[xr] : 0u;
+        }
         unsigned long long orr = 0;   // bit 1 + k <-> x0 + k, bit 0 <-> x0 - 1, bit 33 <-> x0 + 32
 #pragma unroll
-        for (int dz = -1; dz <= 1; ++dz) {
-            const int zz = shift(z, dz, s.nz, s.per_z);
-            if (zz < 0) continue;
-#pragma unroll
-            for (int dy = -1; dy <= 1; ++dy) {
-                const int yy = shift(y, dy, s.ny, s.per_y);
-                if (yy < 0) continue;
-                const long long rbase = ((long long)zz * s.ny + yy) * nxw;
-                const unsigned cw = s.fbits[rbase + xw];
-                const unsigned lw = xl >= 0 ? s.fbits[rbase + xl] : 0u;
-                const unsigned rw = xr >= 0 ? s.fbits[rbase + xr] : 0u;
-                orr |= ((unsigned long long)cw << 1) | (unsigned long long)(lw >> 31) |
-                       ((unsigned long long)(rw & 1u) << 33);
-            }
+        for (int k = 0; k < 9; ++k) {
+            // the neighbour lanes' words: the row (y + dy, z + dz) of a lane in
+            // the same row of words
+            const unsigned l = __shfl_up_sync(full, cw[k], 1), r = __shfl_down_sync(full, cw[k], 1);
+            orr |= ((unsigned long long)cw[k] << 1) | (unsigned long long)((own_l ? lw[k] : l) >> 31) |
+                   ((unsigned long long)((own_r ? rw[k] : r) & 1u) << 33);
         }
         const unsigned long long nb = orr | (orr >> 1) | (orr << 1);   // bit 1 + k: fluid in the 3x3x3 block
-        sol_mask = s.sbits[w] & (unsigned)(nb >> 1);
-        ifc_mask = s.ibits[w];
+        sol_mask = sol & (unsigned)(nb >> 1);
     }
     const int c0 = (int)(w << 5);
     block_append_masks(s, c0, ifc_mask, s.wl, s.wl_count, s.wl_cap, sol_mask, s.sl, s.sl_count, s.sl_cap);
