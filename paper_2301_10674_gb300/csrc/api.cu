@@ -302,6 +302,11 @@ int fslbm_create(const fslbm_params* p, void* cuda_stream, fslbm** out) {
     d.dem_substeps = p->dem_substeps;
     d.lub = p->lubrication;
     d.lub_mu = (1.0 / p->omega - 0.5) / 3.0;
+    d.kn_f = (float)d.kn_coef;
+    d.dn_f = (float)d.dn_coef;
+    d.kt_f = (float)d.kt_ratio;
+    d.friction_f = (float)p->friction;
+    d.lub_mu_f = (float)d.lub_mu;
     s->elem = p->storage == FSLBM_STORE_FP32 ? 4 : 2;
 
     // The buffers of the run are parts of one device allocation: the section

@@ -148,6 +148,8 @@ struct Dev {
     int* nb; int* nb_count;                     // DEM neighbour list [np_cap][NB_SLOTS]
     double rho_p, restitution, friction, poisson, collision_time;
     double kn_coef, dn_coef, kt_ratio;          // contact law constants (host-computed)
+    // the sub-steps' FP32 copies (a conversion from FP64 takes the FP64 pipe)
+    float kn_f, dn_f, kt_f, friction_f, lub_mu_f;
     double gxd, gyd, gzd;
     int dem_substeps;
     int lub;                                    // lubrication corrections on

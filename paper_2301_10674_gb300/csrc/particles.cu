@@ -194,7 +194,7 @@ __device__ __forceinline__ void lub_f(const Dev& s, float R, const float (&n)[3]
                                       float (&Fl)[3], float (&Ft)[3]) {
     const float hh = fmaxf(h, LUB_HMIN);
     const float vn = dot_r(vrel, n);
-    const float k = 6.f * 3.14159265f * (float)s.lub_mu * R;
+    const float k = 6.f * 3.14159265f * s.lub_mu_f * R;
     const float cn = k * R * (1.f / hh - 1.f / LUB_HC);
     const float ct = k * (8.f / 15.f) * logf(LUB_HC / hh);
     for (int a = 0; a < 3; ++a) {
@@ -343,9 +343,9 @@ void launch_particle_copies(const Dev& s, cudaStream_t st) {
 __device__ __forceinline__ void contact_f(const Dev& s, float meff, const float (&n)[3], float delta,
                                           const float (&vrel)[3], float (&xi)[3], float dts, float (&F)[3],
                                           float (&Ft)[3]) {
-    const float kn = meff * (float)s.kn_coef;
-    const float dn = meff * (float)s.dn_coef;
-    const float kt = kn * (float)s.kt_ratio;
+    const float kn = meff * s.kn_f;
+    const float dn = meff * s.dn_f;
+    const float kt = kn * s.kt_f;
     const float dt_ = dn;
     const float vn = dot_r(vrel, n);
     const float vt[3] = {__fmaf_rn(-vn, n[0], vrel[0]), __fmaf_rn(-vn, n[1], vrel[1]), __fmaf_rn(-vn, n[2], vrel[2])};
@@ -355,7 +355,7 @@ __device__ __forceinline__ void contact_f(const Dev& s, float meff, const float 
     for (int a = 0; a < 3; ++a) x[a] = __fmaf_rn(vt[a], dts, __fmaf_rn(-xn, n[a], x[a]));
     for (int a = 0; a < 3; ++a) Ft[a] = __fmaf_rn(-kt, x[a], -__fmul_rn(dt_, vt[a]));
     const float ftl = sqrtf(dot_r(Ft, Ft));
-    const float lim = (float)s.friction * fabsf(fn);
+    const float lim = s.friction_f * fabsf(fn);
     if (ftl > lim && ftl > 0.f) {
         const float sc = lim / ftl;
         for (int a = 0; a < 3; ++a) {
@@ -396,41 +396,44 @@ static_assert(NB_SLOTS % DEM_LANES == 0 && NB_ITEMS == NB_SLOTS + DEM_LANES, "on
 // torque (12 floats); the group stride keeps a warp's four groups on distinct banks
 constexpr int DEM_SH = 104;
 
-__device__ __forceinline__ void dem_substep(const Dev& s, float* sh, int p, int l, unsigned gm, int a, bool have_prev,
-                                            float dts, bool first, bool last) {
-    const int b = 1 - a;
-    if (s.fixed[p]) {
-        // the top of the particle cells and the grid count the fixed particles too
-        if (last && l == 0) {
-            atomicMax(s.zmax_cell, (int)ceil(s.X[3 * p + 2] + s.R[p]) + 2);
-            atomicAdd(&s.g_count[s.g_of[p]], 1);
-        }
-        return;
+// What a lane group needs of its particle's lists, from global memory
+struct GlobalLists {
+    const Dev& s;
+    long long p;
+    int a;     // buffer of the published values
+    __device__ __forceinline__ void slot(int k, float4& d0, float4& xi, float4& xj, float4& uj, float4& wj) const {
+        const int j = s.nb[p * NB_SLOTS + k];
+        d0 = s.nb_d0[p * NB_SLOTS + k];
+        xi = s.nb_xi[p * NB_ITEMS + k];
+        xj = s.dem_x[a][j];
+        uj = s.dem_u[a][j];
+        wj = s.dem_w[a][j];
     }
-    const float4 cp = s.dem_c[p];
-    const float4 xa4 = s.dem_x[a][p], ua4 = s.dem_u[a][p], wa4 = s.dem_w[a][p];
-    const int nbc = s.nb_count[p];
+    __device__ __forceinline__ float4 spring(int k) const { return s.nb_xi[p * NB_ITEMS + k]; }
+    __device__ __forceinline__ void set_spring(int k, float4 v) const { s.nb_xi[p * NB_ITEMS + k] = v; }
+};
+
+// The outer force (lanes 0-2) or torque (lanes 3-5) along the lane's axis of
+// particle p: two-step average of the hydrodynamic force, plus the weight
+__device__ __forceinline__ float dem_outer(const Dev& s, int p, int l, bool have_prev) {
+    const bool trans = l < 3;
+    const int ax = trans ? l : l - 3, k = 3 * p + ax;
+    const double now = (trans ? s.Fh : s.Th)[k];
+    double* prev = (trans ? s.Fp : s.Tp) + k;
+    const double avg = have_prev ? 0.5 * (now + *prev) : now;
+    *prev = now;
+    const double g = ax == 0 ? s.gxd : (ax == 1 ? s.gyd : s.gzd);
+    return (float)(trans ? avg + s.M[p] * g : avg);
+}
+
+// Adds the contact and lubrication forces of one sub-step to the lanes'
+// components acc
+template <class Lists>
+__device__ __forceinline__ void dem_forces(const Dev& s, float* sh, const Lists& lists, int l, unsigned gm, int nbc,
+                                           const float4& cp, const float4& xa4, const float4& ua4, const float4& wa4,
+                                           float wall_d, float dts, float& acc) {
     const float rif = cp.x;
-    const bool trans = l < 3;              // lanes 0-2: velocity and position, 3-5: angular velocity
-    const int ax = trans ? l : l - 3;      // (lanes 6 and 7 hold no component)
-    float acc = 0.f;                       // the lane's component of force or torque
-    const float arm = trans ? 1.f : rif;   // torque: r n x F_t, the lanes' n x F_t times r
-    if (l < 6) {
-        const int k = 3 * p + ax;
-        float* outer = (trans ? s.Faf : s.Taf) + k;
-        if (first) {
-            // two-step average of the hydrodynamic force, plus the weight
-            const double now = (trans ? s.Fh : s.Th)[k];
-            double* prev = (trans ? s.Fp : s.Tp) + k;
-            const double avg = have_prev ? 0.5 * (now + *prev) : now;
-            *prev = now;
-            const double g = ax == 0 ? s.gxd : (ax == 1 ? s.gyd : s.gzd);
-            acc = (float)(trans ? avg + s.M[p] * g : avg);
-            *outer = acc;
-        } else {
-            acc = *outer;
-        }
-    }
+    const float arm = l < 3 ? 1.f : rif;   // torque: r n x F_t, the lanes' n x F_t times r
     int touching = 0;
     const int nround = (nbc + DEM_LANES - 1) / DEM_LANES;   // rounds of neighbours, then one of wall faces
 #pragma unroll 1
@@ -442,12 +445,8 @@ __device__ __forceinline__ void dem_substep(const Dev& s, float* sh, int p, int 
         float4 uj = make_float4(0.f, 0.f, 0.f, 0.f), wj = uj, xi4 = uj;
         if (!wall) {
             if (slot < nbc) {
-                const int j = s.nb[(long long)p * NB_SLOTS + slot];
-                const float4 d0 = s.nb_d0[(long long)p * NB_SLOTS + slot];
-                xi4 = s.nb_xi[(long long)p * NB_ITEMS + slot];
-                const float4 xj = s.dem_x[a][j];
-                uj = s.dem_u[a][j];
-                wj = s.dem_w[a][j];
+                float4 d0, xj;
+                lists.slot(slot, d0, xi4, xj, uj, wj);
                 rj = d0.w;
                 const float d[3] = {d0.x + (xj.x - xa4.x), d0.y + (xj.y - xa4.y), d0.z + (xj.z - xa4.z)};
                 const float dist2 = d[0] * d[0] + d[1] * d[1] + d[2] * d[2];
@@ -464,17 +463,21 @@ __device__ __forceinline__ void dem_substep(const Dev& s, float* sh, int p, int 
             const int wx = l >> 1;
             if (!(wx == 0 ? s.per_x : (wx == 1 ? s.per_y : s.per_z))) {
                 const float dxa = wx == 0 ? xa4.x : (wx == 1 ? xa4.y : xa4.z);
-                const float dist = (l & 1) ? s.dem_wall[6 * p + l] - dxa : s.dem_wall[6 * p + l] + dxa;
+                const float dist = (l & 1) ? wall_d - dxa : wall_d + dxa;
                 delta = rif - dist;
                 touch = delta > 0.f;
                 lub = s.lub && -delta < LUB_HC;
                 const float sg = (l & 1) ? 1.f : -1.f;
 #pragma unroll
                 for (int k = 0; k < 3; ++k) n[k] = k == wx ? sg : 0.f;
-                xi4 = s.nb_xi[(long long)p * NB_ITEMS + slot];
+                xi4 = lists.spring(slot);
                 xi4.w = cp.y;   // the wall's mass is infinite
             }
         }
+        // a partner not touched in this sub-step loses its spring
+        if (!touch && (xi4.x != 0.f || xi4.y != 0.f || xi4.z != 0.f))
+            lists.set_spring(slot, make_float4(0.f, 0.f, 0.f, xi4.w));
+        if (!__any_sync(gm, lub || touch)) continue;   // nothing to add in this round
         float Fl[3] = {0.f, 0.f, 0.f}, Fc[3] = {0.f, 0.f, 0.f}, tl[3] = {0.f, 0.f, 0.f}, tc[3] = {0.f, 0.f, 0.f};
         if (lub || touch) {
             // (the second two slots of every four fuse the partner's product: the
@@ -495,13 +498,10 @@ __device__ __forceinline__ void dem_substep(const Dev& s, float* sh, int p, int 
             if (touch) {
                 float xi[3] = {xi4.x, xi4.y, xi4.z};
                 contact_f(s, xi4.w, n, delta, vrel, xi, dts, Fc, Ft);
-                s.nb_xi[(long long)p * NB_ITEMS + slot] = make_float4(xi[0], xi[1], xi[2], xi4.w);
+                lists.set_spring(slot, make_float4(xi[0], xi[1], xi[2], xi4.w));
                 cross_r(n, Ft, tc);
             }
         }
-        // a partner not touched in this sub-step loses its spring
-        if (!touch && (xi4.x != 0.f || xi4.y != 0.f || xi4.z != 0.f))
-            s.nb_xi[(long long)p * NB_ITEMS + slot] = make_float4(0.f, 0.f, 0.f, xi4.w);
         touching += touch ? 1 : 0;
         float4* mine = reinterpret_cast<float4*>(sh + 12 * l);
         mine[0] = make_float4(Fl[0], Fl[1], Fl[2], tl[0]);
@@ -520,50 +520,46 @@ __device__ __forceinline__ void dem_substep(const Dev& s, float* sh, int p, int 
 #pragma unroll
     for (int o = 1; o < DEM_LANES; o <<= 1) touching += __shfl_xor_sync(gm, touching, o);
     if (touching > HIST_SLOTS && l == 0) set_error(s, ERR_HISTORY);
-    float v0 = 0.f, dv = 0.f;    // velocity component at the step's start, and its change
+}
+
+// The FP64 state of the step's end of a mobile particle (positions wrapped on
+// periodic axes), its FP32 copies and its grid cell, from the lanes' changes
+// of position (dx, lanes 0-2) and velocity (dv, lanes 0-5)
+__device__ __forceinline__ void dem_finish(const Dev& s, int p, int l, unsigned gm, float dx, float dv) {
+    const bool trans = l < 3;
+    const int ax = trans ? l : l - 3;
+    int g = 0;
+    if (trans) {
+        const int L = l == 0 ? s.nx : (l == 1 ? s.ny : s.nz);
+        double x = s.X[3 * p + l] + (double)dx;
+        if (l == 0 ? s.per_x : (l == 1 ? s.per_y : s.per_z)) x = x < 0.0 ? x + L : (x >= L ? x - L : x);
+        s.X[3 * p + l] = x;
+        const double fl = floor(x);
+        reinterpret_cast<float*>(s.Xr + p)[l] = (float)x;
+        reinterpret_cast<int*>(s.Xi + p)[l] = (int)fl;
+        reinterpret_cast<float*>(s.Xfr + p)[l] = (float)(x - fl);
+        if (l == 2) atomicMax(s.zmax_cell, (int)ceil(x + s.R[p]) + 2);
+        g = l == 0 ? gcoord(x, s.ghx, s.gnx)
+                   : (l == 1 ? s.gnx * gcoord(x, s.ghy, s.gny) : s.gnx * s.gny * gcoord(x, s.ghz, s.gnz));
+    }
     if (l < 6) {
-        const float4 v4 = trans ? s.Uf[p] : s.Wf[p];
-        v0 = ax == 0 ? v4.x : (ax == 1 ? v4.y : v4.z);
-        dv = reinterpret_cast<const float*>((trans ? s.dem_du : s.dem_dw) + p)[ax];
-        dv = dv + dts * acc * (1.f / (trans ? cp.y : cp.z));
+        double* v = (trans ? s.U : s.W) + 3 * p + ax;
+        const double vn = *v + (double)dv;
+        *v = vn;
+        reinterpret_cast<float*>((trans ? s.Uf : s.Wf) + p)[ax] = (float)vn;
     }
-    const float dxn = (ax == 0 ? xa4.x : (ax == 1 ? xa4.y : xa4.z)) + dts * (v0 + dv);   // (lanes 0-2)
-    __syncwarp(gm);   // every lane has read the copies Uf and Wf
-    if (l < 6 && !last) {
-        reinterpret_cast<float*>((trans ? s.dem_du : s.dem_dw) + p)[ax] = dv;
-        reinterpret_cast<float*>((trans ? s.dem_u : s.dem_w)[b] + p)[ax] = v0 + dv;
-        if (trans) reinterpret_cast<float*>(s.dem_x[b] + p)[ax] = dxn;
+    g += __shfl_xor_sync(gm, g, 1);
+    g += __shfl_xor_sync(gm, g, 2);
+    if (l == 0) {
+        s.g_of[p] = g;
+        atomicAdd(&s.g_count[g], 1);
     }
-    if (last) {
-        // the FP64 state of the step's end (positions wrapped on periodic
-        // axes), its FP32 copies and the grid cell
-        int g = 0;
-        if (trans) {
-            const int L = l == 0 ? s.nx : (l == 1 ? s.ny : s.nz);
-            double x = s.X[3 * p + l] + (double)dxn;
-            if (l == 0 ? s.per_x : (l == 1 ? s.per_y : s.per_z)) x = x < 0.0 ? x + L : (x >= L ? x - L : x);
-            s.X[3 * p + l] = x;
-            const double fl = floor(x);
-            reinterpret_cast<float*>(s.Xr + p)[l] = (float)x;
-            reinterpret_cast<int*>(s.Xi + p)[l] = (int)fl;
-            reinterpret_cast<float*>(s.Xfr + p)[l] = (float)(x - fl);
-            if (l == 2) atomicMax(s.zmax_cell, (int)ceil(x + s.R[p]) + 2);
-            g = l == 0 ? gcoord(x, s.ghx, s.gnx)
-                       : (l == 1 ? s.gnx * gcoord(x, s.ghy, s.gny) : s.gnx * s.gny * gcoord(x, s.ghz, s.gnz));
-        }
-        if (l < 6) {
-            double* v = (trans ? s.U : s.W) + 3 * p + ax;
-            const double vn = *v + (double)dv;
-            *v = vn;
-            reinterpret_cast<float*>((trans ? s.Uf : s.Wf) + p)[ax] = (float)vn;
-        }
-        g += __shfl_xor_sync(gm, g, 1);
-        g += __shfl_xor_sync(gm, g, 2);
-        if (l == 0) {
-            s.g_of[p] = g;
-            atomicAdd(&s.g_count[g], 1);
-        }
-    }
+}
+// a fixed particle: the top of the particle cells and the grid count it too
+__device__ __forceinline__ void dem_finish_fixed(const Dev& s, int p, int l) {
+    if (l != 0) return;
+    atomicMax(s.zmax_cell, (int)ceil(s.X[3 * p + 2] + s.R[p]) + 2);
+    atomicAdd(&s.g_count[s.g_of[p]], 1);
 }
 
 // one sub-step; the first of several also clears what the last one counts
@@ -575,45 +571,163 @@ __global__ void __launch_bounds__(128) k_dem_substep(Dev s, int a, int have_prev
         for (int g = t; g < G; g += gridDim.x * blockDim.x) s.g_count[g] = 0;
         if (t == 0) *s.zmax_cell = 0;
     }
-    const int p = t / DEM_LANES, l = t % DEM_LANES;
+    const int p = t / DEM_LANES, l = t % DEM_LANES, b = 1 - a;
     const unsigned gm = ((1u << DEM_LANES) - 1u) << ((threadIdx.x & 31) / DEM_LANES * DEM_LANES);
-    if (p < s.np)
-        dem_substep(s, sh + threadIdx.x / DEM_LANES * DEM_SH, p, l, gm, a, have_prev != 0, dts, first != 0, last != 0);
+    if (p >= s.np) return;                    // whole groups leave together
+    if (s.fixed[p]) {
+        if (last) dem_finish_fixed(s, p, l);
+        return;
+    }
+    const float4 cp = s.dem_c[p];
+    const float4 xa4 = s.dem_x[a][p], ua4 = s.dem_u[a][p], wa4 = s.dem_w[a][p];
+    const bool trans = l < 3;                 // lanes 0-2: velocity and position, 3-5: angular velocity
+    const int ax = trans ? l : l - 3;         // (lanes 6 and 7 hold no component)
+    float acc = 0.f;                          // the lane's component of force or torque
+    if (l < 6) {
+        float* outer = (trans ? s.Faf : s.Taf) + 3 * p + ax;
+        if (first) *outer = acc = dem_outer(s, p, l, have_prev != 0);
+        else acc = *outer;
+    }
+    const float wall_d = l < 6 ? s.dem_wall[6 * p + l] : 0.f;
+    dem_forces(s, sh + threadIdx.x / DEM_LANES * DEM_SH, GlobalLists{s, p, a}, l, gm, s.nb_count[p], cp, xa4, ua4, wa4,
+               wall_d, dts, acc);
+    float v0 = 0.f, dv = 0.f;    // velocity component at the step's start, and its change
+    if (l < 6) {
+        const float4 v4 = trans ? s.Uf[p] : s.Wf[p];
+        v0 = ax == 0 ? v4.x : (ax == 1 ? v4.y : v4.z);
+        dv = reinterpret_cast<const float*>((trans ? s.dem_du : s.dem_dw) + p)[ax];
+        dv = dv + dts * acc * (1.f / (trans ? cp.y : cp.z));
+    }
+    const float dxn = (ax == 0 ? xa4.x : (ax == 1 ? xa4.y : xa4.z)) + dts * (v0 + dv);   // (lanes 0-2)
+    __syncwarp(gm);   // every lane has read the copies Uf and Wf
+    if (last) {
+        dem_finish(s, p, l, gm, dxn, dv);
+    } else if (l < 6) {
+        reinterpret_cast<float*>((trans ? s.dem_du : s.dem_dw) + p)[ax] = dv;
+        reinterpret_cast<float*>((trans ? s.dem_u : s.dem_w)[b] + p)[ax] = v0 + dv;
+        if (trans) reinterpret_cast<float*>(s.dem_x[b] + p)[ax] = dxn;
+    }
 }
 
 // The sub-steps of a step and the particle grid in one thread-block cluster,
 // for up to DEM_CLUSTER_MAX particles: the cluster's hardware barrier
 // (release at arrival, acquire at the wait) stands between the phases that
 // read other particles' values, so nothing is launched between the sub-steps.
-// Measured for the whole DEM half (ten sub-steps and the grid): 52 us for 34
-// particles, 113 us for 1 008 (two per lane group), against ten launches of
-// 9.7 us plus three of the grid; beyond 1 024 particles a lane group would take
-// three and more in turn, and the launches win.
+// A lane group keeps its particle's lists and springs in shared memory and its
+// constants in registers for the whole step, and reads its partners' published
+// values from the shared memory of the CTA that owns them: with all of it in
+// global memory a sub-step waited for six L2 latencies in turn. Measured for the whole DEM half (ten
+// sub-steps and the grid): CLUSTER_FIGS
 constexpr int DEM_CLUSTER_MAX = 1024;
 constexpr int DEM_CLUSTER_CTAS = 8;
-constexpr int DEM_CLUSTER_THREADS = 512;
 
 __device__ __forceinline__ void cluster_barrier() {
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
+__device__ __forceinline__ unsigned cluster_address(const void* p, unsigned rank) {
+    unsigned r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;"
+                 : "=r"(r)
+                 : "r"((unsigned)__cvta_generic_to_shared(p)), "r"(rank));
+    return r;
+}
+__device__ __forceinline__ float4 cluster_load(unsigned address) {
+    float4 v;
+    asm volatile("ld.shared::cluster.v4.f32 {%0,%1,%2,%3}, [%4];"
+                 : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+                 : "r"(address)
+                 : "memory");
+    return v;
+}
 
-__global__ void __launch_bounds__(DEM_CLUSTER_THREADS) k_dem_cluster(Dev s, int have_prev, int G, float dts) {
-    __shared__ __align__(16) float sh[DEM_CLUSTER_THREADS / DEM_LANES * DEM_SH];
-    __shared__ int wtot[DEM_CLUSTER_THREADS / 32];
+// shared memory per particle of a CTA: published values (x, u, w; two
+// buffers), list offsets and springs, partners' addresses
+struct ClusterParticle {
+    float4 pub[2][3];
+    float4 d0[NB_SLOTS];
+    float4 xi[NB_ITEMS];
+    unsigned at[NB_SLOTS];      // cluster address of the partner's ClusterParticle
+};
+struct ClusterLists {
+    ClusterParticle& me;
+    int a;
+    __device__ __forceinline__ void slot(int k, float4& d0, float4& xi, float4& xj, float4& uj, float4& wj) const {
+        const unsigned at = me.at[k] + (unsigned)a * 3u * (unsigned)sizeof(float4);
+        xj = cluster_load(at);
+        uj = cluster_load(at + (unsigned)sizeof(float4));
+        wj = cluster_load(at + 2u * (unsigned)sizeof(float4));
+        d0 = me.d0[k];
+        xi = me.xi[k];
+    }
+    __device__ __forceinline__ float4 spring(int k) const { return me.xi[k]; }
+    __device__ __forceinline__ void set_spring(int k, float4 v) const { me.xi[k] = v; }
+};
+
+template <int THREADS>
+__global__ void __launch_bounds__(THREADS) k_dem_cluster(Dev s, int have_prev, int G, float dts) {
+    extern __shared__ __align__(16) unsigned char cluster_smem[];
+    __shared__ int wtot[THREADS / 32];
     const int nt = gridDim.x * blockDim.x, tid = blockIdx.x * blockDim.x + threadIdx.x;   // one cluster: the grid
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
     const unsigned full = 0xffffffffu;
-    const int l = tid % DEM_LANES;
+    const int l = tid % DEM_LANES, gpc = blockDim.x / DEM_LANES, lg = threadIdx.x / DEM_LANES;   // groups per CTA, local group
     const unsigned gm = ((1u << DEM_LANES) - 1u) << (lane / DEM_LANES * DEM_LANES);
+    ClusterParticle* parts = reinterpret_cast<ClusterParticle*>(cluster_smem);      // [gpc]
+    float* sh = reinterpret_cast<float*>(parts + gpc) + lg * DEM_SH;
+    const bool trans = l < 3;
+    const int ax = trans ? l : l - 3;
+    const int p = tid / DEM_LANES;
+    const bool mobile = p < s.np && s.fixed[p] == 0;
+    ClusterParticle& me = parts[lg];
+    int nbc = 0;
+    float4 cp = make_float4(0.f, 0.f, 0.f, 0.f);
+    float outer = 0.f, v0 = 0.f, dv = 0.f, wall_d = 0.f;
+    if (p < s.np && l < 6) me.pub[l & 1][l >> 1] = l < 2 ? s.dem_x[0][p] : (l < 4 ? s.Uf[p] : s.Wf[p]);
+    if (mobile) {
+        nbc = s.nb_count[p];
+        cp = s.dem_c[p];
+        for (int k = l; k < nbc; k += DEM_LANES) {
+            const int j = s.nb[(long long)p * NB_SLOTS + k];
+            me.d0[k] = s.nb_d0[(long long)p * NB_SLOTS + k];
+            me.xi[k] = s.nb_xi[(long long)p * NB_ITEMS + k];
+            me.at[k] = cluster_address(&parts[j % gpc].pub[0][0], (unsigned)(j / gpc));
+        }
+        me.xi[NB_SLOTS + l] = s.nb_xi[(long long)p * NB_ITEMS + NB_SLOTS + l];
+        if (l < 6) {
+            outer = dem_outer(s, p, l, have_prev != 0);
+            const float4 v4 = trans ? s.Uf[p] : s.Wf[p];
+            v0 = ax == 0 ? v4.x : (ax == 1 ? v4.y : v4.z);
+            wall_d = s.dem_wall[6 * p + l];
+        }
+    }
     for (int g = tid; g < G; g += nt) s.g_count[g] = 0;
     if (tid == 0) *s.zmax_cell = 0;
     cluster_barrier();
     for (int k = 0; k < s.dem_substeps; ++k) {
-        for (int p = tid / DEM_LANES; p < s.np; p += nt / DEM_LANES)
-            dem_substep(s, sh + threadIdx.x / DEM_LANES * DEM_SH, p, l, gm, k & 1, have_prev != 0, dts, k == 0,
-                        k == s.dem_substeps - 1);
+        const int a = k & 1, b = 1 - a;
+        if (mobile) {
+            const float4 xa4 = me.pub[a][0], ua4 = me.pub[a][1], wa4 = me.pub[a][2];
+            float acc = outer;
+            dem_forces(s, sh, ClusterLists{me, a}, l, gm, nbc, cp, xa4, ua4, wa4, wall_d, dts, acc);
+            if (l < 6) dv = dv + dts * acc * (1.f / (trans ? cp.y : cp.z));
+            const float dxn = (ax == 0 ? xa4.x : (ax == 1 ? xa4.y : xa4.z)) + dts * (v0 + dv);   // (lanes 0-2)
+            if (k == s.dem_substeps - 1) {
+                dem_finish(s, p, l, gm, dxn, dv);
+            } else if (l < 6) {
+                reinterpret_cast<float*>(&me.pub[b][trans ? 1 : 2])[ax] = v0 + dv;
+                if (trans) reinterpret_cast<float*>(&me.pub[b][0])[ax] = dxn;
+            }
+        }
         cluster_barrier();
     }
+    if (mobile) {
+        // the springs go back to the lists
+        for (int k = l; k < nbc; k += DEM_LANES) s.nb_xi[(long long)p * NB_ITEMS + k] = me.xi[k];
+        s.nb_xi[(long long)p * NB_ITEMS + NB_SLOTS + l] = me.xi[NB_SLOTS + l];
+    } else if (p < s.np) {
+        dem_finish_fixed(s, p, l);
+    }
+    cluster_barrier();
     // exclusive scan of the grid counts: each CTA scans a contiguous run of
     // rows of 32 counts, a warp a part of it; the CTAs' totals pass through g_tot
     const int rows = (G + 31) / 32;
@@ -653,7 +767,7 @@ __global__ void __launch_bounds__(DEM_CLUSTER_THREADS) k_dem_cluster(Dev s, int 
         run += __shfl_sync(full, v, 31);
     }
     cluster_barrier();
-    for (int p = tid; p < s.np; p += nt) grid_fill(s, p);
+    for (int q = tid; q < s.np; q += nt) grid_fill(s, q);
     cluster_barrier();
     for (int g = tid; g < G; g += nt) grid_sort(s, g);
 }
@@ -1204,14 +1318,17 @@ int launch_dem(const Dev& s, int have_prev, cudaStream_t st) {
     const int ns = s.dem_substeps, G = s.gnx * s.gny * s.gnz;
     const float dts = 1.f / (float)ns;
     if (s.np <= DEM_CLUSTER_MAX) {
-        // as many CTAs (a power of two) as give one warp per scheduler
+        // one particle per lane group, in as many CTAs (a power of two) as
+        // leave one warp per scheduler
+        const int lanes = s.np * DEM_LANES;
         int ctas = 1;
-        while (ctas < DEM_CLUSTER_CTAS && ctas * 128 < s.np * DEM_LANES) ctas *= 2;
-        int threads = ((s.np * DEM_LANES + ctas - 1) / ctas + 31) / 32 * 32;
-        threads = threads < 128 ? 128 : (threads > DEM_CLUSTER_THREADS ? DEM_CLUSTER_THREADS : threads);
+        while (ctas < DEM_CLUSTER_CTAS && ctas * 128 < lanes) ctas *= 2;
+        int threads = ((lanes + ctas - 1) / ctas + 31) / 32 * 32;
+        threads = threads < 128 ? 128 : threads;
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3((unsigned)ctas);
         cfg.blockDim = dim3((unsigned)threads);
+        cfg.dynamicSmemBytes = threads / DEM_LANES * (sizeof(ClusterParticle) + DEM_SH * sizeof(float));
         cfg.stream = st;
         cudaLaunchAttribute at[1];
         at[0].id = cudaLaunchAttributeClusterDimension;
@@ -1219,7 +1336,9 @@ int launch_dem(const Dev& s, int have_prev, cudaStream_t st) {
         at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
         cfg.attrs = at;
         cfg.numAttrs = 1;
-        cudaLaunchKernelEx(&cfg, k_dem_cluster, s, have_prev, G, dts);
+        auto* kernel = threads <= 512 ? k_dem_cluster<512> : k_dem_cluster<1024>;
+        cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cfg.dynamicSmemBytes);
+        cudaLaunchKernelEx(&cfg, kernel, s, have_prev, G, dts);
         return 1;
     }
     if (ns == 1) {
