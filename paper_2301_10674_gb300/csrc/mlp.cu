@@ -255,52 +255,64 @@ __device__ __forceinline__ uint64_t splitmix64(uint64_t seed, uint64_t counter) 
 // cube symmetry k: (T v)_i = s_i v_perm(i), perm the (k / 8)-th permutation
 // of (0, 1, 2) in lexicographic order, s_i = -1 where bit i of k % 8 is set
 __device__ __forceinline__ int sym_perm(int k, int i) {
-    constexpr int P[6][3] = {{0, 1, 2}, {0, 2, 1}, {1, 0, 2}, {1, 2, 0}, {2, 0, 1}, {2, 1, 0}};
-    return P[k >> 3][i];
+    // two bits per axis, six per permutation, the first lowest
+    constexpr uint64_t P = 0b000110'010010'001001'100001'011000'100100ull;
+    return (int)(P >> (6 * (k >> 3) + 2 * i)) & 3;
 }
 __device__ __forceinline__ int sym_sign(int k, int i) { return ((k & 7) >> i & 1) ? -1 : 1; }
 
-// the cell whose fill lands in cell qd under symmetry k: c = T^-1 c', i.e.
-// c[perm(i)] = s_i c'[i]
-__device__ __forceinline__ int sym_source(int k, int qd) {
-    const int cdst[3] = {qd % 3 - 1, (qd / 3) % 3 - 1, qd / 9 - 1};
-    int c[3] = {0, 0, 0};
-#pragma unroll
-    for (int i = 0; i < 3; ++i) c[sym_perm(k, i)] = sym_sign(k, i) * cdst[i];
-    return (c[0] + 1) + 3 * (c[1] + 1) + 9 * (c[2] + 1);
+// The cell whose fill lands in cell c' = (x, y, z) under symmetry k is
+// c = T^-1 c', i.e. c[perm(i)] = s_i c'[i]: index 13 + m0 x + m1 y + m2 z with
+// m_i = s_i 3^perm(i)
+__device__ __forceinline__ int sym_stride(int k, int i) {
+    const int p = sym_perm(k, i);
+    return sym_sign(k, i) * (p == 0 ? 1 : (p == 1 ? 3 : 9));
 }
 
 // ------------------------------------------------------------ training
-constexpr int TR_WARPS = 8;
-constexpr int TR_ROWS = 16 * TR_WARPS;   // samples per block
-constexpr int LDS = TR_ROWS + 8;         // padded row: rows g = 0..7 fall in distinct banks
-constexpr int PSTRIDE = 6216;            // floats per block in the partial buffer
-constexpr int LOSS_SLOT = MLP_NPARAM;
+// A batch is summed in chunks of 128 samples, each of 8 tiles of 16: the order
+// of every sum (samples of a chunk in one tensor-core chain, tiles of a chunk
+// and chunks one after the other) is fixed, and two runs give the same bits.
+constexpr int CHUNK_TILES = 8, CHUNK = 16 * CHUNK_TILES;
+constexpr int NBIAS = 2 * MLP_H + MLP_OUT + 1;   // bias gradients and the loss
+constexpr int SLICE_CHUNKS = 128;                // chunks whose operands are held at once
 
-struct TrainSmem {
-    __nv_bfloat16 XT[32][LDS];           // inputs, transposed (column, sample)
-    __nv_bfloat16 H1T[MLP_H][LDS];       // relu(z1)
-    __nv_bfloat16 H2T[MLP_H][LDS];       // relu(z2)
-    __nv_bfloat16 D1T[MLP_H][LDS];       // dL/dz1
-    __nv_bfloat16 D2T[MLP_H][LDS];       // dL/dz2
-    __nv_bfloat16 DYT[16][LDS];          // dL/dy (outputs 4..15 zero)
-    float bsum[TR_WARPS][132];           // per-warp column sums of dz1, dz2, dy
-    float lsum[TR_WARPS];
+// parameters as the operands of a training step
+struct __align__(16) TrainWeights {
+    MlpFwd f;
+    uint2 w2t[8][4][32];     // W2 transposed
+    uint32_t w3t[8][32];     // W3 transposed; outputs 8..15 are zero
+};
+
+// The operands of the weight gradients dW = dZ^T H of one tile of 16 samples,
+// in fragment order with the samples along k, and its sums
+constexpr int SAMPLE_THREADS = 128;
+
+struct __align__(16) TrainOps {
+    uint4 d1[4][32];         // dL/dz1
+    uint4 d2[4][32];         // dL/dz2
+    uint2 h1[8][32];         // relu(z1)
+    uint2 h2[8][32];         // relu(z2)
+    uint2 x[4][32];          // inputs
+    uint2 dy[32];            // dL/dy (rows 8..15 are zero)
+    float sums[NBIAS + 3];   // dz1, dz2, dy, loss
 };
 
 enum : int { TR_FIXED = 0, TR_DRAW_SYM = 1, TR_DRAW = 2 };
 
 struct TrainArgs {
-    const MlpBf16* W;
+    const TrainWeights* W;
     const float* fill;
     const float* target;
     long long n;            // stencils in the set
     int B;                  // samples in the batch
+    int first;              // first sample of the slice
+    int tiles;              // tiles of the slice
     int mode;               // TR_FIXED: sample j is stencil j; TR_DRAW(_SYM): drawn (and mapped)
     uint64_t seed;
     long long step;
     float lam, mu;
-    float* part;            // [blocks][PSTRIDE]
+    TrainOps* ops;          // [tiles]
 };
 
 __device__ __forceinline__ float sum_over_groups(float v) {
@@ -310,55 +322,95 @@ __device__ __forceinline__ float sum_over_groups(float v) {
     return v;
 }
 
-// One block per 128 samples: per-warp forward and backward of 16 samples,
-// then the block's share of the weight gradients dW = dZ^T H as 56
-// tensor-core tiles over K = 128 samples, written with the bias and loss
-// sums to the block's row of the partial buffer.
-__global__ void __launch_bounds__(256) k_mlp_train_block(TrainArgs a) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    TrainSmem& S = *reinterpret_cast<TrainSmem*>(smem_raw);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-    const MlpBf16& W = *a.W;
-    const float invB = 1.f / (float)a.B;
+// 8 x 8 matrix of 16-bit values across the warp (lane (g, t) holds row g,
+// columns 2t and 2t + 1), transposed
+__device__ __forceinline__ uint32_t transposed(uint32_t a) {
+    uint32_t d;
+    asm volatile("movmatrix.sync.aligned.m8n8.trans.b16 %0, %1;" : "=r"(d) : "r"(a));
+    return d;
+}
 
-    // -------- per-warp forward and backward
-    long long src[2];
-    int sym[2];
+// programmatic dependent launch: the previous kernel of the stream is complete
+// and its writes are visible after the first; the next one may start after the
+// second
+__device__ __forceinline__ void wait_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void allow_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+// Forward and backward pass, a warp per 16 samples, and the operands of the
+// weight gradients. Bound by latency: a warp runs about 2000 instructions one
+// after the other, so there is a warp per scheduler and an SM for every four
+// tiles. Weights come in fragment order, all of them at once, to shared memory
+// (read from L2 where they are used: 0.9 us more); the transposes that the
+// gradient products need are made in registers; drawing and gathering the
+// samples, which need no weights, run before the previous launch is waited
+// for. A step with a batch of 4096 takes 9.5 us; with one block of 8 warps per
+// chunk, which also formed the chunk's weight gradients from transposes in
+// shared memory, and a second launch for the sums and the update it took 31 us
+// (24.4 + 5.6 and the gaps).
+__global__ void __launch_bounds__(SAMPLE_THREADS) k_mlp_train_samples(TrainArgs a) {
+    __shared__ TrainWeights W;
+    const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+    const int tile = blockIdx.x * (SAMPLE_THREADS / 32) + (threadIdx.x >> 5);
+    const float invB = 1.f / (float)a.B;
+    uint32_t xf[2][4];
+    float tg[2][4];
     bool valid[2];
+    {
+        float xv[2][8];
 #pragma unroll
-    for (int r = 0; r < 2; ++r) {
-        const long long j = (long long)blockIdx.x * TR_ROWS + warp * 16 + g + 8 * r;
-        valid[r] = j < a.B;
-        src[r] = 0;
-        sym[r] = 0;
-        if (valid[r]) {
-            if (a.mode == TR_FIXED) {
-                src[r] = j;
-            } else {
+        for (int r = 0; r < 2; ++r) {
+            const long long j = a.first + (long long)tile * 16 + g + 8 * r;
+            valid[r] = tile < a.tiles && j < a.B;
+            long long src = j;
+            int sym = 0;
+            if (a.mode != TR_FIXED) {
                 const uint64_t v = splitmix64(a.seed, (uint64_t)a.step * (uint64_t)a.B + (uint64_t)j);
-                src[r] = (long long)(v % (uint64_t)a.n);
-                sym[r] = a.mode == TR_DRAW_SYM ? (int)((v >> 32) % 48ull) : 0;
+                src = (long long)(v % (uint64_t)a.n);
+                sym = a.mode == TR_DRAW_SYM ? (int)((v >> 32) % 48ull) : 0;
+            }
+            const int m0 = sym_stride(sym, 0), m1 = sym_stride(sym, 1), m2 = sym_stride(sym, 2);
+            const float* f = a.fill + src * 27 + 13;
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+                const int col = frag_col(q >> 2, q & 3, t);
+                xv[r][q] = (valid[r] && col < 27)
+                               ? f[m0 * (col % 3 - 1) + m1 * (col / 3 % 3 - 1) + m2 * (col / 9 - 1)]
+                               : 0.f;
+            }
+#pragma unroll
+            for (int i = 0; i < 4; ++i) tg[r][i] = 0.f;
+            if (valid[r]) {
+                const float* tp = a.target + src * 4;
+#pragma unroll
+                for (int i = 0; i < 3; ++i) tg[r][i] = sym_sign(sym, i) * tp[sym_perm(sym, i)];
+                tg[r][3] = tp[3];
             }
         }
-    }
-    float xv[2][8];
 #pragma unroll
-    for (int r = 0; r < 2; ++r)
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            const int col = frag_col(j >> 2, j & 3, t);
-            xv[r][j] = (valid[r] && col < 27) ? a.fill[src[r] * 27 + sym_source(sym[r], col)] : 0.f;
+        for (int kk = 0; kk < 2; ++kk) {
+            xf[kk][0] = pack_bf16(xv[0][4 * kk + 0], xv[0][4 * kk + 1]);
+            xf[kk][1] = pack_bf16(xv[1][4 * kk + 0], xv[1][4 * kk + 1]);
+            xf[kk][2] = pack_bf16(xv[0][4 * kk + 2], xv[0][4 * kk + 3]);
+            xf[kk][3] = pack_bf16(xv[1][4 * kk + 2], xv[1][4 * kk + 3]);
         }
-    uint32_t xf[2][4];
-#pragma unroll
-    for (int kk = 0; kk < 2; ++kk) {
-        xf[kk][0] = pack_bf16(xv[0][4 * kk + 0], xv[0][4 * kk + 1]);
-        xf[kk][1] = pack_bf16(xv[1][4 * kk + 0], xv[1][4 * kk + 1]);
-        xf[kk][2] = pack_bf16(xv[0][4 * kk + 2], xv[0][4 * kk + 3]);
-        xf[kk][3] = pack_bf16(xv[1][4 * kk + 2], xv[1][4 * kk + 3]);
     }
+    wait_previous();
+    allow_next();
+    for (int q = threadIdx.x; q < (int)(sizeof(TrainWeights) / 16); q += SAMPLE_THREADS)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
+                         (uint32_t)__cvta_generic_to_shared(reinterpret_cast<uint4*>(&W) + q)),
+                     "l"(reinterpret_cast<const uint4*>(a.W) + q)
+                     : "memory");
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    __syncthreads();
+    if (tile >= a.tiles) return;
+    TrainOps& O = a.ops[tile];
+#pragma unroll
+    for (int nt = 0; nt < 4; ++nt)
+        O.x[nt][lane] = make_uint2(transposed(xf[nt >> 1][2 * (nt & 1)]), transposed(xf[nt >> 1][2 * (nt & 1) + 1]));
+
     MlpAct act;
-    mlp_forward(W, xf, act);
+    mlp_forward_ops(W.f.w1, W.f.w2, W.f.w3, W.f.b1, W.f.b2, W.f.b3, xf, act);
     float y[2][4];
     mlp_outputs(act, y[0], y[1]);
 
@@ -367,22 +419,14 @@ __global__ void __launch_bounds__(256) k_mlp_train_block(TrainArgs a) {
     float dy[2][4], L[2];
 #pragma unroll
     for (int r = 0; r < 2; ++r) {
-        float tg[4] = {0.f, 0.f, 0.f, 0.f};
-        if (valid[r]) {
-            const float* tp = a.target + src[r] * 4;
-            const int k = sym[r];
-#pragma unroll
-            for (int i = 0; i < 3; ++i) tg[i] = sym_sign(k, i) * tp[sym_perm(k, i)];
-            tg[3] = tp[3];
-        }
         const float n2 = y[r][0] * y[r][0] + y[r][1] * y[r][1] + y[r][2] * y[r][2];
         const float nrm = sqrtf(fmaxf(n2, 1e-30f));
-        const float dot = y[r][0] * tg[0] + y[r][1] * tg[1] + y[r][2] * tg[2];
-        const float dk = y[r][3] - tg[3];
+        const float dot = y[r][0] * tg[r][0] + y[r][1] * tg[r][1] + y[r][2] * tg[r][2];
+        const float dk = y[r][3] - tg[r][3];
         const float pen = 2.f * a.mu * (nrm - 1.f) / nrm;
 #pragma unroll
         for (int i = 0; i < 3; ++i)
-            dy[r][i] = valid[r] ? (-(tg[i] / nrm - dot / (nrm * nrm * nrm) * y[r][i]) + pen * y[r][i]) * invB : 0.f;
+            dy[r][i] = valid[r] ? (-(tg[r][i] / nrm - dot / (nrm * nrm * nrm) * y[r][i]) + pen * y[r][i]) * invB : 0.f;
         dy[r][3] = valid[r] ? 2.f * a.lam * dk * invB : 0.f;
         L[r] = valid[r] ? (1.f - dot / nrm + a.lam * dk * dk + a.mu * (nrm - 1.f) * (nrm - 1.f)) * invB : 0.f;
     }
@@ -394,11 +438,11 @@ __global__ void __launch_bounds__(256) k_mlp_train_block(TrainArgs a) {
 #pragma unroll
     for (int nt = 0; nt < 8; ++nt) {
         float d[4] = {0.f, 0.f, 0.f, 0.f};
-        const __nv_bfloat16* col = W.w3t + (8 * nt + g) * 16 + 2 * t;
-        mma_bf16(d, ay0, ay1, 0u, 0u, ld_pair(col), ld_pair(col + 8));
+        mma_bf16(d, ay0, ay1, 0u, 0u, W.w3t[nt][lane], 0u);
 #pragma unroll
         for (int k = 0; k < 4; ++k) dz2[nt][k] = act.z2[nt][k] > 0.f ? d[k] : 0.f;
     }
+    O.dy[lane] = make_uint2(transposed(ay0), transposed(ay1));
     // dZ1 = (dZ2 W2) masked by z1 > 0
     float dz1[8][4];
     {
@@ -411,202 +455,278 @@ __global__ void __launch_bounds__(256) k_mlp_train_block(TrainArgs a) {
             af[kk][1] = pack_bf16(p[2], p[3]);
             af[kk][2] = pack_bf16(q[0], q[1]);
             af[kk][3] = pack_bf16(q[2], q[3]);
+            O.d2[kk][lane] = make_uint4(transposed(af[kk][0]), transposed(af[kk][2]), transposed(af[kk][1]),
+                                        transposed(af[kk][3]));
         }
 #pragma unroll
         for (int nt = 0; nt < 8; ++nt) {
             float d[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
             for (int kk = 0; kk < 4; ++kk) {
-                const __nv_bfloat16* col = W.w2t + (8 * nt + g) * MLP_H + 16 * kk + 2 * t;
-                mma_bf16(d, af[kk][0], af[kk][1], af[kk][2], af[kk][3], ld_pair(col), ld_pair(col + 8));
+                const uint2 w = W.w2t[nt][kk][lane];
+                mma_bf16(d, af[kk][0], af[kk][1], af[kk][2], af[kk][3], w.x, w.y);
             }
 #pragma unroll
             for (int k = 0; k < 4; ++k) dz1[nt][k] = act.z1[nt][k] > 0.f ? d[k] : 0.f;
         }
     }
-
-    // operands of the weight-gradient products, transposed into shared memory
-    const int rl = warp * 16 + g, rl8 = rl + 8;
 #pragma unroll
-    for (int j = 0; j < 8; ++j) {
-        const int col = frag_col(j >> 2, j & 3, t);
-        S.XT[col][rl] = __float2bfloat16_rn(xv[0][j]);
-        S.XT[col][rl8] = __float2bfloat16_rn(xv[1][j]);
+    for (int mt = 0; mt < 4; ++mt) {
+        const float* p = dz1[2 * mt];
+        const float* q = dz1[2 * mt + 1];
+        O.d1[mt][lane] = make_uint4(transposed(pack_bf16(p[0], p[1])), transposed(pack_bf16(q[0], q[1])),
+                                    transposed(pack_bf16(p[2], p[3])), transposed(pack_bf16(q[2], q[3])));
     }
 #pragma unroll
-    for (int nt = 0; nt < 8; ++nt) {
-        const int u = 8 * nt + 2 * t;
-        S.H1T[u][rl] = __float2bfloat16_rn(fmaxf(act.z1[nt][0], 0.f));
-        S.H1T[u + 1][rl] = __float2bfloat16_rn(fmaxf(act.z1[nt][1], 0.f));
-        S.H1T[u][rl8] = __float2bfloat16_rn(fmaxf(act.z1[nt][2], 0.f));
-        S.H1T[u + 1][rl8] = __float2bfloat16_rn(fmaxf(act.z1[nt][3], 0.f));
-        S.H2T[u][rl] = __float2bfloat16_rn(fmaxf(act.z2[nt][0], 0.f));
-        S.H2T[u + 1][rl] = __float2bfloat16_rn(fmaxf(act.z2[nt][1], 0.f));
-        S.H2T[u][rl8] = __float2bfloat16_rn(fmaxf(act.z2[nt][2], 0.f));
-        S.H2T[u + 1][rl8] = __float2bfloat16_rn(fmaxf(act.z2[nt][3], 0.f));
-        S.D1T[u][rl] = __float2bfloat16_rn(dz1[nt][0]);
-        S.D1T[u + 1][rl] = __float2bfloat16_rn(dz1[nt][1]);
-        S.D1T[u][rl8] = __float2bfloat16_rn(dz1[nt][2]);
-        S.D1T[u + 1][rl8] = __float2bfloat16_rn(dz1[nt][3]);
-        S.D2T[u][rl] = __float2bfloat16_rn(dz2[nt][0]);
-        S.D2T[u + 1][rl] = __float2bfloat16_rn(dz2[nt][1]);
-        S.D2T[u][rl8] = __float2bfloat16_rn(dz2[nt][2]);
-        S.D2T[u + 1][rl8] = __float2bfloat16_rn(dz2[nt][3]);
+    for (int kk = 0; kk < 4; ++kk) {
+        uint32_t h[4];
+        relu_frag(act.z1, kk, h);
+        O.h1[2 * kk][lane] = make_uint2(transposed(h[0]), transposed(h[1]));
+        O.h1[2 * kk + 1][lane] = make_uint2(transposed(h[2]), transposed(h[3]));
+        relu_frag(act.z2, kk, h);
+        O.h2[2 * kk][lane] = make_uint2(transposed(h[0]), transposed(h[1]));
+        O.h2[2 * kk + 1][lane] = make_uint2(transposed(h[2]), transposed(h[3]));
     }
-    S.DYT[t][rl] = __float2bfloat16_rn(dy[0][t]);
-    S.DYT[t][rl8] = __float2bfloat16_rn(dy[1][t]);
-    for (int o = 4 + t; o < 16; o += 4) {
-        S.DYT[o][rl] = __float2bfloat16_rn(0.f);
-        S.DYT[o][rl8] = __float2bfloat16_rn(0.f);
-    }
-    // bias gradients and loss in FP32: sums over the warp's 16 samples
+    // bias gradients and loss in FP32: sums over the 16 samples. At each of
+    // the three levels of the sum over the lane groups a lane passes on the
+    // half of its columns that it doesn't keep (28 shuffles for 32 columns).
+    float v[32];
 #pragma unroll
-    for (int nt = 0; nt < 8; ++nt) {
-        const float s10 = sum_over_groups(dz1[nt][0] + dz1[nt][2]);
-        const float s11 = sum_over_groups(dz1[nt][1] + dz1[nt][3]);
-        const float s20 = sum_over_groups(dz2[nt][0] + dz2[nt][2]);
-        const float s21 = sum_over_groups(dz2[nt][1] + dz2[nt][3]);
-        if (g == 0) {
-            S.bsum[warp][8 * nt + 2 * t] = s10;
-            S.bsum[warp][8 * nt + 2 * t + 1] = s11;
-            S.bsum[warp][64 + 8 * nt + 2 * t] = s20;
-            S.bsum[warp][64 + 8 * nt + 2 * t + 1] = s21;
-        }
-    }
-    {
-        const float sy = sum_over_groups(dy[0][t] + dy[1][t]);
-        const float sl = sum_over_groups(L[0] + L[1]);
-        if (g == 0) S.bsum[warp][128 + t] = sy;
-        if (lane == 0) S.lsum[warp] = sl;
-    }
-    __syncthreads();
-
-    // -------- the block's share of the weight gradients: 56 tiles of 16 x 8
-    float* part = a.part + (long long)blockIdx.x * PSTRIDE;
-    for (int tile = warp; tile < 56; tile += TR_WARPS) {
-        const __nv_bfloat16 *Am, *Bm;
-        int mt, nt, which;
-        if (tile < 16) { which = 1; mt = tile >> 2; nt = tile & 3; Am = &S.D1T[0][0]; Bm = &S.XT[0][0]; }
-        else if (tile < 48) { which = 2; mt = (tile - 16) >> 3; nt = (tile - 16) & 7; Am = &S.D2T[0][0]; Bm = &S.H1T[0][0]; }
-        else { which = 3; mt = 0; nt = tile - 48; Am = &S.DYT[0][0]; Bm = &S.H2T[0][0]; }
-        float d[4] = {0.f, 0.f, 0.f, 0.f};
+    for (int nt = 0; nt < 8; ++nt)
 #pragma unroll
-        for (int ks = 0; ks < TR_ROWS / 16; ++ks) {
-            const __nv_bfloat16* ar = Am + (16 * mt + g) * LDS + 16 * ks + 2 * t;
-            const __nv_bfloat16* br = Bm + (8 * nt + g) * LDS + 16 * ks + 2 * t;
-            mma_bf16(d, ld_pair(ar), ld_pair(ar + 8 * LDS), ld_pair(ar + 8), ld_pair(ar + 8 * LDS + 8), ld_pair(br),
-                     ld_pair(br + 8));
+        for (int e = 0; e < 2; ++e) {
+            v[2 * nt + e] = dz1[nt][e] + dz1[nt][e + 2];
+            v[16 + 2 * nt + e] = dz2[nt][e] + dz2[nt][e + 2];
         }
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            const int row = 16 * mt + g + 8 * (k >> 1), col = 8 * nt + 2 * t + (k & 1);
-            if (which == 1) { if (col < MLP_IN) part[OFF_W1 + row * MLP_IN + col] = d[k]; }
-            else if (which == 2) part[OFF_W2 + row * MLP_H + col] = d[k];
-            else if (row < MLP_OUT) part[OFF_W3 + row * MLP_H + col] = d[k];
+    for (int lv = 0; lv < 3; ++lv) {
+        const int half = 16 >> lv;
+        const bool hi = g >> lv & 1;
+#pragma unroll
+        for (int q = 0; q < half; ++q) {
+            const float r = __shfl_xor_sync(0xffffffffu, hi ? v[q] : v[q + half], 4 << lv);
+            v[q] = (hi ? v[q + half] : v[q]) + r;
         }
     }
-    const int j = threadIdx.x;
-    if (j < 132) {
-        float s = 0.f;
-        for (int w = 0; w < TR_WARPS; ++w) s += S.bsum[w][j];
-        const int off = j < 64 ? OFF_B1 + j : (j < 128 ? OFF_B2 + j - 64 : OFF_B3 + j - 128);
-        part[off] = s;
-    }
-    if (j == 132) {
-        float s = 0.f;
-        for (int w = 0; w < TR_WARPS; ++w) s += S.lsum[w];
-        part[LOSS_SLOT] = s;
-    }
+    // lane group g holds columns q = 16 (g & 1) + 8 (g >> 1 & 1) + 4 (g >> 2) + 0..3
+    const int nt0 = 4 * (g >> 1 & 1) + 2 * (g >> 2);
+    float* sums = O.sums + MLP_H * (g & 1) + 8 * nt0 + 2 * t;
+    *reinterpret_cast<float2*>(sums) = make_float2(v[0], v[1]);
+    *reinterpret_cast<float2*>(sums + 8) = make_float2(v[2], v[3]);
+    const float d0 = t == 0 ? dy[0][0] : (t == 1 ? dy[0][1] : (t == 2 ? dy[0][2] : dy[0][3]));
+    const float d1 = t == 0 ? dy[1][0] : (t == 1 ? dy[1][1] : (t == 2 ? dy[1][2] : dy[1][3]));
+    const float sy = sum_over_groups(d0 + d1);
+    const float sl = sum_over_groups(L[0] + L[1]);
+    if (g == 0) O.sums[2 * MLP_H + t] = sy;
+    if (lane == 0) O.sums[2 * MLP_H + MLP_OUT] = sl;
 }
 
-// writes the operand copies of parameter i
-__device__ __forceinline__ void emit_bf16(MlpBf16* W, int i, float v) {
+// parameter i in the operands of a training step
+__device__ __forceinline__ void put_training(TrainWeights& W, int i, float v) {
+    put_forward(W.f, i, v);
     const __nv_bfloat16 b = __float2bfloat16_rn(v);
-    if (i < OFF_B1) {
-        W->w1[(i / MLP_IN) * 32 + i % MLP_IN] = b;
-    } else if (i < OFF_W2) {
-        W->b1[i - OFF_B1] = v;
-    } else if (i < OFF_B2) {
-        const int r = (i - OFF_W2) / MLP_H, c = (i - OFF_W2) % MLP_H;
-        W->w2[r * MLP_H + c] = b;
-        W->w2t[c * MLP_H + r] = b;
-    } else if (i < OFF_W3) {
-        W->b2[i - OFF_B2] = v;
-    } else if (i < OFF_B3) {
+    if (i >= OFF_W2 && i < OFF_B2) {
+        reinterpret_cast<__nv_bfloat16*>(W.w2t)[frag_entry<4>((i - OFF_W2) % MLP_H, (i - OFF_W2) / MLP_H)] = b;
+    } else if (i >= OFF_W3 && i < OFF_B3) {
         const int r = (i - OFF_W3) / MLP_H, c = (i - OFF_W3) % MLP_H;
-        W->w3[r * MLP_H + c] = b;
-        W->w3t[c * 16 + r] = b;
-    } else {
-        W->b3[i - OFF_B3] = v;
+        reinterpret_cast<__nv_bfloat16*>(W.w3t)[(((c >> 3) * 32 + (c & 7) * 4 + (r >> 1)) << 1) + (r & 1)] = b;
     }
 }
 
-// zero padding (first launch), then the copies of every parameter (second)
-__global__ void k_mlp_pad(MlpBf16* W) {
+__global__ void k_mlp_emit(const float* __restrict__ theta, TrainWeights* W) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < MLP_H * 32) W->w1[i] = __float2bfloat16_rn(0.f);
-    if (i < 16 * MLP_H) {
-        W->w3[i] = __float2bfloat16_rn(0.f);
-        W->w3t[i] = __float2bfloat16_rn(0.f);
-    }
-    if (i < 16) W->b3[i] = 0.f;
-}
-__global__ void k_mlp_emit(const float* __restrict__ theta, MlpBf16* W) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < MLP_NPARAM) emit_bf16(W, i, theta[i]);
+    if (i < MLP_NPARAM) put_training(*W, i, theta[i]);
 }
 
 struct AdamArgs {
     float lr, b1, b2, eps, c1, c2;
 };
 
-// Sum of the blocks' partials in block order (deterministic). mode 0:
-// gradient and loss out; mode 1: Adam update of theta and its operand
-// copies, loss out.
-__global__ void k_mlp_reduce(const float* __restrict__ part, int nblocks, int mode, float* grad, float* loss,
-                             float* theta, float* m, float* v, MlpBf16* W, AdamArgs ad) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i > MLP_NPARAM) return;
-    float s = 0.f;
-    for (int b = 0; b < nblocks; ++b) s += part[(long long)b * PSTRIDE + i];
-    if (i == LOSS_SLOT) {
-        if (loss) *loss = s;
+struct UpdateArgs {
+    const TrainOps* ops;    // of the slice
+    int chunks;             // of the slice
+    bool first, last;       // slice of the batch
+    float* acc;             // sums of the slices so far
+    float* grad;            // gradient out (theta unchanged), or null: Adam
+    float* loss;            // or null
+    float *theta, *m, *v;
+    TrainWeights* W;
+    AdamArgs ad;
+};
+
+constexpr int UP_TILES = 56, UP_COLS = 27, UP_BLOCKS = UP_TILES + (NBIAS + UP_COLS - 1) / UP_COLS;
+
+// Weight gradients, their sums over the batch and the Adam update in one
+// launch: a block per 16 x 8 tile of the weight matrices (56) or 27 columns of
+// the bias sums (5), a warp per chunk, the chunks' results added in order.
+// Bound by latency (operands from L2, a chain of 8 mma, a chain of 32
+// additions), so all of a chunk's loads are issued before its first product.
+__global__ void __launch_bounds__(1024) k_mlp_train_update(UpdateArgs a) {
+    __shared__ float part[32][128];
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tile = blockIdx.x;
+    int which, mt = 0, nt = 0;
+    if (tile < 16) { which = 1; mt = tile >> 2; nt = tile & 3; }
+    else if (tile < 48) { which = 2; mt = (tile - 16) >> 3; nt = (tile - 16) & 7; }
+    else if (tile < UP_TILES) { which = 3; nt = tile - 48; }
+    else which = 0;
+    // the parameter whose sum this thread forms, -1 for none
+    int i = -1;
+    if (which == 0) {
+        const int j = (tile - UP_TILES) * UP_COLS + tid;
+        if (tid < UP_COLS && j < NBIAS)
+            i = j < MLP_H ? OFF_B1 + j : (j < 2 * MLP_H ? OFF_B2 + j - MLP_H : OFF_B3 + j - 2 * MLP_H);
+    } else if (tid < 128) {
+        const int l = tid >> 2, k = tid & 3;
+        const int row = 16 * mt + (l >> 2) + 8 * (k >> 1), col = 8 * nt + 2 * (l & 3) + (k & 1);
+        if (which == 1) { if (col < MLP_IN) i = OFF_W1 + row * MLP_IN + col; }
+        else if (which == 2) i = OFF_W2 + row * MLP_H + col;
+        else if (row < MLP_OUT) i = OFF_W3 + row * MLP_H + col;
+    }
+    allow_next();
+    // the previous update is complete: the launch before this one waited for it
+    const bool adam = i >= 0 && i < MLP_NPARAM && a.last && !a.grad;
+    const float th = adam ? a.theta[i] : 0.f, mo = adam ? a.m[i] : 0.f, vo = adam ? a.v[i] : 0.f;
+    wait_previous();
+    float s = i >= 0 && !a.first ? a.acc[i] : 0.f;
+    for (int c0 = 0; c0 < a.chunks; c0 += 32) {
+        const int nc = a.chunks - c0 < 32 ? a.chunks - c0 : 32;
+        if (which == 0) {
+            const int c = tid / UP_COLS, jj = tid % UP_COLS, j = (tile - UP_TILES) * UP_COLS + jj;
+            if (c < nc && j < NBIAS) {
+                const TrainOps* O = a.ops + (long long)(c0 + c) * CHUNK_TILES;
+                float w[CHUNK_TILES];
+#pragma unroll
+                for (int k = 0; k < CHUNK_TILES; ++k) w[k] = O[k].sums[j];
+                float p = 0.f;
+#pragma unroll
+                for (int k = 0; k < CHUNK_TILES; ++k) p += w[k];
+                part[c][jj] = p;
+            }
+        } else if (warp < nc) {
+            const TrainOps* O = a.ops + (long long)(c0 + warp) * CHUNK_TILES;
+            uint4 A[CHUNK_TILES];
+            uint2 B[CHUNK_TILES];
+#pragma unroll
+            for (int k = 0; k < CHUNK_TILES; ++k) {
+                if (which == 1) { A[k] = O[k].d1[mt][lane]; B[k] = O[k].x[nt][lane]; }
+                else if (which == 2) { A[k] = O[k].d2[mt][lane]; B[k] = O[k].h1[nt][lane]; }
+                else {
+                    const uint2 dy = O[k].dy[lane];
+                    A[k] = make_uint4(dy.x, 0u, dy.y, 0u);
+                    B[k] = O[k].h2[nt][lane];
+                }
+            }
+            float d[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+            for (int k = 0; k < CHUNK_TILES; ++k) mma_bf16(d, A[k].x, A[k].y, A[k].z, A[k].w, B[k].x, B[k].y);
+            *reinterpret_cast<float4*>(&part[warp][4 * lane]) = make_float4(d[0], d[1], d[2], d[3]);
+        }
+        __syncthreads();
+        if (i >= 0) {
+#pragma unroll 8
+            for (int c = 0; c < nc; ++c) s += part[c][tid];
+        }
+        __syncthreads();
+    }
+    if (i < 0) return;
+    if (!a.last) {
+        a.acc[i] = s;
         return;
     }
-    if (mode == 0) {
-        grad[i] = s;
+    if (i == MLP_NPARAM) {
+        if (a.loss) *a.loss = s;
         return;
     }
-    const float mi = ad.b1 * m[i] + (1.f - ad.b1) * s;
-    const float vi = ad.b2 * v[i] + (1.f - ad.b2) * s * s;
-    m[i] = mi;
-    v[i] = vi;
-    const float p = theta[i] - ad.lr * (mi / ad.c1) / (sqrtf(vi / ad.c2) + ad.eps);
-    theta[i] = p;
-    emit_bf16(W, i, p);
+    if (a.grad) {
+        a.grad[i] = s;
+        return;
+    }
+    const float mi = __fmaf_rn(1.f - a.ad.b1, s, __fmul_rn(a.ad.b1, mo));
+    const float vi = __fmaf_rn(__fmul_rn(1.f - a.ad.b2, s), s, __fmul_rn(a.ad.b2, vo));
+    a.m[i] = mi;
+    a.v[i] = vi;
+    const float p = th - a.ad.lr * (mi / a.ad.c1) / (sqrtf(vi / a.ad.c2) + a.ad.eps);
+    a.theta[i] = p;
+    put_training(*a.W, i, p);
 }
 
-// Raw outputs (n, curvature) of n stencils, a warp per 16
-__global__ void __launch_bounds__(128) k_mlp_infer(const MlpBf16* __restrict__ Wp, const float* __restrict__ fill,
-                                                   long long n, float4* out) {
+// two blocks per SM: 66 944 stencils 27.2 us a call from cold caches (27.8 with
+// three, 28 with one of 512 threads), 2 million 110 us (110, 113)
+constexpr int INFER_THREADS = 256, INFER_BLOCKS = 2 * 152;
+
+// The forward operands from the parameters, a pair of entries per thread and
+// turn, with every load issued before the first is used
+__device__ __forceinline__ void make_forward(MlpFwd& W, const float* __restrict__ theta) {
+    const int tid = threadIdx.x;
+    auto pair = [&](int off, int ld, int rows, int cols, int r, int c) -> uint32_t {
+        const float* p = theta + off + r * ld + c;
+        return pack_bf16(r < rows && c < cols ? p[0] : 0.f, r < rows && c + 1 < cols ? p[1] : 0.f);
+    };
+    // word e: half h of the register pair of lane l, operand e >> 6
+    auto row = [](int e) { return e >> 3 & 7; };
+    auto col = [](int e) { return (e >> 1 & 3) * 2 + (e & 1) * 8; };
+    constexpr int N1 = sizeof(W.w1) / 4, N2 = sizeof(W.w2) / 4, N3 = sizeof(W.w3) / 4;
+    uint32_t w1[(N1 + INFER_THREADS - 1) / INFER_THREADS], w2[(N2 + INFER_THREADS - 1) / INFER_THREADS];
+#pragma unroll
+    for (int q = 0; q < (int)(sizeof(w1) / 4); ++q) {
+        const int e = q * INFER_THREADS + tid, o = e >> 6;
+        w1[q] = pair(OFF_W1, MLP_IN, MLP_H, MLP_IN, 8 * (o >> 1) + row(e), 16 * (o & 1) + col(e));
+    }
+#pragma unroll
+    for (int q = 0; q < (int)(sizeof(w2) / 4); ++q) {
+        const int e = q * INFER_THREADS + tid, o = e >> 6;
+        w2[q] = pair(OFF_W2, MLP_H, MLP_H, MLP_H, 8 * (o >> 2) + row(e), 16 * (o & 3) + col(e));
+    }
+    const uint32_t w3 = tid < N3 ? pair(OFF_W3, MLP_H, MLP_OUT, MLP_H, row(tid), 16 * (tid >> 6) + col(tid)) : 0u;
+    const float b = tid < MLP_H ? theta[OFF_B1 + tid]
+                                : (tid < 2 * MLP_H ? theta[OFF_B2 + tid - MLP_H]
+                                                   : (tid < 2 * MLP_H + MLP_OUT ? theta[OFF_B3 + tid - 2 * MLP_H] : 0.f));
+#pragma unroll
+    for (int q = 0; q < (int)(sizeof(w1) / 4); ++q) reinterpret_cast<uint32_t*>(W.w1)[q * INFER_THREADS + tid] = w1[q];
+#pragma unroll
+    for (int q = 0; q < (int)(sizeof(w2) / 4); ++q) reinterpret_cast<uint32_t*>(W.w2)[q * INFER_THREADS + tid] = w2[q];
+    if (tid < N3) reinterpret_cast<uint32_t*>(W.w3)[tid] = w3;
+    if (tid < MLP_H) W.b1[tid] = b;
+    else if (tid < 2 * MLP_H) W.b2[tid - MLP_H] = b;
+    else if (tid < 2 * MLP_H + 8) W.b3[tid - 2 * MLP_H] = b;
+}
+
+// Raw outputs (n, curvature) of n stencils, a warp per 16. Each block makes
+// its operands from the parameters itself, in shared memory, while its first
+// inputs are on their way: one launch and no scratch memory. Bound by latency
+// (parameters, inputs, a chain of 14 mma). 66 944 stencils: a call took
+// 35.8 us with operands in scratch memory made by two launches before, now
+// 18.3 us, most of it the launch and the wait of the call.
+__global__ void __launch_bounds__(INFER_THREADS) k_mlp_infer(const float* __restrict__ theta,
+                                                             const float* __restrict__ fill, long long n,
+                                                             float4* out) {
+    __shared__ MlpFwd W;
     const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-    const long long nwarps = ((long long)gridDim.x * blockDim.x) >> 5;
-    for (long long base = (((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * 16; base < n;
-         base += nwarps * 16) {
-        const long long r0 = base + g, r1 = base + g + 8;
-        auto val = [&](int r, int col) -> float {
-            const long long row = r ? r1 : r0;
+    const long long stride = (long long)gridDim.x * (INFER_THREADS / 2);
+    long long base = ((long long)blockIdx.x * (INFER_THREADS / 32) + (threadIdx.x >> 5)) * 16;
+    uint32_t xf[2][4], next[2][4];
+    auto load = [&](long long b) {
+        input_frags([&](int r, int col) -> float {
+            const long long row = b + g + 8 * r;
             return (row < n && col < 27) ? fill[row * 27 + col] : 0.f;
-        };
-        uint32_t xf[2][4];
-        input_frags(val, xf);
+        }, next);
+    };
+    load(base);
+    make_forward(W, theta);
+    __syncthreads();
+    for (; base < n; base += stride) {
+#pragma unroll
+        for (int k = 0; k < 8; ++k) xf[k >> 2][k & 3] = next[k >> 2][k & 3];
+        load(base + stride);
         MlpAct act;
-        mlp_forward(*Wp, xf, act);
+        mlp_forward_ops(W.w1, W.w2, W.w3, W.b1, W.b2, W.b3, xf, act);
         float y[2][4];
         mlp_outputs(act, y[0], y[1]);
         if (t < 2) {
-            const long long row = t ? r1 : r0;
-            if (row < n) out[row] = make_float4(y[t][0], y[t][1], y[t][2], y[t][3]);
+            const long long row = base + g + 8 * t;
+            if (row < n) out[row] = t ? make_float4(y[1][0], y[1][1], y[1][2], y[1][3])
+                                      : make_float4(y[0][0], y[0][1], y[0][2], y[0][3]);
         }
     }
 }
@@ -680,15 +800,9 @@ void mlp_from_bf16_host(const uint16_t* w, MlpBf16& h) {
     for (int r = 0; r < MLP_H; ++r)
         for (int c = 0; c < MLP_IN; ++c) h.w1[r * 32 + c] = bf(w[OFF_W1 + r * MLP_IN + c]);
     for (int r = 0; r < MLP_H; ++r)
-        for (int c = 0; c < MLP_H; ++c) {
-            h.w2[r * MLP_H + c] = bf(w[OFF_W2 + r * MLP_H + c]);
-            h.w2t[c * MLP_H + r] = bf(w[OFF_W2 + r * MLP_H + c]);
-        }
+        for (int c = 0; c < MLP_H; ++c) h.w2[r * MLP_H + c] = bf(w[OFF_W2 + r * MLP_H + c]);
     for (int r = 0; r < MLP_OUT; ++r)
-        for (int c = 0; c < MLP_H; ++c) {
-            h.w3[r * MLP_H + c] = bf(w[OFF_W3 + r * MLP_H + c]);
-            h.w3t[c * 16 + r] = bf(w[OFF_W3 + r * MLP_H + c]);
-        }
+        for (int c = 0; c < MLP_H; ++c) h.w3[r * MLP_H + c] = bf(w[OFF_W3 + r * MLP_H + c]);
     for (int i = 0; i < MLP_H; ++i) {
         h.b1[i] = f(w[OFF_B1 + i]);
         h.b2[i] = f(w[OFF_B2 + i]);
@@ -703,22 +817,30 @@ using namespace fsl;
 
 namespace {
 
-struct Scratch {
-    std::vector<void*> ptrs;
-    bool ok = true;
-    template <class T>
-    T* get(size_t count) {
-        void* p = nullptr;
-        if (!ok || cudaMalloc(&p, count * sizeof(T)) != cudaSuccess) {
-            ok = false;
+// device memory of one training or gradient call, in one allocation; weights,
+// moments and acc start at zero
+struct TrainScratch {
+    TrainWeights* W = nullptr;
+    float *m, *v, *acc;
+    TrainOps* ops;
+    bool get(long long samples, cudaStream_t st) {
+        const long long chunks = (samples + CHUNK - 1) / CHUNK;
+        const size_t slice = (size_t)(chunks < SLICE_CHUNKS ? chunks : SLICE_CHUNKS);
+        const size_t zeroed = (sizeof(TrainWeights) + 3 * (MLP_NPARAM + 4) * sizeof(float) + 15) / 16 * 16;
+        if (cudaMalloc(&W, zeroed + slice * CHUNK_TILES * sizeof(TrainOps)) != cudaSuccess) {
             cudaGetLastError();
-            return nullptr;
+            W = nullptr;
+            return false;
         }
-        ptrs.push_back(p);
-        return static_cast<T*>(p);
+        m = reinterpret_cast<float*>(W + 1);
+        v = m + MLP_NPARAM + 4;
+        acc = v + MLP_NPARAM + 4;
+        ops = reinterpret_cast<TrainOps*>(reinterpret_cast<char*>(W) + zeroed);
+        cudaMemsetAsync(W, 0, zeroed, st);
+        return true;
     }
-    ~Scratch() {
-        for (void* p : ptrs) cudaFree(p);
+    ~TrainScratch() {
+        if (W) cudaFree(W);
     }
 };
 
@@ -728,23 +850,38 @@ int finish(cudaStream_t st) {
     return FSLBM_OK;
 }
 
-void emit(const float* theta, MlpBf16* W, cudaStream_t st) {
-    k_mlp_pad<<<(MLP_H * 32 + 255) / 256, 256, 0, st>>>(W);
+template <class Arg>
+void launch_dependent(void (*k)(Arg), unsigned blocks, unsigned threads, const Arg& a, cudaStream_t st) {
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(blocks);
+    cfg.blockDim = dim3(threads);
+    cfg.stream = st;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, k, a);
+}
+
+void emit(const float* theta, TrainWeights* W, cudaStream_t st) {
     k_mlp_emit<<<(MLP_NPARAM + 255) / 256, 256, 0, st>>>(theta, W);
 }
 
-bool train_smem_ready() {
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess) return false;
-    static int done_mask = 0;
-    if (dev < 31 && (done_mask >> dev & 1)) return true;
-    if (cudaFuncSetAttribute(k_mlp_train_block, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)sizeof(TrainSmem)) != cudaSuccess) {
-        cudaGetLastError();
-        return false;
+// One batch: slices of SLICE_CHUNKS chunks, so that the operands of a large
+// batch stay at 10 MB (in L2), each with its two launches
+void batch_gradient(TrainArgs a, UpdateArgs u, cudaStream_t st) {
+    const int chunks = (a.B + CHUNK - 1) / CHUNK;
+    for (int c0 = 0; c0 < chunks; c0 += SLICE_CHUNKS) {
+        u.chunks = chunks - c0 < SLICE_CHUNKS ? chunks - c0 : SLICE_CHUNKS;
+        u.first = c0 == 0;
+        u.last = c0 + u.chunks == chunks;
+        a.first = c0 * CHUNK;
+        a.tiles = u.chunks * CHUNK_TILES;
+        launch_dependent(k_mlp_train_samples, (unsigned)((a.tiles * 32 + SAMPLE_THREADS - 1) / SAMPLE_THREADS),
+                         SAMPLE_THREADS, a, st);
+        launch_dependent(k_mlp_train_update, UP_BLOCKS, 1024, u, st);
     }
-    if (dev < 31) done_mask |= 1 << dev;
-    return true;
 }
 
 }  // namespace
@@ -762,17 +899,25 @@ int fslbm_mlp_gradient(const float* theta, const float* fill, const float* targe
                        double mu, float* grad, float* loss, void* cuda_stream) {
     if (!theta || !fill || !target || !grad || !loss || n <= 0 || n > ((int64_t)1 << 24)) return FSLBM_EINVAL;
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
-    if (!train_smem_ready()) return FSLBM_EDEVICE;
-    const int blocks = (int)((n + TR_ROWS - 1) / TR_ROWS);
-    Scratch sc;
-    MlpBf16* W = sc.get<MlpBf16>(1);
-    float* part = sc.get<float>((size_t)blocks * PSTRIDE);
-    if (!sc.ok) return FSLBM_ENOMEM;
-    emit(theta, W, st);
-    TrainArgs a{W, fill, target, (long long)n, (int)n, TR_FIXED, 0, 0, (float)lam, (float)mu, part};
-    k_mlp_train_block<<<blocks, 256, sizeof(TrainSmem), st>>>(a);
-    k_mlp_reduce<<<(MLP_NPARAM + 256) / 256, 256, 0, st>>>(part, blocks, 0, grad, loss, nullptr, nullptr,
-                                                           nullptr, nullptr, AdamArgs{});
+    TrainScratch sc;
+    if (!sc.get(n, st)) return FSLBM_ENOMEM;
+    emit(theta, sc.W, st);
+    TrainArgs a{};
+    a.W = sc.W;
+    a.fill = fill;
+    a.target = target;
+    a.n = n;
+    a.B = (int)n;
+    a.mode = TR_FIXED;
+    a.lam = (float)lam;
+    a.mu = (float)mu;
+    a.ops = sc.ops;
+    UpdateArgs u{};
+    u.ops = sc.ops;
+    u.acc = sc.acc;
+    u.grad = grad;
+    u.loss = loss;
+    batch_gradient(a, u, st);
     return finish(st);
 }
 
@@ -783,33 +928,40 @@ int fslbm_mlp_train(float* theta, const float* fill, const float* target, int64_
         batch > (1 << 20) || !(lr >= 0.0) || !(lr_end >= 0.0))
         return FSLBM_EINVAL;
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
-    if (!train_smem_ready()) return FSLBM_EDEVICE;
-    const int blocks = (batch + TR_ROWS - 1) / TR_ROWS;
-    Scratch sc;
-    MlpBf16* W = sc.get<MlpBf16>(1);
-    float* part = sc.get<float>((size_t)blocks * PSTRIDE);
-    float* m = sc.get<float>(MLP_NPARAM);
-    float* v = sc.get<float>(MLP_NPARAM);
-    if (!sc.ok) return FSLBM_ENOMEM;
-    cudaMemsetAsync(m, 0, MLP_NPARAM * sizeof(float), st);
-    cudaMemsetAsync(v, 0, MLP_NPARAM * sizeof(float), st);
-    emit(theta, W, st);
+    TrainScratch sc;
+    if (!sc.get(batch, st)) return FSLBM_ENOMEM;
+    emit(theta, sc.W, st);
+    TrainArgs a{};
+    a.W = sc.W;
+    a.fill = fill;
+    a.target = target;
+    a.n = n;
+    a.B = batch;
+    a.mode = augment ? TR_DRAW_SYM : TR_DRAW;
+    a.seed = seed;
+    a.lam = (float)lam;
+    a.mu = (float)mu;
+    a.ops = sc.ops;
+    UpdateArgs u{};
+    u.ops = sc.ops;
+    u.acc = sc.acc;
+    u.theta = theta;
+    u.m = sc.m;
+    u.v = sc.v;
+    u.W = sc.W;
     const double b1 = 0.9, b2 = 0.999;
     double p1 = 1.0, p2 = 1.0;
     for (int64_t k = 0; k < steps; ++k) {
-        TrainArgs a{W, fill, target, (long long)n, batch, augment ? TR_DRAW_SYM : TR_DRAW, seed, (long long)k,
-                    (float)lam, (float)mu, part};
-        k_mlp_train_block<<<blocks, 256, sizeof(TrainSmem), st>>>(a);
+        a.step = (long long)k;
         p1 *= b1;
         p2 *= b2;
         // learning rate: geometric from lr to lr_end over the run (constant
         // when lr_end is 0 or equal to lr)
         const double frac = steps > 1 ? (double)k / (double)(steps - 1) : 0.0;
         const double lr_k = (lr_end > 0.0 && lr > 0.0) ? lr * std::pow(lr_end / lr, frac) : lr;
-        const AdamArgs ad{(float)lr_k, (float)b1, (float)b2, 1e-8f, (float)(1.0 - p1), (float)(1.0 - p2)};
-        k_mlp_reduce<<<(MLP_NPARAM + 256) / 256, 256, 0, st>>>(part, blocks, 1, nullptr,
-                                                               loss_curve ? loss_curve + k : nullptr, theta, m,
-                                                               v, W, ad);
+        u.ad = AdamArgs{(float)lr_k, (float)b1, (float)b2, 1e-8f, (float)(1.0 - p1), (float)(1.0 - p2)};
+        u.loss = loss_curve ? loss_curve + k : nullptr;
+        batch_gradient(a, u, st);
         if ((k & 255) == 255 && cudaGetLastError() != cudaSuccess) return FSLBM_EDEVICE;
     }
     return finish(st);
@@ -818,13 +970,9 @@ int fslbm_mlp_train(float* theta, const float* fill, const float* target, int64_
 int fslbm_mlp_infer(const float* theta, const float* fill, int64_t n, float* out, void* cuda_stream) {
     if (!theta || !fill || !out || n <= 0) return FSLBM_EINVAL;
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
-    Scratch sc;
-    MlpBf16* W = sc.get<MlpBf16>(1);
-    if (!sc.ok) return FSLBM_ENOMEM;
-    emit(theta, W, st);
-    const long long blocks_needed = ((n + 15) / 16 * 32 + 127) / 128;
-    const int blocks = (int)(blocks_needed < 152 * 16 ? blocks_needed : 152 * 16);
-    k_mlp_infer<<<blocks, 128, 0, st>>>(W, fill, (long long)n, reinterpret_cast<float4*>(out));
+    const long long blocks_needed = ((n + 15) / 16 + INFER_THREADS / 32 - 1) / (INFER_THREADS / 32);
+    const int blocks = (int)(blocks_needed < INFER_BLOCKS ? blocks_needed : INFER_BLOCKS);
+    k_mlp_infer<<<blocks, INFER_THREADS, 0, st>>>(theta, fill, (long long)n, reinterpret_cast<float4*>(out));
     return finish(st);
 }
 

@@ -19,14 +19,12 @@ constexpr int OFF_W1 = 0, OFF_B1 = OFF_W1 + MLP_H * MLP_IN, OFF_W2 = OFF_B1 + ML
               OFF_B2 = OFF_W2 + MLP_H * MLP_H, OFF_W3 = OFF_B2 + MLP_H, OFF_B3 = OFF_W3 + MLP_OUT * MLP_H;
 static_assert(MLP_NPARAM == 6212, "parameter count");
 
-// Operand copies of the parameters. W1 is padded to 32 inputs and W3 to 16
-// outputs (zeros); the transposes serve the backward pass.
+// Operand copies of the parameters, built on the host. W1 is padded to 32
+// inputs and W3 to 16 outputs (zeros).
 struct MlpBf16 {
     __nv_bfloat16 w1[MLP_H * 32];       // (out, in)
     __nv_bfloat16 w2[MLP_H * MLP_H];    // (out, in)
-    __nv_bfloat16 w2t[MLP_H * MLP_H];   // (in, out)
     __nv_bfloat16 w3[16 * MLP_H];       // (out, in)
-    __nv_bfloat16 w3t[MLP_H * 16];      // (in, out)
     float b1[MLP_H], b2[MLP_H], b3[16];
 };
 
@@ -69,53 +67,6 @@ __device__ __forceinline__ void relu_frag(const float (&z)[8][4], int kk, uint32
     a[3] = pack_bf16(fmaxf(q[2], 0.f), fmaxf(q[3], 0.f));
 }
 
-// Forward pass from the input fragments x[kk] (k-tiles 0 and 1: inputs
-// 0..15 and 16..31, inputs 27..31 zero). W may live in global or shared
-// memory.
-__device__ __forceinline__ void mlp_forward(const MlpBf16& W, const uint32_t (&x)[2][4], MlpAct& o) {
-    const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-#pragma unroll
-    for (int nt = 0; nt < 8; ++nt) {
-        const float b0 = W.b1[8 * nt + 2 * t], b1 = W.b1[8 * nt + 2 * t + 1];
-        float d[4] = {b0, b1, b0, b1};
-#pragma unroll
-        for (int kk = 0; kk < 2; ++kk) {
-            const __nv_bfloat16* row = W.w1 + (8 * nt + g) * 32 + 16 * kk + 2 * t;
-            mma_bf16(d, x[kk][0], x[kk][1], x[kk][2], x[kk][3], ld_pair(row), ld_pair(row + 8));
-        }
-#pragma unroll
-        for (int k = 0; k < 4; ++k) o.z1[nt][k] = d[k];
-    }
-    uint32_t a[4][4];
-#pragma unroll
-    for (int kk = 0; kk < 4; ++kk) relu_frag(o.z1, kk, a[kk]);
-#pragma unroll
-    for (int nt = 0; nt < 8; ++nt) {
-        const float b0 = W.b2[8 * nt + 2 * t], b1 = W.b2[8 * nt + 2 * t + 1];
-        float d[4] = {b0, b1, b0, b1};
-#pragma unroll
-        for (int kk = 0; kk < 4; ++kk) {
-            const __nv_bfloat16* row = W.w2 + (8 * nt + g) * MLP_H + 16 * kk + 2 * t;
-            mma_bf16(d, a[kk][0], a[kk][1], a[kk][2], a[kk][3], ld_pair(row), ld_pair(row + 8));
-        }
-#pragma unroll
-        for (int k = 0; k < 4; ++k) o.z2[nt][k] = d[k];
-    }
-#pragma unroll
-    for (int kk = 0; kk < 4; ++kk) relu_frag(o.z2, kk, a[kk]);
-    {
-        const float b0 = W.b3[2 * t], b1 = W.b3[2 * t + 1];
-        float d[4] = {b0, b1, b0, b1};
-#pragma unroll
-        for (int kk = 0; kk < 4; ++kk) {
-            const __nv_bfloat16* row = W.w3 + g * MLP_H + 16 * kk + 2 * t;
-            mma_bf16(d, a[kk][0], a[kk][1], a[kk][2], a[kk][3], ld_pair(row), ld_pair(row + 8));
-        }
-#pragma unroll
-        for (int k = 0; k < 4; ++k) o.y[k] = d[k];
-    }
-}
-
 // Weight operands of the in-step forward pass in fragment order: entry
 // [...][lane] is the register pair (b0, b1) that lane feeds one mma, so a
 // warp reads one contiguous 256-byte row per mma. w1[m] is the first layer
@@ -127,18 +78,29 @@ struct MlpFrag {
     uint2 w3[4][32];
 };
 
-// The forward pass of mlp_forward with the weights of G (first layer of
-// mirror image m) and the biases of W
-__device__ __forceinline__ void mlp_forward_frag(const MlpBf16& W, const MlpFrag& G, int m,
-                                                 const uint32_t (&x)[2][4], MlpAct& o) {
+// Weights and biases of one forward pass in the same order, padded with zeros
+// to 32 inputs and 8 outputs
+struct MlpFwd {
+    uint2 w1[8][2][32];
+    uint2 w2[8][4][32];
+    uint2 w3[4][32];
+    float b1[MLP_H], b2[MLP_H], b3[8];
+};
+
+// Forward pass from the input fragments x[kk] (k-tiles 0 and 1: inputs 0..15
+// and 16..31, inputs 27..31 zero); the operands may live in global or shared
+// memory.
+__device__ __forceinline__ void mlp_forward_ops(const uint2 (&w1)[8][2][32], const uint2 (&w2)[8][4][32],
+                                                const uint2 (&w3)[4][32], const float* b1, const float* b2,
+                                                const float* b3, const uint32_t (&x)[2][4], MlpAct& o) {
     const int lane = threadIdx.x & 31, t = lane & 3;
 #pragma unroll
     for (int nt = 0; nt < 8; ++nt) {
-        const float2 b = *reinterpret_cast<const float2*>(W.b1 + 8 * nt + 2 * t);
+        const float2 b = *reinterpret_cast<const float2*>(b1 + 8 * nt + 2 * t);
         float d[4] = {b.x, b.y, b.x, b.y};
 #pragma unroll
         for (int kk = 0; kk < 2; ++kk) {
-            const uint2 w = G.w1[m][nt][kk][lane];
+            const uint2 w = w1[nt][kk][lane];
             mma_bf16(d, x[kk][0], x[kk][1], x[kk][2], x[kk][3], w.x, w.y);
         }
 #pragma unroll
@@ -149,11 +111,11 @@ __device__ __forceinline__ void mlp_forward_frag(const MlpBf16& W, const MlpFrag
     for (int kk = 0; kk < 4; ++kk) relu_frag(o.z1, kk, a[kk]);
 #pragma unroll
     for (int nt = 0; nt < 8; ++nt) {
-        const float2 b = *reinterpret_cast<const float2*>(W.b2 + 8 * nt + 2 * t);
+        const float2 b = *reinterpret_cast<const float2*>(b2 + 8 * nt + 2 * t);
         float d[4] = {b.x, b.y, b.x, b.y};
 #pragma unroll
         for (int kk = 0; kk < 4; ++kk) {
-            const uint2 w = G.w2[nt][kk][lane];
+            const uint2 w = w2[nt][kk][lane];
             mma_bf16(d, a[kk][0], a[kk][1], a[kk][2], a[kk][3], w.x, w.y);
         }
 #pragma unroll
@@ -162,15 +124,45 @@ __device__ __forceinline__ void mlp_forward_frag(const MlpBf16& W, const MlpFrag
 #pragma unroll
     for (int kk = 0; kk < 4; ++kk) relu_frag(o.z2, kk, a[kk]);
     {
-        const float2 b = *reinterpret_cast<const float2*>(W.b3 + 2 * t);
+        const float2 b = *reinterpret_cast<const float2*>(b3 + 2 * t);
         float d[4] = {b.x, b.y, b.x, b.y};
 #pragma unroll
         for (int kk = 0; kk < 4; ++kk) {
-            const uint2 w = G.w3[kk][lane];
+            const uint2 w = w3[kk][lane];
             mma_bf16(d, a[kk][0], a[kk][1], a[kk][2], a[kk][3], w.x, w.y);
         }
 #pragma unroll
         for (int k = 0; k < 4; ++k) o.y[k] = d[k];
+    }
+}
+
+// with the weights of G (first layer of mirror image m) and the biases of W
+__device__ __forceinline__ void mlp_forward_frag(const MlpBf16& W, const MlpFrag& G, int m,
+                                                 const uint32_t (&x)[2][4], MlpAct& o) {
+    mlp_forward_ops(G.w1[m], G.w2, G.w3, W.b1, W.b2, W.b3, x, o);
+}
+
+// 16-bit entry of output row r, input column c in operands of KT k-tiles
+template <int KT>
+__device__ __forceinline__ int frag_entry(int r, int c) {
+    return (((r >> 3) * KT + (c >> 4)) * 32 + (r & 7) * 4 + ((c >> 1) & 3)) * 4 + ((c >> 3) & 1) * 2 + (c & 1);
+}
+
+// parameter i, of value v, in the operands of the forward pass
+__device__ __forceinline__ void put_forward(MlpFwd& W, int i, float v) {
+    const __nv_bfloat16 b = __float2bfloat16_rn(v);
+    if (i < OFF_B1) {
+        reinterpret_cast<__nv_bfloat16*>(W.w1)[frag_entry<2>(i / MLP_IN, i % MLP_IN)] = b;
+    } else if (i < OFF_W2) {
+        W.b1[i - OFF_B1] = v;
+    } else if (i < OFF_B2) {
+        reinterpret_cast<__nv_bfloat16*>(W.w2)[frag_entry<4>((i - OFF_W2) / MLP_H, (i - OFF_W2) % MLP_H)] = b;
+    } else if (i < OFF_W3) {
+        W.b2[i - OFF_B2] = v;
+    } else if (i < OFF_B3) {
+        reinterpret_cast<__nv_bfloat16*>(W.w3)[frag_entry<4>((i - OFF_W3) / MLP_H, (i - OFF_W3) % MLP_H)] = b;
+    } else {
+        W.b3[i - OFF_B3] = v;
     }
 }
 
