@@ -330,12 +330,6 @@ __device__ __forceinline__ uint32_t transposed(uint32_t a) {
     return d;
 }
 
-// programmatic dependent launch: the previous kernel of the stream is complete
-// and its writes are visible after the first; the next one may start after the
-// second
-__device__ __forceinline__ void wait_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void allow_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-
 // Forward and backward pass, a warp per 16 samples, and the operands of the
 // weight gradients. Bound by latency: a warp runs about 2000 instructions one
 // after the other, so there is a warp per scheduler and an SM for every four
@@ -850,20 +844,6 @@ int finish(cudaStream_t st) {
     return FSLBM_OK;
 }
 
-template <class Arg>
-void launch_dependent(void (*k)(Arg), unsigned blocks, unsigned threads, const Arg& a, cudaStream_t st) {
-    cudaLaunchAttribute at{};
-    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at.val.programmaticStreamSerializationAllowed = 1;
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3(blocks);
-    cfg.blockDim = dim3(threads);
-    cfg.stream = st;
-    cfg.attrs = &at;
-    cfg.numAttrs = 1;
-    cudaLaunchKernelEx(&cfg, k, a);
-}
-
 void emit(const float* theta, TrainWeights* W, cudaStream_t st) {
     k_mlp_emit<<<(MLP_NPARAM + 255) / 256, 256, 0, st>>>(theta, W);
 }
@@ -878,9 +858,8 @@ void batch_gradient(TrainArgs a, UpdateArgs u, cudaStream_t st) {
         u.last = c0 + u.chunks == chunks;
         a.first = c0 * CHUNK;
         a.tiles = u.chunks * CHUNK_TILES;
-        launch_dependent(k_mlp_train_samples, (unsigned)((a.tiles * 32 + SAMPLE_THREADS - 1) / SAMPLE_THREADS),
-                         SAMPLE_THREADS, a, st);
-        launch_dependent(k_mlp_train_update, UP_BLOCKS, 1024, u, st);
+        launch_after(k_mlp_train_samples, blocks_for(a.tiles * 32, SAMPLE_THREADS), SAMPLE_THREADS, st, a);
+        launch_after(k_mlp_train_update, UP_BLOCKS, 1024, st, u);
     }
 }
 

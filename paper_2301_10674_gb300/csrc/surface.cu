@@ -57,6 +57,7 @@ __device__ __forceinline__ float4 py_normal(const Dev& s, int c) {
 }
 
 __global__ void k_normals(Dev s, float4* out, const int* list, const int* countp) {
+    after_previous();
     for (int i = blockIdx.x * blockDim.x + threadIdx.x, cnt = min(*countp, s.wl_cap); i < cnt;
          i += gridDim.x * blockDim.x) {
         int c = list[i];
@@ -74,6 +75,7 @@ __global__ void k_normals(Dev s, float4* out, const int* list, const int* countp
 // than 30 degrees away falls back too). out[c] = (n, curvature), curvature 0 where the fallback is
 // taken.
 __global__ void __launch_bounds__(128, 5) k_mlp_normals(Dev s, float4* out, const int* list, const int* countp) {
+    after_previous();
     const int count = min(*countp, s.wl_cap);
     const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
     const int nwarps = (gridDim.x * blockDim.x) >> 5;
@@ -206,8 +208,8 @@ __global__ void __launch_bounds__(128, 5) k_mlp_normals(Dev s, float4* out, cons
 // normals of the cells of a list (the interface list, or the cells that
 // convert in this step)
 static int normals_into(const Dev& s, float4* out, const int* list, const int* count, cudaStream_t st) {
-    if (s.mlp) k_mlp_normals<<<152 * 8, 128, 0, st>>>(s, out, list, count);
-    else k_normals<<<LIST_BLOCKS, LIST_THREADS, 0, st>>>(s, out, list, count);
+    if (s.mlp) launch_after(k_mlp_normals, 152 * 8, 128, st, s, out, list, count);
+    else launch_after(k_normals, LIST_BLOCKS, LIST_THREADS, st, s, out, list, count);
     return 1;
 }
 
@@ -224,6 +226,7 @@ static int normals_into(const Dev& s, float4* out, const int* list, const int* c
 // below -eps, or isolation (no gas neighbour -> liquid, no liquid neighbour
 // -> gas). Clears the counts of the lists that the kernels after it fill.
 __global__ void __launch_bounds__(LIST_THREADS) k_candidates(Dev s) {
+    after_previous();
     if (blockIdx.x == 0 && threadIdx.x == 0)
         *s.cl_count = *s.nl_count = *s.tl_count = *s.dl_count = *s.tile_count = 0;
     FOR_LIST(i, s.wl_count) {
@@ -254,6 +257,7 @@ __global__ void __launch_bounds__(LIST_THREADS) k_candidates(Dev s) {
 // cells that still convert are listed (their normals give the excess-mass
 // weights).
 __global__ void __launch_bounds__(LIST_THREADS) k_conflict(Dev s) {
+    after_previous();
     const int cnt = *s.wl_count, stride = gridDim.x * blockDim.x;
     for (int base = blockIdx.x * blockDim.x; base < cnt; base += stride) {
         const int i = base + threadIdx.x;
@@ -290,6 +294,7 @@ __global__ void __launch_bounds__(LIST_THREADS) k_conflict(Dev s) {
 // neighbours (fill levels and types are still those the candidates saw).
 template <bool FD>
 __global__ void __launch_bounds__(LIST_THREADS) k_mark(Dev s) {
+    after_previous();
     const int lane = threadIdx.x & 31;
     const int ncl = min(*s.cl_count, s.wl_cap);
     FOR_WARP(i, ncl) {
@@ -421,6 +426,7 @@ __device__ __forceinline__ void excess_prep(const Dev& s, int c, int lane) {
 // second read and write that of interface cells only.
 template <typename S, int LP>
 __global__ void __launch_bounds__(LIST_THREADS) k_init_and_prep(Dev s) {
+    after_previous();
     const int lane = threadIdx.x & 31;
     const int nnl = min(*s.nl_count, s.nl_cap), ncl = min(*s.cl_count, s.wl_cap);
     FOR_WARP(i, nnl + ncl) {
@@ -466,6 +472,7 @@ __device__ __forceinline__ float gather_excess(const Dev& s, int c, bool& any) {
 // which nothing here writes, and writes its own mass, fill level and flag.
 // Without a converting cell everything stands as the candidates left it.
 __global__ void __launch_bounds__(LIST_THREADS) k_finish_conversion(Dev s) {
+    after_previous();
     if (*s.cl_count == 0) return;
     FOR_LIST(i, s.wl_count) {
         const int c = s.wl[i];
@@ -636,24 +643,24 @@ int launch_normals(const Dev& s, float4* out, cudaStream_t st) { return normals_
 
 template <typename S>
 static void launch_init_and_prep(const Dev& s, int last_parity, cudaStream_t st) {
-    if (last_parity == 0) k_init_and_prep<S, 0><<<LIST_BLOCKS, LIST_THREADS, 0, st>>>(s);
-    else k_init_and_prep<S, 1><<<LIST_BLOCKS, LIST_THREADS, 0, st>>>(s);
+    if (last_parity == 0) launch_after(k_init_and_prep<S, 0>, LIST_BLOCKS, LIST_THREADS, st, s);
+    else launch_after(k_init_and_prep<S, 1>, LIST_BLOCKS, LIST_THREADS, st, s);
 }
 
 int launch_conversion(const Dev& s, int last_parity, cudaStream_t st) {
     k_candidates<<<LIST_BLOCKS, LIST_THREADS, 0, st>>>(s);
-    k_conflict<<<LIST_BLOCKS, LIST_THREADS, 0, st>>>(s);
+    launch_after(k_conflict, LIST_BLOCKS, LIST_THREADS, st, s);
     // the excess-mass weights need the normals of the converting cells only
     if (s.mlp) {
         normals_into(s, s.nrm1, s.cl, s.cl_count, st);
-        k_mark<false><<<LIST_BLOCKS, LIST_THREADS, 0, st>>>(s);
+        launch_after(k_mark<false>, LIST_BLOCKS, LIST_THREADS, st, s);
     } else {
-        k_mark<true><<<LIST_BLOCKS, LIST_THREADS, 0, st>>>(s);
+        launch_after(k_mark<true>, LIST_BLOCKS, LIST_THREADS, st, s);
     }
     if (s.storage == FSLBM_STORE_FP32) launch_init_and_prep<float>(s, last_parity, st);
     else if (s.storage == FSLBM_STORE_FP16) launch_init_and_prep<__half>(s, last_parity, st);
     else launch_init_and_prep<__nv_bfloat16>(s, last_parity, st);
-    k_finish_conversion<<<LIST_BLOCKS, LIST_THREADS, 0, st>>>(s);
+    launch_after(k_finish_conversion, LIST_BLOCKS, LIST_THREADS, st, s);
     return s.mlp ? 6 : 5;
 }
 
@@ -732,6 +739,7 @@ __device__ __forceinline__ void type_nibbles(unsigned v, unsigned& f, unsigned& 
 
 // (also clears the counts of the lists that the second pass fills)
 __global__ void k_type_bits(Dev s) {
+    after_previous();
     const long long w = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (w == 0) *s.wl_count = *s.sl_count = *s.bseg_count = 0;
     if (w >= (s.n >> 5)) return;
@@ -796,6 +804,7 @@ __device__ __forceinline__ void classify_last(const Dev& s, int spread) {
 }
 
 __global__ void k_classify_bits(Dev s, int spread) {
+    after_previous();
     const long long w = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     const int nxw = s.nx >> 5;                      // words per row
     const long long nw = s.n >> 5;
@@ -852,6 +861,7 @@ __global__ void k_classify_bits(Dev s, int spread) {
 // it, dilated by one cell along x, ANDed with its liquid words) and lists it.
 // Rows at or above zmax_cell hold no such cell (no particle reaches them).
 __global__ void k_bed_segments(Dev s) {
+    after_previous();
     constexpr int WPS = BED_SEG / 32;                // words per segment
     const long long sg = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     const int nxw = s.nx >> 5;
@@ -908,6 +918,7 @@ __global__ void k_bed_segments(Dev s) {
 // Fallback for lattices whose x extent is not a multiple of 32: one thread
 // per cell, 26 neighbour reads for solid cells.
 __global__ void k_classify(Dev s, int spread) {
+    after_previous();
     const long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     const bool in = c < s.n;
     int t = 0;
@@ -960,11 +971,11 @@ void launch_check_invariant(const Dev& s, cudaStream_t st) {
 int launch_classify(const Dev& s, bool spread, cudaStream_t st) {
     int k = 1;
     if (s.nx % 32 == 0) {
-        k_type_bits<<<blocks_for(s.n / 32, 256), 256, 0, st>>>(s);
-        k_classify_bits<<<blocks_for(s.n / 32, 128), 128, 0, st>>>(s, spread);
+        launch_after(k_type_bits, blocks_for(s.n / 32, 256), 256, st, s);
+        launch_after(k_classify_bits, blocks_for(s.n / 32, 128), 128, st, s, spread);
         ++k;
         if (s.links_fused) {
-            k_bed_segments<<<blocks_for((long long)s.nsegx * s.ny * s.nz, 128), 128, 0, st>>>(s);
+            launch_after(k_bed_segments, blocks_for((long long)s.nsegx * s.ny * s.nz, 128), 128, st, s);
             ++k;
         }
     } else {
@@ -997,6 +1008,7 @@ void launch_cell_counts(const Dev& s, unsigned long long* out, cudaStream_t st) 
 // the pool's share joins every interface cell; the conversion codes, left
 // only on the cells k_conflict listed, are cleared
 __global__ void k_pool_spread(Dev s) {
+    after_previous();
     const int ncl = min(*s.cl_count, s.wl_cap);
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < ncl; i += gridDim.x * blockDim.x) s.conv[s.cl[i]] = 0;
     const double share = *s.pool_share;
@@ -1010,7 +1022,7 @@ __global__ void k_pool_spread(Dev s) {
 }
 
 int launch_pool_spread(const Dev& s, cudaStream_t st) {
-    k_pool_spread<<<LIST_BLOCKS, LIST_THREADS, 0, st>>>(s);
+    launch_after(k_pool_spread, LIST_BLOCKS, LIST_THREADS, st, s);
     return 1;
 }
 
