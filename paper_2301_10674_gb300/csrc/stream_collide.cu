@@ -1334,13 +1334,29 @@ __global__ void __launch_bounds__(128, bed_min_blocks<PAR>()) k_liquid_pair_bed(
     }
 }
 
+// directions whose pull source x - c_q lies beyond wall face `bit` of a cell
+__host__ __device__ constexpr unsigned wall_sources(unsigned bit) {
+    unsigned m = 0;
+    for (int q = 0; q < 27; ++q) m |= (wall_bits(-cx(q), -cy(q), -cz(q)) & bit) ? 1u << q : 0u;
+    return m;
+}
+
 // Interface cells, from the interface list: gas-pressure reconstruction
 // (Section 2.1), mass exchange, particle links, collision; the cell's own
-// post-collision PDFs come from and go to the side buffer. Four blocks per
-// SM (128 registers, a few dozen bytes of spills) rather than the two that
-// the compiler's 250 registers leave: the kernel waits on dependent gathers.
-template <typename S, int PAR>
-__global__ void __launch_bounds__(128, 4) k_interface(Dev s) {
+// post-collision PDFs come from and go to the side buffer. Bound by latency: a
+// few thousand cells, each a chain of list entry, types, PDFs and fill levels
+// of the neighbours, collision, stores, and code that most warps run once. So
+// all loads of a link of that chain are issued together, the types are kept as
+// two bit planes, what differs between directions is selected rather than
+// branched to, and the fluid-side links (FUSED) are in an instance of their
+// own. Blocks of 64 spread a short list over more SMs; six a SM leave 168
+// registers a thread. Even / odd step, against a form that branched per direction
+// (blocks of 128, 128 registers): 1 270 cells FP32 24 / 30 -> 7.5 / 8.5 us, 22 000
+// cells FP32 23 / 27 -> 10 / 11 us, 71 000 cells FP16 30 / 34 -> 20 / 24 us (8
+// blocks a SM: 10 / 17 us for the 22 000).
+constexpr int IFC_THREADS = 64, IFC_BLOCKS = 6;
+template <typename S, int PAR, bool FUSED>
+__global__ void __launch_bounds__(IFC_THREADS, IFC_BLOCKS) k_interface(Dev s) {
     const int count = min(*s.wl_count, s.wl_cap);
     const int stride = gridDim.x * blockDim.x;
     for (int base = blockIdx.x * blockDim.x; base < count; base += stride) {
@@ -1350,55 +1366,62 @@ __global__ void __launch_bounds__(128, 4) k_interface(Dev s) {
         int lkey = -1;
         float LF[3] = {0.f, 0.f, 0.f}, LT[3] = {0.f, 0.f, 0.f};
         if (work) {
-            const long long cell = s.wl[i];
-            int x, y, z;
-            coords32(s, (int)cell, x, y, z);
+            const int cell = s.wl[i];
             S* f = static_cast<S*>(s.f);
             S* fs = static_cast<S*>(s.fs);
             const long long n = s.n;
-            const int xs[3] = {shift(x, -1, s.nx, s.per_x), x, shift(x, 1, s.nx, s.per_x)};
-            const int ys[3] = {shift(y, -1, s.ny, s.per_y), y, shift(y, 1, s.ny, s.per_y)};
-            const int zs[3] = {shift(z, -1, s.nz, s.per_z), z, shift(z, 1, s.nz, s.per_z)};
-            unsigned wallm = 0, solidm = 0, gasm = 0, liqm = 0;
+            // stored values of the cell's own post-collision PDFs
+            float fo[27];
 #pragma unroll
-            for (int q = 0; q < 27; ++q) {
-                const int sx = xs[1 - cx(q)], sy = ys[1 - cy(q)], sz = zs[1 - cz(q)];
-                if (sx < 0 || sy < 0 || sz < 0) {
-                    wallm |= 1u << q;
-                } else {
-                    const int ts = s.flags[sx + (long long)s.nx * (sy + (long long)s.ny * sz)] & TYPE_MASK;
-                    if (ts == T_SOL) solidm |= 1u << q;
-                    else if (ts == T_GAS) gasm |= 1u << q;
-                    else if (ts == T_LIQ) liqm |= 1u << q;
-                }
-            }
+            for (int q = 0; q < 27; ++q) fo[q] = Store<S>::ld(fs + q * n + cell);
             const float phix = s.phi[cell];
             const float mx = s.mass[cell];
             const float4 nn = s.nrm[cell];
+            int x, y, z;
+            coords32(s, cell, x, y, z);
+            const NbrOffsets o = nbr_offsets(s, x, y, z);
+            unsigned wallm = 0;
+#pragma unroll
+            for (int k = 0; k < 6; ++k) wallm |= (o.wall >> k & 1u) ? wall_sources(1u << k) : 0u;
+            // the pull source of direction q; the cell itself beyond a wall face
+            auto source = [&](int q) -> int {
+                return (wallm >> q & 1u) ? cell : cell + o.ox[1 - cx(q)] + o.oy[1 - cy(q)] + o.oz[1 - cz(q)];
+            };
+            unsigned lo = 0, hi = 0;   // bits of the sources' types: gas 0, liquid 1, interface 2, solid 3
+#pragma unroll
+            for (int q = 0; q < 27; ++q) {
+                const unsigned ts = s.flags[source(q)];
+                lo |= (ts & 1u) << q;
+                hi |= (ts >> 1 & 1u) << q;
+            }
+            const unsigned solidm = lo & hi & ~wallm, liqm = lo & ~hi & ~wallm, ifcm = hi & ~lo & ~wallm;
+            const unsigned gasm = ~(lo | hi | wallm);
             // 16-bit storage: references of the slots (the cell's own z, the
             // pull source's z - c_z in an odd step, the target's z + c_z); h3[k]
             // that of z + k - 1 (the cell's own beyond a wall face, never used)
             const float hz = Store<S>::HREF ? s.href[z] : 0.f;
             float h3[3] = {hz, hz, hz};
             if (Store<S>::HREF && PAR == 1) {
-                if (zs[0] >= 0) h3[0] = s.href[zs[0]];
-                if (zs[2] >= 0) h3[2] = s.href[zs[2]];
+                const int zm = shift(z, -1, s.nz, s.per_z), zp = shift(z, 1, s.nz, s.per_z);
+                if (zm >= 0) h3[0] = s.href[zm];
+                if (zp >= 0) h3[2] = s.href[zp];
             }
-            float fo[27];
+            float v[27], sc[27];
 #pragma unroll
             for (int q = 0; q < 27; ++q) {
-                fo[q] = Store<S>::ld(fs + (long long)q * n + cell);
-                if (Store<S>::HREF) fo[q] += wq(q) * hz;
+                const bool pull = !((wallm | gasm) >> q & 1u);   // fluid or solid source
+                const S* a = PAR == 0 ? f + q * n + cell : f + opp(q) * n + source(q);
+                v[q] = pull ? Store<S>::ld(a) : 0.f;
             }
-            float v[27];
 #pragma unroll
-            for (int q = 0; q < 27; ++q) {
-                const int sx = xs[1 - cx(q)], sy = ys[1 - cy(q)], sz = zs[1 - cz(q)];
-                const bool pull = !(((wallm | gasm) >> q) & 1u);   // fluid or solid source
-                const long long src = pull ? sx + (long long)s.nx * (sy + (long long)s.ny * sz) : cell;
-                const long long a = PAR == 0 ? (long long)q * n + cell : (long long)opp(q) * n + src;
-                v[q] = pull ? Store<S>::ld(f + a) : 0.f;
-                if (Store<S>::HREF && pull) v[q] += wq(q) * (PAR == 0 ? hz : h3[1 - cz(q)]);
+            for (int q = 0; q < 27; ++q) sc[q] = q == 13 ? phix : ((ifcm >> q & 1u) ? s.phi[source(q)] : 0.f);
+            if (Store<S>::HREF) {
+#pragma unroll
+                for (int q = 0; q < 27; ++q) {
+                    fo[q] += wq(q) * hz;
+                    const bool pull = !((wallm | gasm) >> q & 1u);
+                    v[q] = pull ? v[q] + wq(q) * (PAR == 0 ? hz : h3[1 - cz(q)]) : v[q];
+                }
             }
             // own collision velocity from the post-collision PDFs
             float d = 0.f, jx = 0.f, jy = 0.f, jz = 0.f;
@@ -1418,92 +1441,88 @@ __global__ void __launch_bounds__(128, 4) k_interface(Dev s) {
             // kappa the curvature that came with the cell's normal (0 where
             // the finite-difference normal was taken)
             const float rhoG = s.rho_gas + 6.f * s.sigma * nn.w;
+            // fluid sources: mass exchange with the pulled post-collision PDF
             float dm = 0.f;
 #pragma unroll
             for (int q = 0; q < 27; ++q) {
-                const float fob = fo[opp(q)];
-                if ((wallm >> q) & 1u) {
-                    v[q] = fob;
-                    continue;
-                }
-                const int sx = xs[1 - cx(q)], sy = ys[1 - cy(q)], sz = zs[1 - cz(q)];
-                const long long src = sx + (long long)s.nx * (sy + (long long)s.ny * sz);
-                // solid source: the pulled value is the bounce-back value,
-                // placed by the link pass, or formed here from the cell's own
-                // f*_opp(q) (its side-buffer copy) with the momentum exchange
-                // summed per run of equal owner
-                if ((solidm >> q) & 1u) {
-                    if (s.links_fused) {
-                        const int p = s.owner[src];
-                        if (p < 0 || p >= s.np) {
-                            set_error(s, ERR_INVARIANT);
-                            continue;
-                        }
-                        if (p != lkey) {
-                            if (lkey >= 0) flush_direct(s, lkey, LF, LT);
-                            lkey = p;
+                const float e = (liqm >> q & 1u) ? 1.f : 0.5f * (phix + sc[q]);
+                const float t = __fmaf_rn(e, v[q] - fo[opp(q)], dm);
+                dm = ((liqm | ifcm) >> q & 1u) ? t : dm;
+            }
+            // solid sources: the pulled value is the bounce-back value, placed by
+            // the link pass, or formed here from the cell's own f*_opp(q) (its
+            // side-buffer copy) with the momentum exchange summed per run of
+            // equal owner
+            if constexpr (FUSED) {
 #pragma unroll
-                            for (int c = 0; c < 3; ++c) LF[c] = LT[c] = 0.f;
-                        }
-                        const PData P = particle_data(s, p);
-                        const float dx = (float)wrap_int(x - P.xi.x, s.nx, s.per_x) + 0.5f - P.xf.x - 0.5f * cx(q);
-                        const float dy = (float)wrap_int(y - P.xi.y, s.ny, s.per_y) + 0.5f - P.xf.y - 0.5f * cy(q);
-                        const float dz = (float)wrap_int(z - P.xi.z, s.nz, s.per_z) + 0.5f - P.xf.z - 0.5f * cz(q);
-                        const float ubx = P.u.x + (P.w.y * dz - P.w.z * dy);
-                        const float uby = P.u.y + (P.w.z * dx - P.w.x * dz);
-                        const float ubz = P.u.z + (P.w.x * dy - P.w.y * dx);
-                        const float corr = 6.f * wq(q) * (cx(q) * ubx + cy(q) * uby + cz(q) * ubz);
-                        v[q] = fob + corr;
-                        const float sum = fob + v[q];
-                        const float Fx = -cx(q) * sum + ubx * corr;
-                        const float Fy = -cy(q) * sum + uby * corr;
-                        const float Fz = -cz(q) * sum + ubz * corr;
-                        LF[0] += Fx; LF[1] += Fy; LF[2] += Fz;
-                        LT[0] += dy * Fz - dz * Fy;
-                        LT[1] += dz * Fx - dx * Fz;
-                        LT[2] += dx * Fy - dy * Fx;
+                for (int q = 0; q < 27; ++q) {
+                    if (!(solidm >> q & 1u)) continue;
+                    const float fob = fo[opp(q)];
+                    const int p = s.owner[source(q)];
+                    if (p < 0 || p >= s.np) {
+                        set_error(s, ERR_INVARIANT);
+                        continue;
                     }
-                    continue;
+                    if (p != lkey) {
+                        if (lkey >= 0) flush_direct(s, lkey, LF, LT);
+                        lkey = p;
+#pragma unroll
+                        for (int c = 0; c < 3; ++c) LF[c] = LT[c] = 0.f;
+                    }
+                    const PData P = particle_data(s, p);
+                    const float dx = (float)wrap_int(x - P.xi.x, s.nx, s.per_x) + 0.5f - P.xf.x - 0.5f * cx(q);
+                    const float dy = (float)wrap_int(y - P.xi.y, s.ny, s.per_y) + 0.5f - P.xf.y - 0.5f * cy(q);
+                    const float dz = (float)wrap_int(z - P.xi.z, s.nz, s.per_z) + 0.5f - P.xf.z - 0.5f * cz(q);
+                    const float ubx = P.u.x + (P.w.y * dz - P.w.z * dy);
+                    const float uby = P.u.y + (P.w.z * dx - P.w.x * dz);
+                    const float ubz = P.u.z + (P.w.x * dy - P.w.y * dx);
+                    const float corr = 6.f * wq(q) * (cx(q) * ubx + cy(q) * uby + cz(q) * ubz);
+                    v[q] = fob + corr;
+                    const float sum = fob + v[q];
+                    const float Fx = -cx(q) * sum + ubx * corr;
+                    const float Fy = -cy(q) * sum + uby * corr;
+                    const float Fz = -cz(q) * sum + ubz * corr;
+                    LF[0] += Fx; LF[1] += Fy; LF[2] += Fz;
+                    LT[0] += dy * Fz - dz * Fy;
+                    LT[1] += dz * Fx - dx * Fz;
+                    LT[2] += dx * Fy - dy * Fx;
                 }
-                const bool gas = (gasm >> q) & 1u;
-                if (!gas) {
-                    // fluid source: mass exchange with the pulled post-collision PDF
-                    const bool liq = (liqm >> q) & 1u;
-                    const float sc = liq ? 1.f : 0.5f * (phix + s.phi[src]);
-                    dm += sc * (v[q] - fob);
-                }
-                bool rebuild = gas;
-                if (!rebuild && s.recon_normal) rebuild = (nn.x * cx(q) + nn.y * cy(q) + nn.z * cz(q)) < -s.eps_normal;
-                if (rebuild) {
-                    const float cu = cx(q) * urx + cy(q) * ury + cz(q) * urz;
-                    v[q] = wq(q) * (2.f * (rhoG - 1.f) + rhoG * (9.f * cu * cu - 3.f * uur)) - fob;
-                }
+            }
+            // gas sources, and with recon_normal every source on the gas side of
+            // the surface, are rebuilt; beyond a wall face the value bounces back
+#pragma unroll
+            for (int q = 0; q < 27; ++q) {
+                const float fob = fo[opp(q)];
+                bool rebuild = gasm >> q & 1u;
+                if (s.recon_normal)
+                    rebuild = rebuild || (((liqm | ifcm) >> q & 1u) &&
+                                          (nn.x * cx(q) + nn.y * cy(q) + nn.z * cz(q)) < -s.eps_normal);
+                const float cu = cx(q) * urx + cy(q) * ury + cz(q) * urz;
+                const float r = wq(q) * (2.f * (rhoG - 1.f) + rhoG * (9.f * cu * cu - 3.f * uur)) - fob;
+                v[q] = (wallm >> q & 1u) ? fob : (rebuild ? r : v[q]);
             }
             float rho, ux, uy, uz;
             collide_scaled(v, 1.f, s.omega, s.gx, s.gy, s.gz, rho, ux, uy, uz, s.galilean != 0);
-            if (PAR == 0) {
 #pragma unroll
-                for (int q = 0; q < 27; ++q)
-                    Store<S>::st(f + (long long)opp(q) * n + cell, Store<S>::HREF ? v[q] - wq(q) * hz : v[q]);
-            } else {
-#pragma unroll
-                for (int q = 0; q < 27; ++q) {
-                    const int tx = xs[1 + cx(q)], ty = ys[1 + cy(q)], tz = zs[1 + cz(q)];
-                    const bool out = tx < 0 || ty < 0 || tz < 0;
-                    const long long a = out ? (long long)opp(q) * n + cell
-                                            : (long long)q * n + tx + (long long)s.nx * (ty + (long long)s.ny * tz);
-                    Store<S>::st(f + a, Store<S>::HREF ? v[q] - wq(q) * (out ? hz : h3[1 + cz(q)]) : v[q]);
+            for (int q = 0; q < 27; ++q) {
+                if (PAR == 0) {
+                    Store<S>::st(f + opp(q) * n + cell, Store<S>::HREF ? v[q] - wq(q) * hz : v[q]);
+                } else {
+                    // x + c_q is the pull source of direction opp(q)
+                    const bool out = wallm >> opp(q) & 1u;
+                    Store<S>::st(f + (out ? opp(q) : q) * n + source(opp(q)),
+                                 Store<S>::HREF ? v[q] - wq(q) * (out ? hz : h3[1 + cz(q)]) : v[q]);
                 }
             }
 #pragma unroll
             for (int q = 0; q < 27; ++q)
-                Store<S>::st(fs + (long long)q * n + cell, Store<S>::HREF ? v[q] - wq(q) * hz : v[q]);
+                Store<S>::st(fs + q * n + cell, Store<S>::HREF ? v[q] - wq(q) * hz : v[q]);
             // phi = m / rho is refreshed after the sweep: neighbours read the
             // old phi in their mass exchange
             s.mass[cell] = mx + dm;
             s.ru[cell] = make_float4(rho, ux, uy, uz);
         }
-        flush_mem(s, lkey, LF, LT);
+        if constexpr (FUSED) flush_mem(s, lkey, LF, LT);
     }
 }
 
@@ -1598,9 +1617,14 @@ static int bed_blocks() {
     return blocks;
 }
 
+template <typename S, int PAR>
+static void launch_interface(const Dev& s, cudaStream_t st) {
+    if (s.np > 0 && s.links_fused) k_interface<S, PAR, true><<<152 * IFC_BLOCKS, IFC_THREADS, 0, st>>>(s);
+    else k_interface<S, PAR, false><<<152 * IFC_BLOCKS, IFC_THREADS, 0, st>>>(s);
+}
+
 template <typename S>
 static void launch_typed(const Dev& s, int parity, cudaStream_t st, cudaEvent_t links_done) {
-    const int lb = 152 * 8;
     // the particle forces are complete after the link pass, or with fluid-side
     // links after the whole sweep
     const bool early = s.np > 0 && !s.links_fused;
@@ -1625,7 +1649,7 @@ static void launch_typed(const Dev& s, int parity, cudaStream_t st, cudaEvent_t 
             k_liquid<S, 0><<<lgrid, 256, 0, st>>>(s);
         }
         if (s.np > 0 && s.links_fused) k_liquid_pair_bed<S, 0><<<bed_blocks<S, 0>(), 128, 0, st>>>(s);
-        k_interface<S, 0><<<lb, 128, 0, st>>>(s);
+        launch_interface<S, 0>(s, st);
     } else {
         if (s.np > 0 && !s.links_fused) {
             launch_links<S, 1>(s, st);
@@ -1642,7 +1666,7 @@ static void launch_typed(const Dev& s, int parity, cudaStream_t st, cudaEvent_t 
             k_liquid<S, 1><<<lgrid, 256, 0, st>>>(s);
         }
         if (s.np > 0 && s.links_fused) k_liquid_pair_bed<S, 1><<<bed_blocks<S, 1>(), 128, 0, st>>>(s);
-        k_interface<S, 1><<<lb, 128, 0, st>>>(s);
+        launch_interface<S, 1>(s, st);
     }
     if (!early && links_done) cudaEventRecord(links_done, st);
 }

@@ -38,6 +38,7 @@ def _device(sim, mask, fields, offset=0):
     import torch
     host = [sim._alloc(f) for f in fields]
     raw = [torch.zeros(h.nbytes + 16, dtype=torch.uint8, device="cuda") for h in host]
+    torch.cuda.synchronize()             # the buffers' zeroing, on another stream than the run's
     F._check(F.fslbm_get_fields(sim.h, mask, [int(r.data_ptr()) + offset for r in raw], on_device=True), "get")
     return [r.cpu().numpy()[offset:offset + h.nbytes].view(h.dtype).reshape(h.shape) for r, h in zip(raw, host)]
 
