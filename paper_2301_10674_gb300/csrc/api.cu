@@ -368,7 +368,7 @@ int fslbm_create(const fslbm_params* p, void* cuda_stream, fslbm** out) {
             d.bseg_count = counts + 9;
             d.cl_count = counts + 10;
             d.rtail_count = counts + 11;
-            d.g_tot = counts + 16;   // one word per CTA of the DEM cluster (8)
+            d.g_tot = counts + 16;   // one word per CTA of the DEM cluster (up to 16)
         }
         dd = dalloc<double>(s, 4, ok);
         if (ok) {

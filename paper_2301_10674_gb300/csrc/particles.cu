@@ -620,13 +620,15 @@ __global__ void __launch_bounds__(128) k_dem_substep(Dev s, int a, int have_prev
 // constants in registers for the whole step, and reads its partners' published
 // values from the shared memory of the CTA that owns them: with all of it in
 // global memory a sub-step waited for six L2 latencies in turn. The whole DEM
-// half (ten sub-steps and the grid) takes 40 us for 34 particles (54 us with the
-// lists in global memory), 78 us for 1 008 (114 us with 512 threads and two
-// particles per group, whose fewer warps left each waiting for its own
-// arithmetic; 1 024 threads at 64 registers), against ten launches of 9 us plus
-// three of the grid.
-constexpr int DEM_CLUSTER_MAX = 1024;
-constexpr int DEM_CLUSTER_CTAS = 8;
+// half (ten sub-steps and the grid) took 40 us for 34 particles (54 us with the
+// lists in global memory) and 78 us for 1 008 in eight CTAs of 1 024 threads
+// (114 us with 512 threads and two particles per group, whose fewer warps left
+// each waiting for its own arithmetic), against ten launches of 9 us plus three
+// of the grid. 16 CTAs leave a scheduler half the warps: 301x37x75 flume, step
+// 0.1465 -> 0.137 ms; 768x40x96 (1 500 particles, separate launches before) 0.226
+// -> 0.2195 ms.
+constexpr int DEM_CLUSTER_CTAS = 16;       // where the device can place a cluster of 16, else 8
+constexpr int DEM_CLUSTER_MAX = DEM_CLUSTER_CTAS * 1024 / DEM_LANES;
 
 __device__ __forceinline__ void cluster_barrier() {
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
@@ -1325,22 +1327,59 @@ int launch_dem_neighbours(const Dev& s, cudaStream_t st) {
     return 1;
 }
 
+static size_t dem_cluster_smem(int threads) {
+    return (size_t)(threads / DEM_LANES) * (sizeof(ClusterParticle) + DEM_SH * sizeof(float));
+}
+template <class K>
+static void dem_cluster_attributes(K* kernel, int smem) {
+    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+}
+// the largest cluster that this device places with 1024 threads a CTA, found
+// once (a cluster of 16 needs as many SMs of one group)
+static int dem_cluster_ctas() {
+    static const int ctas = [] {
+        cudaLaunchConfig_t cfg = {};
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = DEM_CLUSTER_CTAS;
+        at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+        cfg.gridDim = dim3(DEM_CLUSTER_CTAS);
+        cfg.blockDim = dim3(1024);
+        cfg.dynamicSmemBytes = dem_cluster_smem(1024);
+        cfg.attrs = at;
+        cfg.numAttrs = 1;
+        dem_cluster_attributes(k_dem_cluster<1024>, (int)cfg.dynamicSmemBytes);
+        int clusters = 0;
+        if (cudaOccupancyMaxActiveClusters(&clusters, k_dem_cluster<1024>, &cfg) != cudaSuccess) {
+            cudaGetLastError();
+            clusters = 0;
+        }
+        return clusters > 0 ? DEM_CLUSTER_CTAS : 8;
+    }();
+    return ctas;
+}
+
 int launch_dem(const Dev& s, int have_prev, cudaStream_t st) {
     if (s.np == 0) return 0;
     const int ns = s.dem_substeps, G = s.gnx * s.gny * s.gnz;
     const float dts = 1.f / (float)ns;
-    if (s.np <= DEM_CLUSTER_MAX) {
-        // one particle per lane group, in as many CTAs (a power of two) as
-        // leave one warp per scheduler
+    const int max_ctas = s.np <= DEM_CLUSTER_MAX ? dem_cluster_ctas() : 0;
+    if (s.np <= max_ctas * 1024 / DEM_LANES) {
+        // one particle per lane group. Up to 64 particles in one CTA, whose
+        // partners' values are its own (34 particles: step of the 64x16x32
+        // flume 0.0775 ms, in four CTAs 0.0795); beyond, as many CTAs as leave
+        // each 512 threads, up to the largest cluster (735 particles of the
+        // 301x37x75 flume in 16 CTAs: step 0.137 ms, in 8: 0.1465)
         const int lanes = s.np * DEM_LANES;
         int ctas = 1;
-        while (ctas < DEM_CLUSTER_CTAS && ctas * 128 < lanes) ctas *= 2;
+        while (ctas < max_ctas && ctas * 512 < lanes) ctas *= 2;
         int threads = ((lanes + ctas - 1) / ctas + 31) / 32 * 32;
         threads = threads < 128 ? 128 : threads;
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3((unsigned)ctas);
         cfg.blockDim = dim3((unsigned)threads);
-        cfg.dynamicSmemBytes = threads / DEM_LANES * (sizeof(ClusterParticle) + DEM_SH * sizeof(float));
+        cfg.dynamicSmemBytes = dem_cluster_smem(threads);
         cfg.stream = st;
         cudaLaunchAttribute at[1];
         at[0].id = cudaLaunchAttributeClusterDimension;
@@ -1349,7 +1388,7 @@ int launch_dem(const Dev& s, int have_prev, cudaStream_t st) {
         cfg.attrs = at;
         cfg.numAttrs = 1;
         auto* kernel = threads <= 512 ? k_dem_cluster<512> : k_dem_cluster<1024>;
-        cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cfg.dynamicSmemBytes);
+        dem_cluster_attributes(kernel, (int)cfg.dynamicSmemBytes);
         cudaLaunchKernelEx(&cfg, kernel, s, have_prev, G, dts);
         return 1;
     }

@@ -1,9 +1,9 @@
 """DEM sub-steps and particle grid in one thread-block cluster against the
 separate launches: the same mobile particles settle in a gas-filled box while
 far-away fixed spheres bring the particle count to each side of the cluster
-kernel's sizes (one CTA, several, more than one particle per lane group, and
-beyond its range, where the separate launches run), with ten sub-steps and
-with one."""
+kernel's sizes (one CTA up to 64 particles, several with up to 512 and up to
+1024 threads, and beyond its range, where the separate launches run), with ten
+sub-steps and with one."""
 import numpy as np
 import pytest
 
@@ -46,10 +46,10 @@ def _run(mobile, total, substeps=10):
     return [sim.get(f)[:mobile] for f in z], sim.get(F.FIELD_OWNER)[:30], xyz
 
 
-@pytest.mark.parametrize("mobile,total,substeps", [(1, 1, 10), (5, 33, 10), (300, 512, 10), (300, 513, 10),
-                                                   (300, 1024, 10), (600, 1023, 10), (300, 1000, 1)])
+@pytest.mark.parametrize("mobile,total,substeps", [(1, 1, 10), (5, 33, 10), (40, 64, 10), (40, 65, 10), (300, 513, 10),
+                                                   (300, 1024, 10), (600, 1025, 10), (900, 2048, 10), (300, 1000, 1)])
 def test_cluster_matches_separate_launches(mobile, total, substeps):
-    (xa, ua, wa), oa, start = _run(mobile, 1025 if total > 512 else 8193, substeps)
+    (xa, ua, wa), oa, start = _run(mobile, 2049 if total > 512 else 8193, substeps)
     (xb, ub, wb), ob, _ = _run(mobile, total, substeps)
     assert np.abs(xa - start).max() > 0.1
     if mobile > 5:
