@@ -339,13 +339,14 @@ int fslbm_create(const fslbm_params* p, void* cuda_stream, fslbm** out) {
         if (tcap > n) tcap = n;
         d.tl_cap = (int)tcap;
         d.tl = dalloc<int>(s, tcap, ok);
-        // (with the fill-up to groups of 32 per 4096 cells)
-        const long long scap = std::min(n + 32 * (n / 4096 + 1), (1LL << 31) - 1);
+        // (with the fill-up to groups of 32 per 128 words of a row's cells)
+        const long long twords = (long long)((p->nx + 31) / 32) * p->ny * p->nz;
+        const long long scap = std::min(n + 32 * (twords / 128 + 1), (1LL << 31) - 1);
         d.sl_cap = (int)scap;
         d.sl = dalloc<int>(s, scap, ok);
-        d.fbits = dalloc<unsigned>(s, n / 32 + 1, ok);
-        d.ibits = dalloc<unsigned>(s, n / 32 + 1, ok);
-        d.sbits = dalloc<unsigned>(s, n / 32 + 1, ok);
+        d.fbits = dalloc<unsigned>(s, twords + 1, ok);
+        d.ibits = dalloc<unsigned>(s, twords + 1, ok);
+        d.sbits = dalloc<unsigned>(s, twords + 1, ok);
         d.tw = p->storage != FSLBM_STORE_FP32 && d.idx32 && p->nx % 32 == 0 ? dalloc<unsigned>(s, n / 8 + 1, ok) : nullptr;
         d.tiles = dalloc<int>(s, n / fsl::SP_TILE + 1, ok);
         {
