@@ -16,6 +16,8 @@
 // exchange); the liquid cells (x-adjacent pairs per thread on packed FP32
 // arithmetic; one cell per thread where nx is odd or the lattice needs
 // 64-bit element indices); and the interface cells of the interface list.
+#include <type_traits>
+
 #include "collide_pair.cuh"
 #include "fslbm_dev.cuh"
 
@@ -159,6 +161,13 @@ __global__ void __launch_bounds__(256, liquid_min_blocks<S>()) k_liquid(Dev s) {
 template <typename S, int PAR>
 constexpr int liquid_pair_min_blocks() { return PAR == 0 ? 4 : (sizeof(S) == 2 ? 7 : 5); }
 
+// index type of the pairs on the faces of the lattice: 32 bits at FP32, where
+// they run in the warps of the other pairs (512x40x96: step 0.177 -> 0.174 ms, a
+// 200x72x90 box 0.0875 -> 0.0843);
+// 64 at 16 bits, whose kernel of their own was 0.2% of a step slower with 32
+template <typename S>
+using PairIndex = typename std::conditional<sizeof(S) == 4, unsigned, long long>::type;
+
 // Stream and collide one pair (x even, x + 1) of row `row`; liq: bit 0 cell
 // x liquid, bit 1 cell x + 1 liquid. `interior`: every neighbour of both
 // cells inside the lattice without wrap (always true in an even step, which
@@ -204,15 +213,15 @@ __device__ __forceinline__ void pair_load(const Dev& s, const S* f, int x, int r
         }
     } else {
         const NbrOffsets o0 = nbr_offsets(s, x, y, z), o1 = nbr_offsets(s, x + 1, y, z);
+        const PairIndex<S> n = (PairIndex<S>)s.n;
 #pragma unroll
         for (int q = 0; q < 27; ++q) {
             // source x - c_q beyond a wall face: the cell's own slot (q, x)
             const unsigned wb = wall_bits(-cx(q), -cy(q), -cz(q));
             const int src0 = cell + o0.ox[1 - cx(q)] + o0.oy[1 - cy(q)] + o0.oz[1 - cz(q)];
             const int src1 = cell + 1 + o1.ox[1 - cx(q)] + o1.oy[1 - cy(q)] + o1.oz[1 - cz(q)];
-            const long long a0 = (o0.wall & wb) ? (long long)q * s.n + cell : (long long)opp(q) * s.n + src0;
-            const long long a1 =
-                (o1.wall & wb) ? (long long)q * s.n + cell + 1 : (long long)opp(q) * s.n + src1;
+            const PairIndex<S> a0 = (o0.wall & wb) ? q * n + cell : opp(q) * n + src0;
+            const PairIndex<S> a1 = (o1.wall & wb) ? q * n + (cell + 1) : opp(q) * n + src1;
             v[q] = make_float2((liq & 1u) ? Store<S>::ld_raw(f + a0) : 0.f,
                                (liq & 2u) ? Store<S>::ld_raw(f + a1) : 0.f);
             if (Store<S>::HREF) {
@@ -263,6 +272,7 @@ __device__ __forceinline__ void pair_finish(const Dev& s, S* f, int x, int row, 
         }
     } else {
         const NbrOffsets o0 = nbr_offsets(s, x, y, z), o1 = nbr_offsets(s, x + 1, y, z);
+        const PairIndex<S> n = (PairIndex<S>)s.n;
 #pragma unroll
         for (int q = 0; q < 27; ++q) {
             // target x + c_q beyond a wall face: the cell's own slot (opp(q), x)
@@ -276,12 +286,9 @@ __device__ __forceinline__ void pair_finish(const Dev& s, S* f, int x, int row, 
                 e.y -= (o1.wall & wb) ? ho : ht;
             }
             if (liq & 1u)
-                Store<S>::st_raw(
-                    f + ((o0.wall & wb) ? (long long)opp(q) * s.n + cell : (long long)q * s.n + dst0), e.x);
+                Store<S>::st_raw(f + ((o0.wall & wb) ? opp(q) * n + cell : q * n + dst0), e.x);
             if (liq & 2u)
-                Store<S>::st_raw(
-                    f + ((o1.wall & wb) ? (long long)opp(q) * s.n + cell + 1 : (long long)q * s.n + dst1),
-                    e.y);
+                Store<S>::st_raw(f + ((o1.wall & wb) ? opp(q) * n + (cell + 1) : q * n + dst1), e.y);
         }
     }
 }
@@ -1656,10 +1663,12 @@ static void launch_typed(const Dev& s, int parity, cudaStream_t st, cudaEvent_t 
         }
         if (early && links_done) cudaEventRecord(links_done, st);
         if (use_split(s)) {
-            if constexpr (sizeof(S) == 2) k_liquid_pair_warps<S, 1, 1><<<wblocks, 128, 0, st>>>(s);
-            const long long ne = (2LL * s.nz + 2LL * (s.ny > 2 ? s.ny - 2 : 0)) * (s.nx / 2) +
-                                 2LL * (s.ny > 2 ? s.ny - 2 : 0) * (s.nz > 2 ? s.nz - 2 : 0);
-            k_liquid_pair_edges<S><<<blocks_for(ne, 128), 128, 0, st>>>(s);
+            if constexpr (sizeof(S) == 2) {
+                k_liquid_pair_warps<S, 1, 1><<<wblocks, 128, 0, st>>>(s);
+                const long long ne = (2LL * s.nz + 2LL * (s.ny > 2 ? s.ny - 2 : 0)) * (s.nx / 2) +
+                                     2LL * (s.ny > 2 ? s.ny - 2 : 0) * (s.nz > 2 ? s.nz - 2 : 0);
+                k_liquid_pair_edges<S><<<blocks_for(ne, 128), 128, 0, st>>>(s);
+            }
         } else if (use_pairs(s)) {
             k_liquid_pair<S, 1><<<lgrid, 128, 0, st>>>(s);
         } else {
