@@ -630,8 +630,10 @@ __global__ void __launch_bounds__(128) k_dem_substep(Dev s, int a, int have_prev
 constexpr int DEM_CLUSTER_CTAS = 16;       // where the device can place a cluster of 16, else 8
 constexpr int DEM_CLUSTER_MAX = DEM_CLUSTER_CTAS * 1024 / DEM_LANES;
 
+// (not the .aligned forms, which a warp must execute together: the lane groups
+// of a warp come from loops of different lengths)
 __device__ __forceinline__ void cluster_barrier() {
-    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
 }
 __device__ __forceinline__ unsigned cluster_address(const void* p, unsigned rank) {
     unsigned r;
