@@ -6,6 +6,8 @@
 // cells it covers and uncovers. Particle state and forces are FP64; the map
 // test is evaluated in FP64 without fused multiply-add so that cell types do
 // not depend on contraction choices.
+#include <atomic>
+
 #include "fslbm_dev.cuh"
 
 namespace fsl {
@@ -1332,33 +1334,43 @@ int launch_dem_neighbours(const Dev& s, cudaStream_t st) {
 static size_t dem_cluster_smem(int threads) {
     return (size_t)(threads / DEM_LANES) * (sizeof(ClusterParticle) + DEM_SH * sizeof(float));
 }
-template <class K>
-static void dem_cluster_attributes(K* kernel, int smem) {
-    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+template <int THREADS>
+static void dem_cluster_attributes() {
+    cudaFuncSetAttribute(k_dem_cluster<THREADS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         (int)dem_cluster_smem(THREADS));
+    cudaFuncSetAttribute(k_dem_cluster<THREADS>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
 }
-// the largest cluster that this device places with 1024 threads a CTA, found
-// once (a cluster of 16 needs as many SMs of one group)
+// The largest cluster that this device places with 1024 threads a CTA (a
+// cluster of 16 needs as many SMs of one group), asked at a device's first use.
+// The kernels' attributes are set then too, for their largest blocks, and never
+// again: they belong to the function, and a run that lowered them to its own
+// size would have the launch of a larger run in another thread refused.
 static int dem_cluster_ctas() {
-    static const int ctas = [] {
-        cudaLaunchConfig_t cfg = {};
-        cudaLaunchAttribute at[1];
-        at[0].id = cudaLaunchAttributeClusterDimension;
-        at[0].val.clusterDim.x = DEM_CLUSTER_CTAS;
-        at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
-        cfg.gridDim = dim3(DEM_CLUSTER_CTAS);
-        cfg.blockDim = dim3(1024);
-        cfg.dynamicSmemBytes = dem_cluster_smem(1024);
-        cfg.attrs = at;
-        cfg.numAttrs = 1;
-        dem_cluster_attributes(k_dem_cluster<1024>, (int)cfg.dynamicSmemBytes);
-        int clusters = 0;
-        if (cudaOccupancyMaxActiveClusters(&clusters, k_dem_cluster<1024>, &cfg) != cudaSuccess) {
-            cudaGetLastError();
-            clusters = 0;
-        }
-        return clusters > 0 ? DEM_CLUSTER_CTAS : 8;
-    }();
+    constexpr int DEVICES = 64;
+    static std::atomic<int> known[DEVICES];   // 0: not asked yet
+    int dev = 0;
+    cudaGetDevice(&dev);
+    const int have = dev < DEVICES ? known[dev].load(std::memory_order_acquire) : 0;
+    if (have) return have;
+    dem_cluster_attributes<512>();
+    dem_cluster_attributes<1024>();
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = DEM_CLUSTER_CTAS;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.gridDim = dim3(DEM_CLUSTER_CTAS);
+    cfg.blockDim = dim3(1024);
+    cfg.dynamicSmemBytes = dem_cluster_smem(1024);
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    int clusters = 0;
+    if (cudaOccupancyMaxActiveClusters(&clusters, k_dem_cluster<1024>, &cfg) != cudaSuccess) {
+        cudaGetLastError();
+        clusters = 0;
+    }
+    const int ctas = clusters > 0 ? DEM_CLUSTER_CTAS : 8;
+    if (dev < DEVICES) known[dev].store(ctas, std::memory_order_release);
     return ctas;
 }
 
@@ -1389,9 +1401,7 @@ int launch_dem(const Dev& s, int have_prev, cudaStream_t st) {
         at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
         cfg.attrs = at;
         cfg.numAttrs = 1;
-        auto* kernel = threads <= 512 ? k_dem_cluster<512> : k_dem_cluster<1024>;
-        dem_cluster_attributes(kernel, (int)cfg.dynamicSmemBytes);
-        cudaLaunchKernelEx(&cfg, kernel, s, have_prev, G, dts);
+        cudaLaunchKernelEx(&cfg, threads <= 512 ? k_dem_cluster<512> : k_dem_cluster<1024>, s, have_prev, G, dts);
         return 1;
     }
     if (ns == 1) {
