@@ -967,7 +967,10 @@ __global__ void k_remap_all(Dev s) {
 
 // cells along one axis that a sphere of radius r at a or b can cover, with a
 // cell to spare on each side (the FP32 rounding of the coordinates, below 0.07
-// at 2^20 cells, stays within it)
+// at 2^20 cells, stays within it). On a periodic axis the range is not wrapped,
+// and where it is longer than the axis it is the L + 5 cells around b, which
+// hold the nearest image of every cell (and a few cells twice): offsets from b
+// taken along it are then those of the nearest image.
 __device__ __forceinline__ void bbox_axis(float a, float b, float r, int L, int periodic, int& lo, int& hi) {
     const float mn = fminf(a, b), mx = fmaxf(a, b);
     lo = (int)floorf(mn - r - 0.5f) - 1;
@@ -976,8 +979,9 @@ __device__ __forceinline__ void bbox_axis(float a, float b, float r, int L, int 
         lo = lo < 0 ? 0 : lo;
         hi = hi > L - 1 ? L - 1 : hi;
     } else if (hi - lo + 1 > L) {
-        lo = 0;
-        hi = L - 1;
+        const int c = (int)floorf(b);
+        lo = c - L / 2 - 2;
+        hi = c + (L + 1) / 2 + 2;
     }
 }
 
