@@ -872,6 +872,19 @@ __global__ void k_fixed_map(Dev s) {
     s.fixowner[c] = bestp;
 }
 
+// FP32 offset of cell centre k from the nearest image of a centre with integer
+// part i and fraction f. The real offset is wrapped: the integer difference
+// alone picks the farther image where it is half an even axis.
+__device__ __forceinline__ float cover_offset(int k, int i, float f, int L, int periodic) {
+    float e = (float)(k - i) + (0.5f - f);
+    if (periodic) {
+        const float h = 0.5f * (float)L;
+        if (e > h) e = (float)(k - i - L) + (0.5f - f);
+        else if (e < -h) e = (float)(k - i + L) + (0.5f - f);
+    }
+    return e;
+}
+
 // Calls f(p) for every mobile particle of the k-th grid cell of the ranges
 // that covers cell (x, y, z). |d^2 - r^2| is taken from the FP32 centre first
 // (rounded by up to 1e-4 cells at x = 3072), within its margin from the integer
@@ -902,9 +915,8 @@ __device__ __forceinline__ void for_covers(const Dev& s, int x, int y, int z, co
         if (m32 >= -tol) {
             const int4 xi = s.Xi[p];
             const float4 xf = s.Xfr[p];
-            const float ex = (float)wrap_int(x - xi.x, s.nx, s.per_x) + (0.5f - xf.x),
-                        ey = (float)wrap_int(y - xi.y, s.ny, s.per_y) + (0.5f - xf.y),
-                        ez = (float)wrap_int(z - xi.z, s.nz, s.per_z) + (0.5f - xf.z);
+            const float ex = cover_offset(x, xi.x, xf.x, s.nx, s.per_x), ey = cover_offset(y, xi.y, xf.y, s.ny, s.per_y),
+                        ez = cover_offset(z, xi.z, xf.z, s.nz, s.per_z);
             const float m2 = ex * ex + ey * ey + ez * ez - xr.w * xr.w;
             if (m2 > 1e-2f * tol) continue;
             if (m2 >= -1e-2f * tol) {

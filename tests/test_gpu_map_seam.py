@@ -62,3 +62,18 @@ def test_sphere_crossing_a_seam(shape, periodic, radius):
         assert _wrong(sim, shape, periodic, [radius]) == 0, k
         sim.step(3)
     assert np.sum(sim.get(F.FIELD_TYPE) == 3) > 20
+
+
+@pytest.mark.parametrize("L", [10, 11, 16])
+def test_sphere_that_nearly_spans_an_axis(L):
+    """radii up to half the axis, where a cell's nearest image is not that of
+    the integer parts' difference"""
+    rng = np.random.default_rng(L)
+    n = 14
+    shape, periodic = (n * (L + 2), L, 2 * L + 8), (1, 1, 0)
+    xyz = np.stack([(np.arange(n) + 0.5) * (L + 2), rng.uniform(0, L, n), L + 4 + rng.uniform(-1, 1, n)], 1)
+    radius = 0.5 * L - rng.uniform(0.01, 0.45, n)
+    sim = _sim(shape, periodic, (0.0, 3e-4, 0.0), xyz, radius)
+    for k in range(20):
+        assert _wrong(sim, shape, periodic, radius) == 0, k
+        sim.step(2)
