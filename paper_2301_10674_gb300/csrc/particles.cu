@@ -973,7 +973,8 @@ __device__ void remap_cell(const Dev& s, int c) {
 __global__ void k_remap_all(Dev s) {
     const long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (c >= s.n) return;
-    if ((int)((unsigned)c / ((unsigned)s.nx * (unsigned)s.ny)) > *s.zmax_cell) return;
+    // above every particle's top (z not periodic) nothing covers a cell
+    if (!s.per_z && (int)((unsigned)c / ((unsigned)s.nx * (unsigned)s.ny)) > *s.zmax_cell) return;
     remap_cell(s, (int)c);
 }
 

@@ -77,3 +77,14 @@ def test_sphere_that_nearly_spans_an_axis(L):
     for k in range(20):
         assert _wrong(sim, shape, periodic, radius) == 0, k
         sim.step(2)
+
+
+@pytest.mark.parametrize("fixed", [0, 1])
+@pytest.mark.parametrize("z", [0.7, 23.6])
+def test_sphere_across_the_z_seam_at_set_up(z, fixed):
+    """no other sphere reaches the cells on the far side"""
+    shape, periodic = (16, 16, 24), (1, 1, 1)
+    sim = _sim(shape, periodic, (0.0, 0.0, 1e-3), np.array([[8.2, 8.1, z]]), np.array([3.0]), np.array([fixed], np.uint8))
+    for k in range(10):
+        assert _wrong(sim, shape, periodic, [3.0]) == 0, k
+        sim.step(2)
