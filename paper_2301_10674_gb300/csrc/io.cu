@@ -1048,7 +1048,8 @@ __global__ void k_psd_peak(const double* psd, int nt, int nx, double* out) {
 
 // ------------------------------------------------------------ bed spectrum, factored
 // Series whose rows and columns fit shared memory (both extents up to
-// FFT_MAX) take mixed-radix transforms instead of the direct sums: FP64 runs
+// FFT_MAX) and have no prime factor that makes it the dearer way
+// (fft_cheaper) take mixed-radix transforms instead of the direct sums: FP64 runs
 // at 1/64 of the FP32 rate here, so the operation count is the bound
 // (500 x 3072 samples: 2.4e10 FP64 operations directly, 1.6e8 factored; the call
 // went from 24.7 ms to 0.42 ms, of which 0.11 ms are each of the two transforms;
@@ -1296,27 +1297,63 @@ __global__ void k_fft_peak(const double* peaks, int n, int nx, double* out) {
     }
 }
 
-static bool fft_fits(long long nt, long long nx) { return nt <= FFT_MAX && nx <= FFT_MAX; }
+// columns that a block of k_fft_t transforms at once: whole 64-byte segments
+// while two buffers of them fit twice on an SM, or as many as fit at all
+static int fft_cols(long long nt) {
+    int cols = 4;
+    while (cols > 1 && cols * nt > FFT_MAX) cols /= 2;
+    return cols;
+}
+
+// Whether the factored transforms take less time than the direct sums, both
+// bound by the FP64 pipes: operations per block times the blocks that follow
+// one another on an SM. A prime factor p costs p complex products per value,
+// in one block per two rows (or `cols` columns), where the direct sums spread
+// any extent over nt nx / 256 blocks. Counted per value: 4 p operations for a
+// prime p > 5; 7, 4, 7 and 11 for radix 4, 2, 3 and 5 with their twiddles; 2 per
+// product of the direct sums along x, 6 along t (four operations that wait for
+// their loads); 2.5 per sample for the direct way's mean and peak, each one
+// block. Measured (factored / direct, ms): 20 x 3499 12.3 / 1.16, 100 x 3461
+// 12.1 / 5.1, 300 x 3461 12.1 / 16.3, 691 x 200 2.14 / 1.68, 691 x 400 2.16 / 3.10,
+// 7159 x 20 50.4 / 20.1, 7159 x 200 50.5 / 128, 40 x 5996 9.1 / 5.7, 40 x 6416 2.8 / 6.1,
+// 97 x 97 0.287 / 0.264, 500 x 3072 0.44 / 24.7; the rule takes the faster at each.
+static bool fft_cheaper(long long nt, long long nx) {
+    auto per_value = [](int n) {
+        const Radices f = factor(n);
+        double c = 0.0;
+        for (int i = 0; i < f.n; ++i) {
+            const int r = f.r[i];
+            c += r == 2 ? 4.0 : (r == 3 || r == 4 ? 7.0 : (r == 5 ? 11.0 : 4.0 * r));
+        }
+        return c;
+    };
+    auto waves = [](long long blocks) { return (double)((blocks + 151) / 152); };
+    const long long cols = fft_cols(nt), passes = (nx / 2 + cols) / cols;   // ceil(hx / cols)
+    const double factored = waves((nt + 1) / 2) * (double)nx * per_value((int)nx) +
+                            waves(passes) * (double)(cols * nt) * per_value((int)nt);
+    const double threads = nx < 256 ? (double)((nx + 31) / 32 * 32) : 256.0;
+    const double direct = waves(nt * ((nx + 255) / 256)) * threads * (2.0 * (double)nx + 6.0 * (double)nt) +
+                          2.5 * (double)nt * (double)nx;
+    return factored <= direct;
+}
+static bool use_fft(long long nt, long long nx) { return nt <= FFT_MAX && nx <= FFT_MAX && fft_cheaper(nt, nx); }
 
 // doubles of device scratch of launch_bed_spectrum
 size_t bed_spectrum_work(long long nt, long long nx) {
     const size_t tw = 2 * ((size_t)nx + nt);
-    if (fft_fits(nt, nx)) return tw + 2 * (size_t)nt * (nx / 2 + 1) + FFT_SUMS + 2 * FFT_BLOCKS + 3;
+    if (use_fft(nt, nx)) return tw + 2 * (size_t)nt * (nx / 2 + 1) + FFT_SUMS + 2 * FFT_BLOCKS + 3;
     return tw + 2 * (size_t)nt * nx + 4;
 }
 
 int launch_bed_spectrum(const double* h, int nt, int nx, double* psd, double* work, double* peak3, cudaStream_t st) {
-    if (fft_fits(nt, nx)) {
+    if (use_fft(nt, nx)) {
         // twiddles, the half-spectrum rows, partial sums and peaks
         double2* twx = reinterpret_cast<double2*>(work);
         double2* twt = twx + nx;
         double2* X1 = twt + nt;
         double* sums = reinterpret_cast<double*>(X1 + (size_t)nt * (nx / 2 + 1));
         double* peaks = sums + FFT_SUMS;
-        // columns per block pass: whole 64-byte segments while two buffers of
-        // them fit twice on an SM, or as many as fit at all
-        int cols = 4;
-        while (cols > 1 && cols * nt > FFT_MAX) cols /= 2;
+        const int cols = fft_cols(nt);
         const int hx = nx / 2 + 1;
         const int blocks = std::min(FFT_BLOCKS, (hx + cols - 1) / cols);
         const int smx = 2 * nx * (int)sizeof(double2), smt = 2 * cols * nt * (int)sizeof(double2);
