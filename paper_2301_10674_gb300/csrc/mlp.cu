@@ -577,11 +577,11 @@ __global__ void __launch_bounds__(1024) k_mlp_train_update(UpdateArgs a) {
         else if (which == 2) i = OFF_W2 + row * MLP_H + col;
         else if (row < MLP_OUT) i = OFF_W3 + row * MLP_H + col;
     }
-    allow_next();
-    // the previous update is complete: the launch before this one waited for it
+    // (the update before is complete when the launch in between has waited for
+    // it, but only this grid's own wait makes its writes visible here)
+    after_previous();
     const bool adam = i >= 0 && i < MLP_NPARAM && a.last && !a.grad;
     const float th = adam ? a.theta[i] : 0.f, mo = adam ? a.m[i] : 0.f, vo = adam ? a.v[i] : 0.f;
-    wait_previous();
     float s = i >= 0 && !a.first ? a.acc[i] : 0.f;
     for (int c0 = 0; c0 < a.chunks; c0 += 32) {
         const int nc = a.chunks - c0 < 32 ? a.chunks - c0 : 32;
