@@ -7,6 +7,9 @@
 #include <new>
 #include <vector>
 
+#include <cuda.h>
+
+#include "buffer_check.h"
 #include "fslbm_dev.cuh"
 #include "mlp_dev.cuh"
 
@@ -137,24 +140,38 @@ int launch_check(fslbm* s) {
 }
 
 // Whether a kernel may access [p, p + bytes) of a caller's buffer directly:
-// aligned, and its first and last byte both device memory of the current
-// device. Anything else (another device's memory, host memory passed as
-// device memory, a range that leaves its allocation) keeps the staged copy,
-// which validates it.
+// aligned and inside one allocation of device memory of the current device.
+// Anything else (another device's memory, host memory passed as device
+// memory, a range that leaves its allocation, a range over several mappings)
+// keeps the staged copy, which validates it.
 bool kernel_writable(const void* p, size_t bytes, size_t align) {
-    if (reinterpret_cast<uintptr_t>(p) % align) return false;
+    using Range = CUresult (*)(CUdeviceptr*, size_t*, CUdeviceptr);
+    static const Range range = [] {
+        void* f = nullptr;
+        cudaDriverEntryPointQueryResult found;
+        if (cudaGetDriverEntryPointByVersion("cuMemGetAddressRange", &f, 12000, cudaEnableDefault, &found) != cudaSuccess ||
+            found != cudaDriverEntryPointSuccess) {
+            cudaGetLastError();
+            f = nullptr;
+        }
+        return reinterpret_cast<Range>(f);
+    }();
     int dev = -1;
-    if (cudaGetDevice(&dev) != cudaSuccess) return false;
-    const char* ends[2] = {static_cast<const char*>(p), static_cast<const char*>(p) + bytes - 1};
-    for (const char* e : ends) {
-        cudaPointerAttributes a;
-        if (cudaPointerGetAttributes(&a, e) != cudaSuccess) {
+    if (!range || cudaGetDevice(&dev) != cudaSuccess) return false;
+    return kernel_may_access(p, bytes, align, dev, [&](const void* q, BufferInfo& b) {
+        cudaPointerAttributes at;
+        if (cudaPointerGetAttributes(&at, q) != cudaSuccess) {
             cudaGetLastError();
             return false;
         }
-        if (a.type != cudaMemoryTypeDevice || a.device != dev) return false;
-    }
-    return true;
+        b.device_memory = at.type == cudaMemoryTypeDevice;
+        b.device = at.device;
+        if (!b.device_memory) return true;
+        CUdeviceptr base = 0;
+        if (range(&base, &b.size, reinterpret_cast<CUdeviceptr>(q)) != CUDA_SUCCESS) return false;
+        b.base = static_cast<std::uintptr_t>(base);
+        return true;
+    });
 }
 
 cudaMemcpyKind kind_to(int on_device) { return on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost; }
