@@ -177,9 +177,10 @@ __global__ void __launch_bounds__(GEN_THREADS) k_make_stencils(const double* __r
         // change of g = w - A sin(k u + phase) + A sin(phase) within a cell,
         // row or run, at most: the gradient at the point tested times the
         // extent plus half the largest second derivative A k^2 along u, and
-        // the rounding of an evaluation
+        // the rounding of an evaluation, with that of two arguments of the
+        // sine, each up to 6e-8 of the phase
         const float Ak = Af * kf, h2 = 0.5f * fabsf(Ak * kf);
-        const float tol = 1e-4f * (1.f + fabsf(Af));
+        const float tol = 1e-4f * (1.f + fabsf(Af)) + 1.5e-7f * fabsf(Af * pf);
         const float ec = 0.5f * (fabsf(fe[0]) + fabsf(fe[1]) + fabsf(fe[2])), er = 0.5f * fe[0], es = 0.25f * fe[0];
         const float cell_add = tol + h2 * ec * ec, row_add = tol + h2 * er * er, run_add = tol + h2 * es * es;
         for (int q = 0; q < 27; ++q) {
