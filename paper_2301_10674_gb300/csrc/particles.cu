@@ -142,13 +142,17 @@ __device__ __forceinline__ GRange grange(int k0, int k1, int g, int periodic) {
 }
 
 // ------------------------------------------------------------ DEM
-// minimal image of an integer displacement along a periodic axis
-__device__ __forceinline__ int wrap_int(int d, int L, int periodic) {
+// FP32 displacement d + f (integer and fraction parts) of the nearest image
+// along a periodic axis (|d| <= L). The real displacement is wrapped: the
+// integer part alone picks the farther image where it is half an even axis.
+__device__ __forceinline__ float image_offset(int d, float f, int L, int periodic) {
+    float e = (float)d + f;
     if (periodic) {
-        if (d > L / 2) d -= L;
-        else if (d < -L / 2) d += L;
+        const float h = 0.5f * (float)L;
+        if (e > h) e = (float)(d - L) + f;
+        else if (e < -h) e = (float)(d + L) + f;
     }
-    return d;
+    return e;
 }
 
 // minimal image of a displacement along a periodic axis (|d| < 1.5 L)
@@ -314,9 +318,9 @@ __global__ void k_dem_neighbours(Dev s) {
         const float4 fj = s.Xfr[nj];
         s.nb[(long long)p * NB_SLOTS + lane] = nj;
         s.nb_d0[(long long)p * NB_SLOTS + lane] =
-            make_float4((float)wrap_int(ij.x - ip.x, s.nx, s.per_x) + (fj.x - fp.x),
-                        (float)wrap_int(ij.y - ip.y, s.ny, s.per_y) + (fj.y - fp.y),
-                        (float)wrap_int(ij.z - ip.z, s.nz, s.per_z) + (fj.z - fp.z), cj.x);
+            make_float4(image_offset(ij.x - ip.x, fj.x - fp.x, s.nx, s.per_x),
+                        image_offset(ij.y - ip.y, fj.y - fp.y, s.ny, s.per_y),
+                        image_offset(ij.z - ip.z, fj.z - fp.z, s.nz, s.per_z), cj.x);
         xi.w = cp.y * cj.y / (cp.y + cj.y);
         s.nb_xi[row + lane] = xi;
     }
@@ -872,19 +876,6 @@ __global__ void k_fixed_map(Dev s) {
     s.fixowner[c] = bestp;
 }
 
-// FP32 offset of cell centre k from the nearest image of a centre with integer
-// part i and fraction f. The real offset is wrapped: the integer difference
-// alone picks the farther image where it is half an even axis.
-__device__ __forceinline__ float cover_offset(int k, int i, float f, int L, int periodic) {
-    float e = (float)(k - i) + (0.5f - f);
-    if (periodic) {
-        const float h = 0.5f * (float)L;
-        if (e > h) e = (float)(k - i - L) + (0.5f - f);
-        else if (e < -h) e = (float)(k - i + L) + (0.5f - f);
-    }
-    return e;
-}
-
 // Calls f(p) for every mobile particle of the k-th grid cell of the ranges
 // that covers cell (x, y, z). |d^2 - r^2| is taken from the FP32 centre first
 // (rounded by up to 1e-4 cells at x = 3072), within its margin from the integer
@@ -915,8 +906,9 @@ __device__ __forceinline__ void for_covers(const Dev& s, int x, int y, int z, co
         if (m32 >= -tol) {
             const int4 xi = s.Xi[p];
             const float4 xf = s.Xfr[p];
-            const float ex = cover_offset(x, xi.x, xf.x, s.nx, s.per_x), ey = cover_offset(y, xi.y, xf.y, s.ny, s.per_y),
-                        ez = cover_offset(z, xi.z, xf.z, s.nz, s.per_z);
+            const float ex = image_offset(x - xi.x, 0.5f - xf.x, s.nx, s.per_x),
+                        ey = image_offset(y - xi.y, 0.5f - xf.y, s.ny, s.per_y),
+                        ez = image_offset(z - xi.z, 0.5f - xf.z, s.nz, s.per_z);
             const float m2 = ex * ex + ey * ey + ez * ez - xr.w * xr.w;
             if (m2 > 1e-2f * tol) continue;
             if (m2 >= -1e-2f * tol) {
