@@ -188,8 +188,8 @@ COMPARE_FORMS = (("fp32", "fd"), ("fp16", "fd"), ("bf16", "fd"), ("fp32", "mlp")
 # even and odd steps averaged, from one ncu capture on the 1024x64x128 flume.
 # It is valid while the sweep's sources hash to `sources`, and is scaled to a
 # run by its fluid cells.
-SWEEP_TRAFFIC = {"sources": "6c065cbb4f1e0bb9", "workload": "precision-1024x64x128",
-                 "per_fluid_cell": {"fp16": 192.3, "fp32": 377.8, "bf16": 192.5}}
+SWEEP_TRAFFIC = {"sources": "d16f940ba01f3cc2", "workload": "precision-1024x64x128",
+                 "per_fluid_cell": {"fp16": 192.3, "fp32": 377.9, "bf16": 192.4}}
 SWEEP_SOURCES = ("paper_2301_10674_gb300/csrc/stream_collide.cu", "paper_2301_10674_gb300/csrc/fslbm_dev.cuh",
                  "paper_2301_10674_gb300/csrc/collide_pair.cuh")
 

@@ -174,7 +174,6 @@ struct Dev {
     int mlp_mirror;
     int* shared;
     uint8_t* dirty;
-    uint8_t* scratch_a; uint8_t* scratch_b;     // byte fields for the neighbourhood OR
     int* dl; int* dl_count; int dl_cap;
     // static map of the fixed particles
     unsigned long long* fixkey;
@@ -228,12 +227,7 @@ __device__ __forceinline__ float slot_ref(const Dev& s, long long i) {
     const long long c = i - (long long)q * s.n;
     return wq(q) * s.href[(int)(c / ((long long)s.nx * s.ny))];
 }
-// f - w at PDF slot i, in any storage format
-__device__ __forceinline__ float ld_any(const Dev& s, const void* base, long long i) {
-    if (s.storage == FSLBM_STORE_FP32) return static_cast<const float*>(base)[i];
-    if (s.storage == FSLBM_STORE_FP16) return Store<__half>::ld(static_cast<const __half*>(base) + i) + slot_ref(s, i);
-    return __bfloat162float(static_cast<const __nv_bfloat16*>(base)[i]) + slot_ref(s, i);
-}
+// stores f - w at PDF slot i, in any storage format
 __device__ __forceinline__ void st_any(const Dev& s, void* base, long long i, float v) {
     if (s.storage == FSLBM_STORE_FP32) static_cast<float*>(base)[i] = v;
     else if (s.storage == FSLBM_STORE_FP16) Store<__half>::st(static_cast<__half*>(base) + i, v - slot_ref(s, i));
@@ -575,14 +569,8 @@ __device__ __forceinline__ void warp_append(const Dev& s, bool pred, int v, int*
     }
 }
 
-// post-collision PDFs of a cell read from the AA layout (outside the
+// post-collision PDFs of a cell written to the AA layout (outside the
 // stream-collide kernel, where no slot is being rewritten)
-__device__ __forceinline__ void load_fstar(const Dev& s, long long cell, int last_parity, float (&f)[27]) {
-    int x, y, z;
-    coords(s, cell, x, y, z);
-#pragma unroll
-    for (int q = 0; q < 27; ++q) f[q] = ld_any(s, s.f, fstar_slot(s, q, x, y, z, cell, last_parity));
-}
 __device__ __forceinline__ void store_fstar(const Dev& s, long long cell, int last_parity, const float (&f)[27]) {
     int x, y, z;
     coords(s, cell, x, y, z);
@@ -599,8 +587,8 @@ __device__ __forceinline__ long long pdf_slot(const Dev& s, int q, long long c, 
     return own ? (long long)opp(q) * s.n + c
                : (long long)q * s.n + c + (o.ox[1 + cx(q)] + o.oy[1 + cy(q)] + o.oz[1 + cz(q)]);
 }
-// f - w from a stored value and its slot's reference (the rounding of ld_any
-// and, with -h, of st_any: product, then sum)
+// f - w from a stored value and its slot's reference (and the other
+// way with -h, with the rounding of st_any: product, then sum)
 template <typename S>
 __device__ __forceinline__ float with_ref(float v, int q, float h) {
     return Store<S>::HREF ? __fadd_rn(v, __fmul_rn(wq(q), h)) : v;

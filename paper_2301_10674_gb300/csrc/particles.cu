@@ -821,10 +821,8 @@ __device__ __forceinline__ GRange cover_range(int k, double r_max, double h, int
 }
 
 // best covering particle (lowest metric, then lowest index) among the
-// particles of the selected kind near cell (x, y, z); every covering mobile
-// particle of a cell covered more than once is flagged as sharing cells
-__device__ void best_cover(const Dev& s, int x, int y, int z, int want_fixed, double& best, int& bestp,
-                           int* ncover = nullptr, int* cov = nullptr) {
+// particles of the selected kind near cell (x, y, z)
+__device__ void best_cover(const Dev& s, int x, int y, int z, int want_fixed, double& best, int& bestp) {
     const double xc = x + 0.5, yc = y + 0.5, zc = z + 0.5;
     const GRange ra = cover_range(x, s.r_max, s.ghx, s.gnx, s.per_x);
     const GRange rb = cover_range(y, s.r_max, s.ghy, s.gny, s.per_y);
@@ -851,10 +849,6 @@ __device__ void best_cover(const Dev& s, int x, int y, int z, int want_fixed, do
                     double m = map_metric(image_centre(x, Xp[0], s.nx, s.per_x), image_centre(y, Xp[1], s.ny, s.per_y),
                                           image_centre(z, Xp[2], s.nz, s.per_z), Xp, r);
                     if (m > 0.0) continue;
-                    if (ncover) {
-                        if (*ncover < 4) cov[*ncover] = p;
-                        (*ncover)++;
-                    }
                     if (m < best || (m == best && p < bestp)) {
                         best = m;
                         bestp = p;

@@ -884,9 +884,10 @@ __global__ void __launch_bounds__(256, 3) k_solid_links(Dev s) {
 // the kernel above waits for three in turn. For 16-bit storage (rows of 32
 // cells, 32-bit indices), where the pass is bound by latency: the sweep of the
 // 3072x96x320 flume at FP16 went from 3.39 to 3.06 ms, of 1024x64x128 from 0.349
-// to 0.315 ms. At FP32 the pass moves its 9 GB at the HBM rate either way
-// (sweep 4.00 ms with the kernel above, 4.02 to 4.08 ms with this one), so it
-// stays with the flag bytes and saves the words.
+// to 0.315 ms. At FP32 the pass is short of the HBM rate too (3.6 to 3.8 TB/s of
+// 6.7), but this form gained nothing there (sweep of the large flume 4.00 ms
+// with the kernel above, 4.02 to 4.08 ms with this one), so it stays with the
+// flag bytes and saves the words.
 // bit of direction q in the per-plane masks: 2 (c_x + 1) + 6 (c_y + 1) of plane c_z + 1
 __device__ __forceinline__ bool fluid_bit(const unsigned (&m)[3], int q) {
     return (m[cz(q) + 1] >> (2 * (cx(q) + 1) + 6 * (cy(q) + 1))) & 1u;
